@@ -122,7 +122,9 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     float *Cc = kind == kKindFactored ? after_m + n : nullptr;
 
     // ---- tile geometry and item counts (the planner's, plan_geometry) ---------------
-    const bool wg_aligned = !f32 && (((uintptr_t)weight | (uintptr_t)grad) & 15) == 0;  // row tiles: bf16 only
+    // row tiles: bf16 only, and every array that they bulk-copy (the momentum too: the caller's
+    // state is only 4-byte aligned) starts on a 16-byte boundary
+    const bool wg_aligned = !f32 && (((uintptr_t)weight | (uintptr_t)grad | (uintptr_t)M) & 15) == 0;
     const int64_t tiles64 = kind == kKindFactored ? ((m + 255) / 256) * ((n + 255) / 256)
                                                   : (numel + kFlatTileElems - 1) / kFlatTileElems;
     if (tiles64 > (int64_t(1) << 31)) return SKEW_EINVAL;
