@@ -35,7 +35,7 @@ struct TPlan {
     int64_t n = 0, m = 0, numel = 0;
     int64_t moff = -1, voff = -1, roff = -1, coff = -1;  // floats into the state
     uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0;
-    uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0, at_rows = 0, atiles = 0, fci = 0;
+    uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0, at_rows = 0, atiles = 0, fci = 0, nu2 = 0;
     uint32_t f32 = 0;         // SKEW_F_FP32: fp32 weights and gradient
     // bytes into the workspace
     size_t ws_rowp = 0, ws_colp = 0, ws_bsc = 0, ws_rsum = 0, ws_u2 = 0, ws_pp = 0, ws_rmin = 0, ws_fsum = 0, ws_fmin = 0;
@@ -118,6 +118,7 @@ static void geometry(TPlan &p, bool wg_aligned) {
     p.at_rows = g.at_rows;
     p.atiles = g.atiles;
     p.fci = g.fci;
+    p.nu2 = u2_len(g);
 }
 
 extern "C" {
@@ -286,7 +287,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             p.ws_fmin = w; w = align_up(w + 4 * size_t(p.nfc), 256);
         }
         p.ws_u2 = w;
-        w = align_up(w + 8 * size_t(p.ntiles), 256);
+        w = align_up(w + 8 * size_t(p.nu2), 256);
     }
     h->ws_bytes = w;
     *out = h;

@@ -159,7 +159,7 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
         o_fsum = off; off = align256(off + 8 * size_t(G.nfc));
         o_fmin = off; off = align256(off + 4 * size_t(G.nfc));
     }
-    const size_t o_u2 = off;     off = align256(off + 8 * size_t(G.ntiles));
+    const size_t o_u2 = off;     off = align256(off + 8 * size_t(u2_len(G)));
     if (off > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
 
     // ---- device address of the fixed array on the current device ---------------------

@@ -144,6 +144,14 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
     return g;
 }
 
+// Entries of a tensor's sums of U^2.
+inline uint32_t u2_len(const TileGeom &g) {
+    return g.rowpath && 2 * g.atiles > g.ntiles ? 2 * g.atiles : g.ntiles;
+}
+
+// Where a row-path tensor whose clamp may bind gets its sum(U^2): phase B, or phase C (clip factor 1).
+enum SumWhere : uint32_t { kPhaseB = 1, kSumInC = 2 };
+
 // Device descriptor of one tensor (lives in the workspace).
 struct TensorDev {
     uint16_t *w;        // bf16 weights, n*m, row-major (borrowed)
@@ -156,11 +164,13 @@ struct TensorDev {
     float *colp;        // strip path: column partials of g^2 [rowtiles][m]
     float *bsc;         // factored: 1/sqrt(C_j) [m]
     double *rsum;       // factored: sums of R per finalize-row item [nfr] / per row tile [rtiles]
-    float2 *pp;         // row path: per row tile and column, (sum of g^2, sum of g^2 / R_i) [rtiles][m]
+    float2 *pp;         // row path: per row tile and column, (sum of g^2, sum of g^2 / R_i) [rtiles][m];
+                        // then an item's sum of g^2 in the first entry of its columns
     float *rmin;        // row path: smallest positive R_i per row tile [rtiles]
     double *fsum;       // row path: sum of P_j / C_j per finalize item [nfc]
     float *fmin;        // row path: smallest C_j with P_j > 0 per finalize item [nfc]
-    float2 *u2;         // per tile sum of (U / coef)^2 as a (hi, lo) pair [ntiles]
+    float2 *u2;         // sums of (U / coef)^2 as (hi, lo) pairs: per phase-B tile [ntiles], or on the
+                        // row path per half of a phase-C tile [2 atiles] (u2_len)
     int64_t n, m, numel;
     uint32_t tid;       // dither tensor id
     uint64_t base;      // dither index of element 0 (a matrix of a stacked tensor: its offset)
@@ -193,7 +203,7 @@ struct TensorScal {
     float coefC;        // lr * kappa * coef, the factor applied to (y / D)
     uint32_t cntF;      // finalize items done
     uint32_t cntB;      // update-RMS tiles done
-    uint32_t fallback;  // row path: 1 if sum(U^2) needs phase B (a clamp may bind)
+    uint32_t fallback;  // row path, when a clamp may bind: SumWhere of sum(U^2); else 0
     uint32_t zflag;     // row path: a row with R_i == 0 holds a nonzero gradient
     uint32_t pad;
 };

@@ -1,0 +1,35 @@
+"""Row-path tensors whose eps clamp binds (eps = 1e-8, App. A), on both routes to sum(U^2): summed in
+phase C where a bound proves that the update is not clipped (d = 1), and by phase B where it may be
+(d = 0.05). Weights, state and the scalars (sum(U^2), RMS, clip factor) against the oracle; whole and
+half phase-C tiles, last tiles without a second half, one-row matrices, stacks, zero-gradient experts."""
+import pytest
+
+from paper_2607_19058_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+E, B = WL.TIER_EXPERT, WL.TIER_BACKBONE
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2607_19058_gb300 import _build
+    _build.build()
+    import oracle
+    oracle.build()
+
+
+@pytest.mark.parametrize("clip_d", [1.0, 0.05])
+def test_clamped_tensors(clip_d):
+    import parity
+    specs = [WL.Spec("e301x4096", (301, 4096), E, expert=0), WL.Spec("b301x4096", (301, 4096), B),
+             WL.Spec("e1x4096", (1, 4096), E, expert=1), WL.Spec("b2101x512", (2101, 512), B),
+             WL.Spec("e2049x1024", (2049, 1024), E, expert=5), WL.Spec("s3x70x2048", (3, 70, 2048), E),
+             WL.Spec("e2300x4096", (2300, 4096), E, expert=6)]
+    h = parity.Harness(WL.Workload("clamp", specs, WL.HP(), "toy", steps=3),
+                       hp_override=dict(eps=1e-8, lr=3e-4, weight_decay=0.05, clip_d=clip_d))
+    for t in range(1, 4):
+        rep = h.step(t, seed=5 * t, **({"gscale": 0.37} if t == 2 else {}))
+        assert (rep.clipped > 0) == (clip_d < 1.0)
+    h.opt.sync_status()
+    h.close()
