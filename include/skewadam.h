@@ -149,8 +149,8 @@ typedef struct {
     int32_t vectorized; /* 1 if the 16-byte vector path serves it (after bind) */
     int64_t rows, cols, numel;
     int64_t m_offset, v_offset, r_offset, c_offset;
-    int32_t rowpath;    /* 1 if phase A runs on whole rows and sum(U^2) needs no  */
-                        /* second pass over G unless a clamp may bind (bilinear) */
+    int32_t rowpath;    /* 1 at the widths 512, 1024, 2048 and 4096 (bf16, 16-byte */
+                        /* aligned), whose phase A always runs on whole rows       */
     int32_t stack;      /* matrices of a stacked tensor (ndim 3), else 0; then   */
                         /* rows / cols are one matrix's, numel the whole stack's, */
                         /* and each state array holds the E matrices' in order   */
@@ -307,7 +307,8 @@ const char *skew_kernel_name(int32_t k);
  * fed to the dither (use the tensor's index in a skew_create list to get the
  * same bits as skew_step); step, lr, seed as for skew_step; stream: a
  * cudaStream_t. Updates weight and state in place, asynchronously on stream,
- * with the same kernels and results as skew_step on a one-tensor handle.
+ * with the same kernels and results as skew_step on a one-tensor handle (up to
+ * summation order at the few sizes whose row tiles must be larger to fit the scratch).
  *
  * Every call looks up the array's device address on the current device with
  * cudaGetSymbolAddress. The first such lookup on a device may load the

@@ -102,8 +102,8 @@ static void resolve(int ndim, int tier, int policy, uint32_t flags, TPlan &p) {
 
 // Tile geometry (plan_geometry): strip tiles of (tile_rows rows) x (8*LC
 // columns) or flat tiles of kFlatTileElems elements, and for the row path whole-row tiles.
-static void geometry(TPlan &p, bool wg_aligned) {
-    const TileGeom g = plan_geometry(p.kind, p.momentum, wg_aligned, p.n, p.m, p.numel);
+static void geometry(TPlan &p, bool row_aligned, int64_t rest) {
+    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, p.n, p.m, p.numel, rest);
     p.lcl = g.lcl;
     p.strips = g.strips;
     p.rowtiles = g.rowtiles;
@@ -150,6 +150,9 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         return fail(nullptr, SKEW_ENOMEM, "out of host memory");
     }
     const int64_t kMaxExtent = int64_t(1) << 40;
+    // whole-row tiles are for bf16 rows on 16-byte boundaries
+    auto row_aligned = [](const TPlan &q) { return !q.f32 && (((uintptr_t)q.w | (uintptr_t)q.g) & 15) == 0; };
+    int64_t any_bytes = 0;  // bytes of G of the matrices that only kRowAny's whole-row tiles serve
     for (int32_t k = 0; k < n_params; ++k) {
         const skew_param_desc_t &d = params[k];
         TPlan p;
@@ -182,15 +185,27 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.tid = (uint32_t)k;
                 q.base = (uint64_t)(e * p.numel);
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
-                // whole-row tiles and 16-byte vectors are for bf16 rows
-                geometry(q, !q.f32 && (((uintptr_t)q.w | (uintptr_t)q.g) & 15) == 0);
-                h->n_rowpath += q.rowpath;
+                geometry(q, row_aligned(q), kWholeGroup);
+                if (q.rowpath == kRowAny) any_bytes += 2 * q.numel;
                 h->t.push_back(q);
             }
         } catch (...) {
             delete h;
             return fail(nullptr, SKEW_ENOMEM, "out of host memory");
         }
+    }
+    const bool any = any_bytes >= kAnyGroupBytes;
+    int64_t rest = 0;
+    for (size_t k = h->t.size(); k-- > 0;) {  // row tiles by the bytes that follow, from the last matrix back
+        TPlan &q = h->t[k];
+        if (q.rowpath == kRowNone) continue;
+        if (q.rowpath == kRowAny && !any) {
+            geometry(q, false, kWholeGroup);
+            continue;
+        }
+        rest += 2 * q.numel;
+        geometry(q, true, rest);
+        ++h->n_rowpath;
     }
     const int32_t n_plans = (int32_t)h->t.size();
 
@@ -229,13 +244,14 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 for (uint32_t i = 0; i < p.ntiles; ++i) h->itemsC.push_back(make_uint2(q, i));
             }
         }
-        // the last phase-C row tiles of momentum-free matrices run as two half tiles each
-        // (tiles of momentum matrices and tile indices past the mask keep whole tiles)
+        // the last phase-C row tiles run as two half tiles each (small tiles and tile indices past
+        // the mask keep whole tiles)
         std::vector<uint2> tail;
         const size_t ncr = h->itemsCR.size(), nsplit = std::min<size_t>(ncr, kApplyTailSplit);
         for (size_t k = ncr - nsplit; k < ncr; ++k) {
             const uint2 it = h->itemsCR[k];
-            if (!h->t[it.x].momentum && it.y <= kTileMask) {
+            const TPlan &p = h->t[it.x];
+            if (2 * p.m * p.at_rows >= kSplitTileBytes && it.y <= kTileMask) {
                 tail.push_back(make_uint2(it.x, it.y | kHalfTile));
                 tail.push_back(make_uint2(it.x, it.y | kHalfTile | kSecondHalf));
             } else {
@@ -329,7 +345,7 @@ int skew_tensor_info(const skew_handle_t *h, int32_t tid, skew_tensor_info_t *ou
     out->v_offset = p.voff;
     out->r_offset = p.roff;
     out->c_offset = p.coff;
-    out->rowpath = (int32_t)p.rowpath;
+    out->rowpath = p.rowpath == kRowFixed;
     out->stack = h->desc[tid].ndim == 3 ? (int32_t)h->count[tid] : 0;
     return SKEW_OK;
 }
@@ -377,6 +393,8 @@ int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace
         T.n = p.n;
         T.m = p.m;
         T.numel = p.numel;
+        T.inv_n = 1.0 / (double)p.n;
+        T.inv_numel = 1.0 / (double)p.numel;
         T.tid = p.tid;
         T.base = p.base;
         T.kind = p.kind;

@@ -30,6 +30,7 @@
 // tiles), phase C takes a clamp-free path. Every wait on a bulk copy is bounded
 // and reports a copy that does not land through the status word.
 #include <cuda_runtime.h>
+#include <cstddef>
 #include <type_traits>
 #include <stdint.h>
 
@@ -342,7 +343,7 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t *p, uint32_t v) {
 struct Smem {
     float colred[kThreads * 8];  // column partials of a sum-of-squares tile
     float2 red2[kThreads / 32];
-    double redd[kThreads / 32];
+    double redd[3 * (kThreads / 32)];
     int last;
 };
 
@@ -922,14 +923,14 @@ template <typename V>
 __device__ __forceinline__ V strided_sum(const V *p, int64_t stride, uint32_t cnt) {
     V s = V(0);
     uint32_t r = 0;
-    for (; r + 8 <= cnt; r += 8) {
+    for (; r < cnt; r += 8) {
         V v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = __ldcg(p + int64_t(r + q) * stride);
+        for (int q = 0; q < 8; ++q) v[q] = r + q < cnt ? __ldcg(p + int64_t(r + q) * stride) : V(0);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) s += v[q];
+        for (int q = 0; q < 8; ++q)
+            if (r + q < cnt) s += v[q];
     }
-    for (; r < cnt; ++r) s += __ldcg(p + int64_t(r) * stride);
     return s;
 }
 
@@ -957,8 +958,9 @@ __device__ __forceinline__ double update_coef(const StepArgs &A, const TensorDev
 __device__ void set_clip(const StepArgs &A, const TensorDev &T, TensorScal &S, double s) {
     const double coef = update_coef(A, T);
     const double su2 = s * coef * coef;
-    const double rms = sqrt(su2 / (double)T.numel);
-    const double kappa = 1.0 / fmax(1.0, rms / (double)A.clip_d);
+    const double rms = sqrt(su2 * T.inv_numel);
+    const double d = (double)A.clip_d;
+    const double kappa = rms > d ? d / rms : 1.0;  // a NaN RMS clips nothing, as fmax(1, NaN) = 1
     S.sumsq = su2;
     S.rms = rms;
     S.kappa = kappa;
@@ -988,7 +990,7 @@ __device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem 
     if (j < T.m) {
         const float2 *p = T.pp + j;
         uint32_t r = sl;
-        // loads issued 32 (then 16) at a time ahead of the adds, which go in tile order
+        // loads issued 32 at a time ahead of the adds, which go in tile order
         for (; r + 31 * tpc < T.rtiles; r += 32 * tpc) {
             float2 v[32];
 #pragma unroll
@@ -999,20 +1001,18 @@ __device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem 
                 pa.add(v[q].y);
             }
         }
-        for (; r + 15 * tpc < T.rtiles; r += 16 * tpc) {
-            float2 v[16];
+        // the rest eight at a time (one at a time each tile would cost a trip to L2)
+        for (; r < T.rtiles; r += 8 * tpc) {
+            float2 v[8];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] = __ldcg(p + int64_t(r + q * tpc) * T.m);
+            for (int q = 0; q < 8; ++q)
+                if (r + q * tpc < T.rtiles) v[q] = __ldcg(p + int64_t(r + q * tpc) * T.m);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                cs += v[q].x;
-                pa.add(v[q].y);
-            }
-        }
-        for (; r < T.rtiles; r += tpc) {
-            const float2 v = __ldcg(p + int64_t(r) * T.m);
-            cs += v.x;
-            pa.add(v.y);
+            for (int q = 0; q < 8; ++q)
+                if (r + q * tpc < T.rtiles) {
+                    cs += v[q].x;
+                    pa.add(v[q].y);
+                }
         }
     }
     // the column's tpc parts in slice order
@@ -1089,25 +1089,36 @@ __device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem 
     for (int o = 16; o; o >>= 1) {
         rmn = fminf(rmn, __shfl_xor_sync(kAll, rmn, o));
         cmn = fminf(cmn, __shfl_xor_sync(kAll, cmn, o));
+        rs += __shfl_xor_sync(kAll, rs, o);
+        fs += __shfl_xor_sync(kAll, fs, o);
+        gs += __shfl_xor_sync(kAll, gs, o);
     }
     if ((threadIdx.x & 31) == 0) {  // colred was last read before the barrier above
-        sm.colred[threadIdx.x >> 5] = rmn;
-        sm.colred[kThreads / 32 + (threadIdx.x >> 5)] = cmn;
+        const int w = threadIdx.x >> 5;
+        sm.colred[w] = rmn;
+        sm.colred[kThreads / 32 + w] = cmn;
+        sm.redd[w] = rs;
+        sm.redd[kThreads / 32 + w] = fs;
+        sm.redd[2 * (kThreads / 32) + w] = gs;
     }
-    rs = block_sum_d(rs, sm.redd);  // its barriers also publish the minima
-    fs = block_sum_d(fs, sm.redd);
-    gs = block_sum_d(gs, sm.redd);
+    __syncthreads();
     if (threadIdx.x == 0) {
+        rs = fs = gs = 0.0;
+#pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) {
             rmn = fminf(rmn, sm.colred[w]);
             cmn = fminf(cmn, sm.colred[kThreads / 32 + w]);
+            rs += sm.redd[w];
+            fs += sm.redd[kThreads / 32 + w];
+            gs += sm.redd[2 * (kThreads / 32) + w];
         }
-        const double rbar = rs / (double)T.n;
+        const double rbar = rs * T.inv_n;
         set_rbar(S, rbar);
-        const double a2 = rmn < inf ? rbar / (double)rmn : 0.0;  // max_i a_i^2 over rows with R_i > 0
-        const double b2 = cmn < inf ? 1.0 / (double)cmn : 0.0;   // max_j b_j^2 over columns holding gradient
+        // max_i a_i^2 = Rbar / min R_i over rows with R_i > 0; max_j b_j^2 = 1 / min C_j over columns
+        // holding gradient (0 without any). Multiplied out: fp64 divides are slow here.
+        const bool some = rmn < inf && cmn < inf;
         const double ce2 = (double)A.ce * (double)A.ce;
-        if (__ldcg(&S.zflag) == 0u && a2 * b2 <= ce2 * (1.0 - 1e-6)) {
+        if (__ldcg(&S.zflag) == 0u && (!some || rbar <= ce2 * (1.0 - 1e-6) * ((double)rmn * (double)cmn))) {
             set_clip(A, T, S, fs * rbar);
         } else {
             // A clamp may bind, and it only lowers |U|: no element is above its unclamped value or
@@ -1119,7 +1130,7 @@ __device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem 
             // 850M parameters 1724 -> 1205 us (phase B 572 us, the sums 32 us of phase C).
             const double ub = T.momentum ? fs * rbar : fmin(fs * rbar, gs * ce2);
             const double coef = update_coef(A, T);
-            if (__ldcg(&S.zflag) == 0u && sqrt(ub * coef * coef / (double)T.numel) <= (double)A.clip_d * (1.0 - 1e-4)) {
+            if (__ldcg(&S.zflag) == 0u && ub * coef * coef * T.inv_numel <= (double)A.clip_d * (double)A.clip_d * (1.0 - 1e-4)) {
                 S.kappa = 1.0;
                 S.coefC = (float)((double)A.lr * coef);
                 S.fallback = kSumInC;
@@ -1172,7 +1183,7 @@ __device__ void phase_F(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm)
     double s = 0.0;  // the CTA sums the row items' partials (fixed partition and tree)
     for (uint32_t f = threadIdx.x; f < T.nfr; f += kThreads) s += __ldcg(T.rsum + f);
     s = block_sum_d(s, sm.redd);
-    if (threadIdx.x == 0) set_rbar(S, s / (double)T.n);
+    if (threadIdx.x == 0) set_rbar(S, s * T.inv_n);
 }
 
 // ---------------------------------------------------------------------------
@@ -1335,27 +1346,34 @@ __device__ void phase_B(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm,
 // ---------------------------------------------------------------------------
 // Phase C: decoupled decay, clipped update, dithered bf16 write-back.
 // ---------------------------------------------------------------------------
+// The dithered bf16 values of eight elements whose first has index e0 (a multiple of 8 with the
+// tensor's base).
+__device__ __forceinline__ void round8(const float (&x)[8], const Dith &d, uint64_t e0, uint4 &out) {
+    uint32_t r[8], o[4];
+    dither8(e0, d, r);
+    // a NaN anywhere makes the sum NaN (so does Inf - Inf): only then test per element
+    const float any = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+    if (any == any) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)  // top halves of (bits + draw) of the two elements
+            o[q] = __byte_perm(__float_as_uint(x[2 * q]) + r[2 * q], __float_as_uint(x[2 * q + 1]) + r[2 * q + 1],
+                               0x7632);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q] = sr_bf16(x[2 * q], r[2 * q]) | (sr_bf16(x[2 * q + 1], r[2 * q + 1]) << 16);
+    }
+    out = make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // x of eight elements -> dithered bf16, stored at w + e0 (16-byte store when VEC).
 template <bool VEC>
 __device__ __forceinline__ void write8(uint16_t *__restrict__ w, const Dith &d, int64_t e0, int valid, bool aligned8,
                                        const float (&x)[8], const Pol &pol) {
     uint32_t r[8];
     if (VEC) {
-        dither8((uint64_t)e0, d, r);
-        uint32_t o[4];
-        // a NaN anywhere makes the sum NaN (so does Inf - Inf): only then test per element
-        const float any = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
-        if (any == any) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)  // top halves of (bits + draw) of the two elements
-                o[q] = __byte_perm(__float_as_uint(x[2 * q]) + r[2 * q], __float_as_uint(x[2 * q + 1]) + r[2 * q + 1],
-                                   0x7632);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                o[q] = sr_bf16(x[2 * q], r[2 * q]) | (sr_bf16(x[2 * q + 1], r[2 * q + 1]) << 16);
-        }
-        st16_hint(w + e0, make_uint4(o[0], o[1], o[2], o[3]), pol.drop);
+        uint4 o;
+        round8(x, d, (uint64_t)e0, o);
+        st16_hint(w + e0, o, pol.drop);
     } else {
         if (aligned8) dither8((uint64_t)e0, d, r);
 #pragma unroll
@@ -1731,16 +1749,16 @@ struct MomRowSmem {
     int fail;
 };
 
-// Issues the bulk copies of chunk c of row tile `tile` (rows of x = G in phase A,
+// Issues the bulk copies of chunk c of the tile whose first row is r0 (rows of x = G in phase A,
 // W in phase C, and the same rows of M) into ring slot c % kMomStages.
-__device__ __forceinline__ void mom_issue(const TensorDev &T, const uint16_t *x, uint32_t tile, uint32_t c,
+__device__ __forceinline__ void mom_issue(const TensorDev &T, const uint16_t *x, int64_t r0, uint32_t c,
                                           uint4 (*buf)[kMomSlot16], uint64_t *full, uint64_t pol) {
-    const RowChunk ch = row_chunk(T, tile, c);
-    const uint32_t bx = ch.rows * (uint32_t)T.m * 2u;
+    const int64_t i0 = r0 + int64_t(c) * T.cr;
+    const uint32_t bx = (uint32_t)min(T.n - i0, (int64_t)T.cr) * (uint32_t)T.m * 2u;
     const int st = c % kMomStages;
     mbar_expect_tx(&full[st], 3u * bx);
-    bulk_g2s(buf[st], x + ch.i0 * T.m, bx, &full[st], pol);
-    bulk_g2s(buf[st] + kMomGBytes / 16, T.M + ch.i0 * T.m, 2u * bx, &full[st], pol);
+    bulk_g2s(buf[st], x + i0 * T.m, bx, &full[st], pol);
+    bulk_g2s(buf[st] + kMomGBytes / 16, T.M + i0 * T.m, 2u * bx, &full[st], pol);
 }
 
 // k_rowsq for momentum tensors on TPB threads, rows of m = 8 V: chunks of CS = 1024 / V
@@ -1755,7 +1773,7 @@ __device__ void rowsq_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal
     const L lay;
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    const uint32_t nch = (uint32_t)min((int64_t)kMomChunks, (T.n - int64_t(tile) * T.rt_rows + T.cr - 1) / T.cr);
+    const uint32_t nch = (uint32_t)min((int64_t)(T.rt_rows / T.cr), (T.n - int64_t(tile) * T.rt_rows + T.cr - 1) / T.cr);
     if (threadIdx.x == 0) {
         for (int st = 0; st < kMomStages; ++st) mbar_init(&sm.full[st], 1);
         fence_mbar_init();
@@ -1763,7 +1781,7 @@ __device__ void rowsq_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal
     }
     __syncthreads();
     if (threadIdx.x == 0)
-        for (uint32_t c = 0; c < nch && c < (uint32_t)kMomStages; ++c) mom_issue(T, T.g, tile, c, sm.buf, sm.full, pol);
+        for (uint32_t c = 0; c < nch && c < (uint32_t)kMomStages; ++c) mom_issue(T, T.g, int64_t(tile) * T.rt_rows, c, sm.buf, sm.full, pol);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const GScale gsc = grad_scale(A);
@@ -1816,7 +1834,7 @@ __device__ void rowsq_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal
         // refill from warp 1: warp 0 forms the chunk's row scales, which the CTA waits for
         if (tid == 32 && c >= 1 && c - 1 + kMomStages < nch) {
             fence_proxy_async_smem();
-            mom_issue(T, T.g, tile, c - 1 + kMomStages, sm.buf, sm.full, pol);
+            mom_issue(T, T.g, int64_t(tile) * T.rt_rows, c - 1 + kMomStages, sm.buf, sm.full, pol);
         }
         float Rn = 0.f;
         if (tid < (int)ch.rows) {
@@ -1942,7 +1960,7 @@ struct MomApplySmem {
 // Phase C of a momentum row tile: as apply_rows_body with y = the new M (Algorithm 1,
 // backbone branch: U = coef M / D).
 template <int TPB, int V, bool FAST>
-__device__ bool apply_rows_mom_body(const StepArgs &A, const TensorDev &T, uint32_t tile,
+__device__ bool apply_rows_mom_body(const StepArgs &A, const TensorDev &T, int64_t r0,
                                     const float (&b)[RowLayout<TPB, V>::NV][8], float coefC, MomApplySmem &sm,
                                     uint32_t nch, uint64_t pol, Acc2 &acc) {
     using L = RowLayout<TPB, V>;
@@ -1959,7 +1977,7 @@ __device__ bool apply_rows_mom_body(const StepArgs &A, const TensorDev &T, uint3
     const Pol sp;
     for (uint32_t c = 0; c < nch; ++c) {
         const int st = c % kMomStages;
-        const int64_t i0 = int64_t(tile) * T.at_rows + int64_t(c) * CA;
+        const int64_t i0 = r0 + int64_t(c) * CA;
         const int rows = (int)min((int64_t)CA, T.n - i0);
         const bool ok = mbar_wait(&sm.full[st], (c / kMomStages) & 1u);
         const uint4 *bw = sm.buf[st];
@@ -2008,22 +2026,24 @@ __device__ bool apply_rows_mom_body(const StepArgs &A, const TensorDev &T, uint3
         }
         if (tid == 0 && c + kMomStages < nch) {
             fence_proxy_async_smem();
-            mom_issue(T, T.w, tile, c + kMomStages, sm.buf, sm.full, pol);
+            mom_issue(T, T.w, r0, c + kMomStages, sm.buf, sm.full, pol);
         }
     }
     return true;
 }
 
 template <int TPB, int V>
-__device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t tile,
+__device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t item,
                                     MomApplySmem &sm) {
     using L = RowLayout<TPB, V>;
     constexpr int NV = L::NV;
     const L lay;
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    const int64_t r0 = int64_t(tile) * T.at_rows;
-    const uint32_t rows_t = (uint32_t)min((int64_t)T.at_rows, T.n - r0);
+    const uint32_t trows = (item & kHalfTile) ? T.at_rows / 2 : T.at_rows;
+    const int64_t r0 = int64_t(item & kTileMask) * T.at_rows + ((item & kSecondHalf) ? trows : 0);
+    if (r0 >= T.n) return;  // the second half of a matrix's short last tile
+    const uint32_t rows_t = (uint32_t)min((int64_t)trows, T.n - r0);
     const uint32_t nch = (rows_t + T.cr - 1) / T.cr;
     if (threadIdx.x == 0) {
         for (int st = 0; st < kMomStages; ++st) mbar_init(&sm.full[st], 1);
@@ -2031,7 +2051,7 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
     }
     __syncthreads();
     if (threadIdx.x == 0)
-        for (uint32_t c = 0; c < nch && c < (uint32_t)kMomStages; ++c) mom_issue(T, T.w, tile, c, sm.buf, sm.full, pol);
+        for (uint32_t c = 0; c < nch && c < (uint32_t)kMomStages; ++c) mom_issue(T, T.w, r0, c, sm.buf, sm.full, pol);
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
     float ma = 0.f, mb = 0.f;
@@ -2072,10 +2092,473 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
     Acc2 acc;
     bool done;
     if (!sum && ma * mb <= A.ce)
-        done = apply_rows_mom_body<TPB, V, true>(A, T, tile, b, coefC, sm, nch, pol, acc);
+        done = apply_rows_mom_body<TPB, V, true>(A, T, r0, b, coefC, sm, nch, pol, acc);
     else
-        done = apply_rows_mom_body<TPB, V, false>(A, T, tile, b, coefC, sm, nch, pol, acc);
-    if (sum && done) publish_sum(A, T, S, tile, rows_t, acc, sm.sum);
+        done = apply_rows_mom_body<TPB, V, false>(A, T, r0, b, coefC, sm, nch, pol, acc);
+    if (sum && done) publish_sum(A, T, S, item, rows_t, acc, sm.sum);
+}
+
+// ---------------------------------------------------------------------------
+// Row path for any other width m = 8 V in [256, 4096] (phase A; phase C is
+// apply_flat_tile). The same algorithm as rowsq_tile / rowsq_mom_tile on a layout
+// formed at run time: a row belongs to wpr = ceil(V / (32 NV)) warps, of which a
+// thread owns vectors vi, vi + 32 wpr, ... (columns stay in its registers), and
+// rpp = 8 / wpr rows go side by side; warps past rpp * wpr, and lanes past the row's
+// end, only keep the barriers (at worst 3 of 8 warps, m = 1032 to 1280). A chunk is
+// K rpp whole rows (at most 32 KB of G, or 48 KB of G and M), in as many ring slots
+// as 96 KB holds. What bounds it: the chain of two passes and two barriers per chunk, as
+// for the fixed widths (ncu: barrier stalls first), with fewer of the eight warps working.
+// 512 MiB of G: m = 1536 126 us (4.2 TB/s, after a write-back of the last launch's dirty
+// L2), 768 129, 3072 131, against 105 to 117 us at the fixed widths; with momentum 212 to
+// 217 us (6.2 TB/s of G and M) at every width. Branches on the lanes past a row's end made
+// it 536 us where reading zeros instead takes 405 (930M parameters in 3072 x 1536 experts).
+// ---------------------------------------------------------------------------
+constexpr int kGenStages = 8;
+constexpr int kGenRingBytes = 3 * 32768;
+
+struct GenSmem {
+    uint4 ring[kGenRingBytes / 16];
+    uint4 zero[2];      // what the lanes past a row's end (and rows past the matrix) read
+    uint64_t full[kGenStages];
+    float part[8][8];   // per-warp row partial sums of the chunk
+    float inv[64];      // 1 / R_i of the chunk's rows (0: no contribution)
+    double rsum[2];
+    float rmin[2];
+};
+constexpr uint32_t kGenZero = kGenRingBytes / 16;  // index of `zero` from `ring`
+static_assert(offsetof(GenSmem, zero) == 16 * kGenZero, "zero follows the ring");
+
+template <int NV, bool MOM>
+__device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t tile, GenSmem &sm) {
+    constexpr int K = gen_rows_per_thread(NV, MOM);
+    // with one vector per thread and row the chunk stays in registers from pass 1 to pass 2, as in
+    // rowsq_tile: its squares, or with momentum g (M is still read from the slot)
+    constexpr bool kHold = NV == 1, kEarly = kHold && !MOM;
+    const uint32_t V = (uint32_t)T.m / 8u, m = (uint32_t)T.m;
+    const uint32_t wpr = (V + 32 * NV - 1) / (32 * NV), rpp = 8 / wpr, lpr = 32 * wpr;
+    const uint32_t cr = T.cr, gbytes = cr * m * 2u, slot = MOM ? 3u * gbytes : gbytes;
+    const uint32_t stages = min((uint32_t)kGenStages, (uint32_t)kGenRingBytes / slot);
+    const int64_t row0 = int64_t(tile) * T.rt_rows, n = T.n;
+    const uint32_t rows_t = (uint32_t)min((int64_t)T.rt_rows, n - row0);
+    const uint32_t nch = (rows_t + cr - 1) / cr;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float *__restrict__ Mt = MOM ? T.M + row0 * T.m : nullptr;
+    float *__restrict__ Rt = T.R + row0;
+    char *ring = reinterpret_cast<char *>(sm.ring);
+    // (the issuing thread reads its addresses from the descriptor each time: they would cost
+    // every thread registers)
+    auto issue = [&](uint32_t c, uint32_t st) {
+        const uint32_t rows = min(cr, rows_t - c * cr), bx = rows * m * 2u;
+        const int64_t e0 = (int64_t(tile) * T.rt_rows + c * cr) * T.m;
+        uint64_t pol;
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+        mbar_expect_tx(&sm.full[st], MOM ? 3u * bx : bx);
+        bulk_g2s(ring + st * slot, T.g + e0, bx, &sm.full[st], pol);
+        if (MOM) bulk_g2s(ring + st * slot + gbytes, T.M + e0, 2u * bx, &sm.full[st], pol);
+    };
+    if (tid == 0) {
+        for (uint32_t st = 0; st < stages; ++st) mbar_init(&sm.full[st], 1);
+        fence_mbar_init();
+    }
+    if (tid < 8) reinterpret_cast<uint32_t *>(sm.zero)[tid] = 0u;
+    __syncthreads();
+    if (tid == 0)
+        for (uint32_t c = 0; c < nch && c < stages; ++c) issue(c, c);
+
+    const uint32_t rp = warp / wpr, vi = (warp - rp * wpr) * 32u + lane;
+    const bool on = rp < rpp;  // the warp has rows (the same for its lanes)
+    bool act[NV];              // the thread has vector vi + v lpr
+    uint32_t step[NV];         // vectors from one of its rows to the next
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        act[v] = on && vi + v * lpr < V;
+        step[v] = act[v] ? rpp * V : 0u;
+    }
+    const uint32_t kr = tid / rpp, w0 = (tid - kr * rpp) * wpr;  // threads < cr: chunk row tid is k = kr of row-in-pass tid % rpp
+    const GScale gsc = grad_scale(A);
+    const float b2 = A.b2, c2m = __fdiv_rn(gsc.c2, (float)m);
+    const float2 b12 = make_float2(A.b1, A.b1), c12 = make_float2(gsc.c1, gsc.c1);
+    // per column pair: sums of g^2, the compensated (hi, lo) sum of y^2 / R_i (y = g, or the new
+    // M with momentum) and its open fp32 part
+    float2 cs[NV][4], ph[NV][4], pl[NV][4], t[NV][4];
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cs[v][q] = ph[v][q] = pl[v][q] = t[v][q] = make_float2(0.f, 0.f);
+    const float inf = __int_as_float(0x7F800000);
+    double rsum = 0.0;  // threads < cr: sum and smallest positive R of this chunk-row position
+    float rmin = inf;
+    bool zero_row = false;
+
+    uint32_t c = 0, st = 0, par = 0;
+    for (; c < nch; ++c) {
+        const uint32_t rows = min(cr, rows_t - c * cr);
+        float rold = 0.f;
+        if (tid < (int)rows) rold = __ldcg(Rt + c * cr + tid);
+        const bool ok = mbar_wait(&sm.full[st], par);
+        // the thread's first vector of the chunk's G, and of its M (indices from the ring's start);
+        // a lane without a vector reads zeros, so that the passes need no branches
+        uint32_t ig[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) ig[v] = act[v] ? st * (slot / 16) + rp * V + vi + v * lpr : kGenZero;
+        const bool full = rows == cr;  // every chunk but the tile's last needs no row bound checks
+        // pass 1: row and column sums of g^2
+        float rs[K];
+        float2 hold[kHold ? K : 1][4];
+        auto pass1 = [&](auto full_c) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                float2 r2 = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const bool in = decltype(full_c)::value || rp + rpp * k < rows;
+                    float2 g[4];
+                    unpack_bf8x2(sm.ring[in ? ig[v] + k * step[v] : kGenZero], g);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 g2 = __fmul2_rn(g[q], g[q]);  // exact
+                        cs[v][q] = __fadd2_rn(cs[v][q], g2);
+                        r2 = __fadd2_rn(r2, g2);
+                        if constexpr (kHold) hold[k][q] = MOM ? g[q] : g2;
+                    }
+                }
+                rs[k] = r2.x + r2.y;
+            }
+        };
+        if (on) {
+            if (full)
+                pass1(std::true_type{});
+            else
+                pass1(std::false_type{});
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) rs[k] = 0.f;
+        }
+        int j;
+        const float tot = warp_sum_transposed<K>(rs, j);
+        if ((lane & (K == 8 ? 3 : K == 4 ? 7 : 15)) == 0) sm.part[warp][j] = tot;
+        if (__syncthreads_or(!ok)) break;  // every slot before this one has landed
+        // the slot of chunk c (when its values are held), or else of chunk c - 1, is free: refill it
+        // (from the last warp: the first ones form the chunk's row scales, which the CTA waits for)
+        if (tid == kRowThreads - 32 && (kEarly || c >= 1) && c - (kEarly ? 0 : 1) + stages < nch) {
+            fence_proxy_async_smem();
+            issue(c - (kEarly ? 0 : 1) + stages, kEarly ? st : st == 0 ? stages - 1 : st - 1);
+        }
+        float Rn = 0.f, sum = 0.f;
+        if (tid < (int)rows) {
+            float p[8];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) p[w] = w < (int)wpr ? sm.part[w0 + w][kr] : 0.f;
+            sum = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+            Rn = fmaf(b2, rold, c2m * sum);  // c2m = c2 / m, rounded once
+            sm.inv[tid] = Rn > 0.f && Rn < inf ? __frcp_rn(Rn) : 0.f;
+        }
+        __syncthreads();
+        if (tid < (int)rows) {  // the row's R and the tile's statistics, off the barrier's path
+            Rt[c * cr + tid] = Rn;
+            rsum += (double)Rn;
+            if (Rn > 0.f && Rn < inf)
+                rmin = fminf(rmin, Rn);
+            else if (MOM || !(Rn == 0.f && sum == 0.f))
+                zero_row = true;  // content (or, with momentum, perhaps an old M) in a row with R_i == 0, or a non-finite R_i
+        }
+        // pass 2: y^2 / R_i, summed in fp32 over four chunks per column, then folded into (hi, lo);
+        // with momentum M <- b1 M + (1 - b1) g, stored here
+        auto pass2 = [&](auto full_c) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const uint32_t r = rp + rpp * k;
+                const bool in = decltype(full_c)::value || r < rows;
+                const float iv = in ? sm.inv[r] : 0.f;
+                const float2 iv2 = make_float2(iv, iv);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    float2 y[4];
+                    if constexpr (kHold) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) y[q] = hold[k][q];
+                    } else {
+                        unpack_bf8x2(sm.ring[in ? ig[v] + k * step[v] : kGenZero], y);
+                    }
+                    if constexpr (MOM) {
+                        // M's vector: twice G's distance from the slot's start, past its G
+                        const uint32_t im = gbytes / 16 - st * (slot / 16) + 2 * (ig[v] + k * step[v]);
+                        const float4 *bm = reinterpret_cast<const float4 *>(sm.ring + (in && act[v] ? im : kGenZero));
+                        const float4 m0 = bm[0], m1 = bm[1];
+                        y[0] = __ffma2_rn(b12, make_float2(m0.x, m0.y), __fmul2_rn(c12, y[0]));
+                        y[1] = __ffma2_rn(b12, make_float2(m0.z, m0.w), __fmul2_rn(c12, y[1]));
+                        y[2] = __ffma2_rn(b12, make_float2(m1.x, m1.y), __fmul2_rn(c12, y[2]));
+                        y[3] = __ffma2_rn(b12, make_float2(m1.z, m1.w), __fmul2_rn(c12, y[3]));
+                        if (act[v] && in) {
+                            float4 *dst = reinterpret_cast<float4 *>(Mt + uint64_t(c * cr + r) * m + 8 * (vi + v * lpr));
+                            dst[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
+                            dst[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        t[v][q] = __ffma2_rn(kEarly ? y[q] : __fmul2_rn(y[q], y[q]), iv2, t[v][q]);
+                }
+            }
+        };
+        if (on) {
+            if (full)
+                pass2(std::true_type{});
+            else
+                pass2(std::false_type{});
+        }
+        if ((c & 3u) == 3u || c + 1 == nch) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float2 s2, e2;
+                    two_sum2(ph[v][q], t[v][q], s2, e2);
+                    ph[v][q] = s2;
+                    pl[v][q] = __fadd2_rn(pl[v][q], e2);
+                    t[v][q] = make_float2(0.f, 0.f);
+                }
+        }
+        if (++st == stages) {
+            st = 0;
+            par ^= 1u;
+        }
+    }
+    if (c < nch) {
+        // a chunk did not land in time: as in rowsq_tile
+        if (tid == 0) drain_copies(A.err, sm.full, stages, c, min(nch, kEarly || c == 0 ? c + stages : c + stages - 1));
+        return;
+    }
+    // per-tile partials, as rowsq_tile's
+    float2 *pp = T.pp + int64_t(tile) * m;
+    if (rpp == 1) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (act[v]) {
+                float4 *pp4 = reinterpret_cast<float4 *>(pp + 8 * (vi + v * lpr));
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    pp4[q] = make_float4(cs[v][q].x, pair_f(ph[v][q].x, pl[v][q].x), cs[v][q].y,
+                                         pair_f(ph[v][q].y, pl[v][q].y));
+            }
+        }
+    } else {  // NV == 1: rpp rows of at most 128 vectors side by side
+        float *mcs = reinterpret_cast<float *>(sm.ring);          // [256][8]
+        float2 *mpp = reinterpret_cast<float2 *>(sm.ring + 512);  // [256][8] (hi, lo)
+        __syncthreads();  // the ring is free: every chunk is consumed
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            mcs[tid * 8 + 2 * q] = cs[0][q].x;
+            mcs[tid * 8 + 2 * q + 1] = cs[0][q].y;
+            mpp[tid * 8 + 2 * q] = make_float2(ph[0][q].x, pl[0][q].x);
+            mpp[tid * 8 + 2 * q + 1] = make_float2(ph[0][q].y, pl[0][q].y);
+        }
+        __syncthreads();
+        for (uint32_t e = tid; e < m; e += kRowThreads) {
+            float cc = 0.f;
+            Acc2 pq;
+            for (uint32_t r = 0; r < rpp; ++r) {
+                cc += mcs[r * lpr * 8 + e];
+                const float2 h = mpp[r * lpr * 8 + e];
+                pq.add(h.x);
+                pq.lo += h.y;
+            }
+            pp[e] = make_float2(cc, pair_f(pq.hi, pq.lo));
+        }
+    }
+    if (zero_row) atomicOr(&S.zflag, 1u);
+    if (warp < 2) {  // at most 64 rows per chunk: the chunk-row positions are lanes of warps 0 and 1
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            rsum += __shfl_xor_sync(kAll, rsum, o);
+            rmin = fminf(rmin, __shfl_xor_sync(kAll, rmin, o));
+        }
+        if (lane == 0) {
+            sm.rsum[warp] = rsum;
+            sm.rmin[warp] = rmin;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        T.rsum[tile] = sm.rsum[0] + sm.rsum[1];
+        T.rmin[tile] = fminf(sm.rmin[0], sm.rmin[1]);
+    }
+}
+
+// Phase C of these widths: given the step's scalars it is elementwise, so the tile's rows are one
+// run of 16-byte vectors, cut into chunks of 1024 (16 KB of W, and 16 KB of G or 32 KB of M) that
+// need not end with a row, and every thread works whatever the width. Row scales and all m column
+// scales sit in shared memory; a thread steps its row and column by 256 vectors without dividing.
+// Per element the arithmetic is apply_fact_tile's, bit for bit. Bound by HBM: 930M parameters in
+// 3072 x 1536 experts 994 us on strip tiles, 826 us (6.75 TB/s) here.
+constexpr uint32_t kFlatChunk = 1024;  // vectors
+
+struct FlatSmem {
+    uint4 ring[kGenRingBytes / 16];  // [W | G] x 3 slots, or [W | M] x 2
+    uint64_t full[4];
+    float red[2 * kRowThreads / 32];
+    float ab[kFlatScales];  // b_j [m], then a_i of the tile's rows
+    SumSmem sum;
+};
+
+// Issues the copies of chunk c of the tile (vectors of rows r0, ...) into slot st.
+template <bool MOM>
+__device__ __forceinline__ void flat_issue(const TensorDev &T, int64_t r0, uint32_t total, uint32_t c, uint32_t st,
+                                           FlatSmem &sm, uint64_t pol) {
+    constexpr uint32_t kSlot16 = MOM ? 3 * kFlatChunk : 2 * kFlatChunk;
+    const uint32_t bytes = min(kFlatChunk, total - c * kFlatChunk) * 16u;
+    const uint64_t e0 = uint64_t(r0) * (uint64_t)T.m + uint64_t(c) * kFlatChunk * 8u;
+    uint4 *dst = sm.ring + st * kSlot16;
+    mbar_expect_tx(&sm.full[st], MOM ? 3u * bytes : 2u * bytes);
+    bulk_g2s(dst, T.w + e0, bytes, &sm.full[st], pol);
+    if (MOM)
+        bulk_g2s(dst + kFlatChunk, T.M + e0, 2u * bytes, &sm.full[st], pol);
+    else
+        bulk_g2s(dst + kFlatChunk, T.g + e0, bytes, &sm.full[st], pol);
+}
+
+template <bool MOM, bool FAST>
+__device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r0, uint32_t total, float coefC,
+                                FlatSmem &sm, uint64_t pol, Acc2 &acc) {
+    constexpr uint32_t kStages = MOM ? 2 : 3, kSlot16 = MOM ? 3 * kFlatChunk : 2 * kFlatChunk;
+    const uint32_t V = (uint32_t)T.m / 8u, nch = (total + kFlatChunk - 1) / kFlatChunk;
+    const int tid = threadIdx.x;
+    uint16_t *__restrict__ w_ = T.w + r0 * T.m;
+    const Dith d = dith_of(A, T);
+    const uint64_t el0 = uint64_t(r0) * (uint64_t)T.m;
+    const float wdf = T.decay ? A.wdf : 1.0f, ce = A.ce;
+    const float2 wdf2 = make_float2(wdf, wdf);
+    const Pol sp;
+    const float *__restrict__ sb = sm.ab, *__restrict__ sa = sm.ab + 8 * V;
+    uint32_t row = tid / V, col = tid - row * V;  // of vector tid of the tile
+    const uint32_t dq = kRowThreads / V, dr = kRowThreads - dq * V;
+    uint32_t st = 0, par = 0;
+    for (uint32_t c = 0; c < nch; ++c) {
+        const uint32_t cnt = min(kFlatChunk, total - c * kFlatChunk);
+        const bool ok = mbar_wait(&sm.full[st], par);
+        const uint4 *bw = sm.ring + st * kSlot16, *by = bw + kFlatChunk;
+#pragma unroll
+        for (uint32_t k = 0; k < kFlatChunk / kRowThreads; ++k) {
+            const uint32_t f = k * kRowThreads + tid;
+            if (f < cnt) {
+                const float a = sa[row];
+                const float4 b0 = *reinterpret_cast<const float4 *>(sb + 8 * col);
+                const float4 b1 = *reinterpret_cast<const float4 *>(sb + 8 * col + 4);
+                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                float y[8], w[8], x[8];
+                if constexpr (MOM) {
+                    const float4 m0 = reinterpret_cast<const float4 *>(by)[2 * f];
+                    const float4 m1 = reinterpret_cast<const float4 *>(by)[2 * f + 1];
+                    y[0] = m0.x; y[1] = m0.y; y[2] = m0.z; y[3] = m0.w;
+                    y[4] = m1.x; y[5] = m1.y; y[6] = m1.z; y[7] = m1.w;
+                } else {
+                    unpack_bf8(by[f], y);
+                }
+                unpack_bf8(bw[f], w);
+                if constexpr (FAST) {
+                    const float cr = -coefC * a;
+                    const float2 cr2 = make_float2(cr, cr);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 xx = __ffma2_rn(__fmul2_rn(cr2, make_float2(b[2 * q], b[2 * q + 1])),
+                                                     make_float2(y[2 * q], y[2 * q + 1]),
+                                                     __fmul2_rn(make_float2(w[2 * q], w[2 * q + 1]), wdf2));
+                        x[2 * q] = xx.x;
+                        x[2 * q + 1] = xx.y;
+                    }
+                } else {
+                    float u[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        u[q] = y[q] * fminf(a * b[q], ce);
+                        x[q] = fmaf(-coefC, u[q], w[q] * wdf);
+                    }
+                    acc.add(sumsq8(u));
+                }
+                const uint64_t e0 = uint64_t(c * kFlatChunk + f) * 8u;
+                uint4 o;
+                round8(x, d, el0 + e0, o);
+                st16_hint(w_ + e0, o, sp.drop);
+            }
+            row += dq;
+            col += dr;
+            if (col >= V) {
+                col -= V;
+                ++row;
+            }
+        }
+        // every thread is done with the slot: refill it
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0) drain_copies(A.err, sm.full, kStages, c, min(nch, c + kStages));
+            return false;
+        }
+        if (tid == 0 && c + kStages < nch) {
+            fence_proxy_async_smem();
+            flat_issue<MOM>(T, r0, total, c + kStages, st, sm, pol);
+        }
+        if (++st == kStages) {
+            st = 0;
+            par ^= 1u;
+        }
+    }
+    return true;
+}
+
+template <bool MOM>
+__device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t item, FlatSmem &sm) {
+    constexpr uint32_t kStages = MOM ? 2 : 3;
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    const uint32_t trows = (item & kHalfTile) ? T.at_rows / 2 : T.at_rows;
+    const int64_t r0 = int64_t(item & kTileMask) * T.at_rows + ((item & kSecondHalf) ? trows : 0);
+    if (r0 >= T.n) return;  // the second half of a matrix's short last tile
+    const uint32_t m = (uint32_t)T.m, rows_t = (uint32_t)min((int64_t)trows, T.n - r0), total = rows_t * (m / 8u);
+    const uint32_t nch = (total + kFlatChunk - 1) / kFlatChunk;
+    if (threadIdx.x == 0) {
+        for (uint32_t st = 0; st < kStages; ++st) mbar_init(&sm.full[st], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (uint32_t c = 0; c < nch && c < kStages; ++c) flat_issue<MOM>(T, r0, total, c, c, sm, pol);
+    const float rbar_s = __ldcg(&S.rbar_s);
+    const int rbar_e = __ldcg(&S.rbar_e);
+    float ma = 0.f, mb = 0.f;
+    for (uint32_t j = threadIdx.x; j < m / 4; j += kRowThreads) {
+        const float4 b = __ldcg(reinterpret_cast<const float4 *>(T.bsc) + j);
+        reinterpret_cast<float4 *>(sm.ab)[j] = b;
+        mb = fmaxf(fmaxf(mb, fmaxf(nan_to_inf(b.x), nan_to_inf(b.y))), fmaxf(nan_to_inf(b.z), nan_to_inf(b.w)));
+    }
+    for (uint32_t r = threadIdx.x; r < rows_t; r += kRowThreads) {
+        const float a = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
+        sm.ab[m + r] = a;
+        ma = fmaxf(ma, nan_to_inf(a));
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        ma = fmaxf(ma, __shfl_xor_sync(kAll, ma, o));
+        mb = fmaxf(mb, __shfl_xor_sync(kAll, mb, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        sm.red[threadIdx.x >> 5] = ma;
+        sm.red[kRowThreads / 32 + (threadIdx.x >> 5)] = mb;
+    }
+    __syncthreads();
+    ma = mb = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRowThreads / 32; ++w) {
+        ma = fmaxf(ma, sm.red[w]);
+        mb = fmaxf(mb, sm.red[kRowThreads / 32 + w]);
+    }
+    const float coefC = __ldcg(&S.coefC);
+    const bool sum = __ldcg(&S.fallback) == kSumInC;
+    Acc2 acc;
+    bool done;
+    if (!sum && ma * mb <= A.ce)
+        done = apply_flat_body<MOM, true>(A, T, r0, total, coefC, sm, pol, acc);
+    else
+        done = apply_flat_body<MOM, false>(A, T, r0, total, coefC, sm, pol, acc);
+    if (sum && done) publish_sum(A, T, S, item, rows_t, acc, sm.sum);
 }
 
 // ---------------------------------------------------------------------------
@@ -2103,6 +2586,22 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     const uint2 it = items[blockIdx.x];
     const TensorDev &T = A.tensors[it.x];
     TensorScal &S = A.scal[it.x];
+    if (T.rowpath == kRowAny) {
+        GenSmem &gs = *reinterpret_cast<GenSmem *>(dyn_smem);
+        const bool wide = T.m > 2048;
+        if (T.momentum) {
+            if (wide)
+                rowsq_gen_tile<2, true>(A, T, S, it.y, gs);
+            else
+                rowsq_gen_tile<1, true>(A, T, S, it.y, gs);
+        } else {
+            if (wide)
+                rowsq_gen_tile<2, false>(A, T, S, it.y, gs);
+            else
+                rowsq_gen_tile<1, false>(A, T, S, it.y, gs);
+        }
+        return;
+    }
     if (T.momentum) {
         MomRowSmem &ms = *reinterpret_cast<MomRowSmem *>(dyn_smem);
         switch (T.m) {
@@ -2129,6 +2628,14 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     const uint2 it = items[blockIdx.x];
     const TensorDev &T = A.tensors[it.x];
     TensorScal &S = A.scal[it.x];
+    if (T.rowpath == kRowAny) {
+        FlatSmem &fs = *reinterpret_cast<FlatSmem *>(dyn_smem);
+        if (T.momentum)
+            apply_flat_tile<true>(A, T, S, it.y, fs);
+        else
+            apply_flat_tile<false>(A, T, S, it.y, fs);
+        return;
+    }
     if (T.momentum) {
         MomApplySmem &ms = *reinterpret_cast<MomApplySmem *>(dyn_smem);
         switch (T.m) {
@@ -2240,6 +2747,8 @@ int launch_wait_selftest(uint32_t *err, void *stream) {
     return (int)cudaGetLastError();
 }
 
+constexpr size_t max3(size_t a, size_t b, size_t c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
+
 int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *const *ev) {
     cudaStream_t s = (cudaStream_t)stream;
     auto mark = [&](int k) {
@@ -2249,7 +2758,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     if (L.nA) k_sumsq<<<L.nA, kThreads, 0, s>>>(A, L.itemsA);
     mark(1);
     if (L.nR) {
-        constexpr size_t kSm = sizeof(RowSmem) > sizeof(MomRowSmem) ? sizeof(RowSmem) : sizeof(MomRowSmem);
+        constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem));
         const cudaError_t e = cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
         k_rowsq<<<L.nR, kRowThreads, kSm, s>>>(A, L.itemsR);
@@ -2264,8 +2773,8 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     if (L.nC) k_apply<<<L.nC, kThreads, 0, s>>>(A, L.itemsC);
     mark(6);
     if (L.nCR) {
-        constexpr size_t kSm =
-            sizeof(ApplyRowSmem) > sizeof(MomApplySmem) ? sizeof(ApplyRowSmem) : sizeof(MomApplySmem);
+        constexpr size_t kSm = max3(sizeof(ApplyRowSmem), sizeof(MomApplySmem), sizeof(FlatSmem));
+        static_assert(2 * (kSm + 1024) <= 228 * 1024, "two CTAs per SM");
         const cudaError_t e = cudaFuncSetAttribute(k_apply_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
         k_apply_rows<<<L.nCR, kRowThreads, kSm, s>>>(A, L.itemsCR);

@@ -42,6 +42,53 @@ unsigned char *scratch_base() {
     return static_cast<unsigned char *>(p);
 }
 
+// Where one tensor's scratch lies in the fixed array, its item counts and the bytes it takes.
+struct Layout {
+    uint32_t nA, nR, nF, nB, nC, nCR;
+    size_t scal, fb, tens, iA, iR, iF, iB, iC, iCR, rowp, colp, bsc, rsum, pp, rmin, fsum, fmin, u2, bytes;
+};
+
+Layout layout_of(const TileGeom &G, uint32_t kind, int64_t n, int64_t m) {
+    Layout o{};
+    const bool fact = kind == kKindFactored, row = fact && G.rowpath;
+    o.nA = fact && !row ? G.ntiles : 0;
+    o.nR = row ? G.rtiles : 0;
+    o.nF = fact ? G.nfr + G.nfc : 0;
+    o.nB = row ? 0 : G.ntiles;
+    o.nC = row ? 0 : G.ntiles;
+    o.nCR = row ? G.atiles : 0;
+    size_t off = align256(kErrOffset + 16);  // the status word comes first
+    auto put = [&](size_t &at, size_t bytes) {
+        at = off;
+        off = align256(off + bytes);
+    };
+    put(o.scal, sizeof(TensorScal));
+    put(o.fb, 8);
+    put(o.tens, sizeof(TensorDev));
+    put(o.iA, sizeof(uint2) * o.nA);
+    put(o.iR, sizeof(uint2) * o.nR);
+    put(o.iF, sizeof(uint2) * o.nF);
+    put(o.iB, sizeof(uint2) * o.nB);
+    put(o.iC, sizeof(uint2) * o.nC);
+    put(o.iCR, sizeof(uint2) * o.nCR);
+    if (fact && !row) {
+        put(o.rowp, 4 * size_t(G.strips) * n);
+        put(o.colp, 4 * size_t(G.rowtiles) * m);
+        put(o.bsc, 4 * size_t(m));
+        put(o.rsum, 8 * size_t(G.nfr));
+    } else if (row) {
+        put(o.pp, 8 * size_t(G.rtiles) * m);
+        put(o.bsc, 4 * size_t(m));
+        put(o.rsum, 8 * size_t(G.rtiles));
+        put(o.rmin, 4 * size_t(G.rtiles));
+        put(o.fsum, 8 * size_t(G.nfc));
+        put(o.fmin, 4 * size_t(G.nfc));
+    }
+    put(o.u2, 8 * size_t(u2_len(G)));
+    o.bytes = off;
+    return o;
+}
+
 struct SetupTables {
     uint2 *A;
     uint32_t nA;
@@ -128,39 +175,23 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     const int64_t tiles64 = kind == kKindFactored ? ((m + 255) / 256) * ((n + 255) / 256)
                                                   : (numel + kFlatTileElems - 1) / kFlatTileElems;
     if (tiles64 > (int64_t(1) << 31)) return SKEW_EINVAL;
-    const TileGeom G = plan_geometry(kind, momentum, wg_aligned, n, m, numel);
-    const bool fact = kind == kKindFactored, row = fact && G.rowpath;
-    const uint32_t nA = fact && !row ? G.ntiles : 0, nR = row ? G.rtiles : 0, nF = fact ? G.nfr + G.nfc : 0;
-    const uint32_t nB = row ? 0 : G.ntiles, nC = row ? 0 : G.ntiles, nCR = row ? G.atiles : 0;
-
-    // ---- scratch layout inside the fixed array --------------------------------------
-    size_t off = align256(kErrOffset + 16);  // the status word comes first
-    const size_t o_scal = off;   off = align256(off + sizeof(TensorScal));
-    const size_t o_fb = off;     off = align256(off + 8);
-    const size_t o_err = kErrOffset;
-    const size_t o_tens = off;   off = align256(off + sizeof(TensorDev));
-    const size_t o_iA = off;     off = align256(off + sizeof(uint2) * nA);
-    const size_t o_iR = off;     off = align256(off + sizeof(uint2) * nR);
-    const size_t o_iF = off;     off = align256(off + sizeof(uint2) * nF);
-    const size_t o_iB = off;     off = align256(off + sizeof(uint2) * nB);
-    const size_t o_iC = off;     off = align256(off + sizeof(uint2) * nC);
-    const size_t o_iCR = off;    off = align256(off + sizeof(uint2) * nCR);
-    size_t o_rowp = 0, o_colp = 0, o_bsc = 0, o_rsum = 0, o_pp = 0, o_rmin = 0, o_fsum = 0, o_fmin = 0;
-    if (fact && !row) {
-        o_rowp = off; off = align256(off + 4 * size_t(G.strips) * n);
-        o_colp = off; off = align256(off + 4 * size_t(G.rowtiles) * m);
-        o_bsc = off;  off = align256(off + 4 * size_t(m));
-        o_rsum = off; off = align256(off + 8 * size_t(G.nfr));
-    } else if (row) {
-        o_pp = off;   off = align256(off + 8 * size_t(G.rtiles) * m);
-        o_bsc = off;  off = align256(off + 4 * size_t(m));
-        o_rsum = off; off = align256(off + 8 * size_t(G.rtiles));
-        o_rmin = off; off = align256(off + 4 * size_t(G.rtiles));
-        o_fsum = off; off = align256(off + 8 * size_t(G.nfc));
-        o_fmin = off; off = align256(off + 4 * size_t(G.nfc));
+    // What the entry point takes is set by the full-sized row tiles of the fixed widths and by the
+    // strip tiles at the others; a matrix whose own tiles (as skew_step cuts it) need more scratch
+    // than there is runs on those.
+    TileGeom G = plan_geometry(kind, momentum, wg_aligned, n, m, numel, 2 * numel);
+    if (G.rowpath == kRowAny && 2 * numel < kAnyGroupBytes) G = plan_geometry(kind, momentum, false, n, m, numel, kWholeGroup);
+    Layout o = layout_of(G, kind, n, m);
+    if (G.rowpath) {
+        const TileGeom most = plan_geometry(kind, momentum, G.rowpath == kRowFixed, n, m, numel, kWholeGroup);
+        const Layout om = layout_of(most, kind, n, m);
+        if (om.bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;
+        if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) {
+            G = most;
+            o = om;
+        }
     }
-    const size_t o_u2 = off;     off = align256(off + 8 * size_t(u2_len(G)));
-    if (off > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
+    if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
+    const bool fact = kind == kKindFactored, row = fact && G.rowpath;
 
     // ---- device address of the fixed array on the current device ---------------------
     int dev = 0;
@@ -176,18 +207,20 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     td.v = v;
     td.R = R;
     td.C = Cc;
-    td.rowp = fact && !row ? (float *)(base + o_rowp) : nullptr;
-    td.colp = fact && !row ? (float *)(base + o_colp) : nullptr;
-    td.bsc = fact ? (float *)(base + o_bsc) : nullptr;
-    td.rsum = fact ? (double *)(base + o_rsum) : nullptr;
-    td.pp = row ? (float2 *)(base + o_pp) : nullptr;
-    td.rmin = row ? (float *)(base + o_rmin) : nullptr;
-    td.fsum = row ? (double *)(base + o_fsum) : nullptr;
-    td.fmin = row ? (float *)(base + o_fmin) : nullptr;
-    td.u2 = (float2 *)(base + o_u2);
+    td.rowp = fact && !row ? (float *)(base + o.rowp) : nullptr;
+    td.colp = fact && !row ? (float *)(base + o.colp) : nullptr;
+    td.bsc = fact ? (float *)(base + o.bsc) : nullptr;
+    td.rsum = fact ? (double *)(base + o.rsum) : nullptr;
+    td.pp = row ? (float2 *)(base + o.pp) : nullptr;
+    td.rmin = row ? (float *)(base + o.rmin) : nullptr;
+    td.fsum = row ? (double *)(base + o.fsum) : nullptr;
+    td.fmin = row ? (float *)(base + o.fmin) : nullptr;
+    td.u2 = (float2 *)(base + o.u2);
     td.n = n;
     td.m = m;
     td.numel = numel;
+    td.inv_n = 1.0 / (double)n;
+    td.inv_numel = 1.0 / (double)numel;
     td.tid = tensor_id;
     td.kind = kind;
     td.momentum = momentum;
@@ -215,10 +248,10 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     // ---- per-step scalars, as skew_step forms them ------------------------------------
     const StepCoefs k = step_coefs(H, step);
     StepArgs a{};
-    a.tensors = (const TensorDev *)(base + o_tens);
-    a.scal = (TensorScal *)(base + o_scal);
-    a.err = (uint32_t *)(base + o_err);
-    a.fb = (uint32_t *)(base + o_fb);
+    a.tensors = (const TensorDev *)(base + o.tens);
+    a.scal = (TensorScal *)(base + o.scal);
+    a.err = (uint32_t *)(base + kErrOffset);
+    a.fb = (uint32_t *)(base + o.fb);
     a.b1 = H.beta1;
     a.b2 = k.b2;
     a.c1 = (float)(1.0 - (double)H.beta1);
@@ -241,25 +274,25 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     }
 
     cudaStream_t s = (cudaStream_t)stream;
-    SetupTables tb{(uint2 *)(base + o_iA), nA, (uint2 *)(base + o_iR), nR, (uint2 *)(base + o_iF), nF,
-                   (uint2 *)(base + o_iB), nB, (uint2 *)(base + o_iC), nC, (uint2 *)(base + o_iCR), nCR};
-    k_noalloc_setup<<<8, 256, 0, s>>>(td, (TensorDev *)(base + o_tens), (TensorScal *)(base + o_scal),
-                                      (uint32_t *)(base + o_fb), tb);
+    SetupTables tb{(uint2 *)(base + o.iA), o.nA, (uint2 *)(base + o.iR), o.nR, (uint2 *)(base + o.iF), o.nF,
+                   (uint2 *)(base + o.iB), o.nB, (uint2 *)(base + o.iC), o.nC, (uint2 *)(base + o.iCR), o.nCR};
+    k_noalloc_setup<<<8, 256, 0, s>>>(td, (TensorDev *)(base + o.tens), (TensorScal *)(base + o.scal),
+                                      (uint32_t *)(base + o.fb), tb);
     e = cudaGetLastError();
     if (e != cudaSuccess) return SKEW_ECUDA;
-    const LaunchPlan lp{nA,
-                        nR,
-                        nF,
-                        nB,
+    const LaunchPlan lp{o.nA,
+                        o.nR,
+                        o.nF,
+                        o.nB,
                         nFB,
-                        nC,
-                        nCR,
-                        (const uint2 *)(base + o_iA),
-                        (const uint2 *)(base + o_iR),
-                        (const uint2 *)(base + o_iF),
-                        (const uint2 *)(base + o_iB),
-                        (const uint2 *)(base + o_iC),
-                        (const uint2 *)(base + o_iCR)};
+                        o.nC,
+                        o.nCR,
+                        (const uint2 *)(base + o.iA),
+                        (const uint2 *)(base + o.iR),
+                        (const uint2 *)(base + o.iF),
+                        (const uint2 *)(base + o.iB),
+                        (const uint2 *)(base + o.iC),
+                        (const uint2 *)(base + o.iCR)};
     e = (cudaError_t)launch_phases(a, lp, stream, nullptr);
     if (e != cudaSuccess) return SKEW_ECUDA;
     return SKEW_OK;

@@ -39,9 +39,22 @@ constexpr int kRowStages = 3;
 // launch's last wave ends sooner. An item's tile field then carries kHalfTile, plus
 // kSecondHalf for the second half (results do not depend on the split).
 constexpr uint32_t kApplyTailSplit = 2u * 2u * 152u;
+constexpr int64_t kSplitTileBytes = 512 << 10;  // smaller tiles (of W) stay whole
 constexpr uint32_t kHalfTile = 1u << 31, kSecondHalf = 1u << 30, kTileMask = kSecondHalf - 1u;
 constexpr int kMomGBytes = 16384;
 constexpr int kMomChunks = 64;
+
+// Row path of the widths m = 8 V in [kAnyMin, kAnyMax] that are not 512, 1024, 2048 or 4096
+// (rowsq_gen_tile, apply_flat_tile): rows per thread and phase-A chunk at NV vectors per
+// thread and row, and the floats of shared memory that hold phase C's scales.
+// Below 256 columns a row fills less than a warp, and above 4096 the column sums of a row do
+// not fit the registers of two 256-thread CTAs per SM: both stay on the strip tiles. Against
+// the strip tiles (three reads of G): 930M parameters in 3072 x 1536 experts 1872 -> 1259 us.
+enum RowPath : uint32_t { kRowNone = 0, kRowFixed = 1, kRowAny = 2 };
+constexpr int64_t kAnyMin = 256, kAnyMax = 4096;
+constexpr int64_t kAnyTileBytes = 1 << 20;  // bf16 bytes of a tile in phases A and C, as of the fixed widths
+constexpr int kFlatScales = 4200;
+__host__ __device__ constexpr int gen_rows_per_thread(int nv, bool mom) { return (nv == 1 ? 8 : 4) / (mom ? 2 : 1); }
 
 enum Kind : uint32_t { kKindFull = 0, kKindFactored = 1 };
 
@@ -98,14 +111,43 @@ inline StepCoefs step_coefs(const skew_hparams_t &H, int64_t step) {
 struct TileGeom {
     uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0;
     uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0;
-    uint32_t at_rows = 0, atiles = 0;  // row path: phase-C row tiles (momentum tensors: the phase-A tiles)
+    uint32_t at_rows = 0, atiles = 0;  // row path: phase-C row tiles
     uint32_t fci = 0;  // row path: columns per finalize item (kFinChunk / fci threads per column)
 };
 
+constexpr int64_t kWholeGroup = int64_t(1) << 60;  // as `rest`: full-sized tiles
+
+// Chunks (of `chunk` bytes) in the row tiles of a matrix of `own` bytes when the step's row-path
+// matrices from it on, in launch order, hold `rest` bytes: `most` while that gives `waves` waves of
+// two CTAs on each of the 152 SMs or more, then ever smaller tiles, so that the launch's last tiles
+// end together and a small step still fills the chip, down to `least`. 680M parameters with momentum
+// on the experts 1960 -> 1881 us (k_rowsq 1080 -> 1021, k_apply_rows 811 -> 775 us); 850M without
+// 1205 -> 1172 us (k_rowsq 350 -> 321); the 6.78B set 8377 -> 8358. Phase A takes one wave without
+// momentum (a second one costs the finalize more partials than it saves: k_rowsq 331, not 321) and
+// two with it, phase C three. `parts`: tiles a matrix may have before its column partials would outgrow the
+// no-alloc scratch; it then keeps to one wave of tiles, up to twice `most` each.
+inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_t chunk, int64_t least, int64_t most,
+                                int64_t parts) {
+    const int64_t ctas = 2 * 152;
+    auto per = [chunk](int64_t bytes, int64_t tiles) { return (bytes + tiles * chunk - 1) / (tiles * chunk); };
+    int64_t t = per(rest, ctas * waves);
+    t = t < least ? least : t > most ? most : t;
+    if (parts && rest < kWholeGroup && own > t * chunk * parts && own <= 2 * most * chunk * ctas) t = per(own, ctas);
+    return (uint32_t)t;
+}
+
+// Below this many bytes of G in all the matrices that only kRowAny serves, its three launches beside
+// the strip tiles' four cost a step more than the second read of G that they save: with one such
+// matrix of 8 MB among small ones (24 ragged tensors) 242 us against 214, with 320 MB among fixed
+// widths (a 2048-wide model) 435 us against 499.
+constexpr int64_t kAnyGroupBytes = 16 << 20;
+
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
-// gradient pointers are 16-byte aligned. Counts fit 32 bits for n, m <= 2^40
+// gradient pointers are 16-byte aligned; `rest`: bytes of G of the step's row-path
+// matrices from this one on. Counts fit 32 bits for n, m <= 2^40
 // and n*m <= 2^62 only when the caller has checked the tile count (planner).
-inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, int64_t n, int64_t m, int64_t numel) {
+inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, int64_t n, int64_t m, int64_t numel,
+                              int64_t rest) {
     TileGeom g;
     if (kind == kKindFactored) {
         const int64_t vecs = (m + 7) / 8;  // 8-column groups per row
@@ -120,13 +162,33 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
         g.ntiles = g.strips * g.rowtiles;
         g.nfc = (uint32_t)((m + kFinChunk - 1) / kFinChunk);
         // Whole-row phases A and C: factored matrices of width 512, 1024, 2048
-        // or 4096 (64 to 512 16-byte vectors per row), with or without momentum.
-        g.rowpath = (wg_aligned && (m == 512 || m == 1024 || m == 2048 || m == 4096)) ? 1u : 0u;
+        // or 4096 (64 to 512 16-byte vectors per row), with or without momentum, and
+        // (kRowAny) every other multiple of 8 between kAnyMin and kAnyMax.
+        const bool fixed = m == 512 || m == 1024 || m == 2048 || m == 4096;
+        g.rowpath = !wg_aligned ? kRowNone
+                    : fixed     ? kRowFixed
+                    : (m % 8 == 0 && m >= kAnyMin && m <= kAnyMax) ? kRowAny : kRowNone;
         if (g.rowpath) {
-            g.cr = (uint32_t)((momentum ? kMomGBytes : kRowChunkBytes) / (2 * m));
-            g.rt_rows = g.cr * (momentum ? kMomChunks : m == 4096 && n >= 2048 ? kRowChunksWide : kRowChunks);
+            const int64_t own = 2 * numel;
+            if (g.rowpath == kRowFixed) {
+                const int64_t chunk = momentum ? kMomGBytes : kRowChunkBytes;
+                g.cr = (uint32_t)(chunk / (2 * m));
+                const int64_t most = momentum ? kMomChunks : m == 4096 && n >= 2048 ? kRowChunksWide : kRowChunks;
+                g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, 65536 / chunk, most, (12 << 20) / (8 * m));
+                const uint32_t at = row_tile_chunks(own, rest, 3, chunk, 32768 / chunk, (1 << 20) / chunk, 0);
+                g.at_rows = g.cr * (momentum ? (at + 1) / 2 * 2 : at);  // a half tile is whole phase-C chunks
+            } else {
+                const int nv = m > 2048 ? 2 : 1;
+                const int64_t wpr = (m / 8 + 32 * nv - 1) / (32 * nv);
+                g.cr = (uint32_t)(gen_rows_per_thread(nv, momentum != 0) * (8 / wpr));
+                const int64_t chunk = 2 * m * g.cr, least = 65536 / chunk;
+                g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, least < 1 ? 1 : least, kAnyTileBytes / chunk,
+                                                   (12 << 20) / (8 * m));
+                int64_t at = 2 * row_tile_chunks(own, rest, 3, 4 * m, (32768 + 4 * m - 1) / (4 * m), kAnyTileBytes / (4 * m), 0);
+                if (at > kFlatScales - m) at = kFlatScales - m;
+                g.at_rows = (uint32_t)(at / 2 * 2);
+            }
             g.rtiles = (uint32_t)((n + g.rt_rows - 1) / g.rt_rows);
-            g.at_rows = momentum ? g.rt_rows : g.cr * kRowChunks;
             g.atiles = (uint32_t)((n + g.at_rows - 1) / g.at_rows);
             g.nfr = 0;
             // tall matrices: up to 8 threads share a column, each adding every 8th tile
@@ -172,6 +234,7 @@ struct TensorDev {
     float2 *u2;         // sums of (U / coef)^2 as (hi, lo) pairs: per phase-B tile [ntiles], or on the
                         // row path per half of a phase-C tile [2 atiles] (u2_len)
     int64_t n, m, numel;
+    double inv_n, inv_numel;  // 1 / n, 1 / numel
     uint32_t tid;       // dither tensor id
     uint64_t base;      // dither index of element 0 (a matrix of a stacked tensor: its offset)
     uint32_t kind, momentum, decay;
@@ -183,12 +246,12 @@ struct TensorDev {
     uint32_t tile_rows; // factored: rows per tile = 32 * (256 / LC)
     uint32_t ntiles;    // update tiles of this tensor
     uint32_t nfr, nfc;  // factored: finalize items over rows / columns
-    uint32_t rowpath;   // 1: whole-row phase A (k_rowsq) and the bilinear sum of U^2
+    uint32_t rowpath;   // RowPath; nonzero: whole-row phase A (k_rowsq) and the bilinear sum of U^2
     uint32_t cr;        // row path: rows per chunk
     uint32_t rt_rows;   // row path: rows per phase-A row tile
     uint32_t rtiles;    // row path: phase-A row tiles
     uint32_t fci;       // row path: columns per finalize item
-    uint32_t at_rows;   // row path: rows per phase-C row tile (<= 1024)
+    uint32_t at_rows;   // row path: rows per phase-C row tile (<= 1024 at the fixed widths)
     uint32_t atiles;    // row path: phase-C row tiles
 };
 

@@ -1,0 +1,62 @@
+"""Whole-row tiles at widths other than 512, 1024, 2048 and 4096 (any multiple of 8 from 256 to 4096),
+against the oracle: the narrowest and widest, widths whose rows take 1 to 8 warps and one or two
+vectors per thread, ragged last tiles and chunks, one-row matrices, stacks, with and without momentum."""
+import pytest
+import torch
+
+from paper_2607_19058_gb300 import skewadam as S
+from paper_2607_19058_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+E, B = WL.TIER_EXPERT, WL.TIER_BACKBONE
+#          rows, width: 64-row chunks; 2 warps a row; 5 of 8 warps; a partial last warp; 1 row side by side;
+#          two vectors a thread, the second for few lanes; three quarters of the warps; the widest
+SHAPES = [(2113, 256), (1, 256), (700, 264), (333, 776), (517, 1032), (131, 1408), (9, 2040), (130, 2056), (257, 2880),
+          (301, 3072), (5, 4088), (267, 4088)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2607_19058_gb300 import _build
+    _build.build()
+    import oracle
+    oracle.build()
+
+
+def _workload():
+    specs = [WL.Spec(f"{'eb'[t]}{n}x{m}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1)
+             for k, (n, m) in enumerate(SHAPES) for t in (0, 1)]
+    specs += [WL.Spec("se", (3, 130, 1536), E), WL.Spec("sb", (2, 67, 768), B)]
+    return WL.Workload("widths", specs, WL.HP(), "toy", steps=3)
+
+
+@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05)], ids=["eps1e-30", "paper"])
+def test_any_width_rows(hp):
+    """eps = 1e-8 binds the clamp at step 1; experts 5 to 7 have zero gradients on odd steps."""
+    import parity
+    h = parity.Harness(_workload(), hp_override=hp)
+    for t in range(1, 4):
+        h.step(t, seed=17 * t, **({"gscale": 0.37} if t == 2 else {}))
+    h.opt.sync_status()
+    h.close()
+
+
+@pytest.mark.parametrize("shape,tier", [((700, 264), E), ((517, 1032), B), ((301, 3072), E), ((2049, 1408), E)])
+def test_noalloc_matches_the_handle(shape, tier):
+    torch.manual_seed(0)
+    w0 = (torch.randn(shape, device="cuda") * 0.02).to(torch.bfloat16)
+    g = torch.empty(shape, dtype=torch.bfloat16, device="cuda")
+    hp = S.hparams(0.9, 0.999, 1e-30, 1.0, 0.1, S.POLICY_TIERED)
+    w_ref, w_na = w0.clone(), w0.clone()
+    ref = S.SkewAdam([(w_ref, g, tier)], hp)
+    state = torch.zeros(ref.state_bytes // 4, dtype=torch.float32, device="cuda")
+    for t in (1, 2):
+        g.copy_((torch.randn(shape, device="cuda") * 1e-3).to(torch.bfloat16))
+        ref.step(t, 1e-3, 77)
+        S.skew_step_tensor_noalloc(w_na.data_ptr(), g.data_ptr(), 2, shape[0], shape[1], tier, 0, hp, state.data_ptr(),
+                                   ref.state_bytes, 0, t, 1e-3, 77, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert torch.equal(w_ref.view(torch.int16), w_na.view(torch.int16))
+        assert torch.equal(ref.state[: ref.state_bytes].view(torch.float32), state)
+    ref.close()
