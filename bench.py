@@ -147,8 +147,12 @@ def byte_model(opt, n_tensors):
     """Algorithmic minimum bytes of one step and of each kernel's own traffic."""
     N = N_mom = N_full = N_fact = N_nomom = N_row = N_rowm = 0
     rc = rc_row = 0
-    for k in range(n_tensors):
-        i = opt.info(k)
+    infos = [opt.info(k) for k in range(n_tensors)]
+    # whole-row tiles: the fixed widths, and any multiple of 8 from 256 to 4096 where such matrices
+    # hold 2 MiB of gradient or more
+    other = [i for i in infos if i.kind == 1 and not i.rowpath and i.vectorized and 256 <= i.cols <= 4096]
+    any_width = 2 * sum(i.numel for i in other) >= 2 << 20
+    for i in infos:
         E = max(1, i.stack)  # a stack of E matrices: rows / cols are one matrix's
         N += i.numel
         if i.momentum:
@@ -157,7 +161,7 @@ def byte_model(opt, n_tensors):
             N_nomom += i.numel
         if i.kind == 0:
             N_full += i.numel
-        elif i.rowpath:
+        elif i.rowpath or (any_width and i.vectorized and 256 <= i.cols <= 4096):
             N_row += i.numel
             N_rowm += i.numel if i.momentum else 0
             rc_row += E * (i.rows + i.cols)
@@ -166,14 +170,22 @@ def byte_model(opt, n_tensors):
             rc += E * (i.rows + i.cols)
     step_min = 6 * N + 8 * N_mom + 8 * N_full + 8 * (rc + rc_row)
     N_rest = N - N_row  # tensors of the strip / flat tiles
+    mom_rest = N_mom - N_rowm
+    mom_full = sum(i.numel for i in infos if i.kind == 0 and i.momentum)
+    sumsq = 2 * N_fact                                            # read G of strip-path factored matrices
+    rms_full = 2 * N_full + 8 * mom_full + 8 * N_full             # read G; M, v read + write
+    rms_fact = 2 * N_fact + 8 * (mom_rest - mom_full)
+    apply = 4 * N_rest + 2 * (N_nomom - (N_row - N_rowm)) + 4 * mom_rest + 4 * N_full
+    rows = N_row > 0  # the row path's launches then run the strip and flat tiles too
     kernels = {
-        "k_sumsq": 2 * N_fact,                                   # read G of strip-path factored matrices
-        "k_rowsq": 2 * N_row + 8 * N_rowm + 8 * rc_row,          # read G (and M r/w) of row-path matrices; R r/w
+        "k_sumsq": 0 if rows else sumsq,
+        # read G (and M r/w) of row-path matrices; R r/w
+        "k_rowsq": 2 * N_row + 8 * N_rowm + 8 * rc_row + (sumsq + rms_full if rows else 0),
         "k_finalize": 8 * (rc + rc_row),                         # R, C read + write
-        "k_rms": 2 * N_rest + 8 * (N_mom - N_rowm) + 8 * N_full,  # read G; M, v read + write
-        "k_fallback": 0,                                          # runs only when a clamp may bind
-        "k_apply": 4 * N_rest + 2 * (N_nomom - (N_row - N_rowm)) + 4 * (N_mom - N_rowm) + 4 * N_full,
-        "k_apply_rows": 6 * N_row - 2 * N_rowm + 4 * N_rowm,     # W r/w and G (or the new M) read
+        "k_rms": 0 if rows else rms_full + rms_fact,
+        "k_fallback": rms_fact if rows else 0,                    # and phase B of queued row-path tensors
+        "k_apply": 0 if rows else apply,
+        "k_apply_rows": 6 * N_row - 2 * N_rowm + 4 * N_rowm + (apply if rows else 0),  # W r/w and G (or the new M) read
     }
     return dict(N=N, N_mom=N_mom, N_full=N_full, rc=rc, step_min=step_min, kernels=kernels)
 

@@ -54,8 +54,9 @@ struct skew_handle {
     std::vector<uint32_t> first, count;    // per descriptor: its first plan and how many
     size_t state_bytes = 0, ws_bytes = 0;
     size_t ws_scal = 0, ws_fb = 0, ws_err = 0, ws_tab = 0, ws_tab_end = 0;
-    size_t ws_tens = 0, ws_itemsA = 0, ws_itemsR = 0, ws_itemsF = 0, ws_itemsB = 0, ws_itemsC = 0, ws_itemsCR = 0;
-    std::vector<uint2> itemsA, itemsR, itemsF, itemsB, itemsC, itemsCR;  // per phase, tensors in order
+    size_t ws_tens = 0, ws_itemsA = 0, ws_itemsF = 0, ws_itemsB = 0, ws_itemsC = 0;
+    std::vector<uint2> itemsA, itemsF, itemsB, itemsC;  // A + R, F, B, C + CR: per phase, tensors in order
+    uint32_t nA = 0, nC = 0;  // items of A before those of R, of C before those of CR
     uint32_t n_rowpath = 0;  // tensors on the row path
     uint32_t fb_ctas = 0;    // CTAs of the row path's phase-B launch (set at bind)
     char *state = nullptr, *ws = nullptr;
@@ -69,7 +70,7 @@ struct skew_handle {
     }
 };
 
-// What the profiler times per step: the grouped launches (an empty phase times ~0).
+// What the profiler times per step: the grouped launches (one that the step does not make times ~0).
 constexpr int kProfLaunches = kLaunches;
 const char *const kProfNames[kProfLaunches] = {"k_sumsq", "k_rowsq",  "k_finalize", "k_rms",
                                                "k_fallback", "k_apply", "k_apply_rows"};
@@ -228,28 +229,32 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     // Item tables: every factored tensor's tiles (phase A), finalize items
     // (phase F) and every tensor's tiles (phases B and C), tensors in order.
     try {
+        std::vector<uint2> itemsR, itemsCR;
+        auto all = [](std::vector<uint2> &v, int q, uint32_t n) {
+            for (uint32_t i = 0; i < n; ++i) v.push_back(make_uint2(q, i));
+        };
         for (int q = 0; q < n_plans; ++q) {
             const TPlan &p = h->t[q];
-            if (p.kind == kKindFactored) {
-                if (p.rowpath)
-                    for (uint32_t i = 0; i < p.rtiles; ++i) h->itemsR.push_back(make_uint2(q, i));
-                else
-                    for (uint32_t i = 0; i < p.ntiles; ++i) h->itemsA.push_back(make_uint2(q, i));
-                for (uint32_t i = 0; i < p.nfr + p.nfc; ++i) h->itemsF.push_back(make_uint2(q, i));
-            }
+            const bool fact = p.kind == kKindFactored;
             if (p.rowpath) {
-                for (uint32_t i = 0; i < p.atiles; ++i) h->itemsCR.push_back(make_uint2(q, i));
+                all(itemsR, q, p.rtiles);
+                all(itemsCR, q, p.atiles);
             } else {
-                for (uint32_t i = 0; i < p.ntiles; ++i) h->itemsB.push_back(make_uint2(q, i));
-                for (uint32_t i = 0; i < p.ntiles; ++i) h->itemsC.push_back(make_uint2(q, i));
+                if (fact) all(h->itemsA, q, p.ntiles);
+                // flat tiles of phase B need no earlier phase: with row tiles they go with phase A
+                all(!fact && h->n_rowpath ? h->itemsA : h->itemsB, q, p.ntiles);
+                all(h->itemsC, q, p.ntiles);
             }
+            if (fact) all(h->itemsF, q, p.nfr + p.nfc);
         }
+        h->nA = (uint32_t)h->itemsA.size();
+        h->nC = (uint32_t)h->itemsC.size();
         // the last phase-C row tiles run as two half tiles each (small tiles and tile indices past
         // the mask keep whole tiles)
         std::vector<uint2> tail;
-        const size_t ncr = h->itemsCR.size(), nsplit = std::min<size_t>(ncr, kApplyTailSplit);
+        const size_t ncr = itemsCR.size(), nsplit = std::min<size_t>(ncr, kApplyTailSplit);
         for (size_t k = ncr - nsplit; k < ncr; ++k) {
-            const uint2 it = h->itemsCR[k];
+            const uint2 it = itemsCR[k];
             const TPlan &p = h->t[it.x];
             if (2 * p.m * p.at_rows >= kSplitTileBytes && it.y <= kTileMask) {
                 tail.push_back(make_uint2(it.x, it.y | kHalfTile));
@@ -258,8 +263,10 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 tail.push_back(it);
             }
         }
-        h->itemsCR.resize(ncr - nsplit);
-        h->itemsCR.insert(h->itemsCR.end(), tail.begin(), tail.end());
+        itemsCR.resize(ncr - nsplit);
+        itemsCR.insert(itemsCR.end(), tail.begin(), tail.end());
+        h->itemsA.insert(h->itemsA.end(), itemsR.begin(), itemsR.end());
+        h->itemsC.insert(h->itemsC.end(), itemsCR.begin(), itemsCR.end());
     } catch (...) {
         delete h;
         return fail(nullptr, SKEW_ENOMEM, "out of host memory");
@@ -282,11 +289,9 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         w = align_up(w + sizeof(uint2) * v.size(), 256);
     };
     table(h->ws_itemsA, h->itemsA);
-    table(h->ws_itemsR, h->itemsR);
     table(h->ws_itemsF, h->itemsF);
     table(h->ws_itemsB, h->itemsB);
     table(h->ws_itemsC, h->itemsC);
-    table(h->ws_itemsCR, h->itemsCR);
     h->ws_tab_end = w;
     for (auto &p : h->t) {
         if (p.kind == kKindFactored && !p.rowpath) {
@@ -323,9 +328,9 @@ int32_t skew_num_tensors(const skew_handle_t *h) { return h ? (int32_t)h->desc.s
 
 int64_t skew_launches_per_step(const skew_handle_t *h) {
     if (!h) return 0;
-    return int64_t(!h->itemsA.empty()) + int64_t(!h->itemsR.empty()) + int64_t(!h->itemsF.empty()) +
-           int64_t(!h->itemsB.empty()) + int64_t(h->n_rowpath > 0) + int64_t(!h->itemsC.empty()) +
-           int64_t(!h->itemsCR.empty());
+    if (h->n_rowpath) return 4;  // k_rowsq, k_finalize, k_fallback, k_apply_rows
+    return int64_t(!h->itemsA.empty()) + int64_t(!h->itemsF.empty()) + int64_t(!h->itemsB.empty()) +
+           int64_t(!h->itemsC.empty());
 }
 
 const char *skew_last_error(const skew_handle_t *h) { return h ? h->err.c_str() : g_create_err.c_str(); }
@@ -427,11 +432,9 @@ int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace
         if (!v.empty()) std::memcpy(img.data() + (at - h->ws_tab), v.data(), v.size() * sizeof(uint2));
     };
     put(h->ws_itemsA, h->itemsA);
-    put(h->ws_itemsR, h->itemsR);
     put(h->ws_itemsF, h->itemsF);
     put(h->ws_itemsB, h->itemsB);
     put(h->ws_itemsC, h->itemsC);
-    put(h->ws_itemsCR, h->itemsCR);
 
     cudaError_t e;
     if (!img.empty()) {
@@ -504,10 +507,9 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
     cudaError_t e = cudaMemsetAsync(h->ws + h->ws_scal, 0, h->ws_fb + 4 - h->ws_scal, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "reset of per-step scalars");
     auto items = [&](size_t at) { return reinterpret_cast<const uint2 *>(h->ws + at); };
-    const LaunchPlan L{(uint32_t)h->itemsA.size(), (uint32_t)h->itemsR.size(), (uint32_t)h->itemsF.size(),
-                       (uint32_t)h->itemsB.size(), h->n_rowpath ? h->fb_ctas : 0u, (uint32_t)h->itemsC.size(),
-                       (uint32_t)h->itemsCR.size(), items(h->ws_itemsA), items(h->ws_itemsR), items(h->ws_itemsF),
-                       items(h->ws_itemsB), items(h->ws_itemsC), items(h->ws_itemsCR)};
+    const LaunchPlan L{h->nA, (uint32_t)h->itemsA.size() - h->nA, (uint32_t)h->itemsF.size(), (uint32_t)h->itemsB.size(),
+                       h->n_rowpath ? h->fb_ctas : 0u, h->nC, (uint32_t)h->itemsC.size() - h->nC,
+                       items(h->ws_itemsA), items(h->ws_itemsF), items(h->ws_itemsB), items(h->ws_itemsC)};
     e = (cudaError_t)launch_phases(a, L, s, reinterpret_cast<void *const *>(ev));
     if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch");
     return SKEW_OK;

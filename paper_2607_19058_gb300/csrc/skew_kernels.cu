@@ -1,7 +1,9 @@
 // Device kernels of libskewadam (sm_103a).
 //
-// One SkewAdam step (paper Sec. 3, Eq. 1, Algorithm 1) as seven grouped launches in
-// stream order, each over an item table of (tensor, tile) pairs:
+// One SkewAdam step (paper Sec. 3, Eq. 1, Algorithm 1) as grouped launches in stream
+// order, each over an item table of (tensor, tile) pairs; a step with row-path tensors
+// takes k_rowsq, k_finalize, k_fallback and k_apply_rows, which also run its strip and flat
+// tiles, any other k_sumsq, k_finalize, k_rms and k_apply:
 //   k_sumsq      phase A, strip tiles: per-row and per-column sums of g^2 of a
 //                factored matrix (Eq. 1), column partials per row tile (no atomics);
 //   k_rowsq      phase A, whole-row tiles of factored matrices 512 to 4096 wide:
@@ -1312,20 +1314,11 @@ __device__ Acc2 rms_full_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
     return acc;
 }
 
-__device__ void phase_B(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, const Meta &meta, const Pol &pol) {
+// Stores a phase-B tile's sum of (U / coef)^2; the last tile of the tensor forms sum(U^2), RMS and
+// the clip factor (fixed summation order).
+__device__ void finish_B(const StepArgs &A, uint32_t t, uint32_t local, const Acc2 &acc, Smem &sm) {
     const TensorDev &T = A.tensors[t];
     TensorScal &S = A.scal[t];
-    Acc2 acc;
-    if (T.kind == kKindFactored) {
-        if (T.vec)
-            acc = T.momentum ? rms_fact_tile<true, true>(A, T, local, meta, pol)
-                             : rms_fact_tile<true, false>(A, T, local, meta, pol);
-        else
-            acc = T.momentum ? rms_fact_tile<false, true>(A, T, local, meta, pol)
-                             : rms_fact_tile<false, false>(A, T, local, meta, pol);
-    } else {
-        acc = T.vec ? rms_full_tile<true>(A, T, local, pol) : rms_full_tile<false>(A, T, local, pol);
-    }
     const float2 tsum = block_sum2(acc, sm.red2);
     if (threadIdx.x == 0) {
         T.u2[local] = tsum;
@@ -1333,7 +1326,6 @@ __device__ void phase_B(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm,
     }
     __syncthreads();
     if (!sm.last) return;
-    // Last tile of the tensor: sum(U^2), RMS, clip factor (fixed summation order).
     double s = 0.0;
     for (uint32_t k = threadIdx.x; k < T.ntiles; k += kThreads) {
         const float2 p = __ldcg(T.u2 + k);
@@ -1341,6 +1333,25 @@ __device__ void phase_B(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm,
     }
     s = block_sum_d(s, sm.redd);
     if (threadIdx.x == 0) set_clip(A, T, S, s);
+}
+
+__device__ void phase_B_full(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, const Pol &pol) {
+    const TensorDev &T = A.tensors[t];
+    const Acc2 acc = T.vec ? rms_full_tile<true>(A, T, local, pol) : rms_full_tile<false>(A, T, local, pol);
+    finish_B(A, t, local, acc, sm);
+}
+
+__device__ void phase_B_fact(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+    const TensorDev &T = A.tensors[t];
+    (void)fill_meta(T, A.scal[t], local, A.ce, meta);
+    Acc2 acc;
+    if (T.vec)
+        acc = T.momentum ? rms_fact_tile<true, true>(A, T, local, meta, pol)
+                         : rms_fact_tile<true, false>(A, T, local, meta, pol);
+    else
+        acc = T.momentum ? rms_fact_tile<false, true>(A, T, local, meta, pol)
+                         : rms_fact_tile<false, false>(A, T, local, meta, pol);
+    finish_B(A, t, local, acc, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -2566,19 +2577,58 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
 // parameter (constant bank), so the dither keys and step scalars are uniform
 // operands of every warp.
 // ---------------------------------------------------------------------------
+__device__ void phase_A_strip(const TensorDev &T, uint32_t tile, Smem &sm, const Pol &pol) {
+    if (T.vec)
+        sumsq_tile<true>(T, tile, sm, pol);
+    else
+        sumsq_tile<false>(T, tile, sm, pol);
+}
+
+// Phase C of a strip or flat tile.
+__device__ void phase_C(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
+                        const Pol &pol) {
+    if (T.kind == kKindFactored) {
+        const bool fast = fill_meta(T, S, tile, A.ce, meta);
+        if (T.vec) {
+            if (T.momentum) {
+                if (fast)
+                    apply_fact_tile<true, true, true>(A, T, S, tile, meta, pol);
+                else
+                    apply_fact_tile<true, true, false>(A, T, S, tile, meta, pol);
+            } else {
+                if (fast)
+                    apply_fact_tile<true, false, true>(A, T, S, tile, meta, pol);
+                else
+                    apply_fact_tile<true, false, false>(A, T, S, tile, meta, pol);
+            }
+        } else {
+            if (T.momentum)
+                apply_fact_tile<false, true, false>(A, T, S, tile, meta, pol);
+            else
+                apply_fact_tile<false, false, false>(A, T, S, tile, meta, pol);
+        }
+    } else {
+        if (T.vec)
+            apply_full_tile<true>(A, T, S, tile, pol);
+        else
+            apply_full_tile<false>(A, T, S, tile, pol);
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_SUMSQ)
     k_sumsq(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Smem sm;
-    const Pol pol;
     const uint2 it = items[blockIdx.x];
-    const TensorDev &T = A.tensors[it.x];
-    if (T.vec)
-        sumsq_tile<true>(T, it.y, sm, pol);
-    else
-        sumsq_tile<false>(T, it.y, sm, pol);
+    phase_A_strip(A.tensors[it.x], it.y, sm, Pol());
 }
 
-// Row path, phase A: one row tile per CTA (dynamic shared memory: RowSmem).
+// A step with row-path tensors runs its strip and flat tiles in the row path's launches, ahead of
+// the row tiles: phase B of the flat tiles needs nothing from phase A or the finalize, so it comes
+// with phase A. Such a step has four launches instead of seven, and the light tiles' latency (a
+// launch of its own took 12 to 25 us each for phases A, B and C) hides behind the row tiles.
+
+// Row path, phase A: one row tile per CTA (dynamic shared memory: RowSmem), and before them the
+// phase-A strip tiles and phase-B flat tiles.
 __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     k_rowsq(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
@@ -2586,6 +2636,14 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     const uint2 it = items[blockIdx.x];
     const TensorDev &T = A.tensors[it.x];
     TensorScal &S = A.scal[it.x];
+    if (T.rowpath == kRowNone) {
+        Smem &ss = *reinterpret_cast<Smem *>(dyn_smem);
+        if (T.kind == kKindFactored)
+            phase_A_strip(T, it.y, ss, Pol());
+        else
+            phase_B_full(A, it.x, it.y, ss, Pol());
+        return;
+    }
     if (T.rowpath == kRowAny) {
         GenSmem &gs = *reinterpret_cast<GenSmem *>(dyn_smem);
         const bool wide = T.m > 2048;
@@ -2620,7 +2678,8 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     }
 }
 
-// Row path, phase C: one row tile per CTA (dynamic shared memory: ApplyRowSmem).
+// Row path, phase C: one row tile per CTA (dynamic shared memory: ApplyRowSmem), and before them
+// the phase-C strip and flat tiles.
 __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     k_apply_rows(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
@@ -2628,6 +2687,10 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     const uint2 it = items[blockIdx.x];
     const TensorDev &T = A.tensors[it.x];
     TensorScal &S = A.scal[it.x];
+    if (T.rowpath == kRowNone) {
+        phase_C(A, T, S, it.y, *reinterpret_cast<Meta *>(dyn_smem), Pol());
+        return;
+    }
     if (T.rowpath == kRowAny) {
         FlatSmem &fs = *reinterpret_cast<FlatSmem *>(dyn_smem);
         if (T.momentum)
@@ -2657,19 +2720,23 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
 // Phase B of the row-path tensors whose finalize found that a clamp may bind
 // (queued in A.fb): the CTAs of this grid share the tiles of all queued tensors, laid end to end
 // (starting every tensor at CTA 0 would give the first CTAs a tile of each small one).
-__global__ void __launch_bounds__(kThreads, 2) k_fallback(const __grid_constant__ StepArgs A) {
+// The first nB CTAs run the phase-B strip tiles of the other tensors.
+__global__ void __launch_bounds__(kThreads, 2)
+    k_fallback(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items, uint32_t nB) {
     __shared__ Smem sm;
     __shared__ Meta meta;
     const Pol pol;
-    const uint32_t cnt = __ldcg(A.fb);
-    uint32_t tile = blockIdx.x;  // of queued tensor q
+    if (blockIdx.x < nB) {
+        const uint2 it = items[blockIdx.x];
+        phase_B_fact(A, it.x, it.y, sm, meta, pol);
+        return;
+    }
+    const uint32_t cnt = __ldcg(A.fb), ctas = gridDim.x - nB;
+    uint32_t tile = blockIdx.x - nB;  // of queued tensor q
     for (uint32_t q = 0; q < cnt; ++q) {
-        const uint32_t t = __ldcg(A.fb + 1 + q);
-        const TensorDev &T = A.tensors[t];
-        const uint32_t nt = T.ntiles;
-        for (; tile < nt; tile += gridDim.x) {
-            (void)fill_meta(T, A.scal[t], tile, A.ce, meta);
-            phase_B(A, t, tile, sm, meta, pol);
+        const uint32_t t = __ldcg(A.fb + 1 + q), nt = A.tensors[t].ntiles;
+        for (; tile < nt; tile += ctas) {
+            phase_B_fact(A, t, tile, sm, meta, pol);
             __syncthreads();
         }
         tile -= nt;
@@ -2686,46 +2753,18 @@ __global__ void __launch_bounds__(kThreads, SKEW_MINB_RMS)
     k_rms(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Smem sm;
     __shared__ Meta meta;
-    const Pol pol;
     const uint2 it = items[blockIdx.x];
-    const TensorDev &T = A.tensors[it.x];
-    if (T.kind == kKindFactored) (void)fill_meta(T, A.scal[it.x], it.y, A.ce, meta);
-    phase_B(A, it.x, it.y, sm, meta, pol);
+    if (A.tensors[it.x].kind == kKindFactored)
+        phase_B_fact(A, it.x, it.y, sm, meta, Pol());
+    else
+        phase_B_full(A, it.x, it.y, sm, Pol());
 }
 
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_APPLY)
     k_apply(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Meta meta;
-    const Pol pol;
     const uint2 it = items[blockIdx.x];
-    const TensorDev &T = A.tensors[it.x];
-    const TensorScal &S = A.scal[it.x];
-    if (T.kind == kKindFactored) {
-        const bool fast = fill_meta(T, S, it.y, A.ce, meta);
-        if (T.vec) {
-            if (T.momentum) {
-                if (fast)
-                    apply_fact_tile<true, true, true>(A, T, S, it.y, meta, pol);
-                else
-                    apply_fact_tile<true, true, false>(A, T, S, it.y, meta, pol);
-            } else {
-                if (fast)
-                    apply_fact_tile<true, false, true>(A, T, S, it.y, meta, pol);
-                else
-                    apply_fact_tile<true, false, false>(A, T, S, it.y, meta, pol);
-            }
-        } else {
-            if (T.momentum)
-                apply_fact_tile<false, true, false>(A, T, S, it.y, meta, pol);
-            else
-                apply_fact_tile<false, false, false>(A, T, S, it.y, meta, pol);
-        }
-    } else {
-        if (T.vec)
-            apply_full_tile<true>(A, T, S, it.y, pol);
-        else
-            apply_full_tile<false>(A, T, S, it.y, pol);
-    }
+    phase_C(A, A.tensors[it.x], A.scal[it.x], it.y, meta, Pol());
 }
 
 // Self-test of the bounded wait: one thread waits, exactly as the row kernels wait for
@@ -2754,30 +2793,32 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     auto mark = [&](int k) {
         if (ev) cudaEventRecord((cudaEvent_t)ev[k], s);
     };
+    const bool rows = L.nR != 0;
     mark(0);
-    if (L.nA) k_sumsq<<<L.nA, kThreads, 0, s>>>(A, L.itemsA);
+    if (L.nA && !rows) k_sumsq<<<L.nA, kThreads, 0, s>>>(A, L.itemsA);
     mark(1);
-    if (L.nR) {
+    if (rows) {
         constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem));
         const cudaError_t e = cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
-        k_rowsq<<<L.nR, kRowThreads, kSm, s>>>(A, L.itemsR);
+        k_rowsq<<<L.nA + L.nR, kRowThreads, kSm, s>>>(A, L.itemsA);
     }
     mark(2);
     if (L.nF) k_finalize<<<L.nF, kThreads, 0, s>>>(A, L.itemsF);
     mark(3);
-    if (L.nB) k_rms<<<L.nB, kThreads, 0, s>>>(A, L.itemsB);
+    if (L.nB && !rows) k_rms<<<L.nB, kThreads, 0, s>>>(A, L.itemsB);
     mark(4);
-    if (L.nFB) k_fallback<<<L.nFB, kThreads, 0, s>>>(A);
+    if (rows) k_fallback<<<L.nB + L.nFB, kThreads, 0, s>>>(A, L.itemsB, L.nB);
     mark(5);
-    if (L.nC) k_apply<<<L.nC, kThreads, 0, s>>>(A, L.itemsC);
+    if (L.nC && !rows) k_apply<<<L.nC, kThreads, 0, s>>>(A, L.itemsC);
     mark(6);
-    if (L.nCR) {
+    if (rows) {
         constexpr size_t kSm = max3(sizeof(ApplyRowSmem), sizeof(MomApplySmem), sizeof(FlatSmem));
         static_assert(2 * (kSm + 1024) <= 228 * 1024, "two CTAs per SM");
+        static_assert(sizeof(Meta) <= kSm && sizeof(Smem) <= kSm, "light tiles");
         const cudaError_t e = cudaFuncSetAttribute(k_apply_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
-        k_apply_rows<<<L.nCR, kRowThreads, kSm, s>>>(A, L.itemsCR);
+        k_apply_rows<<<L.nC + L.nCR, kRowThreads, kSm, s>>>(A, L.itemsC);
     }
     mark(7);
     return (int)cudaGetLastError();

@@ -287,12 +287,10 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
                         nFB,
                         o.nC,
                         o.nCR,
-                        (const uint2 *)(base + o.iA),
-                        (const uint2 *)(base + o.iR),
+                        (const uint2 *)(base + (row ? o.iR : o.iA)),
                         (const uint2 *)(base + o.iF),
                         (const uint2 *)(base + o.iB),
-                        (const uint2 *)(base + o.iC),
-                        (const uint2 *)(base + o.iCR)};
+                        (const uint2 *)(base + (row ? o.iCR : o.iC))};
     e = (cudaError_t)launch_phases(a, lp, stream, nullptr);
     if (e != cudaSuccess) return SKEW_ECUDA;
     return SKEW_OK;

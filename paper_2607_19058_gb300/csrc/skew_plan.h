@@ -136,11 +136,10 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
     return (uint32_t)t;
 }
 
-// Below this many bytes of G in all the matrices that only kRowAny serves, its three launches beside
-// the strip tiles' four cost a step more than the second read of G that they save: with one such
-// matrix of 8 MB among small ones (24 ragged tensors) 242 us against 214, with 320 MB among fixed
-// widths (a 2048-wide model) 435 us against 499.
-constexpr int64_t kAnyGroupBytes = 16 << 20;
+// Below this many bytes of G in all the matrices that only kRowAny serves, the strip tiles' second
+// read of G costs a step no more than k_fallback and the row tiles' ramps: 2048 x 1408 on its own
+// (5.8 MB) takes 51 us on strip tiles and 44 us on row tiles, the smallest steps the reverse.
+constexpr int64_t kAnyGroupBytes = 2 << 20;
 
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
 // gradient pointers are 16-byte aligned; `rest`: bytes of G of the step's row-path
@@ -293,24 +292,27 @@ struct StepArgs {
 
 // The phases of one step: item lists (tensor, local tile / item) in device
 // memory and their lengths.
-//   A  strip-tile sums of squares (strip-path factored tensors)
+//   A  strip-tile sums of squares (strip-path factored tensors); in a step with row
+//      tiles, also the update-RMS tiles of full tensors
 //   R  row-tile sums of squares and bilinear partials (row-path tensors)
 //   F  finalize items (rows and columns; columns only on the row path)
-//   B  update-RMS tiles (strip-path factored and full tensors)
+//   B  update-RMS tiles (strip-path factored tensors; without row tiles full tensors too)
 //   FB phase B of the row-path tensors whose finalize asked for it (nFB CTAs)
-//   C  apply strip tiles (tensors not on the row path)
+//   C  apply strip and flat tiles (tensors not on the row path)
 //   CR apply row tiles (row-path tensors)
+// The items of R follow those of A, and those of CR those of C.
 struct LaunchPlan {
     uint32_t nA, nR, nF, nB, nFB, nC, nCR;
-    const uint2 *itemsA, *itemsR, *itemsF, *itemsB, *itemsC, *itemsCR;
+    const uint2 *itemsA, *itemsF, *itemsB, *itemsC;
 };
 
 constexpr int kLaunches = 7;
 
-// Enqueues the phases of `L` as grouped launches (A, R, F, B, FB, C, CR; empty
-// ones skipped) on `stream`, each given the step parameters by value. If `ev` is
-// not null it holds kLaunches + 1 cudaEvent_t, recorded before the first launch
-// and after each of the seven. Returns a cudaError_t value.
+// Enqueues the phases of `L` as grouped launches (A, F, B, C; with row tiles A + R, F,
+// B + FB, C + CR; empty ones skipped) on `stream`, each given the step parameters by value. If `ev` is
+// not null it holds kLaunches + 1 cudaEvent_t, recorded before the first launch and after
+// each of the seven kernels' places (k_sumsq, k_rowsq, k_finalize, k_rms, k_fallback, k_apply,
+// k_apply_rows). Returns a cudaError_t value.
 int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *const *ev);
 
 // Enqueues the bounded-wait self-test (one thread waits on an mbarrier phase that
