@@ -34,7 +34,7 @@ struct TPlan {
     int kind = 0, momentum = 0, decay = 0, vec = 0;
     int64_t n = 0, m = 0, numel = 0;
     int64_t moff = -1, voff = -1, roff = -1, coff = -1;  // floats into the state
-    uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0;
+    uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0, nbc = 0, fvpt = 0;
     uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0, at_rows = 0, atiles = 0, fci = 0, nu2 = 0;
     uint32_t f32 = 0;         // SKEW_F_FP32: fp32 weights and gradient
     // bytes into the workspace
@@ -58,6 +58,7 @@ struct skew_handle {
     std::vector<uint2> itemsA, itemsF, itemsB, itemsC;  // A + R, F, B, C + CR: per phase, tensors in order
     uint32_t nA = 0, nC = 0;  // items of A before those of R, of C before those of CR
     uint32_t n_rowpath = 0;  // tensors on the row path
+    bool ride = false;       // the strip and flat tiles go into the row tiles' launches
     uint32_t fb_ctas = 0;    // CTAs of the row path's phase-B launch (set at bind)
     char *state = nullptr, *ws = nullptr;
     bool bound = false;
@@ -101,10 +102,14 @@ static void resolve(int ndim, int tier, int policy, uint32_t flags, TPlan &p) {
     p.decay = (int)decay;
 }
 
+static bool wg_aligned(const TPlan &p) { return (((uintptr_t)p.w | (uintptr_t)p.g) & 15) == 0; }
+
 // Tile geometry (plan_geometry): strip tiles of (tile_rows rows) x (8*LC
 // columns) or flat tiles of kFlatTileElems elements, and for the row path whole-row tiles.
-static void geometry(TPlan &p, bool row_aligned, int64_t rest) {
-    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, p.n, p.m, p.numel, rest);
+static void geometry(TPlan &p, bool row_aligned, bool small, int64_t rest) {
+    // the state buffer starts on a 256-byte boundary
+    const bool vec = row_vectors(p.f32 != 0, wg_aligned(p), p.moff < 0 || p.moff % 4 == 0, p.m);
+    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, small, p.n, p.m, p.numel, rest);
     p.lcl = g.lcl;
     p.strips = g.strips;
     p.rowtiles = g.rowtiles;
@@ -120,6 +125,8 @@ static void geometry(TPlan &p, bool row_aligned, int64_t rest) {
     p.atiles = g.atiles;
     p.fci = g.fci;
     p.nu2 = u2_len(g);
+    p.nbc = g.nbc;
+    p.fvpt = g.fvpt;
 }
 
 extern "C" {
@@ -152,7 +159,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     }
     const int64_t kMaxExtent = int64_t(1) << 40;
     // whole-row tiles are for bf16 rows on 16-byte boundaries
-    auto row_aligned = [](const TPlan &q) { return !q.f32 && (((uintptr_t)q.w | (uintptr_t)q.g) & 15) == 0; };
+    auto row_aligned = [](const TPlan &q) { return !q.f32 && wg_aligned(q); };
     int64_t any_bytes = 0;  // bytes of G of the matrices that only kRowAny's whole-row tiles serve
     for (int32_t k = 0; k < n_params; ++k) {
         const skew_param_desc_t &d = params[k];
@@ -186,7 +193,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.tid = (uint32_t)k;
                 q.base = (uint64_t)(e * p.numel);
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
-                geometry(q, row_aligned(q), kWholeGroup);
+                geometry(q, row_aligned(q), false, kWholeGroup);  // which path
                 if (q.rowpath == kRowAny) any_bytes += 2 * q.numel;
                 h->t.push_back(q);
             }
@@ -194,19 +201,6 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             delete h;
             return fail(nullptr, SKEW_ENOMEM, "out of host memory");
         }
-    }
-    const bool any = any_bytes >= kAnyGroupBytes;
-    int64_t rest = 0;
-    for (size_t k = h->t.size(); k-- > 0;) {  // row tiles by the bytes that follow, from the last matrix back
-        TPlan &q = h->t[k];
-        if (q.rowpath == kRowNone) continue;
-        if (q.rowpath == kRowAny && !any) {
-            geometry(q, false, kWholeGroup);
-            continue;
-        }
-        rest += 2 * q.numel;
-        geometry(q, true, rest);
-        ++h->n_rowpath;
     }
     const int32_t n_plans = (int32_t)h->t.size();
 
@@ -226,6 +220,24 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         if (p.kind == kKindFactored) { p.coff = off; off += p.m; }
     h->state_bytes = size_t(off) * 4;
 
+    // Tiles, now that the paths and the state's alignment are known: the row tiles by the bytes that
+    // follow, from the last matrix back.
+    const bool any = any_bytes >= kAnyGroupBytes;
+    int64_t rest = 0, light = 0, fact = 0;  // elements off the row path, and of factored tensors
+    for (TPlan &q : h->t) {
+        if (q.rowpath == kRowAny && !any) q.rowpath = kRowNone;
+        if (!q.rowpath) light += q.numel;
+        if (q.kind == kKindFactored) fact += q.numel;
+    }
+    for (size_t k = h->t.size(); k-- > 0;) {
+        TPlan &q = h->t[k];
+        const bool row = q.rowpath != kRowNone;
+        if (row) rest += 2 * q.numel;
+        geometry(q, row, fact < kSmallStrip, rest);
+        h->n_rowpath += row;
+    }
+    h->ride = h->n_rowpath && light <= kRideElems;
+
     // Item tables: every factored tensor's tiles (phase A), finalize items
     // (phase F) and every tensor's tiles (phases B and C), tensors in order.
     try {
@@ -241,9 +253,9 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 all(itemsCR, q, p.atiles);
             } else {
                 if (fact) all(h->itemsA, q, p.ntiles);
-                // flat tiles of phase B need no earlier phase: with row tiles they go with phase A
-                all(!fact && h->n_rowpath ? h->itemsA : h->itemsB, q, p.ntiles);
-                all(h->itemsC, q, p.ntiles);
+                // flat tiles of phase B need no earlier phase: riding, they go with phase A
+                all(!fact && h->ride ? h->itemsA : h->itemsB, q, p.nbc);
+                all(h->itemsC, q, p.nbc);
             }
             if (fact) all(h->itemsF, q, p.nfr + p.nfc);
         }
@@ -328,9 +340,10 @@ int32_t skew_num_tensors(const skew_handle_t *h) { return h ? (int32_t)h->desc.s
 
 int64_t skew_launches_per_step(const skew_handle_t *h) {
     if (!h) return 0;
-    if (h->n_rowpath) return 4;  // k_rowsq, k_finalize, k_fallback, k_apply_rows
-    return int64_t(!h->itemsA.empty()) + int64_t(!h->itemsF.empty()) + int64_t(!h->itemsB.empty()) +
-           int64_t(!h->itemsC.empty());
+    // with row tiles k_rowsq, k_fallback and k_apply_rows; the others where they have items of their own
+    const uint32_t rows = h->n_rowpath > 0;
+    return 3 * rows + int64_t(!h->itemsF.empty()) +
+           (h->ride ? 0 : int64_t(h->nA > 0) + int64_t(!h->itemsB.empty()) + int64_t(h->nC > 0));
 }
 
 const char *skew_last_error(const skew_handle_t *h) { return h ? h->err.c_str() : g_create_err.c_str(); }
@@ -412,6 +425,10 @@ int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace
             vec = vec && (p.m % 8 == 0);
         p.vec = vec ? 1 : 0;
         T.vec = p.vec;
+        T.wal = al16(T.w) && al16(T.g);
+        T.sal = (!T.M || al16(T.M)) && (!T.v || al16(T.v));
+        T.nbc = p.nbc;
+        T.fvpt = p.fvpt;
         T.f32 = p.f32;
         T.lcl = p.lcl;
         T.strips = p.strips;
@@ -508,7 +525,7 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
     if (e != cudaSuccess) return cuda_fail(h, e, "reset of per-step scalars");
     auto items = [&](size_t at) { return reinterpret_cast<const uint2 *>(h->ws + at); };
     const LaunchPlan L{h->nA, (uint32_t)h->itemsA.size() - h->nA, (uint32_t)h->itemsF.size(), (uint32_t)h->itemsB.size(),
-                       h->n_rowpath ? h->fb_ctas : 0u, h->nC, (uint32_t)h->itemsC.size() - h->nC,
+                       h->n_rowpath ? h->fb_ctas : 0u, h->nC, (uint32_t)h->itemsC.size() - h->nC, h->ride,
                        items(h->ws_itemsA), items(h->ws_itemsF), items(h->ws_itemsB), items(h->ws_itemsC)};
     e = (cudaError_t)launch_phases(a, L, s, reinterpret_cast<void *const *>(ev));
     if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch");

@@ -102,48 +102,46 @@ __device__ __forceinline__ void unpack_bf8x2(uint4 u, float2 (&o)[4]) {
 
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-// Eight bf16 values (scalar path: elements >= valid read as 0).
-__device__ __forceinline__ void load_bf8_scalar(const uint16_t *p, int valid, float (&o)[8]) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) o[c] = c < valid ? bf16_to_f32(p[c]) : 0.f;
-}
-
-// Elements e0 .. e0+7 of a weight or gradient array on the scalar path (elements
-// >= valid read as 0): bf16, or fp32 for a tensor kept in fp32 (its array pointer
-// then addresses floats).
-__device__ __forceinline__ void load8_elem(const uint16_t *base, bool f32, int64_t e0, int valid, float (&o)[8]) {
+// Elements e0 .. e0 + 7 of a weight or gradient array (elements >= valid read as 0): bf16, or fp32
+// for a tensor kept in fp32 (its array pointer then addresses floats). `wide`: the address is on
+// the boundary that 16-byte loads need.
+__device__ __forceinline__ void load8_elem(const uint16_t *base, bool f32, bool wide, int64_t e0, int valid,
+                                           float (&o)[8], const Pol &pol) {
     if (f32) {
         const float *p = reinterpret_cast<const float *>(base) + e0;
+        if (wide && valid == 8) {
+            const uint4 a = ld16_hint(p, pol.drop), b = ld16_hint(p + 4, pol.drop);
+            const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int c = 0; c < 8; ++c) o[c] = c < valid ? p[c] : 0.f;
+            for (int c = 0; c < 8; ++c) o[c] = __uint_as_float(w[c]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] = c < valid ? p[c] : 0.f;
+        }
+    } else if (wide && valid == 8) {
+        unpack_bf8(ld16_hint(base + e0, pol.drop), o);
     } else {
-        load_bf8_scalar(base + e0, valid, o);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) o[c] = c < valid ? bf16_to_f32(base[e0 + c]) : 0.f;
     }
 }
 
-// Eight fp32 values; `cg` reads through L2 only (values an earlier phase wrote).
-template <bool VEC>
-__device__ __forceinline__ void load_f8(const float *p, int valid, float (&o)[8], bool cg) {
-    if (VEC) {
-        float4 a, b;
-        if (cg) {
-            a = __ldcg(reinterpret_cast<const float4 *>(p));
-            b = __ldcg(reinterpret_cast<const float4 *>(p + 4));
-        } else {
-            a = *reinterpret_cast<const float4 *>(p);
-            b = *reinterpret_cast<const float4 *>(p + 4);
-        }
+// Eight fp32 state values (`wide`: on a 16-byte boundary), read through L2 (an earlier launch of
+// the step may have written them).
+__device__ __forceinline__ void load_f8(const float *p, bool wide, int valid, float (&o)[8]) {
+    if (wide && valid == 8) {
+        const float4 a = __ldcg(reinterpret_cast<const float4 *>(p));
+        const float4 b = __ldcg(reinterpret_cast<const float4 *>(p + 4));
         o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
         o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
     } else {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) o[c] = c < valid ? (cg ? __ldcg(p + c) : p[c]) : 0.f;
+        for (int c = 0; c < 8; ++c) o[c] = c < valid ? __ldcg(p + c) : 0.f;
     }
 }
 
-template <bool VEC>
-__device__ __forceinline__ void store_f8(float *p, int valid, const float (&o)[8]) {
-    if (VEC) {
+__device__ __forceinline__ void store_f8(float *p, bool wide, int valid, const float (&o)[8]) {
+    if (wide && valid == 8) {
         *reinterpret_cast<float4 *>(p) = make_float4(o[0], o[1], o[2], o[3]);
         *reinterpret_cast<float4 *>(p + 4) = make_float4(o[4], o[5], o[6], o[7]);
     } else {
@@ -199,13 +197,35 @@ __device__ __forceinline__ void dither8(uint64_t idx0, const Dith &d, uint32_t (
     }
 }
 
-__device__ __forceinline__ uint32_t dither1(uint64_t idx, const Dith &d) {
-    idx += d.base;
-    const uint64_t blk = idx >> 3;
-    const uint4 o = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), d.tid, d.step, d.k0, d.k1);
-    const uint32_t k = (uint32_t)(idx & 7);
-    const uint32_t w = k < 2 ? o.x : k < 4 ? o.y : k < 6 ? o.z : o.w;
-    return (w >> (16 * (k & 1))) & 0xFFFFu;
+// The same for an idx0 whose dither index (with the tensor's base) need not be a multiple of 8:
+// the eight halves start inside a Philox block and may run into the next.
+__device__ __forceinline__ void dither8_any(uint64_t idx0, const Dith &d, uint32_t (&r)[8]) {
+    const uint64_t i = idx0 + d.base, blk = i >> 3;
+    const uint32_t s = (uint32_t)(i & 7);
+    const uint4 a = philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), d.tid, d.step, d.k0, d.k1);
+    uint32_t w[8] = {a.x, a.y, a.z, a.w, 0u, 0u, 0u, 0u};
+    if (s) {
+        const uint64_t nxt = blk + 1;
+        const uint4 b = philox4x32_10((uint32_t)nxt, (uint32_t)(nxt >> 32), d.tid, d.step, d.k0, d.k1);
+        w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+        if (s & 4) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) w[k] = w[k + 2];
+        }
+        if (s & 2) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) w[k] = w[k + 1];
+        }
+        if (s & 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = __funnelshift_r(w[k], w[k + 1], 16);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        r[2 * q] = w[q] & 0xFFFFu;
+        r[2 * q + 1] = w[q] >> 16;
+    }
 }
 
 // Dithered rounding to bf16: add the 16-bit draw to the fp32 bit pattern and
@@ -445,11 +465,12 @@ __device__ void sumsq_tile(const TensorDev &T, uint32_t tile, Smem &sm, const Po
     const int64_t n = T.n, m = T.m, row0 = F.row0, RG = F.RG, col0 = F.col0;
     const uint32_t LC = F.LC;
     const bool act = F.act, lane0 = F.lane == 0;
+    const int vpt = (int)(T.tile_rows / F.RG);  // rows per thread: 8 or kVecPerThread
     float col[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if constexpr (VEC) {
         constexpr int KCH = 8;  // row-vectors requested before the first is used
 #pragma unroll 1
-        for (int k0 = 0; k0 < kVecPerThread; k0 += KCH) {
+        for (int k0 = 0; k0 < vpt; k0 += KCH) {
             uint4 raw[KCH];
 #pragma unroll
             for (int q = 0; q < KCH; ++q) {
@@ -504,16 +525,28 @@ __device__ void sumsq_tile(const TensorDev &T, uint32_t tile, Smem &sm, const Po
             }
         }
     } else {
-        for (int k = 0; k < kVecPerThread; ++k) {
-            const int64_t i = row0 + k * RG;
-            float g[8];
-            if (act && i < n)
-                load8_elem(g_, T.f32, i * m + col0, F.valid, g);
-            else
+        constexpr int KCH = 4;  // rows requested before the first is used
+        // a row starts on a 16-byte boundary only where the width keeps it there (fp32 rows)
+        const bool wide = T.wal && (m & (T.f32 ? 3 : 7)) == 0;
+#pragma unroll 1
+        for (int k0 = 0; k0 < vpt; k0 += KCH) {
+            if (int64_t(F.rt) * T.tile_rows + k0 * RG >= n) break;  // past the last row for every thread
+            float g[KCH][8];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) g[c] = 0.f;
-            const float rs = sumsq_row(g, col, LC);
-            if (lane0 && i < n) rowp[i] = rs;
+            for (int q = 0; q < KCH; ++q) {
+                const int64_t i = row0 + (k0 + q) * RG;
+                if (act && i < n)
+                    load8_elem(g_, T.f32, wide, i * m + col0, F.valid, g[q], pol);
+                else
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) g[q][c] = 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < KCH; ++q) {
+                const int64_t i = row0 + (k0 + q) * RG;
+                const float rs = sumsq_row(g[q], col, LC);
+                if (lane0 && i < n) rowp[i] = rs;
+            }
         }
     }
 #pragma unroll
@@ -1168,9 +1201,16 @@ __device__ void phase_F(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm)
         rd = block_sum_d(rd, sm.redd);
         if (threadIdx.x == 0) T.rsum[local] = rd;
     } else {
-        const int64_t j = int64_t(local - T.nfr) * kFinChunk + threadIdx.x;
-        if (threadIdx.x < kFinChunk && j < T.m) {
-            const float cs = strided_sum(T.colp + j, T.m, T.rowtiles);
+        // fci columns per item, kFinChunk / fci threads per column, each with every (kFinChunk / fci)-th tile
+        const int fci = (int)T.fci, tpc = kFinChunk / fci, cix = threadIdx.x % fci, sl = threadIdx.x / fci;
+        const int64_t j = int64_t(local - T.nfr) * fci + cix;
+        float cs = 0.f;
+        if (j < T.m && sl < (int)T.rowtiles)
+            cs = strided_sum(T.colp + int64_t(sl) * T.m + j, T.m * tpc, (T.rowtiles - sl + tpc - 1) / tpc);
+        sm.colred[threadIdx.x] = cs;
+        __syncthreads();
+        if (sl == 0 && j < T.m) {
+            for (int k = 1; k < tpc; ++k) cs += sm.colred[k * fci + cix];
             const float mean = __fdiv_rn(cs, (float)T.n);
             const float Cn = fmaf(A.b2, T.C[j], grad_scale(A).c2 * mean);
             T.C[j] = Cn;
@@ -1200,7 +1240,7 @@ __device__ __forceinline__ void rms_row(const float (&y)[8], float a, const floa
     acc.add(sumsq8(u));
 }
 
-template <bool VEC, bool MOM>
+template <bool MOM>
 __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t tile, const Meta &meta,
                               const Pol &pol) {
     const FactTile F(T, tile);
@@ -1209,18 +1249,18 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
     const uint16_t *__restrict__ g_ = T.g;
     float *__restrict__ M_ = T.M;
     const int64_t n = T.n, m = T.m, row0 = F.row0, RG = F.RG, col0 = F.col0;
-    const int valid = F.valid;
     const float b1 = A.b1, c1 = grad_scale(A).c1, ce = A.ce;
     const bool mnew = MOM && T.rowpath;  // phase B of a queued row-path tensor: M is already new
     const float *rows = meta.rows + F.rg;
+    const int vpt = (int)(T.tile_rows / F.RG);
     float b[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) b[c] = meta.cols[F.lane * 8 + c];
-    if constexpr (VEC) {
+    {
         // row-vectors requested together: eight when only g streams, four with the momentum
         constexpr int KCH = MOM ? 4 : 8;
 #pragma unroll 1
-        for (int k0 = 0; k0 < kVecPerThread; k0 += KCH) {
+        for (int k0 = 0; k0 < vpt; k0 += KCH) {
             uint4 graw[KCH];
             float4 mraw[MOM ? KCH : 1][2];
 #pragma unroll
@@ -1248,68 +1288,184 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
                         } else {
 #pragma unroll
                             for (int c = 0; c < 8; ++c) y[c] = fmaf(b1, mm[c], c1 * y[c]);
-                            store_f8<true>(M_ + i * m + col0, 8, y);
+                            store_f8(M_ + i * m + col0, true, 8, y);
                         }
                     }
                     rms_row(y, rows[(k0 + q) * RG], b, 8, ce, acc);
                 }
             }
         }
-    } else {
-        for (int k = 0; k < kVecPerThread; ++k) {
-            const int64_t i = row0 + k * RG;
-            if (i >= n) break;
-            float y[8];
-            load8_elem(g_, T.f32, i * m + col0, valid, y);
-            if (MOM) {
-                float mm[8];
-                load_f8<false>(M_ + i * m + col0, valid, mm, false);
-                if (mnew) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) y[c] = mm[c];
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) y[c] = fmaf(b1, mm[c], c1 * y[c]);
-                    store_f8<false>(M_ + i * m + col0, valid, y);
-                }
-            }
-            rms_row(y, rows[k * RG], b, valid, ce, acc);
-        }
     }
     return acc;
 }
 
-template <bool VEC>
+// ---------------------------------------------------------------------------
+// Phases B and C of factored tensors without 16-byte row-vectors (fp32, widths that are not a
+// multiple of 8, unaligned pointers): flat tiles of 8 consecutive elements per thread and round, which
+// are loaded wide wherever the arrays start on a 16-byte boundary and draw one Philox block, whatever
+// the width. Bound by latency; the row-vectors' layout had 8 narrow loads per row, a Philox block per
+// element and 32 rows per thread one after another (k_apply, 42829 x 58 bf16: 103 -> 17 us; 3467 x
+// 1072 fp32 with momentum: 45 -> 22; 24 ragged tensors of 13M elements in all: a step 215 -> 161).
+// ---------------------------------------------------------------------------
+struct FlatPos {
+    int64_t row, col;    // of element e0
+    int64_t dq, dr;      // one round of the CTA, 8 kThreads elements, in rows and columns
+    __device__ FlatPos(const TensorDev &T, int64_t e0) {
+        if (T.numel < (int64_t(1) << 31)) {  // 64-bit divides are long here
+            row = (uint32_t)e0 / (uint32_t)T.m;
+            dq = 8u * kThreads / (uint32_t)T.m;
+        } else {
+            row = e0 / T.m;
+            dq = (8 * kThreads) / T.m;
+        }
+        col = e0 - row * T.m;
+        dr = 8 * kThreads - dq * T.m;
+    }
+    __device__ void next(int64_t m) {
+        row += dq;
+        col += dr;
+        if (col >= m) {
+            col -= m;
+            ++row;
+        }
+    }
+};
+
+// The scales of a flat tile: a_i of its rows, then b_j of all columns, in shared memory where they
+// fit (`in`; read from L2 by every thread, the few columns of a narrow matrix are one hot line).
+struct FlatMeta {
+    const float *a, *b;
+    int64_t row0;
+    float rbar_s;
+    int rbar_e;
+    bool in;
+    __device__ FlatMeta(const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta) {
+        const int64_t elems = int64_t(8 * kThreads) * T.fvpt, e0 = int64_t(tile) * elems;
+        const int64_t e1 = min(e0 + elems, T.numel) - 1, m = T.m;
+        const bool narrow = T.numel < (int64_t(1) << 31);  // 64-bit divides are long here
+        row0 = narrow ? (uint32_t)e0 / (uint32_t)m : e0 / m;
+        const int64_t rows = (narrow ? (uint32_t)e1 / (uint32_t)m : e1 / m) - row0 + 1;
+        rbar_s = __ldcg(&S.rbar_s);
+        rbar_e = __ldcg(&S.rbar_e);
+        float *pool = reinterpret_cast<float *>(&meta);
+        in = rows + m <= kSmemFloats + kStripCols;
+        a = pool;
+        b = pool + rows;
+        if (in) {
+            for (int r = threadIdx.x; r < (int)rows; r += kThreads) pool[r] = row_scale(__ldcg(T.R + row0 + r), rbar_s, rbar_e);
+            for (int j = threadIdx.x; j < (int)m; j += kThreads) pool[rows + j] = __ldcg(T.bsc + j);
+            __syncthreads();
+        }
+    }
+    // min(a_i b_j, 1/sqrt(eps)) of the `valid` elements from (row, col) on
+    __device__ __forceinline__ void scales(const TensorDev &T, const FlatPos &P, int valid, float ce, float (&sc)[8]) const {
+        const int64_t m = T.m;
+        if (in) {
+            int r = (int)(P.row - row0), j = (int)P.col;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                sc[c] = c < valid ? fminf(a[r] * b[j], ce) : 0.f;
+                const bool wrap = ++j == (int)m;
+                j = wrap ? 0 : j;
+                r += wrap;
+            }
+        } else {
+            int64_t r = P.row, j = P.col;
+            float ar = row_scale(__ldcg(T.R + r), rbar_s, rbar_e);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                sc[c] = c < valid ? fminf(ar * __ldcg(T.bsc + j), ce) : 0.f;
+                if (++j == m) {
+                    j = 0;
+                    if (++r < T.n) ar = row_scale(__ldcg(T.R + r), rbar_s, rbar_e);
+                }
+            }
+        }
+    }
+};
+constexpr uint32_t kFlatAhead = 2;  // rounds of a flat tile whose loads are issued together
+
+__device__ Acc2 rms_flat_tile(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
+                              const Pol &pol) {
+    const GScale gsc = grad_scale(A);
+    const FlatMeta F(T, S, tile, meta);
+    Acc2 acc;
+    const int64_t numel = T.numel;
+    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
+    FlatPos P(T, e0);
+    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
+        float y[kFlatAhead][8], mm[kFlatAhead][8];
+        FlatPos Q[kFlatAhead] = {P, P};
+#pragma unroll
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            Q[h] = P;
+            if (e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
+                if (T.momentum) load_f8(T.M + e, T.sal, valid, mm[h]);
+            }
+            P.next(T.m);
+        }
+#pragma unroll
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                float sc[8], u[8];
+                if (T.momentum) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) y[h][c] = fmaf(A.b1, mm[h][c], gsc.c1 * y[h][c]);
+                    store_f8(T.M + e, T.sal, valid, y[h]);
+                }
+                F.scales(T, Q[h], valid, A.ce, sc);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) u[c] = c < valid ? y[h][c] * sc[c] : 0.f;
+                acc.add(sumsq8(u));
+            }
+        }
+        e0 += kFlatAhead * 8 * kThreads;
+    }
+    return acc;
+}
+
 __device__ Acc2 rms_full_tile(const StepArgs &A, const TensorDev &T, uint32_t tile, const Pol &pol) {
     const GScale gsc = grad_scale(A);
+    const int64_t numel = T.numel;
     Acc2 acc;
-    for (int k = 0; k < kFlatVecPerThread; ++k) {
-        const int64_t e0 = 8 * (int64_t(tile) * kThreads * kFlatVecPerThread + int64_t(k) * kThreads + threadIdx.x);
-        if (e0 >= T.numel) break;
-        const int valid = (int)min(int64_t(8), T.numel - e0);
-        float g[8], v[8], y[8];
-        if (VEC)
-            unpack_bf8(ld16_hint(T.g + e0, pol.drop), g);
-        else
-            load8_elem(T.g, T.f32, e0, valid, g);
-        load_f8<VEC>(T.v + e0, valid, v, false);
+    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
+    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
+        float g[kFlatAhead][8], v[kFlatAhead][8], mm[kFlatAhead][8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = fmaf(A.b2, v[c], gsc.c2 * (g[c] * g[c]));
-        store_f8<VEC>(T.v + e0, valid, v);
-        if (T.momentum) {
-            float mm[8];
-            load_f8<VEC>(T.M + e0, valid, mm, false);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) y[c] = fmaf(A.b1, mm[c], gsc.c1 * g[c]);
-            store_f8<VEC>(T.M + e0, valid, y);
-        } else {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) y[c] = g[c];
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (k + h < T.fvpt && e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                load8_elem(T.g, T.f32, T.wal, e, valid, g[h], pol);
+                load_f8(T.v + e, T.sal, valid, v[h]);
+                if (T.momentum) load_f8(T.M + e, T.sal, valid, mm[h]);
+            }
         }
-        float u[8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) u[c] = c < valid ? y[c] * fminf(__frsqrt_rn(v[c]), A.ce) : 0.f;
-        acc.add(sumsq8(u));
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (k + h < T.fvpt && e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                float u[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[h][c] = fmaf(A.b2, v[h][c], gsc.c2 * (g[h][c] * g[h][c]));
+                store_f8(T.v + e, T.sal, valid, v[h]);
+                if (T.momentum) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) g[h][c] = fmaf(A.b1, mm[h][c], gsc.c1 * g[h][c]);
+                    store_f8(T.M + e, T.sal, valid, g[h]);
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) u[c] = c < valid ? g[h][c] * fminf(__frsqrt_rn(v[h][c]), A.ce) : 0.f;
+                acc.add(sumsq8(u));
+            }
+        }
+        e0 += kFlatAhead * 8 * kThreads;
     }
     return acc;
 }
@@ -1322,12 +1478,12 @@ __device__ void finish_B(const StepArgs &A, uint32_t t, uint32_t local, const Ac
     const float2 tsum = block_sum2(acc, sm.red2);
     if (threadIdx.x == 0) {
         T.u2[local] = tsum;
-        sm.last = (atom_add_acq_rel(&S.cntB, 1u) == T.ntiles - 1);
+        sm.last = (atom_add_acq_rel(&S.cntB, 1u) == T.nbc - 1);
     }
     __syncthreads();
     if (!sm.last) return;
     double s = 0.0;
-    for (uint32_t k = threadIdx.x; k < T.ntiles; k += kThreads) {
+    for (uint32_t k = threadIdx.x; k < T.nbc; k += kThreads) {
         const float2 p = __ldcg(T.u2 + k);
         s += pair_value(p.x, p.y);
     }
@@ -1337,21 +1493,33 @@ __device__ void finish_B(const StepArgs &A, uint32_t t, uint32_t local, const Ac
 
 __device__ void phase_B_full(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, const Pol &pol) {
     const TensorDev &T = A.tensors[t];
-    const Acc2 acc = T.vec ? rms_full_tile<true>(A, T, local, pol) : rms_full_tile<false>(A, T, local, pol);
+    const Acc2 acc = rms_full_tile(A, T, local, pol);
     finish_B(A, t, local, acc, sm);
 }
 
-__device__ void phase_B_fact(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+__device__ void phase_B_strip(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
     const TensorDev &T = A.tensors[t];
     (void)fill_meta(T, A.scal[t], local, A.ce, meta);
-    Acc2 acc;
-    if (T.vec)
-        acc = T.momentum ? rms_fact_tile<true, true>(A, T, local, meta, pol)
-                         : rms_fact_tile<true, false>(A, T, local, meta, pol);
+    finish_B(A, t, local,
+             T.momentum ? rms_fact_tile<true>(A, T, local, meta, pol) : rms_fact_tile<false>(A, T, local, meta, pol), sm);
+}
+
+__device__ void phase_B_flat(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+    const TensorDev &T = A.tensors[t];
+    finish_B(A, t, local, rms_flat_tile(A, T, A.scal[t], local, meta, pol), sm);
+}
+
+__device__ void phase_B_fact(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+    if (A.tensors[t].vec)
+        phase_B_strip(A, t, local, sm, meta, pol);
     else
-        acc = T.momentum ? rms_fact_tile<false, true>(A, T, local, meta, pol)
-                         : rms_fact_tile<false, false>(A, T, local, meta, pol);
-    finish_B(A, t, local, acc, sm);
+        phase_B_flat(A, t, local, sm, meta, pol);
+}
+
+// The same for k_fallback's own items, out of line: inlined beside the queue's tiles, which are strip
+// tiles, it makes those spill (a queue of 62M elements of 1024 and 496 columns 56 us slower).
+__device__ __noinline__ void phase_B_own(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta) {
+    phase_B_fact(A, t, local, sm, meta, Pol());
 }
 
 // ---------------------------------------------------------------------------
@@ -1376,44 +1544,40 @@ __device__ __forceinline__ void round8(const float (&x)[8], const Dith &d, uint6
     out = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// x of eight elements -> dithered bf16, stored at w + e0 (16-byte store when VEC).
-template <bool VEC>
-__device__ __forceinline__ void write8(uint16_t *__restrict__ w, const Dith &d, int64_t e0, int valid, bool aligned8,
-                                       const float (&x)[8], const Pol &pol) {
-    uint32_t r[8];
-    if (VEC) {
-        uint4 o;
-        round8(x, d, (uint64_t)e0, o);
-        st16_hint(w + e0, o, pol.drop);
-    } else {
-        if (aligned8) dither8((uint64_t)e0, d, r);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            if (c < valid) {
-                const uint32_t rc = aligned8 ? r[c] : dither1((uint64_t)(e0 + c), d);
-                w[e0 + c] = (uint16_t)sr_bf16(x[c], rc);
-            }
-        }
-    }
+// x of eight elements -> dithered bf16, one 16-byte store at w + e0.
+__device__ __forceinline__ void write8(uint16_t *__restrict__ w, const Dith &d, int64_t e0, const float (&x)[8],
+                                       const Pol &pol) {
+    uint4 o;
+    round8(x, d, (uint64_t)e0, o);
+    st16_hint(w + e0, o, pol.drop);
 }
 
-// Scalar-path write-back of elements e0 .. e0+valid-1: the dithered bf16 rounding,
-// or for a tensor kept in fp32 the fp32 value x itself.
-__device__ __forceinline__ void store8_elem(const TensorDev &T, uint16_t *w, const Dith &d, int64_t e0, int valid,
-                                            const float (&x)[8], const Pol &pol) {
+// Write-back of elements e0 .. e0 + valid - 1 at any alignment: the dithered bf16 rounding, or for a
+// tensor kept in fp32 the fp32 value x itself.
+__device__ __forceinline__ void store8_elem(const TensorDev &T, const Dith &d, int64_t e0, int valid, const float (&x)[8],
+                                            const Pol &pol) {
     if (T.f32) {
-        float *p = reinterpret_cast<float *>(w) + e0;
+        store_f8(reinterpret_cast<float *>(T.w) + e0, T.wal, valid, x);
+        return;
+    }
+    uint32_t r[8];
+    dither8_any((uint64_t)e0, d, r);
+    uint32_t h[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) h[c] = sr_bf16(x[c], r[c]);
+    if (T.wal && valid == 8) {
+        st16_hint(T.w + e0, make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16)),
+                  pol.drop);
+    } else {
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-            if (c < valid) p[c] = x[c];
-    } else {
-        write8<false>(w, d, e0, valid, ((e0 + d.base) & 7) == 0, x, pol);
+            if (c < valid) T.w[e0 + c] = (uint16_t)h[c];
     }
 }
 
 // FAST: no element of the tile reaches the clamp (fill_meta), so the update is
 // (-lr*kappa*coef * a_i) * b_j * y, one multiply and one fma per element.
-template <bool VEC, bool MOM, bool FAST>
+template <bool MOM, bool FAST>
 __device__ void apply_fact_tile(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile,
                                 const Meta &meta, const Pol &pol) {
     const FactTile F(T, tile);
@@ -1422,7 +1586,7 @@ __device__ void apply_fact_tile(const StepArgs &A, const TensorDev &T, const Ten
     const float *__restrict__ M_ = T.M;
     uint16_t *__restrict__ w_ = T.w;
     const int64_t n = T.n, m = T.m, row0 = F.row0, RG = F.RG, col0 = F.col0;
-    const int valid = F.valid;
+    const int vpt = (int)(T.tile_rows / F.RG);
     const Dith d = dith_of(A, T);
     const float coefC = __ldcg(&S.coefC);
     const float wdf = T.decay ? A.wdf : 1.0f;
@@ -1431,10 +1595,10 @@ __device__ void apply_fact_tile(const StepArgs &A, const TensorDev &T, const Ten
     float b[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) b[c] = meta.cols[F.lane * 8 + c];
-    if constexpr (VEC) {
+    {
         constexpr int KCH = 4;  // row-vectors (with their weights) requested together
 #pragma unroll 1
-        for (int k0 = 0; k0 < kVecPerThread; k0 += KCH) {
+        for (int k0 = 0; k0 < vpt; k0 += KCH) {
             uint4 wraw[KCH], graw[MOM ? 1 : KCH];
             float4 mraw[MOM ? KCH : 1][2];
 #pragma unroll
@@ -1480,57 +1644,90 @@ __device__ void apply_fact_tile(const StepArgs &A, const TensorDev &T, const Ten
 #pragma unroll
                         for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[c] * fminf(a * b[c], ce), w[c] * wdf);
                     }
-                    write8<true>(w_, d, i * m + col0, 8, true, x, pol);
+                    write8(w_, d, i * m + col0, x, pol);
                 }
             }
-        }
-    } else {
-        for (int k = 0; k < kVecPerThread; ++k) {
-            const int64_t i = row0 + k * RG;
-            if (i >= n) break;
-            const int64_t e0 = i * m + col0;
-            float y[8], w[8], x[8];
-            if (MOM)
-                load_f8<false>(M_ + e0, valid, y, true);
-            else
-                load8_elem(g_, T.f32, e0, valid, y);
-            load8_elem(w_, T.f32, e0, valid, w);
-            const float a = rows[k * RG];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[c] * fminf(a * b[c], ce), w[c] * wdf);
-            store8_elem(T, w_, d, e0, valid, x, pol);
         }
     }
 }
 
-template <bool VEC>
+__device__ void apply_flat_any(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
+                               const Pol &pol) {
+    const FlatMeta F(T, S, tile, meta);
+    const float coefC = __ldcg(&S.coefC);
+    const float wdf = T.decay ? A.wdf : 1.0f;
+    const Dith d = dith_of(A, T);
+    const int64_t numel = T.numel;
+    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
+    FlatPos P(T, e0);
+    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
+        float y[kFlatAhead][8], w[kFlatAhead][8];
+        FlatPos Q[kFlatAhead] = {P, P};
+#pragma unroll
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            Q[h] = P;
+            if (e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                if (T.momentum)
+                    load_f8(T.M + e, T.sal, valid, y[h]);
+                else
+                    load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
+                load8_elem(T.w, T.f32, T.wal, e, valid, w[h], pol);
+            }
+            P.next(T.m);
+        }
+#pragma unroll
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                float sc[8], x[8];
+                F.scales(T, Q[h], valid, A.ce, sc);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[h][c] * sc[c], w[h][c] * wdf);
+                store8_elem(T, d, e, valid, x, pol);
+            }
+        }
+        e0 += kFlatAhead * 8 * kThreads;
+    }
+}
+
 __device__ void apply_full_tile(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile,
                                 const Pol &pol) {
     const float coefC = __ldcg(&S.coefC);
     const float wdf = T.decay ? A.wdf : 1.0f;
-    for (int k = 0; k < kFlatVecPerThread; ++k) {
-        const int64_t e0 = 8 * (int64_t(tile) * kThreads * kFlatVecPerThread + int64_t(k) * kThreads + threadIdx.x);
-        if (e0 >= T.numel) break;
-        const int valid = (int)min(int64_t(8), T.numel - e0);
-        float y[8], v[8], w[8], x[8];
-        if (T.momentum)
-            load_f8<VEC>(T.M + e0, valid, y, true);
-        else if (VEC)
-            unpack_bf8(ld16_hint(T.g + e0, pol.drop), y);
-        else
-            load8_elem(T.g, T.f32, e0, valid, y);
-        load_f8<VEC>(T.v + e0, valid, v, true);
-        if (VEC)
-            unpack_bf8(ld16_hint(T.w + e0, pol.drop), w);
-        else
-            load8_elem(T.w, T.f32, e0, valid, w);
+    const Dith d = dith_of(A, T);
+    const int64_t numel = T.numel;
+    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
+    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
+        float y[kFlatAhead][8], v[kFlatAhead][8], w[kFlatAhead][8];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[c] * fminf(__frsqrt_rn(v[c]), A.ce), w[c] * wdf);
-        const Dith dd = dith_of(A, T);  // on the vector path e0 and base are multiples of 8
-        if (VEC)
-            write8<true>(T.w, dd, e0, valid, true, x, pol);
-        else
-            store8_elem(T, T.w, dd, e0, valid, x, pol);
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (k + h < T.fvpt && e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                if (T.momentum)
+                    load_f8(T.M + e, T.sal, valid, y[h]);
+                else
+                    load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
+                load_f8(T.v + e, T.sal, valid, v[h]);
+                load8_elem(T.w, T.f32, T.wal, e, valid, w[h], pol);
+            }
+        }
+#pragma unroll
+        for (uint32_t h = 0; h < kFlatAhead; ++h) {
+            const int64_t e = e0 + h * 8 * kThreads;
+            if (k + h < T.fvpt && e < numel) {
+                const int valid = (int)min(int64_t(8), numel - e);
+                float x[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    x[c] = fmaf(-coefC, y[h][c] * fminf(__frsqrt_rn(v[h][c]), A.ce), w[h][c] * wdf);
+                store8_elem(T, d, e, valid, x, pol);
+            }
+        }
+        e0 += kFlatAhead * 8 * kThreads;
     }
 }
 
@@ -1649,7 +1846,7 @@ __device__ bool apply_rows_body(const StepArgs &A, const TensorDev &T, int64_t r
                         }
                         acc.add(sumsq8(u));
                     }
-                    write8<true>(w_, d, (i0 + r) * m + 8 * (v * TPB + lay.vi), 8, true, x, sp);
+                    write8(w_, d, (i0 + r) * m + 8 * (v * TPB + lay.vi), x, sp);
                 }
             }
         }
@@ -2026,7 +2223,7 @@ __device__ bool apply_rows_mom_body(const StepArgs &A, const TensorDev &T, int64
                         }
                         acc.add(sumsq8(u));
                     }
-                    write8<true>(w_, d, (i0 + r) * m + 8 * vec, 8, true, x, sp);
+                    write8(w_, d, (i0 + r) * m + 8 * vec, x, sp);
                 }
             }
         }
@@ -2587,31 +2784,23 @@ __device__ void phase_A_strip(const TensorDev &T, uint32_t tile, Smem &sm, const
 // Phase C of a strip or flat tile.
 __device__ void phase_C(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
                         const Pol &pol) {
-    if (T.kind == kKindFactored) {
-        const bool fast = fill_meta(T, S, tile, A.ce, meta);
-        if (T.vec) {
-            if (T.momentum) {
-                if (fast)
-                    apply_fact_tile<true, true, true>(A, T, S, tile, meta, pol);
-                else
-                    apply_fact_tile<true, true, false>(A, T, S, tile, meta, pol);
-            } else {
-                if (fast)
-                    apply_fact_tile<true, false, true>(A, T, S, tile, meta, pol);
-                else
-                    apply_fact_tile<true, false, false>(A, T, S, tile, meta, pol);
-            }
-        } else {
-            if (T.momentum)
-                apply_fact_tile<false, true, false>(A, T, S, tile, meta, pol);
-            else
-                apply_fact_tile<false, false, false>(A, T, S, tile, meta, pol);
-        }
+    if (T.kind != kKindFactored) {
+        apply_full_tile(A, T, S, tile, pol);
+    } else if (!T.vec) {
+        apply_flat_any(A, T, S, tile, meta, pol);
     } else {
-        if (T.vec)
-            apply_full_tile<true>(A, T, S, tile, pol);
-        else
-            apply_full_tile<false>(A, T, S, tile, pol);
+        const bool fast = fill_meta(T, S, tile, A.ce, meta);
+        if (T.momentum) {
+            if (fast)
+                apply_fact_tile<true, true>(A, T, S, tile, meta, pol);
+            else
+                apply_fact_tile<true, false>(A, T, S, tile, meta, pol);
+        } else {
+            if (fast)
+                apply_fact_tile<false, true>(A, T, S, tile, meta, pol);
+            else
+                apply_fact_tile<false, false>(A, T, S, tile, meta, pol);
+        }
     }
 }
 
@@ -2623,7 +2812,7 @@ __global__ void __launch_bounds__(kThreads, SKEW_MINB_SUMSQ)
 }
 
 // A step with row-path tensors runs its strip and flat tiles in the row path's launches, ahead of
-// the row tiles: phase B of the flat tiles needs nothing from phase A or the finalize, so it comes
+// the row tiles, unless there are many of them (kRideElems): phase B of the flat tiles needs nothing from phase A or the finalize, so it comes
 // with phase A. Such a step has four launches instead of seven, and the light tiles' latency (a
 // launch of its own took 12 to 25 us each for phases A, B and C) hides behind the row tiles.
 
@@ -2725,18 +2914,18 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_fallback(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items, uint32_t nB) {
     __shared__ Smem sm;
     __shared__ Meta meta;
-    const Pol pol;
     if (blockIdx.x < nB) {
         const uint2 it = items[blockIdx.x];
-        phase_B_fact(A, it.x, it.y, sm, meta, pol);
+        phase_B_own(A, it.x, it.y, sm, meta);
         return;
     }
+    const Pol pol;
     const uint32_t cnt = __ldcg(A.fb), ctas = gridDim.x - nB;
     uint32_t tile = blockIdx.x - nB;  // of queued tensor q
     for (uint32_t q = 0; q < cnt; ++q) {
-        const uint32_t t = __ldcg(A.fb + 1 + q), nt = A.tensors[t].ntiles;
+        const uint32_t t = __ldcg(A.fb + 1 + q), nt = A.tensors[t].nbc;
         for (; tile < nt; tile += ctas) {
-            phase_B_fact(A, t, tile, sm, meta, pol);
+            phase_B_strip(A, t, tile, sm, meta, pol);
             __syncthreads();
         }
         tile -= nt;
@@ -2794,23 +2983,24 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
         if (ev) cudaEventRecord((cudaEvent_t)ev[k], s);
     };
     const bool rows = L.nR != 0;
+    const uint32_t rA = L.ride ? L.nA : 0, rB = L.ride ? L.nB : 0, rC = L.ride ? L.nC : 0;  // with the row tiles
     mark(0);
-    if (L.nA && !rows) k_sumsq<<<L.nA, kThreads, 0, s>>>(A, L.itemsA);
+    if (L.nA > rA) k_sumsq<<<L.nA, kThreads, 0, s>>>(A, L.itemsA);
     mark(1);
     if (rows) {
         constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem));
         const cudaError_t e = cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
-        k_rowsq<<<L.nA + L.nR, kRowThreads, kSm, s>>>(A, L.itemsA);
+        k_rowsq<<<rA + L.nR, kRowThreads, kSm, s>>>(A, L.itemsA + (L.nA - rA));
     }
     mark(2);
     if (L.nF) k_finalize<<<L.nF, kThreads, 0, s>>>(A, L.itemsF);
     mark(3);
-    if (L.nB && !rows) k_rms<<<L.nB, kThreads, 0, s>>>(A, L.itemsB);
+    if (L.nB > rB) k_rms<<<L.nB, kThreads, 0, s>>>(A, L.itemsB);
     mark(4);
-    if (rows) k_fallback<<<L.nB + L.nFB, kThreads, 0, s>>>(A, L.itemsB, L.nB);
+    if (rows) k_fallback<<<rB + L.nFB, kThreads, 0, s>>>(A, L.itemsB, rB);
     mark(5);
-    if (L.nC && !rows) k_apply<<<L.nC, kThreads, 0, s>>>(A, L.itemsC);
+    if (L.nC > rC) k_apply<<<L.nC, kThreads, 0, s>>>(A, L.itemsC);
     mark(6);
     if (rows) {
         constexpr size_t kSm = max3(sizeof(ApplyRowSmem), sizeof(MomApplySmem), sizeof(FlatSmem));
@@ -2818,7 +3008,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
         static_assert(sizeof(Meta) <= kSm && sizeof(Smem) <= kSm, "light tiles");
         const cudaError_t e = cudaFuncSetAttribute(k_apply_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm);
         if (e != cudaSuccess) return (int)e;
-        k_apply_rows<<<L.nC + L.nCR, kRowThreads, kSm, s>>>(A, L.itemsC);
+        k_apply_rows<<<rC + L.nCR, kRowThreads, kSm, s>>>(A, L.itemsC + (L.nC - rC));
     }
     mark(7);
     return (int)cudaGetLastError();

@@ -54,8 +54,8 @@ Layout layout_of(const TileGeom &G, uint32_t kind, int64_t n, int64_t m) {
     o.nA = fact && !row ? G.ntiles : 0;
     o.nR = row ? G.rtiles : 0;
     o.nF = fact ? G.nfr + G.nfc : 0;
-    o.nB = row ? 0 : G.ntiles;
-    o.nC = row ? 0 : G.ntiles;
+    o.nB = row ? 0 : G.nbc;
+    o.nC = row ? 0 : G.nbc;
     o.nCR = row ? G.atiles : 0;
     size_t off = align256(kErrOffset + 16);  // the status word comes first
     auto put = [&](size_t &at, size_t bytes) {
@@ -176,21 +176,22 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
                                                   : (numel + kFlatTileElems - 1) / kFlatTileElems;
     if (tiles64 > (int64_t(1) << 31)) return SKEW_EINVAL;
     // What the entry point takes is set by the full-sized row tiles of the fixed widths and by the
-    // strip tiles at the others; a matrix whose own tiles (as skew_step cuts it) need more scratch
-    // than there is runs on those.
-    TileGeom G = plan_geometry(kind, momentum, wg_aligned, n, m, numel, 2 * numel);
-    if (G.rowpath == kRowAny && 2 * numel < kAnyGroupBytes) G = plan_geometry(kind, momentum, false, n, m, numel, kWholeGroup);
+    // full-sized strip tiles at the others; a matrix whose own tiles (as skew_step cuts it) need more
+    // scratch than there is runs on those.
+    const bool vec = row_vectors(f32, (((uintptr_t)weight | (uintptr_t)grad) & 15) == 0, ((uintptr_t)M & 15) == 0, m);
+    TileGeom most = plan_geometry(kind, momentum, wg_aligned, vec, false, n, m, numel, kWholeGroup);
+    const bool any = most.rowpath == kRowAny;
+    if (any) most = plan_geometry(kind, momentum, false, vec, false, n, m, numel, kWholeGroup);
+    TileGeom limit = most;
+    limit.nbc = limit.ntiles;
+    if (layout_of(limit, kind, n, m).bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
+    const bool on_rows = any ? 2 * numel >= kAnyGroupBytes : most.rowpath != kRowNone;
+    TileGeom G = plan_geometry(kind, momentum, on_rows, vec, numel < kSmallStrip, n, m, numel, 2 * numel);
     Layout o = layout_of(G, kind, n, m);
-    if (G.rowpath) {
-        const TileGeom most = plan_geometry(kind, momentum, G.rowpath == kRowFixed, n, m, numel, kWholeGroup);
-        const Layout om = layout_of(most, kind, n, m);
-        if (om.bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;
-        if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) {
-            G = most;
-            o = om;
-        }
+    if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) {
+        G = most;
+        o = layout_of(G, kind, n, m);
     }
-    if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
     const bool fact = kind == kKindFactored, row = fact && G.rowpath;
 
     // ---- device address of the fixed array on the current device ---------------------
@@ -226,9 +227,11 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     td.momentum = momentum;
     td.decay = decay;
     auto al16 = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
-    bool vec = !f32 && al16(td.w) && al16(td.g) && (!td.M || al16(td.M));
-    vec = kind == kKindFull ? (vec && numel % 8 == 0 && al16(td.v)) : (vec && m % 8 == 0);
-    td.vec = vec ? 1 : 0;
+    td.vec = kind == kKindFactored ? vec : 0;
+    td.wal = al16(td.w) && al16(td.g);
+    td.sal = (!td.M || al16(td.M)) && (!td.v || al16(td.v));
+    td.nbc = G.nbc;
+    td.fvpt = G.fvpt;
     td.f32 = f32 ? 1u : 0u;
     td.lcl = G.lcl;
     td.strips = G.strips;
@@ -287,6 +290,7 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
                         nFB,
                         o.nC,
                         o.nCR,
+                        false,
                         (const uint2 *)(base + (row ? o.iR : o.iA)),
                         (const uint2 *)(base + o.iF),
                         (const uint2 *)(base + o.iB),

@@ -14,9 +14,20 @@ namespace skew {
 // Every kernel runs 256-thread CTAs; a thread owns 8 consecutive bf16 elements
 // (one 16-byte vector) of up to kVecPerThread rows (strip tiles: 64 Ki elements)
 // or of kFlatVecPerThread flat vectors (full-second-moment tiles: 8 Ki elements,
-// so that the router and the vectors, small, spread over many CTAs).
+// so that the router and the vectors, small, spread over many CTAs). Where a step's
+// strip-path matrices hold fewer than kSmallStrip elements, strip tiles have
+// kVecSmall rows per thread and flat tiles of factored tensors kFlatVecPerThread
+// vectors, else kVecPerThread of both: 608 full tiles fill two waves of two CTAs
+// per SM, and below that a tile's rounds, one after another, set the time (296K
+// elements in 39 tensors: a step 46 -> 37 us).
 constexpr int kThreads = 256;
 constexpr int kVecPerThread = 32;
+constexpr int kVecSmall = 8;
+constexpr int64_t kSmallStrip = int64_t(2 * 2 * 152) * 65536;
+// A step with row tiles runs its strip and flat tiles in their launches while these hold at most
+// kRideElems elements: more of them are faster in launches of their own, where four CTAs share an SM
+// (1.15B elements of 4864 and 7128 columns beside one 4095 x 1000 matrix: 2316 against 2586 us).
+constexpr int64_t kRideElems = int64_t(32) << 20;
 constexpr int kFlatVecPerThread = 4;
 constexpr int64_t kFlatTileElems = int64_t(kThreads) * kFlatVecPerThread * 8;
 constexpr int kFinChunk = 256;  // rows / columns per finalize item
@@ -110,9 +121,10 @@ inline StepCoefs step_coefs(const skew_hparams_t &H, int64_t step) {
 // tensor is always cut the same way and results are bit-identical).
 struct TileGeom {
     uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0;
+    uint32_t nbc = 0, fvpt = 0;  // tiles of phases B and C; vectors per thread of a flat tile
     uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0;
     uint32_t at_rows = 0, atiles = 0;  // row path: phase-C row tiles
-    uint32_t fci = 0;  // row path: columns per finalize item (kFinChunk / fci threads per column)
+    uint32_t fci = 0;  // columns per finalize item (kFinChunk / fci threads per column)
 };
 
 constexpr int64_t kWholeGroup = int64_t(1) << 60;  // as `rest`: full-sized tiles
@@ -142,11 +154,12 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
 constexpr int64_t kAnyGroupBytes = 2 << 20;
 
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
-// gradient pointers are 16-byte aligned; `rest`: bytes of G of the step's row-path
+// gradient pointers are 16-byte aligned; `vec`: row-vectors may be 16-byte accesses (row_vectors);
+// `small`: the step's factored matrices hold fewer than kSmallStrip elements; `rest`: bytes of G of the step's row-path
 // matrices from this one on. Counts fit 32 bits for n, m <= 2^40
 // and n*m <= 2^62 only when the caller has checked the tile count (planner).
-inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, int64_t n, int64_t m, int64_t numel,
-                              int64_t rest) {
+inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, bool vec, bool small, int64_t n,
+                              int64_t m, int64_t numel, int64_t rest) {
     TileGeom g;
     if (kind == kKindFactored) {
         const int64_t vecs = (m + 7) / 8;  // 8-column groups per row
@@ -156,7 +169,7 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
             ++g.lcl;
         }
         g.strips = (uint32_t)((m + 8 * lc - 1) / (8 * lc));
-        g.tile_rows = (uint32_t)(kVecPerThread * (kThreads / lc));
+        g.tile_rows = (uint32_t)((small ? kVecSmall : kVecPerThread) * (kThreads / lc));
         g.rowtiles = (uint32_t)((n + g.tile_rows - 1) / g.tile_rows);
         g.ntiles = g.strips * g.rowtiles;
         g.nfc = (uint32_t)((m + kFinChunk - 1) / kFinChunk);
@@ -197,17 +210,38 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
             g.nfc = (uint32_t)((m + g.fci - 1) / g.fci);
         } else {
             g.nfr = (uint32_t)((n + kFinChunk - 1) / kFinChunk);
+            // tall matrices: up to 32 threads share a column (one adds 8 tiles per trip to L2)
+            uint32_t tpc = 1;
+            while (tpc < 32 && g.rowtiles > 32u * tpc) tpc <<= 1;
+            g.fci = (uint32_t)(kFinChunk / tpc);
+            g.nfc = (uint32_t)((m + g.fci - 1) / g.fci);
+        }
+        g.nbc = g.ntiles;
+        if (!g.rowpath && !vec) {
+            // (big tiles of a narrow matrix would hold more rows than their scales have room for)
+            g.fvpt = (uint32_t)(small || (m < 64 && rest < kWholeGroup) ? kFlatVecPerThread : kVecPerThread);
+            const int64_t tile = int64_t(kThreads) * 8 * g.fvpt;
+            g.nbc = (uint32_t)((numel + tile - 1) / tile);
         }
     } else {
-        g.rowtiles = (uint32_t)((numel + kFlatTileElems - 1) / kFlatTileElems);
-        g.ntiles = g.rowtiles;
+        // one round per thread spreads a small tensor over more CTAs
+        g.fvpt = numel < 2 * 152 * kFlatTileElems ? 1 : kFlatVecPerThread;
+        const int64_t tile = int64_t(kThreads) * 8 * g.fvpt;
+        g.rowtiles = (uint32_t)((numel + tile - 1) / tile);
+        g.ntiles = g.nbc = g.rowtiles;
     }
     return g;
 }
 
+// Whether a factored tensor's row-vectors may be 16-byte accesses: bf16, every row of W, G and M on
+// a 16-byte boundary.
+inline bool row_vectors(bool f32, bool wg_aligned, bool m_aligned, int64_t m) {
+    return !f32 && wg_aligned && m_aligned && m % 8 == 0;
+}
+
 // Entries of a tensor's sums of U^2.
 inline uint32_t u2_len(const TileGeom &g) {
-    return g.rowpath && 2 * g.atiles > g.ntiles ? 2 * g.atiles : g.ntiles;
+    return g.rowpath && 2 * g.atiles > g.nbc ? 2 * g.atiles : g.nbc;
 }
 
 // Where a row-path tensor whose clamp may bind gets its sum(U^2): phase B, or phase C (clip factor 1).
@@ -230,7 +264,7 @@ struct TensorDev {
     float *rmin;        // row path: smallest positive R_i per row tile [rtiles]
     double *fsum;       // row path: sum of P_j / C_j per finalize item [nfc]
     float *fmin;        // row path: smallest C_j with P_j > 0 per finalize item [nfc]
-    float2 *u2;         // sums of (U / coef)^2 as (hi, lo) pairs: per phase-B tile [ntiles], or on the
+    float2 *u2;         // sums of (U / coef)^2 as (hi, lo) pairs: per phase-B tile [nbc], or on the
                         // row path per half of a phase-C tile [2 atiles] (u2_len)
     int64_t n, m, numel;
     double inv_n, inv_numel;  // 1 / n, 1 / numel
@@ -238,18 +272,20 @@ struct TensorDev {
     uint64_t base;      // dither index of element 0 (a matrix of a stacked tensor: its offset)
     uint32_t kind, momentum, decay;
     uint32_t vec;       // 1: 16-byte vector loads / stores are legal (bf16 tensors only)
+    uint32_t wal, sal;  // 1: w and g (M and v) start on 16-byte boundaries
     uint32_t f32;       // 1: weights and gradient are fp32 (w, g then address floats; no dither)
     uint32_t lcl;       // factored: log2 of lanes along a row (LC)
     uint32_t strips;    // factored: column strips of 8*LC columns
     uint32_t rowtiles;  // factored: row tiles of tile_rows rows; full: flat tiles
     uint32_t tile_rows; // factored: rows per tile = 32 * (256 / LC)
-    uint32_t ntiles;    // update tiles of this tensor
+    uint32_t ntiles;    // strip tiles (full: flat tiles) of this tensor
+    uint32_t nbc, fvpt; // tiles of phases B and C; vectors per thread of a flat tile
     uint32_t nfr, nfc;  // factored: finalize items over rows / columns
     uint32_t rowpath;   // RowPath; nonzero: whole-row phase A (k_rowsq) and the bilinear sum of U^2
     uint32_t cr;        // row path: rows per chunk
     uint32_t rt_rows;   // row path: rows per phase-A row tile
     uint32_t rtiles;    // row path: phase-A row tiles
-    uint32_t fci;       // row path: columns per finalize item
+    uint32_t fci;       // columns per finalize item
     uint32_t at_rows;   // row path: rows per phase-C row tile (<= 1024 at the fixed widths)
     uint32_t atiles;    // row path: phase-C row tiles
 };
@@ -292,17 +328,19 @@ struct StepArgs {
 
 // The phases of one step: item lists (tensor, local tile / item) in device
 // memory and their lengths.
-//   A  strip-tile sums of squares (strip-path factored tensors); in a step with row
-//      tiles, also the update-RMS tiles of full tensors
+//   A  strip-tile sums of squares (strip-path factored tensors); when riding, also
+//      the update-RMS tiles of full tensors
 //   R  row-tile sums of squares and bilinear partials (row-path tensors)
 //   F  finalize items (rows and columns; columns only on the row path)
-//   B  update-RMS tiles (strip-path factored tensors; without row tiles full tensors too)
+//   B  update-RMS tiles (strip-path factored tensors; unless riding, full tensors too)
 //   FB phase B of the row-path tensors whose finalize asked for it (nFB CTAs)
 //   C  apply strip and flat tiles (tensors not on the row path)
 //   CR apply row tiles (row-path tensors)
-// The items of R follow those of A, and those of CR those of C.
+// The items of R follow those of A, and those of CR those of C; `ride`: A, B and C go into the launches
+// of the row tiles (R, FB and CR).
 struct LaunchPlan {
     uint32_t nA, nR, nF, nB, nFB, nC, nCR;
+    bool ride;
     const uint2 *itemsA, *itemsF, *itemsB, *itemsC;
 };
 

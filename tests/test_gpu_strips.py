@@ -1,0 +1,42 @@
+"""Strip and flat tiles against the oracle: factored tensors without 16-byte row-vectors (odd widths
+below and above 8, fp32, unaligned pointers, stacks whose matrices start inside a Philox block), at
+both tile sizes (few strip-path elements, and many)."""
+import pytest
+
+from paper_2607_19058_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+E, B, R = WL.TIER_EXPERT, WL.TIER_BACKBONE, WL.TIER_ROUTER
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2607_19058_gb300 import _build
+    _build.build()
+    import oracle
+    oracle.build()
+
+
+def _specs():
+    shapes = [(1, 1), (3000, 1), (1025, 2), (700, 7), (257, 9), (1, 8191), (300, 127), (37, 333), (129, 1001), (513, 60),
+              (70, 4100), (9, 5000)]
+    out = [WL.Spec(f"{'eb'[t]}{n}x{m}{'f' if f else ''}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1, fp32=f)
+           for k, (n, m) in enumerate(shapes) for t in (0, 1) for f in (False, True)]
+    out += [WL.Spec(f"s{k}x{n}x{m}", (k, n, m), t) for k, n, m, t in ((3, 5, 7, E), (5, 33, 13, B), (2, 3, 1, E))]
+    return out + [WL.Spec("v4099", (4099,), B), WL.Spec("v4099f", (4099,), B, fp32=True), WL.Spec("r33x65", (33, 65), R),
+                  WL.Spec("r3x33x65", (3, 33, 65), R)]
+
+
+@pytest.mark.parametrize("many", [False, True], ids=["few", "many"])
+@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05)], ids=["eps1e-30", "paper"])
+def test_flat_and_strip_tiles(many, hp):
+    import parity
+    specs = _specs()
+    misalign = tuple(range(0, len(specs), 5))
+    if many:  # past the line where strip tiles grow to 32 rows per thread
+        specs += [WL.Spec("e4100x8200", (4100, 8200), E, expert=0), WL.Spec("b7001x901", (7001, 901), B)]
+    h = parity.Harness(WL.Workload("strips", specs, WL.HP(), "toy", steps=2), hp_override=hp, misalign=misalign)
+    for t in (1, 2):
+        h.step(t, seed=23 * t, **({"gscale": 0.37} if t == 2 else {}))
+    h.close()
