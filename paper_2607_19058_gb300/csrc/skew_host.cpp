@@ -521,7 +521,7 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
         ev = h->prof_ev.data() + size_t(h->prof_used) * (kProfLaunches + 1);
         ++h->prof_used;
     }
-    cudaError_t e = cudaMemsetAsync(h->ws + h->ws_scal, 0, h->ws_fb + 4 - h->ws_scal, s);
+    cudaError_t e = (cudaError_t)launch_reset(h->ws + h->ws_scal, h->ws_fb + 4 - h->ws_scal, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "reset of per-step scalars");
     auto items = [&](size_t at) { return reinterpret_cast<const uint2 *>(h->ws + at); };
     const LaunchPlan L{h->nA, (uint32_t)h->itemsA.size() - h->nA, (uint32_t)h->itemsF.size(), (uint32_t)h->itemsB.size(),

@@ -336,13 +336,17 @@ struct StepArgs {
 //   FB phase B of the row-path tensors whose finalize asked for it (nFB CTAs)
 //   C  apply strip and flat tiles (tensors not on the row path)
 //   CR apply row tiles (row-path tensors)
-// The items of R follow those of A, and those of CR those of C; `ride`: A, B and C go into the launches
+// A null table stands for tensor 0's tiles in order. The items of R follow those of A, and those of CR those of C; `ride`: A, B and C go into the launches
 // of the row tiles (R, FB and CR).
 struct LaunchPlan {
     uint32_t nA, nR, nF, nB, nFB, nC, nCR;
     bool ride;
     const uint2 *itemsA, *itemsF, *itemsB, *itemsC;
 };
+
+// Enqueues the clearing of the per-step scalars and of the phase-B queue's length at `p` (a multiple of
+// 4 bytes). Returns a cudaError_t value.
+int launch_reset(void *p, size_t bytes, void *stream);
 
 constexpr int kLaunches = 7;
 
