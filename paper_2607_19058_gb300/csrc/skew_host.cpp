@@ -58,6 +58,7 @@ struct skew_handle {
     std::vector<uint2> itemsA, itemsF, itemsB, itemsC;  // A + R, F, B, C + CR: per phase, tensors in order
     uint32_t nA = 0, nC = 0;  // items of A before those of R, of C before those of CR
     uint32_t n_rowpath = 0;  // tensors on the row path
+    SmallPlan small;         // not used unless small.ctas
     bool ride = false;       // the strip and flat tiles go into the row tiles' launches
     uint32_t fb_ctas = 0;    // CTAs of the row path's phase-B launch (set at bind)
     char *state = nullptr, *ws = nullptr;
@@ -238,6 +239,13 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     }
     h->ride = h->n_rowpath && light <= kRideElems;
 
+    // a step of small tensors only: one launch
+    h->small = plan_small(n_plans, [&](auto &&f) {
+        for (const TPlan &q : h->t)
+            if (!f(q.kind == kKindFactored ? q.n : q.numel, q.kind == kKindFactored ? q.m : 1)) return false;
+        return true;
+    });
+
     // Item tables: every factored tensor's tiles (phase A), finalize items
     // (phase F) and every tensor's tiles (phases B and C), tensors in order.
     try {
@@ -340,6 +348,7 @@ int32_t skew_num_tensors(const skew_handle_t *h) { return h ? (int32_t)h->desc.s
 
 int64_t skew_launches_per_step(const skew_handle_t *h) {
     if (!h) return 0;
+    if (h->small.ctas) return 1;
     // with row tiles k_rowsq, k_fallback and k_apply_rows; the others where they have items of their own
     const uint32_t rows = h->n_rowpath > 0;
     return 3 * rows + int64_t(!h->itemsF.empty()) +
@@ -444,6 +453,14 @@ int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace
         T.at_rows = p.at_rows;
         T.atiles = p.atiles;
         T.fci = p.fci;
+        T.srows = 0;
+        if (h->small.ctas) {
+            if (!fact) {  // stepped as numel x 1
+                T.n = p.numel;
+                T.m = 1;
+            }
+            T.srows = (uint32_t)small_rows(T.n, h->small.ctas);
+        }
     }
     auto put = [&](size_t at, const std::vector<uint2> &v) {
         if (!v.empty()) std::memcpy(img.data() + (at - h->ws_tab), v.data(), v.size() * sizeof(uint2));
@@ -520,6 +537,12 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
     if (h->prof_used < h->prof_max) {
         ev = h->prof_ev.data() + size_t(h->prof_used) * (kProfLaunches + 1);
         ++h->prof_used;
+    }
+    if (h->small.ctas) {
+        const cudaError_t r =
+            (cudaError_t)launch_small(a, nullptr, (uint32_t)h->t.size(), h->small, s, reinterpret_cast<void *const *>(ev));
+        if (r != cudaSuccess) return cuda_fail(h, r, "kernel launch");
+        return SKEW_OK;
     }
     cudaError_t e = (cudaError_t)launch_reset(h->ws + h->ws_scal, h->ws_fb + 4 - h->ws_scal, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "reset of per-step scalars");

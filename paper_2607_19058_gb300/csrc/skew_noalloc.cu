@@ -252,6 +252,16 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     }
 
     cudaStream_t s = (cudaStream_t)stream;
+    const SmallPlan sp = plan_small(1, [&](auto &&f) { return f(fact ? n : numel, fact ? m : 1); });
+    if (sp.ctas) {  // one launch, which needs of the scratch only the scalars
+        if (!fact) {
+            td.n = numel;
+            td.m = 1;
+        }
+        td.srows = (uint32_t)small_rows(td.n, sp.ctas);
+        a.tensors = nullptr;
+        return launch_small(a, &td, 1, sp, stream, nullptr) == (int)cudaSuccess ? SKEW_OK : SKEW_ECUDA;
+    }
     k_noalloc_setup<<<1, 1, 0, s>>>(td, (TensorDev *)(base + o.tens), (TensorScal *)(base + o.scal),
                                     (uint32_t *)(base + o.fb));
     e = cudaGetLastError();

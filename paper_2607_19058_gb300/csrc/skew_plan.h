@@ -288,6 +288,7 @@ struct TensorDev {
     uint32_t fci;       // columns per finalize item
     uint32_t at_rows;   // row path: rows per phase-C row tile (<= 1024 at the fixed widths)
     uint32_t atiles;    // row path: phase-C row tiles
+    uint32_t srows;     // k_small: rows (full: elements, m = 1) of a CTA's slice
 };
 
 // Per-tensor scalars of the current step (zeroed at the start of every step).
@@ -348,7 +349,66 @@ struct LaunchPlan {
 // 4 bytes). Returns a cudaError_t value.
 int launch_reset(void *p, size_t bytes, void *stream);
 
-constexpr int kLaunches = 7;
+constexpr int kLaunches = 7;  // kernels a step may launch in turn
+
+// A step of small tensors only runs as one launch, a cluster of `ctas` CTAs per tensor (k_small).
+constexpr int kSmallThreads = 512;
+constexpr size_t kSmallHeadBytes = 4096;                     // fixed part of its shared memory
+constexpr size_t kSmallSmem = 224 * 1024;                    // most that it takes
+constexpr int64_t kSmallCtas = 256;                          // CTAs of a launch
+struct SmallPlan {
+    uint32_t ctas = 0;  // 0: not a step for k_small
+    size_t smem = 0;
+};
+
+// Rows (elements of a full tensor, stepped as n x 1) of a CTA's slice, a multiple of 8 so that a slice
+// starts on a Philox block and a 16-byte boundary where the tensor does.
+inline int64_t small_rows(int64_t n, uint32_t ctas) { return ((n + ctas - 1) / ctas + 7) / 8 * 8; }
+
+// Shared memory of one CTA's slice: its elements, row scales and twice the columns as fp32.
+inline int64_t small_bytes(int64_t n, int64_t m, uint32_t ctas) {
+    const int64_t rows = small_rows(n, ctas);
+    return (int64_t)kSmallHeadBytes + 4 * (rows * m + rows + 2 * m);
+}
+
+// Adds one tensor (full: n = numel, m = 1) to the plan of a step over `tensors` of them: the fewest CTAs
+// whose shared memory holds a slice, in clusters of at most 8.
+inline bool small_fits(int64_t n, int64_t m, uint32_t ctas) {
+    return n <= (int64_t(1) << 22) && m <= (int64_t(1) << 16) && small_bytes(n, m, ctas) <= (int64_t)kSmallSmem;
+}
+
+// The rule: every tensor of the step fits, with at most kSmallCtas CTAs in all (two waves at one CTA per
+// SM, one at two): beyond, the strip tiles' four launches are as fast. Slices are then halved while that
+// holds: the toy MoE's 39 tensors take 21 us in clusters of two, 17 in clusters of four.
+template <typename Each>
+inline SmallPlan plan_small(int64_t tensors, Each each) {
+    SmallPlan P;
+    if (tensors < 1 || tensors > kSmallCtas) return P;
+    auto fits = [&](uint32_t c) { return each([c](int64_t n, int64_t m) { return small_fits(n, m, c); }); };
+    uint32_t c = 1;
+    while (c <= 8 && !fits(c)) c *= 2;
+    if (c > 8 || tensors * c > kSmallCtas) return P;
+    // smaller slices, while they still hold 4 elements per thread
+    while (c < 8 && tensors * c * 2 <= kSmallCtas &&
+           !each([c](int64_t n, int64_t m) { return small_rows(n, 2 * c) * m < 4 * kSmallThreads; }))
+        c *= 2;
+    P.ctas = c;
+    int64_t most = 0;
+    each([&](int64_t n, int64_t m) {
+        const int64_t b = small_bytes(n, m, c);
+        most = b > most ? b : most;
+        return true;
+    });
+    P.smem = size_t(most);
+    return P;
+}
+
+// Enqueues the step of `tensors` small tensors (A.tensors, or `one` when that is null) as one launch;
+// `ev` as for launch_phases (its time is that of the last place). Returns a cudaError_t value.
+struct TensorDev;
+int launch_small(const StepArgs &A, const TensorDev *one, uint32_t tensors, const SmallPlan &P, void *stream,
+                 void *const *ev);
+
 
 // Enqueues the phases of `L` as grouped launches (A, F, B, C; with row tiles A + R, F,
 // B + FB, C + CR; empty ones skipped) on `stream`, each given the step parameters by value. If `ev` is
