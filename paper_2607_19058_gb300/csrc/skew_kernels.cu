@@ -2308,7 +2308,7 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
 }
 
 // ---------------------------------------------------------------------------
-// Row path for any other width m = 8 V in [256, 4096] (phase A; phase C is
+// Row path for any other width m = 8 V in [128, 4096] (phase A; phase C is
 // apply_flat_tile). The same algorithm as rowsq_tile / rowsq_mom_tile on a layout
 // formed at run time: a row belongs to wpr = ceil(V / (32 NV)) warps, of which a
 // thread owns vectors vi, vi + 32 wpr, ... (columns stay in its registers), and

@@ -58,11 +58,12 @@ constexpr int kMomChunks = 64;
 // Row path of the widths m = 8 V in [kAnyMin, kAnyMax] that are not 512, 1024, 2048 or 4096
 // (rowsq_gen_tile, apply_flat_tile): rows per thread and phase-A chunk at NV vectors per
 // thread and row, and the floats of shared memory that hold phase C's scales.
-// Below 256 columns a row fills less than a warp, and above 4096 the column sums of a row do
+// Below 128 columns a row fills less than half a warp (20M parameters of a 256-wide model with experts
+// of 248 columns: strip tiles below 256 91 us, below 128 72 us), and above 4096 the column sums of a row do
 // not fit the registers of two 256-thread CTAs per SM: both stay on the strip tiles. Against
 // the strip tiles (three reads of G): 930M parameters in 3072 x 1536 experts 1872 -> 1259 us.
 enum RowPath : uint32_t { kRowNone = 0, kRowFixed = 1, kRowAny = 2 };
-constexpr int64_t kAnyMin = 256, kAnyMax = 4096;
+constexpr int64_t kAnyMin = 128, kAnyMax = 4096;
 constexpr int64_t kAnyTileBytes = 1 << 20;  // bf16 bytes of a tile in phases A and C, as of the fixed widths
 constexpr int kFlatScales = 4200;
 __host__ __device__ constexpr int gen_rows_per_thread(int nv, bool mom) { return (nv == 1 ? 8 : 4) / (mom ? 2 : 1); }
@@ -138,11 +139,15 @@ constexpr int64_t kWholeGroup = int64_t(1) << 60;  // as `rest`: full-sized tile
 // momentum (a second one costs the finalize more partials than it saves: k_rowsq 331, not 321) and
 // two with it, phase C three. `parts`: tiles a matrix may have before its column partials would outgrow the
 // no-alloc scratch; it then keeps to one wave of tiles, up to twice `most` each.
+// (Tiles below kWaveTileBytes come in one wave, which saves the second wave's ramps: k_apply_rows of
+// 118M parameters in 816 x 408 experts 162 -> 149 us.)
+constexpr int64_t kWaveTileBytes = 128 << 10;
 inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_t chunk, int64_t least, int64_t most,
                                 int64_t parts) {
     const int64_t ctas = 2 * 152;
     auto per = [chunk](int64_t bytes, int64_t tiles) { return (bytes + tiles * chunk - 1) / (tiles * chunk); };
-    int64_t t = per(rest, ctas * waves);
+    int64_t t = per(rest, ctas), whole = kWaveTileBytes / chunk;  // a single wave of small tiles: no second ramp
+    if (t > whole) t = per(rest, ctas * waves) > whole ? per(rest, ctas * waves) : whole;
     t = t < least ? least : t > most ? most : t;
     if (parts && rest < kWholeGroup && own > t * chunk * parts && own <= 2 * most * chunk * ctas) t = per(own, ctas);
     return (uint32_t)t;

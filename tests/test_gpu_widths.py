@@ -1,4 +1,4 @@
-"""Whole-row tiles at widths other than 512, 1024, 2048 and 4096 (any multiple of 8 from 256 to 4096),
+"""Whole-row tiles at widths other than 512, 1024, 2048 and 4096 (any multiple of 8 from 128 to 4096),
 against the oracle: the narrowest and widest, widths whose rows take 1 to 8 warps and one or two
 vectors per thread, ragged last tiles and chunks, one-row matrices, stacks, with and without momentum."""
 import pytest
@@ -10,9 +10,9 @@ from paper_2607_19058_gb300 import workloads as WL
 pytestmark = pytest.mark.gpu
 
 E, B = WL.TIER_EXPERT, WL.TIER_BACKBONE
-#          rows, width: 64-row chunks; 2 warps a row; 5 of 8 warps; a partial last warp; 1 row side by side;
+#          rows, width: rows of half a warp; 64-row chunks; 2 warps a row; 5 of 8 warps; a partial last warp; 1 row side by side;
 #          two vectors a thread, the second for few lanes; three quarters of the warps; the widest
-SHAPES = [(2113, 256), (1, 256), (700, 264), (333, 776), (517, 1032), (131, 1408), (9, 2040), (130, 2056), (257, 2880),
+SHAPES = [(2113, 128), (700, 200), (2113, 256), (1, 256), (700, 264), (333, 776), (517, 1032), (131, 1408), (9, 2040), (130, 2056), (257, 2880),
           (301, 3072), (5, 4088), (267, 4088)]
 
 
