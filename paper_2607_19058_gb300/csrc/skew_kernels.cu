@@ -2317,9 +2317,9 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
 // K rpp whole rows (at most 32 KB of G, or 48 KB of G and M), in as many ring slots
 // as 96 KB holds. What bounds it: the chain of two passes and two barriers per chunk, as
 // for the fixed widths (ncu: barrier stalls first), with fewer of the eight warps working.
-// 512 MiB of G: m = 1536 126 us (4.2 TB/s, after a write-back of the last launch's dirty
-// L2), 768 129, 3072 131, against 105 to 117 us at the fixed widths; with momentum 212 to
-// 217 us (6.2 TB/s of G and M) at every width. Branches on the lanes past a row's end made
+// 512 MiB of G: m = 1536 117 us (4.6 TB/s, after a write-back of the last launch's dirty
+// L2), 768 120, 1408 124, 3072 127, against 105 to 110 us at the fixed widths; with momentum
+// 210 to 219 us (6.2 TB/s of G and M) at every width. Branches on the lanes past a row's end made
 // it 536 us where reading zeros instead takes 405 (930M parameters in 3072 x 1536 experts).
 // ---------------------------------------------------------------------------
 constexpr int kGenStages = 8;
@@ -2333,6 +2333,7 @@ struct GenSmem {
     float inv[64];      // 1 / R_i of the chunk's rows (0: no contribution)
     double rsum[2];
     float rmin[2];
+    uint32_t first;     // 1: the layout starts with the third warp
 };
 constexpr uint32_t kGenZero = kGenRingBytes / 16;  // index of `zero` from `ring`
 static_assert(offsetof(GenSmem, zero) == 16 * kGenZero, "zero follows the ring");
@@ -2368,13 +2369,20 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
     if (tid == 0) {
         for (uint32_t st = 0; st < stages; ++st) mbar_init(&sm.full[st], 1);
         fence_mbar_init();
+        // the warps left idle sit on the same two of the SM's four schedulers in every CTA: the CTAs in
+        // the SM's second half of warp slots start with the third warp (a hint; any value is right).
+        // 512 MiB of G, before: 126 us at m = 1536, 129 at 768, 133 at 1408
+        uint32_t slot;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+        sm.first = (slot >> 3) & 1u;
     }
     if (tid < 8) reinterpret_cast<uint32_t *>(sm.zero)[tid] = 0u;
     __syncthreads();
     if (tid == 0)
         for (uint32_t c = 0; c < nch && c < stages; ++c) issue(c, c);
 
-    const uint32_t rp = warp / wpr, vi = (warp - rp * wpr) * 32u + lane;
+    const uint32_t lw = (warp + 2 * sm.first) & 7u;  // the warp's place in the layout
+    const uint32_t rp = lw / wpr, vi = (lw - rp * wpr) * 32u + lane;
     const bool on = rp < rpp;  // the warp has rows (the same for its lanes)
     bool act[NV];              // the thread has vector vi + v lpr
     uint32_t step[NV];         // vectors from one of its rows to the next
@@ -2445,7 +2453,7 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
         }
         int j;
         const float tot = warp_sum_transposed<K>(rs, j);
-        if ((lane & (K == 8 ? 3 : K == 4 ? 7 : 15)) == 0) sm.part[warp][j] = tot;
+        if ((lane & (K == 8 ? 3 : K == 4 ? 7 : 15)) == 0) sm.part[lw][j] = tot;
         if (__syncthreads_or(!ok)) break;  // every slot before this one has landed
         // the slot of chunk c (when its values are held), or else of chunk c - 1, is free: refill it
         // (from the last warp: the first ones form the chunk's row scales, which the CTA waits for)
@@ -2557,10 +2565,11 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
         __syncthreads();  // the ring is free: every chunk is consumed
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            mcs[tid * 8 + 2 * q] = cs[0][q].x;
-            mcs[tid * 8 + 2 * q + 1] = cs[0][q].y;
-            mpp[tid * 8 + 2 * q] = make_float2(ph[0][q].x, pl[0][q].x);
-            mpp[tid * 8 + 2 * q + 1] = make_float2(ph[0][q].y, pl[0][q].y);
+            const uint32_t o = (lw * 32 + lane) * 8 + 2 * q;
+            mcs[o] = cs[0][q].x;
+            mcs[o + 1] = cs[0][q].y;
+            mpp[o] = make_float2(ph[0][q].x, pl[0][q].x);
+            mpp[o + 1] = make_float2(ph[0][q].y, pl[0][q].y);
         }
         __syncthreads();
         for (uint32_t e = tid; e < m; e += kRowThreads) {
