@@ -56,6 +56,7 @@ struct skew_handle {
     size_t ws_scal = 0, ws_fb = 0, ws_err = 0, ws_tab = 0, ws_tab_end = 0;
     size_t ws_tens = 0, ws_itemsA = 0, ws_itemsF = 0, ws_itemsB = 0, ws_itemsC = 0;
     std::vector<uint2> itemsA, itemsF, itemsB, itemsC;  // A + R, F, B, C + CR: per phase, tensors in order
+    uint32_t nRW = 0;         // items of R that go to k_rowsq_wide (the last)
     uint32_t nA = 0, nC = 0;  // items of A before those of R, of C before those of CR
     uint32_t n_rowpath = 0;  // tensors on the row path
     SmallPlan small;         // not used unless small.ctas
@@ -161,7 +162,8 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     const int64_t kMaxExtent = int64_t(1) << 40;
     // whole-row tiles are for bf16 rows on 16-byte boundaries
     auto row_aligned = [](const TPlan &q) { return !q.f32 && wg_aligned(q); };
-    int64_t any_bytes = 0;  // bytes of G of the matrices that only kRowAny's whole-row tiles serve
+    int64_t any_narrow = 0, any_wide = 0;  // bytes of G of the matrices that only kRowAny's row tiles serve
+    bool fixed = false;                    // matrices of the fixed widths
     for (int32_t k = 0; k < n_params; ++k) {
         const skew_param_desc_t &d = params[k];
         TPlan p;
@@ -195,7 +197,8 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.base = (uint64_t)(e * p.numel);
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
                 geometry(q, row_aligned(q), false, kWholeGroup);  // which path
-                if (q.rowpath == kRowAny) any_bytes += 2 * q.numel;
+                if (q.rowpath == kRowAny) (q.m > kAnyNarrow ? any_wide : any_narrow) += 2 * q.numel;
+                fixed |= q.rowpath == kRowFixed;
                 h->t.push_back(q);
             }
         } catch (...) {
@@ -223,10 +226,10 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
 
     // Tiles, now that the paths and the state's alignment are known: the row tiles by the bytes that
     // follow, from the last matrix back.
-    const bool any = any_bytes >= kAnyGroupBytes;
+    const AnyWidths any = any_widths(any_narrow, any_wide, fixed);
     int64_t rest = 0, light = 0, fact = 0;  // elements off the row path, and of factored tensors
     for (TPlan &q : h->t) {
-        if (q.rowpath == kRowAny && !any) q.rowpath = kRowNone;
+        if (q.rowpath == kRowAny && !(q.m > kAnyNarrow ? any.wide : any.narrow)) q.rowpath = kRowNone;
         if (!q.rowpath) light += q.numel;
         if (q.kind == kKindFactored) fact += q.numel;
     }
@@ -249,7 +252,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     // Item tables: every factored tensor's tiles (phase A), finalize items
     // (phase F) and every tensor's tiles (phases B and C), tensors in order.
     try {
-        std::vector<uint2> itemsR, itemsCR;
+        std::vector<uint2> itemsR, itemsRW, itemsCR;
         auto all = [](std::vector<uint2> &v, int q, uint32_t n) {
             for (uint32_t i = 0; i < n; ++i) v.push_back(make_uint2(q, i));
         };
@@ -257,7 +260,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             const TPlan &p = h->t[q];
             const bool fact = p.kind == kKindFactored;
             if (p.rowpath) {
-                all(itemsR, q, p.rtiles);
+                all(p.rowpath == kRowAny && p.m > kAnyNarrow ? itemsRW : itemsR, q, p.rtiles);
                 all(itemsCR, q, p.atiles);
             } else {
                 if (fact) all(h->itemsA, q, p.ntiles);
@@ -286,6 +289,8 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         itemsCR.resize(ncr - nsplit);
         itemsCR.insert(itemsCR.end(), tail.begin(), tail.end());
         h->itemsA.insert(h->itemsA.end(), itemsR.begin(), itemsR.end());
+        h->itemsA.insert(h->itemsA.end(), itemsRW.begin(), itemsRW.end());
+        h->nRW = (uint32_t)itemsRW.size();
         h->itemsC.insert(h->itemsC.end(), itemsCR.begin(), itemsCR.end());
     } catch (...) {
         delete h;
@@ -350,8 +355,8 @@ int64_t skew_launches_per_step(const skew_handle_t *h) {
     if (!h) return 0;
     if (h->small.ctas) return 1;
     // with row tiles k_rowsq, k_fallback and k_apply_rows; the others where they have items of their own
-    const uint32_t rows = h->n_rowpath > 0;
-    return 3 * rows + int64_t(!h->itemsF.empty()) +
+    const uint32_t rows = h->n_rowpath > 0, rA = h->ride ? h->nA : 0;
+    return 2 * rows + int64_t(rA + (h->itemsA.size() - h->nA) > h->nRW) + int64_t(h->nRW > 0) + int64_t(!h->itemsF.empty()) +
            (h->ride ? 0 : int64_t(h->nA > 0) + int64_t(!h->itemsB.empty()) + int64_t(h->nC > 0));
 }
 
@@ -548,7 +553,7 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
     if (e != cudaSuccess) return cuda_fail(h, e, "reset of per-step scalars");
     auto items = [&](size_t at) { return reinterpret_cast<const uint2 *>(h->ws + at); };
     const LaunchPlan L{h->nA, (uint32_t)h->itemsA.size() - h->nA, (uint32_t)h->itemsF.size(), (uint32_t)h->itemsB.size(),
-                       h->n_rowpath ? h->fb_ctas : 0u, h->nC, (uint32_t)h->itemsC.size() - h->nC, h->ride,
+                       h->n_rowpath ? h->fb_ctas : 0u, h->nC, (uint32_t)h->itemsC.size() - h->nC, h->nRW, h->ride,
                        items(h->ws_itemsA), items(h->ws_itemsF), items(h->ws_itemsB), items(h->ws_itemsC)};
     e = (cudaError_t)launch_phases(a, L, s, reinterpret_cast<void *const *>(ev));
     if (e != cudaSuccess) return cuda_fail(h, e, "kernel launch");

@@ -2308,7 +2308,7 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
 }
 
 // ---------------------------------------------------------------------------
-// Row path for any other width m = 8 V in [128, 4096] (phase A; phase C is
+// Row path for any other width m = 8 V in [128, 8192] (phase A; phase C is
 // apply_flat_tile). The same algorithm as rowsq_tile / rowsq_mom_tile on a layout
 // formed at run time: a row belongs to wpr = ceil(V / (32 NV)) warps, of which a
 // thread owns vectors vi, vi + 32 wpr, ... (columns stay in its registers), and
@@ -2321,33 +2321,40 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
 // L2), 768 120, 1408 124, 3072 127, against 105 to 110 us at the fixed widths; with momentum
 // 210 to 219 us (6.2 TB/s of G and M) at every width. Branches on the lanes past a row's end made
 // it 536 us where reading zeros instead takes 405 (930M parameters in 3072 x 1536 experts).
+// Widths above 4096 have CTAs of W = 16 warps, one per SM, and a ring of twice the size:
+// 512 MiB of G at m = 5120 147 us, 7168 129, 8192 124; a step of 1.16B parameters of 4864
+// and 7128 columns 2314 us on strip tiles and 1653 so.
 // ---------------------------------------------------------------------------
 constexpr int kGenStages = 8;
-constexpr int kGenRingBytes = 3 * 32768;
+constexpr int kGenRingBytes = 3 * 32768;  // of the 8-warp tile
 
+// W warps: 8, or 16 for the widths above 4096.
+template <int W>
 struct GenSmem {
-    uint4 ring[kGenRingBytes / 16];
+    uint4 ring[W / 8 * kGenRingBytes / 16];
     uint4 zero[2];      // what the lanes past a row's end (and rows past the matrix) read
     uint64_t full[kGenStages];
-    float part[8][8];   // per-warp row partial sums of the chunk
+    float part[W][8];   // per-warp row partial sums of the chunk
     float inv[64];      // 1 / R_i of the chunk's rows (0: no contribution)
     double rsum[2];
     float rmin[2];
     uint32_t first;     // 1: the layout starts with the third warp
 };
-constexpr uint32_t kGenZero = kGenRingBytes / 16;  // index of `zero` from `ring`
-static_assert(offsetof(GenSmem, zero) == 16 * kGenZero, "zero follows the ring");
+static_assert(offsetof(GenSmem<8>, zero) == kGenRingBytes, "zero follows the ring");
+static_assert(offsetof(GenSmem<16>, zero) == 2 * kGenRingBytes, "zero follows the ring");
 
-template <int NV, bool MOM>
-__device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t tile, GenSmem &sm) {
+template <int W, int NV, bool MOM>
+__device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t tile, GenSmem<W> &sm) {
+    constexpr uint32_t kGenZero = W / 8 * kGenRingBytes / 16;  // index of `zero` from `ring`
+    constexpr int TPB = 32 * W;
     constexpr int K = gen_rows_per_thread(NV, MOM);
     // with one vector per thread and row the chunk stays in registers from pass 1 to pass 2, as in
     // rowsq_tile: its squares, or with momentum g (M is still read from the slot)
     constexpr bool kHold = NV == 1, kEarly = kHold && !MOM;
     const uint32_t V = (uint32_t)T.m / 8u, m = (uint32_t)T.m;
-    const uint32_t wpr = (V + 32 * NV - 1) / (32 * NV), rpp = 8 / wpr, lpr = 32 * wpr;
+    const uint32_t wpr = (V + 32 * NV - 1) / (32 * NV), rpp = W / wpr, lpr = 32 * wpr;
     const uint32_t cr = T.cr, gbytes = cr * m * 2u, slot = MOM ? 3u * gbytes : gbytes;
-    const uint32_t stages = min((uint32_t)kGenStages, (uint32_t)kGenRingBytes / slot);
+    const uint32_t stages = min((uint32_t)kGenStages, 16u * kGenZero / slot);
     const int64_t row0 = int64_t(tile) * T.rt_rows, n = T.n;
     const uint32_t rows_t = (uint32_t)min((int64_t)T.rt_rows, n - row0);
     const uint32_t nch = (rows_t + cr - 1) / cr;
@@ -2374,14 +2381,14 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
         // 512 MiB of G, before: 126 us at m = 1536, 129 at 768, 133 at 1408
         uint32_t slot;
         asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-        sm.first = (slot >> 3) & 1u;
+        sm.first = W == 8 ? (slot >> 3) & 1u : 0u;
     }
     if (tid < 8) reinterpret_cast<uint32_t *>(sm.zero)[tid] = 0u;
     __syncthreads();
     if (tid == 0)
         for (uint32_t c = 0; c < nch && c < stages; ++c) issue(c, c);
 
-    const uint32_t lw = (warp + 2 * sm.first) & 7u;  // the warp's place in the layout
+    const uint32_t lw = (warp + 2 * sm.first) & (W - 1u);  // the warp's place in the layout
     const uint32_t rp = lw / wpr, vi = (lw - rp * wpr) * 32u + lane;
     const bool on = rp < rpp;  // the warp has rows (the same for its lanes)
     bool act[NV];              // the thread has vector vi + v lpr
@@ -2457,16 +2464,21 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
         if (__syncthreads_or(!ok)) break;  // every slot before this one has landed
         // the slot of chunk c (when its values are held), or else of chunk c - 1, is free: refill it
         // (from the last warp: the first ones form the chunk's row scales, which the CTA waits for)
-        if (tid == kRowThreads - 32 && (kEarly || c >= 1) && c - (kEarly ? 0 : 1) + stages < nch) {
+        if (tid == TPB - 32 && (kEarly || c >= 1) && c - (kEarly ? 0 : 1) + stages < nch) {
             fence_proxy_async_smem();
             issue(c - (kEarly ? 0 : 1) + stages, kEarly ? st : st == 0 ? stages - 1 : st - 1);
         }
         float Rn = 0.f, sum = 0.f;
         if (tid < (int)rows) {
-            float p[8];
+            float p[W];
 #pragma unroll
-            for (int w = 0; w < 8; ++w) p[w] = w < (int)wpr ? sm.part[w0 + w][kr] : 0.f;
-            sum = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+            for (int w = 0; w < W; ++w) p[w] = w < (int)wpr ? sm.part[w0 + w][kr] : 0.f;
+#pragma unroll
+            for (int h = W / 2; h; h >>= 1)
+#pragma unroll
+                for (int w = 0; w < W / 2; ++w)
+                    if (w < h) p[w] += p[w + h];
+            sum = p[0];
             Rn = fmaf(b2, rold, c2m * sum);  // c2m = c2 / m, rounded once
             sm.inv[tid] = Rn > 0.f && Rn < inf ? __frcp_rn(Rn) : 0.f;
         }
@@ -2572,7 +2584,7 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
             mpp[o + 1] = make_float2(ph[0][q].y, pl[0][q].y);
         }
         __syncthreads();
-        for (uint32_t e = tid; e < m; e += kRowThreads) {
+        for (uint32_t e = tid; e < m; e += TPB) {
             float cc = 0.f;
             Acc2 pq;
             for (uint32_t r = 0; r < rpp; ++r) {
@@ -2609,24 +2621,36 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
 // scales sit in shared memory; a thread steps its row and column by 256 vectors without dividing.
 // Per element the arithmetic is apply_fact_tile's, bit for bit. Bound by HBM: 930M parameters in
 // 3072 x 1536 experts 994 us on strip tiles, 826 us (6.75 TB/s) here.
-constexpr uint32_t kFlatChunk = 1024;  // vectors
-
+// Above 4096 columns the column scales take 16 to 32 KB, and the ring's chunks are half as long.
 struct FlatSmem {
-    uint4 ring[kGenRingBytes / 16];  // [W | G] x 3 slots, or [W | M] x 2
     uint64_t full[4];
     float red[2 * kRowThreads / 32];
-    float ab[kFlatScales];  // b_j [m], then a_i of the tile's rows
     SumSmem sum;
+    uint4 data[kFlatBytes / 16];  // the ring, then b_j [m] and a_i of the tile's rows
 };
 
+template <bool MOM, bool WIDE>
+struct FlatRing {
+    static constexpr uint32_t kChunk = WIDE ? 512 : 1024;                       // vectors
+    static constexpr uint32_t kSlot16 = (MOM ? 3 : 2) * kChunk;                 // [W | G] or [W | M]
+    static constexpr uint32_t kStages = (MOM ? 2 : 3) + (WIDE ? 1 : 0);
+    static constexpr uint32_t kWords = kSlot16 * kStages;
+    static constexpr int kScales = (int)(kFlatBytes / 4 - 4 * kWords);          // floats left
+    static __device__ float *scales(FlatSmem &sm) { return reinterpret_cast<float *>(sm.data + kWords); }
+};
+static_assert(FlatRing<false, false>::kScales >= kFlatScales && FlatRing<true, false>::kScales >= kFlatScales &&
+                  FlatRing<false, true>::kScales >= kFlatWideScales && FlatRing<true, true>::kScales >= kFlatWideScales,
+              "the planner's rows fit");
+
 // Issues the copies of chunk c of the tile (vectors of rows r0, ...) into slot st.
-template <bool MOM>
+template <bool MOM, bool WIDE>
 __device__ __forceinline__ void flat_issue(const TensorDev &T, int64_t r0, uint32_t total, uint32_t c, uint32_t st,
                                            FlatSmem &sm, uint64_t pol) {
-    constexpr uint32_t kSlot16 = MOM ? 3 * kFlatChunk : 2 * kFlatChunk;
+    using F = FlatRing<MOM, WIDE>;
+    constexpr uint32_t kFlatChunk = F::kChunk, kSlot16 = F::kSlot16;
     const uint32_t bytes = min(kFlatChunk, total - c * kFlatChunk) * 16u;
     const uint64_t e0 = uint64_t(r0) * (uint64_t)T.m + uint64_t(c) * kFlatChunk * 8u;
-    uint4 *dst = sm.ring + st * kSlot16;
+    uint4 *dst = sm.data + st * kSlot16;
     mbar_expect_tx(&sm.full[st], MOM ? 3u * bytes : 2u * bytes);
     bulk_g2s(dst, T.w + e0, bytes, &sm.full[st], pol);
     if (MOM)
@@ -2635,10 +2659,11 @@ __device__ __forceinline__ void flat_issue(const TensorDev &T, int64_t r0, uint3
         bulk_g2s(dst + kFlatChunk, T.g + e0, bytes, &sm.full[st], pol);
 }
 
-template <bool MOM, bool FAST>
+template <bool MOM, bool WIDE, bool FAST>
 __device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r0, uint32_t total, float coefC,
                                 FlatSmem &sm, uint64_t pol, Acc2 &acc) {
-    constexpr uint32_t kStages = MOM ? 2 : 3, kSlot16 = MOM ? 3 * kFlatChunk : 2 * kFlatChunk;
+    using F = FlatRing<MOM, WIDE>;
+    constexpr uint32_t kStages = F::kStages, kSlot16 = F::kSlot16, kFlatChunk = F::kChunk;
     const uint32_t V = (uint32_t)T.m / 8u, nch = (total + kFlatChunk - 1) / kFlatChunk;
     const int tid = threadIdx.x;
     uint16_t *__restrict__ w_ = T.w + r0 * T.m;
@@ -2647,14 +2672,14 @@ __device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r
     const float wdf = T.decay ? A.wdf : 1.0f, ce = A.ce;
     const float2 wdf2 = make_float2(wdf, wdf);
     const Pol sp;
-    const float *__restrict__ sb = sm.ab, *__restrict__ sa = sm.ab + 8 * V;
+    const float *__restrict__ sb = F::scales(sm), *__restrict__ sa = sb + 8 * V;
     uint32_t row = tid / V, col = tid - row * V;  // of vector tid of the tile
     const uint32_t dq = kRowThreads / V, dr = kRowThreads - dq * V;
     uint32_t st = 0, par = 0;
     for (uint32_t c = 0; c < nch; ++c) {
         const uint32_t cnt = min(kFlatChunk, total - c * kFlatChunk);
         const bool ok = mbar_wait(&sm.full[st], par);
-        const uint4 *bw = sm.ring + st * kSlot16, *by = bw + kFlatChunk;
+        const uint4 *bw = sm.data + st * kSlot16, *by = bw + kFlatChunk;
 #pragma unroll
         for (uint32_t k = 0; k < kFlatChunk / kRowThreads; ++k) {
             const uint32_t f = k * kRowThreads + tid;
@@ -2712,7 +2737,7 @@ __device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r
         }
         if (tid == 0 && c + kStages < nch) {
             fence_proxy_async_smem();
-            flat_issue<MOM>(T, r0, total, c + kStages, st, sm, pol);
+            flat_issue<MOM, WIDE>(T, r0, total, c + kStages, st, sm, pol);
         }
         if (++st == kStages) {
             st = 0;
@@ -2722,9 +2747,11 @@ __device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r
     return true;
 }
 
-template <bool MOM>
+template <bool MOM, bool WIDE>
 __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t item, FlatSmem &sm) {
-    constexpr uint32_t kStages = MOM ? 2 : 3;
+    using F = FlatRing<MOM, WIDE>;
+    constexpr uint32_t kStages = F::kStages, kFlatChunk = F::kChunk;
+    float *ab = F::scales(sm);
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     const uint32_t trows = (item & kHalfTile) ? T.at_rows / 2 : T.at_rows;
@@ -2738,18 +2765,18 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     }
     __syncthreads();
     if (threadIdx.x == 0)
-        for (uint32_t c = 0; c < nch && c < kStages; ++c) flat_issue<MOM>(T, r0, total, c, c, sm, pol);
+        for (uint32_t c = 0; c < nch && c < kStages; ++c) flat_issue<MOM, WIDE>(T, r0, total, c, c, sm, pol);
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
     float ma = 0.f, mb = 0.f;
     for (uint32_t j = threadIdx.x; j < m / 4; j += kRowThreads) {
         const float4 b = __ldcg(reinterpret_cast<const float4 *>(T.bsc) + j);
-        reinterpret_cast<float4 *>(sm.ab)[j] = b;
+        reinterpret_cast<float4 *>(ab)[j] = b;
         mb = fmaxf(fmaxf(mb, fmaxf(nan_to_inf(b.x), nan_to_inf(b.y))), fmaxf(nan_to_inf(b.z), nan_to_inf(b.w)));
     }
     for (uint32_t r = threadIdx.x; r < rows_t; r += kRowThreads) {
         const float a = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
-        sm.ab[m + r] = a;
+        ab[m + r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
     }
 #pragma unroll
@@ -2773,9 +2800,9 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     Acc2 acc;
     bool done;
     if (!sum && ma * mb <= A.ce)
-        done = apply_flat_body<MOM, true>(A, T, r0, total, coefC, sm, pol, acc);
+        done = apply_flat_body<MOM, WIDE, true>(A, T, r0, total, coefC, sm, pol, acc);
     else
-        done = apply_flat_body<MOM, false>(A, T, r0, total, coefC, sm, pol, acc);
+        done = apply_flat_body<MOM, WIDE, false>(A, T, r0, total, coefC, sm, pol, acc);
     if (sum && done) publish_sum(A, T, S, item, rows_t, acc, sm.sum);
 }
 
@@ -3110,18 +3137,18 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
         return;
     }
     if (T.rowpath == kRowAny) {
-        GenSmem &gs = *reinterpret_cast<GenSmem *>(dyn_smem);
-        const bool wide = T.m > 2048;
+        GenSmem<8> &gs = *reinterpret_cast<GenSmem<8> *>(dyn_smem);
+        const bool two = T.m > 2048;
         if (T.momentum) {
-            if (wide)
-                rowsq_gen_tile<2, true>(A, T, S, it.y, gs);
+            if (two)
+                rowsq_gen_tile<8, 2, true>(A, T, S, it.y, gs);
             else
-                rowsq_gen_tile<1, true>(A, T, S, it.y, gs);
+                rowsq_gen_tile<8, 1, true>(A, T, S, it.y, gs);
         } else {
-            if (wide)
-                rowsq_gen_tile<2, false>(A, T, S, it.y, gs);
+            if (two)
+                rowsq_gen_tile<8, 2, false>(A, T, S, it.y, gs);
             else
-                rowsq_gen_tile<1, false>(A, T, S, it.y, gs);
+                rowsq_gen_tile<8, 1, false>(A, T, S, it.y, gs);
         }
         return;
     }
@@ -3143,6 +3170,19 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     }
 }
 
+// Row path, phase A of the widths above 4096: one row tile per CTA, one CTA per SM.
+__global__ void __launch_bounds__(kWideThreads, 1)
+    k_rowsq_wide(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
+    extern __shared__ uint4 dyn_smem[];
+    GenSmem<16> &gs = *reinterpret_cast<GenSmem<16> *>(dyn_smem);
+    const uint2 it = begin_item(items);
+    const TensorDev &T = A.tensors[it.x];
+    if (T.momentum)
+        rowsq_gen_tile<16, 2, true>(A, T, A.scal[it.x], it.y, gs);
+    else
+        rowsq_gen_tile<16, 2, false>(A, T, A.scal[it.x], it.y, gs);
+}
+
 // Row path, phase C: one row tile per CTA (dynamic shared memory: ApplyRowSmem), and before them
 // the phase-C strip and flat tiles.
 __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
@@ -3158,10 +3198,18 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     }
     if (T.rowpath == kRowAny) {
         FlatSmem &fs = *reinterpret_cast<FlatSmem *>(dyn_smem);
-        if (T.momentum)
-            apply_flat_tile<true>(A, T, S, it.y, fs);
-        else
-            apply_flat_tile<false>(A, T, S, it.y, fs);
+        const bool wide = T.m > kAnyNarrow;
+        if (T.momentum) {
+            if (wide)
+                apply_flat_tile<true, true>(A, T, S, it.y, fs);
+            else
+                apply_flat_tile<true, false>(A, T, S, it.y, fs);
+        } else {
+            if (wide)
+                apply_flat_tile<false, true>(A, T, S, it.y, fs);
+            else
+                apply_flat_tile<false, false>(A, T, S, it.y, fs);
+        }
         return;
     }
     if (T.momentum) {
@@ -3333,9 +3381,15 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     if (L.nA > rA) run(launch(k_sumsq, L.nA, kThreads, 0, s, A, L.itemsA));
     mark(1);
     if (rows) {
-        constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem));
+        constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem<8>));
         run(cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm));
-        run(launch(k_rowsq, rA + L.nR, kRowThreads, kSm, s, A, past(L.itemsA, L.nA - rA)));
+        if (rA + L.nR > L.nRW) run(launch(k_rowsq, rA + L.nR - L.nRW, kRowThreads, kSm, s, A, past(L.itemsA, L.nA - rA)));
+        constexpr size_t kWide = sizeof(GenSmem<16>);
+        static_assert(kWide <= 227 * 1024, "one CTA per SM");
+        if (L.nRW) {
+            run(cudaFuncSetAttribute(k_rowsq_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWide));
+            run(launch(k_rowsq_wide, L.nRW, kWideThreads, kWide, s, A, past(L.itemsA, L.nA + L.nR - L.nRW)));
+        }
     }
     mark(2);
     if (L.nF) run(launch(k_finalize, L.nF, kThreads, 0, s, A, L.itemsF));

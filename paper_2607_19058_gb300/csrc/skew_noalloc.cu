@@ -160,7 +160,8 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     TileGeom limit = most;
     limit.nbc = limit.ntiles;
     if (layout_of(limit, kind, n, m).bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
-    const bool on_rows = any ? 2 * numel >= kAnyGroupBytes : most.rowpath != kRowNone;
+    const AnyWidths w = m > kAnyNarrow ? any_widths(0, 2 * numel, false) : any_widths(2 * numel, 0, false);
+    const bool on_rows = any ? (m > kAnyNarrow ? w.wide : w.narrow) : most.rowpath != kRowNone;
     TileGeom G = plan_geometry(kind, momentum, on_rows, vec, numel < kSmallStrip, n, m, numel, 2 * numel);
     Layout o = layout_of(G, kind, n, m);
     if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) {
@@ -266,7 +267,8 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
                                     (uint32_t *)(base + o.fb));
     e = cudaGetLastError();
     if (e != cudaSuccess) return SKEW_ECUDA;
-    const LaunchPlan lp{o.nA, o.nR, o.nF, o.nB, nFB, o.nC, o.nCR, false, nullptr, nullptr, nullptr, nullptr};
+    const uint32_t nRW = G.rowpath == kRowAny && m > kAnyNarrow ? o.nR : 0;
+    const LaunchPlan lp{o.nA, o.nR, o.nF, o.nB, nFB, o.nC, o.nCR, nRW, false, nullptr, nullptr, nullptr, nullptr};
     e = (cudaError_t)launch_phases(a, lp, stream, nullptr);
     if (e != cudaSuccess) return SKEW_ECUDA;
     return SKEW_OK;

@@ -63,9 +63,11 @@ constexpr int kMomChunks = 64;
 // not fit the registers of two 256-thread CTAs per SM: both stay on the strip tiles. Against
 // the strip tiles (three reads of G): 930M parameters in 3072 x 1536 experts 1872 -> 1259 us.
 enum RowPath : uint32_t { kRowNone = 0, kRowFixed = 1, kRowAny = 2 };
-constexpr int64_t kAnyMin = 128, kAnyMax = 4096;
+constexpr int64_t kAnyMin = 128, kAnyNarrow = 4096, kAnyMax = 8192;
+constexpr int kWideThreads = 512;
 constexpr int64_t kAnyTileBytes = 1 << 20;  // bf16 bytes of a tile in phases A and C, as of the fixed widths
-constexpr int kFlatScales = 4200;
+constexpr int kFlatBytes = 115072;  // phase C's ring and scales
+constexpr int kFlatScales = 4184, kFlatWideScales = 10336;  // scales that fit beside the ring
 __host__ __device__ constexpr int gen_rows_per_thread(int nv, bool mom) { return (nv == 1 ? 8 : 4) / (mom ? 2 : 1); }
 
 enum Kind : uint32_t { kKindFull = 0, kKindFactored = 1 };
@@ -149,7 +151,7 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
     int64_t t = per(rest, ctas), whole = kWaveTileBytes / chunk;  // a single wave of small tiles: no second ramp
     if (t > whole) t = per(rest, ctas * waves) > whole ? per(rest, ctas * waves) : whole;
     t = t < least ? least : t > most ? most : t;
-    if (parts && rest < kWholeGroup && own > t * chunk * parts && own <= 2 * most * chunk * ctas) t = per(own, ctas);
+    if (parts && rest < kWholeGroup && own > t * chunk * parts && own <= 2 * most * chunk * ctas) t = per(own, parts < ctas ? parts : ctas);
     return (uint32_t)t;
 }
 
@@ -157,6 +159,22 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
 // read of G costs a step no more than k_fallback and the row tiles' ramps: 2048 x 1408 on its own
 // (5.8 MB) takes 51 us on strip tiles and 44 us on row tiles, the smallest steps the reverse.
 constexpr int64_t kAnyGroupBytes = 2 << 20;
+// Beside row tiles of other widths, those above kAnyNarrow need a launch of their own, and below this
+// many bytes of G the strip tiles, which ride along, are faster (260M parameters, 23 MB of them 5632
+// wide: 379 us against 407; 1.16B parameters of 4864 and 7128 columns: 2314 against 1653).
+constexpr int64_t kWideGroupBytes = 64 << 20;
+
+// Which widths that only kRowAny serves take row tiles in a step: `narrow` and `wide` bytes of G of its
+// matrices up to and above kAnyNarrow columns, `fixed`: it has matrices of the fixed widths.
+struct AnyWidths {
+    bool narrow, wide;
+};
+inline AnyWidths any_widths(int64_t narrow, int64_t wide, bool fixed) {
+    AnyWidths w;
+    w.wide = wide >= kWideGroupBytes || (!fixed && narrow < kAnyGroupBytes && wide >= kAnyGroupBytes);
+    w.narrow = narrow >= kAnyGroupBytes || (w.wide && narrow > 0);
+    return w;
+}
 
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
 // gradient pointers are 16-byte aligned; `vec`: row-vectors may be 16-byte accesses (row_vectors);
@@ -195,14 +213,16 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
                 const uint32_t at = row_tile_chunks(own, rest, 3, chunk, 32768 / chunk, (1 << 20) / chunk, 0);
                 g.at_rows = g.cr * (momentum ? (at + 1) / 2 * 2 : at);  // a half tile is whole phase-C chunks
             } else {
-                const int nv = m > 2048 ? 2 : 1;
+                const int nv = m > 2048 ? 2 : 1, warps = m > kAnyNarrow ? 16 : 8;
                 const int64_t wpr = (m / 8 + 32 * nv - 1) / (32 * nv);
-                g.cr = (uint32_t)(gen_rows_per_thread(nv, momentum != 0) * (8 / wpr));
+                g.cr = (uint32_t)(gen_rows_per_thread(nv, momentum != 0) * (warps / wpr));
                 const int64_t chunk = 2 * m * g.cr, least = 65536 / chunk;
-                g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, least < 1 ? 1 : least, kAnyTileBytes / chunk,
+                g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, least < 1 ? 1 : least,
+                                                   (warps / 8) * kAnyTileBytes / chunk,
                                                    (12 << 20) / (8 * m));
                 int64_t at = 2 * row_tile_chunks(own, rest, 3, 4 * m, (32768 + 4 * m - 1) / (4 * m), kAnyTileBytes / (4 * m), 0);
-                if (at > kFlatScales - m) at = kFlatScales - m;
+                const int64_t fit = (m > kAnyNarrow ? kFlatWideScales : kFlatScales) - m;
+                if (at > fit) at = fit;
                 g.at_rows = (uint32_t)(at / 2 * 2);
             }
             g.rtiles = (uint32_t)((n + g.rt_rows - 1) / g.rt_rows);
@@ -346,6 +366,7 @@ struct StepArgs {
 // of the row tiles (R, FB and CR).
 struct LaunchPlan {
     uint32_t nA, nR, nF, nB, nFB, nC, nCR;
+    uint32_t nRW;  // of the nR, those of widths above kAnyNarrow (last)
     bool ride;
     const uint2 *itemsA, *itemsF, *itemsB, *itemsC;
 };

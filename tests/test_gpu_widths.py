@@ -1,4 +1,4 @@
-"""Whole-row tiles at widths other than 512, 1024, 2048 and 4096 (any multiple of 8 from 128 to 4096),
+"""Whole-row tiles at widths other than 512, 1024, 2048 and 4096 (any multiple of 8 from 128 to 8192),
 against the oracle: the narrowest and widest, widths whose rows take 1 to 8 warps and one or two
 vectors per thread, ragged last tiles and chunks, one-row matrices, stacks, with and without momentum."""
 import pytest
@@ -11,9 +11,11 @@ pytestmark = pytest.mark.gpu
 
 E, B = WL.TIER_EXPERT, WL.TIER_BACKBONE
 #          rows, width: rows of half a warp; 64-row chunks; 2 warps a row; 5 of 8 warps; a partial last warp; 1 row side by side;
-#          two vectors a thread, the second for few lanes; three quarters of the warps; the widest
+#          two vectors a thread, the second for few lanes; three quarters of the warps; the widest of 8 warps
 SHAPES = [(2113, 128), (700, 200), (2113, 256), (1, 256), (700, 264), (333, 776), (517, 1032), (131, 1408), (9, 2040), (130, 2056), (257, 2880),
           (301, 3072), (5, 4088), (267, 4088)]
+# 16 warps a row tile (in a step without the others: see the planner's any_widths)
+WIDE = [(1, 4104), (130, 4104), (77, 5632), (131, 7128), (300, 8192)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -24,25 +26,27 @@ def _built():
     oracle.build()
 
 
-def _workload():
+def _workload(shapes):
     specs = [WL.Spec(f"{'eb'[t]}{n}x{m}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1)
-             for k, (n, m) in enumerate(SHAPES) for t in (0, 1)]
-    specs += [WL.Spec("se", (3, 130, 1536), E), WL.Spec("sb", (2, 67, 768), B)]
+             for k, (n, m) in enumerate(shapes) for t in (0, 1)]
+    m0, m1 = (1536, 768) if shapes is SHAPES else (4800, 5000)
+    specs += [WL.Spec("se", (3, 130, m0), E), WL.Spec("sb", (2, 67, m1), B)]
     return WL.Workload("widths", specs, WL.HP(), "toy", steps=3)
 
 
+@pytest.mark.parametrize("shapes", [SHAPES, WIDE], ids=["to4096", "to8192"])
 @pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05)], ids=["eps1e-30", "paper"])
-def test_any_width_rows(hp):
+def test_any_width_rows(shapes, hp):
     """eps = 1e-8 binds the clamp at step 1; experts 5 to 7 have zero gradients on odd steps."""
     import parity
-    h = parity.Harness(_workload(), hp_override=hp)
+    h = parity.Harness(_workload(shapes), hp_override=hp)
     for t in range(1, 4):
         h.step(t, seed=17 * t, **({"gscale": 0.37} if t == 2 else {}))
     h.opt.sync_status()
     h.close()
 
 
-@pytest.mark.parametrize("shape,tier", [((700, 264), E), ((517, 1032), B), ((301, 3072), E), ((2049, 1408), E)])
+@pytest.mark.parametrize("shape,tier", [((700, 264), E), ((517, 1032), B), ((301, 3072), E), ((2049, 1408), E), ((300, 7128), B), ((700, 8192), E)])
 def test_noalloc_matches_the_handle(shape, tier):
     torch.manual_seed(0)
     w0 = (torch.randn(shape, device="cuda") * 0.02).to(torch.bfloat16)
