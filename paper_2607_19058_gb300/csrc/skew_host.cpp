@@ -545,7 +545,7 @@ int skew_step_scaled(skew_handle_t *h, int64_t step, float lr, uint64_t seed, co
     }
     if (h->small.ctas) {
         const cudaError_t r =
-            (cudaError_t)launch_small(a, nullptr, (uint32_t)h->t.size(), h->small, s, reinterpret_cast<void *const *>(ev));
+            (cudaError_t)launch_small(a, (uint32_t)h->t.size(), h->small, s, reinterpret_cast<void *const *>(ev));
         if (r != cudaSuccess) return cuda_fail(h, r, "kernel launch");
         return SKEW_OK;
     }

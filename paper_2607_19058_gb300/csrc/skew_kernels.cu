@@ -409,16 +409,20 @@ __device__ bool fill_meta(const TensorDev &T, const TensorScal &S, uint32_t tile
     const uint32_t s = tile % T.strips, rt = tile / T.strips, width = 8u << T.lcl;
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
+    // (held apart from the descriptor, which the stores to shared memory may alias)
+    const float *R = T.R, *bsc = T.bsc;
+    const int64_t n = T.n, m = T.m;
+    const uint32_t tile_rows = T.tile_rows;
     float ma = 0.f, mb = 0.f;
-    for (uint32_t r = threadIdx.x; r < T.tile_rows; r += kThreads) {
-        const int64_t i = int64_t(rt) * T.tile_rows + r;
-        const float a = i < T.n ? row_scale(__ldcg(T.R + i), rbar_s, rbar_e) : 0.f;
+    for (uint32_t r = threadIdx.x; r < tile_rows; r += kThreads) {
+        const int64_t i = int64_t(rt) * tile_rows + r;
+        const float a = i < n ? row_scale(__ldcg(R + i), rbar_s, rbar_e) : 0.f;
         meta.rows[r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
     }
     for (uint32_t c = threadIdx.x; c < width; c += kThreads) {
         const int64_t j = int64_t(s) * width + c;
-        const float b = j < T.m ? __ldcg(T.bsc + j) : 0.f;
+        const float b = j < m ? __ldcg(bsc + j) : 0.f;
         meta.cols[c] = b;
         mb = fmaxf(mb, nan_to_inf(b));
     }
@@ -1012,8 +1016,7 @@ __device__ void set_clip(const StepArgs &A, const TensorDev &T, TensorScal &S, d
 // of P_j / C_j are compensated fp32 (hi, lo) pairs: fp64 arithmetic runs at a
 // small fraction of the fp32 rate here, and every term is non-negative, so a
 // pair keeps the sum to about fp64 accuracy and each quotient to one fp32 rounding.
-__device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm) {
-    const TensorDev &T = A.tensors[t];
+__device__ void phase_F_row(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm) {
     TensorScal &S = A.scal[t];
     const float inf = __int_as_float(0x7F800000);
     // the item's fci columns, kFinChunk / fci threads per column: thread tid adds the
@@ -1182,11 +1185,10 @@ __device__ void phase_F_row(const StepArgs &A, uint32_t t, uint32_t local, Smem 
 // ---------------------------------------------------------------------------
 // Phase F: factor EMAs, 1/sqrt(C_j), mean(R) (Eq. 1).
 // ---------------------------------------------------------------------------
-__device__ void phase_F(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm) {
-    const TensorDev &T = A.tensors[t];
+__device__ void phase_F(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm) {
     TensorScal &S = A.scal[t];
     if (T.rowpath) {
-        phase_F_row(A, t, local, sm);
+        phase_F_row(A, T, t, local, sm);
         return;
     }
     if (local < T.nfr) {
@@ -1353,8 +1355,10 @@ struct FlatMeta {
         a = pool;
         b = pool + rows;
         if (in) {
-            for (int r = threadIdx.x; r < (int)rows; r += kThreads) pool[r] = row_scale(__ldcg(T.R + row0 + r), rbar_s, rbar_e);
-            for (int j = threadIdx.x; j < (int)m; j += kThreads) pool[rows + j] = __ldcg(T.bsc + j);
+            // (pointers held apart from the descriptor, which the stores to shared memory may alias)
+            const float *R = T.R + row0, *bsc = T.bsc;
+            for (int r = threadIdx.x; r < (int)rows; r += kThreads) pool[r] = row_scale(__ldcg(R + r), rbar_s, rbar_e);
+            for (int j = threadIdx.x; j < (int)m; j += kThreads) pool[rows + j] = __ldcg(bsc + j);
             __syncthreads();
         }
     }
@@ -1473,8 +1477,7 @@ __device__ Acc2 rms_full_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
 
 // Stores a phase-B tile's sum of (U / coef)^2; the last tile of the tensor forms sum(U^2), RMS and
 // the clip factor (fixed summation order).
-__device__ void finish_B(const StepArgs &A, uint32_t t, uint32_t local, const Acc2 &acc, Smem &sm) {
-    const TensorDev &T = A.tensors[t];
+__device__ void finish_B(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, const Acc2 &acc, Smem &sm) {
     TensorScal &S = A.scal[t];
     const float2 tsum = block_sum2(acc, sm.red2);
     if (threadIdx.x == 0) {
@@ -1492,35 +1495,33 @@ __device__ void finish_B(const StepArgs &A, uint32_t t, uint32_t local, const Ac
     if (threadIdx.x == 0) set_clip(A, T, S, s);
 }
 
-__device__ void phase_B_full(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, const Pol &pol) {
-    const TensorDev &T = A.tensors[t];
+__device__ void phase_B_full(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, const Pol &pol) {
     const Acc2 acc = rms_full_tile(A, T, local, pol);
-    finish_B(A, t, local, acc, sm);
+    finish_B(A, T, t, local, acc, sm);
 }
 
-__device__ void phase_B_strip(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
-    const TensorDev &T = A.tensors[t];
+__device__ void phase_B_strip(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
     (void)fill_meta(T, A.scal[t], local, A.ce, meta);
-    finish_B(A, t, local,
+    finish_B(A, T, t, local,
              T.momentum ? rms_fact_tile<true>(A, T, local, meta, pol) : rms_fact_tile<false>(A, T, local, meta, pol), sm);
 }
 
-__device__ void phase_B_flat(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
-    const TensorDev &T = A.tensors[t];
-    finish_B(A, t, local, rms_flat_tile(A, T, A.scal[t], local, meta, pol), sm);
+__device__ void phase_B_flat(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+    finish_B(A, T, t, local, rms_flat_tile(A, T, A.scal[t], local, meta, pol), sm);
 }
 
-__device__ void phase_B_fact(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
-    if (A.tensors[t].vec)
-        phase_B_strip(A, t, local, sm, meta, pol);
+__device__ void phase_B_fact(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
+    if (T.vec)
+        phase_B_strip(A, T, t, local, sm, meta, pol);
     else
-        phase_B_flat(A, t, local, sm, meta, pol);
+        phase_B_flat(A, T, t, local, sm, meta, pol);
 }
 
 // The same for k_fallback's own items, out of line: inlined beside the queue's tiles, which are strip
 // tiles, it makes those spill (a queue of 62M elements of 1024 and 496 columns 56 us slower).
-__device__ __noinline__ void phase_B_own(const StepArgs &A, uint32_t t, uint32_t local, Smem &sm, Meta &meta) {
-    phase_B_fact(A, t, local, sm, meta, Pol());
+__device__ __noinline__ void phase_B_own(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm,
+                                         Meta &meta) {
+    phase_B_fact(A, T, t, local, sm, meta, Pol());
 }
 
 // ---------------------------------------------------------------------------
@@ -1891,8 +1892,9 @@ __device__ void apply_rows_tile(const StepArgs &A, const TensorDev &T, TensorSca
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
     float ma = 0.f, mb = 0.f;
+    const float *R = T.R + r0;  // (the stores may alias the descriptor)
     for (uint32_t r = threadIdx.x; r < rows_t; r += TPB) {
-        const float a = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
+        const float a = row_scale(__ldcg(R + r), rbar_s, rbar_e);
         sm.a[r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
     }
@@ -2264,8 +2266,9 @@ __device__ void apply_rows_mom_tile(const StepArgs &A, const TensorDev &T, Tenso
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
     float ma = 0.f, mb = 0.f;
+    const float *R = T.R + r0;  // (the stores may alias the descriptor)
     for (uint32_t r = threadIdx.x; r < rows_t; r += TPB) {
-        const float a = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
+        const float a = row_scale(__ldcg(R + r), rbar_s, rbar_e);
         sm.a[r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
     }
@@ -2769,13 +2772,15 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     const float rbar_s = __ldcg(&S.rbar_s);
     const int rbar_e = __ldcg(&S.rbar_e);
     float ma = 0.f, mb = 0.f;
+    const float4 *bsc = reinterpret_cast<const float4 *>(T.bsc);  // (the stores may alias the descriptor)
+    const float *R = T.R + r0;
     for (uint32_t j = threadIdx.x; j < m / 4; j += kRowThreads) {
-        const float4 b = __ldcg(reinterpret_cast<const float4 *>(T.bsc) + j);
+        const float4 b = __ldcg(bsc + j);
         reinterpret_cast<float4 *>(ab)[j] = b;
         mb = fmaxf(fmaxf(mb, fmaxf(nan_to_inf(b.x), nan_to_inf(b.y))), fmaxf(nan_to_inf(b.z), nan_to_inf(b.w)));
     }
     for (uint32_t r = threadIdx.x; r < rows_t; r += kRowThreads) {
-        const float a = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
+        const float a = row_scale(__ldcg(R + r), rbar_s, rbar_e);
         ab[m + r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
     }
@@ -3091,27 +3096,42 @@ __device__ void phase_C(const StepArgs &A, const TensorDev &T, const TensorScal 
 // CTA's (tensor, tile) table, written at bind; null: tensor 0, tiles in order.
 // A step of 296K elements in 39 tensors 37 -> 28 us, 2048 x 1408 alone 43 -> 35, the 6.78B set 8357 -> 8322.
 __device__ __forceinline__ void wait_previous_launch() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-__device__ __forceinline__ uint2 begin_item(const uint2 *__restrict__ items) {
+__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A CTA's item, with its tensor's descriptor copied to shared memory: one trip to L2 for all of it, where
+// reading fields as they are needed, between barriers, is a chain of trips. Both come from bind and are
+// read before the wait; the no-alloc step, without tables, passes its descriptor as a parameter.
+// Against reading fields from L2: 24 ragged tensors 150 -> 135 us, a 432-wide model 69 -> 61, a 2048-wide
+// one 378 -> 369, the 6.78B set 8349 -> 8318.
+__device__ __forceinline__ uint2 begin_item(const uint2 *__restrict__ items, const StepArgs &A, TensorDev &td) {
+    constexpr uint32_t kWords = sizeof(TensorDev) / 4;
+    static_assert(sizeof(TensorDev) % 4 == 0 && kWords <= kThreads, "one word per thread");
+    let_next_launch_start();
     const uint2 it = items ? items[blockIdx.x] : make_uint2(0u, blockIdx.x);
+    if (threadIdx.x < kWords)
+        reinterpret_cast<uint32_t *>(&td)[threadIdx.x] =
+            items ? __ldcg(reinterpret_cast<const uint32_t *>(A.tensors + it.x) + threadIdx.x)
+                  : reinterpret_cast<const uint32_t *>(&A.one)[threadIdx.x];
     wait_previous_launch();
+    __syncthreads();
     return it;
 }
 
 // Clears the per-step scalars and the length of the phase-B queue (words of 4 bytes).
 __global__ void k_reset(uint32_t *p, uint32_t words) {
-    wait_previous_launch();
+    let_next_launch_start();
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < words; k += gridDim.x * blockDim.x) p[k] = 0u;
 }
 
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_SUMSQ)
     k_sumsq(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Smem sm;
-    const uint2 it = begin_item(items);
-    phase_A_strip(A.tensors[it.x], it.y, sm, Pol());
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    phase_A_strip(td, it.y, sm, Pol());
 }
 
 // A step with row-path tensors runs its strip and flat tiles in the row path's launches, ahead of
@@ -3125,15 +3145,16 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     k_rowsq(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
     RowSmem &sm = *reinterpret_cast<RowSmem *>(dyn_smem);
-    const uint2 it = begin_item(items);
-    const TensorDev &T = A.tensors[it.x];
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    const TensorDev &T = td;
     TensorScal &S = A.scal[it.x];
     if (T.rowpath == kRowNone) {
         Smem &ss = *reinterpret_cast<Smem *>(dyn_smem);
         if (T.kind == kKindFactored)
             phase_A_strip(T, it.y, ss, Pol());
         else
-            phase_B_full(A, it.x, it.y, ss, Pol());
+            phase_B_full(A, T, it.x, it.y, ss, Pol());
         return;
     }
     if (T.rowpath == kRowAny) {
@@ -3175,8 +3196,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     k_rowsq_wide(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
     GenSmem<16> &gs = *reinterpret_cast<GenSmem<16> *>(dyn_smem);
-    const uint2 it = begin_item(items);
-    const TensorDev &T = A.tensors[it.x];
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    const TensorDev &T = td;
     if (T.momentum)
         rowsq_gen_tile<16, 2, true>(A, T, A.scal[it.x], it.y, gs);
     else
@@ -3189,8 +3211,9 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     k_apply_rows(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
     ApplyRowSmem &sm = *reinterpret_cast<ApplyRowSmem *>(dyn_smem);
-    const uint2 it = begin_item(items);
-    const TensorDev &T = A.tensors[it.x];
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    const TensorDev &T = td;
     TensorScal &S = A.scal[it.x];
     if (T.rowpath == kRowNone) {
         phase_C(A, T, S, it.y, *reinterpret_cast<Meta *>(dyn_smem), Pol());
@@ -3239,18 +3262,22 @@ __global__ void __launch_bounds__(kThreads, 2)
     __shared__ Smem sm;
     __shared__ Meta meta;
     if (blockIdx.x < nB) {
-        const uint2 it = begin_item(items);
-        phase_B_own(A, it.x, it.y, sm, meta);
+        __shared__ TensorDev td;
+        const uint2 it = begin_item(items, A, td);
+        phase_B_own(A, td, it.x, it.y, sm, meta);
         return;
     }
+    let_next_launch_start();
     wait_previous_launch();
     const Pol pol;
     const uint32_t cnt = __ldcg(A.fb), ctas = gridDim.x - nB;
     uint32_t tile = blockIdx.x - nB;  // of queued tensor q
     for (uint32_t q = 0; q < cnt; ++q) {
-        const uint32_t t = __ldcg(A.fb + 1 + q), nt = A.tensors[t].nbc;
+        const uint32_t t = __ldcg(A.fb + 1 + q);
+        const TensorDev &T = A.tensors ? A.tensors[t] : A.one;
+        const uint32_t nt = T.nbc;
         for (; tile < nt; tile += ctas) {
-            phase_B_strip(A, t, tile, sm, meta, pol);
+            phase_B_strip(A, T, t, tile, sm, meta, pol);
             __syncthreads();
         }
         tile -= nt;
@@ -3259,34 +3286,38 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 __global__ void __launch_bounds__(kThreads) k_finalize(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Smem sm;
-    const uint2 it = begin_item(items);
-    phase_F(A, it.x, it.y, sm);
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    phase_F(A, td, it.x, it.y, sm);
 }
 
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_RMS)
     k_rms(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Smem sm;
     __shared__ Meta meta;
-    const uint2 it = begin_item(items);
-    if (A.tensors[it.x].kind == kKindFactored)
-        phase_B_fact(A, it.x, it.y, sm, meta, Pol());
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    const TensorDev &T = td;
+    if (T.kind == kKindFactored)
+        phase_B_fact(A, T, it.x, it.y, sm, meta, Pol());
     else
-        phase_B_full(A, it.x, it.y, sm, Pol());
+        phase_B_full(A, T, it.x, it.y, sm, Pol());
 }
 
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_APPLY)
     k_apply(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     __shared__ Meta meta;
-    const uint2 it = begin_item(items);
-    phase_C(A, A.tensors[it.x], A.scal[it.x], it.y, meta, Pol());
+    __shared__ TensorDev td;
+    const uint2 it = begin_item(items, A, td);
+    phase_C(A, td, A.scal[it.x], it.y, meta, Pol());
 }
 
-// One cluster per tensor of the handle, or (tensors null) the one tensor `one`.
+// One cluster per tensor of the handle, or (tensors null) the one tensor A.one.
 __global__ void __launch_bounds__(kSmallThreads, 2)
-    k_small(const __grid_constant__ StepArgs A, const __grid_constant__ TensorDev one) {
+    k_small(const __grid_constant__ StepArgs A) {
     extern __shared__ uint4 dyn_smem[];
     const uint32_t t = blockIdx.x / cooperative_groups::this_cluster().num_blocks();
-    small_step(A, A.tensors ? A.tensors[t] : one, A.scal + t, reinterpret_cast<float *>(dyn_smem));
+    small_step(A, A.tensors ? A.tensors[t] : A.one, A.scal + t, reinterpret_cast<float *>(dyn_smem));
 }
 
 // Self-test of the bounded wait: one thread waits, exactly as the row kernels wait for
@@ -3331,8 +3362,7 @@ cudaError_t launch(void (*k)(P...), uint32_t grid, uint32_t threads, size_t smem
 
 }  // namespace
 
-int launch_small(const StepArgs &A, const TensorDev *one, uint32_t tensors, const SmallPlan &P, void *stream,
-                 void *const *ev) {
+int launch_small(const StepArgs &A, uint32_t tensors, const SmallPlan &P, void *stream, void *const *ev) {
     cudaStream_t s = (cudaStream_t)stream;
     static_assert(kSmallHeadBytes >= (sizeof(SmallSmem) + 15) / 16 * 16, "k_small's shared memory");
     if (ev)
@@ -3350,8 +3380,7 @@ int launch_small(const StepArgs &A, const TensorDev *one, uint32_t tensors, cons
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    const TensorDev none{};
-    e = cudaLaunchKernelEx(&cfg, k_small, A, one ? *one : none);
+    e = cudaLaunchKernelEx(&cfg, k_small, A);
     if (ev) cudaEventRecord((cudaEvent_t)ev[kLaunches], s);
     return (int)e;
 }
@@ -3385,7 +3414,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
         run(cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm));
         if (rA + L.nR > L.nRW) run(launch(k_rowsq, rA + L.nR - L.nRW, kRowThreads, kSm, s, A, past(L.itemsA, L.nA - rA)));
         constexpr size_t kWide = sizeof(GenSmem<16>);
-        static_assert(kWide <= 227 * 1024, "one CTA per SM");
+        static_assert(kWide + 1024 <= 227 * 1024, "one CTA per SM");
         if (L.nRW) {
             run(cudaFuncSetAttribute(k_rowsq_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWide));
             run(launch(k_rowsq_wide, L.nRW, kWideThreads, kWide, s, A, past(L.itemsA, L.nA + L.nR - L.nRW)));
@@ -3402,7 +3431,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     mark(6);
     if (rows) {
         constexpr size_t kSm = max3(sizeof(ApplyRowSmem), sizeof(MomApplySmem), sizeof(FlatSmem));
-        static_assert(2 * (kSm + 1024) <= 228 * 1024, "two CTAs per SM");
+        static_assert(2 * (kSm + 1024 + (sizeof(TensorDev) + 127) / 128 * 128) <= 228 * 1024, "two CTAs per SM");
         static_assert(sizeof(Meta) <= kSm && sizeof(Smem) <= kSm, "light tiles");
         run(cudaFuncSetAttribute(k_apply_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm));
         run(launch(k_apply_rows, rC + L.nCR, kRowThreads, kSm, s, A, past(L.itemsC, L.nC - rC)));

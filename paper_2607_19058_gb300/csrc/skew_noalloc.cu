@@ -89,14 +89,6 @@ Layout layout_of(const TileGeom &G, uint32_t kind, int64_t n, int64_t m) {
     return o;
 }
 
-// Writes the descriptor and clears the scalars and the phase-B queue (the step's completion counters
-// must start at zero). The item tables of a single tensor are the identity: none are written.
-__global__ void k_noalloc_setup(TensorDev td, TensorDev *dst, TensorScal *scal, uint32_t *fb) {
-    *dst = td;
-    *scal = TensorScal{};
-    fb[0] = 0u;
-}
-
 }  // namespace
 }  // namespace skew
 
@@ -227,7 +219,6 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     // ---- per-step scalars, as skew_step forms them ------------------------------------
     const StepCoefs k = step_coefs(H, step);
     StepArgs a{};
-    a.tensors = (const TensorDev *)(base + o.tens);
     a.scal = (TensorScal *)(base + o.scal);
     a.err = (uint32_t *)(base + kErrOffset);
     a.fb = (uint32_t *)(base + o.fb);
@@ -260,12 +251,12 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
             td.m = 1;
         }
         td.srows = (uint32_t)small_rows(td.n, sp.ctas);
-        a.tensors = nullptr;
-        return launch_small(a, &td, 1, sp, stream, nullptr) == (int)cudaSuccess ? SKEW_OK : SKEW_ECUDA;
+        a.one = td;
+        return launch_small(a, 1, sp, stream, nullptr) == (int)cudaSuccess ? SKEW_OK : SKEW_ECUDA;
     }
-    k_noalloc_setup<<<1, 1, 0, s>>>(td, (TensorDev *)(base + o.tens), (TensorScal *)(base + o.scal),
-                                    (uint32_t *)(base + o.fb));
-    e = cudaGetLastError();
+    a.one = td;
+    // the scalars and the phase-B queue's length lie together: the step's completion counters start at zero
+    e = (cudaError_t)launch_reset(base + o.scal, o.fb + 4 - o.scal, stream);
     if (e != cudaSuccess) return SKEW_ECUDA;
     const uint32_t nRW = G.rowpath == kRowAny && m > kAnyNarrow ? o.nR : 0;
     const LaunchPlan lp{o.nA, o.nR, o.nF, o.nB, nFB, o.nC, o.nCR, nRW, false, nullptr, nullptr, nullptr, nullptr};

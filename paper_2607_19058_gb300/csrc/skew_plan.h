@@ -335,7 +335,8 @@ static_assert(sizeof(TensorScal) == 64, "TensorScal layout");
 
 // Per-step parameters, passed by value to every kernel (a kernel parameter).
 struct StepArgs {
-    const TensorDev *tensors;
+    const TensorDev *tensors;  // null: the one tensor `one` (the no-alloc step)
+    TensorDev one;
     TensorScal *scal;
     uint32_t *err;         // sticky status word (nonzero: a bounded wait gave up)
     uint32_t *fb;          // [0]: row-path tensors that need phase B, [1..]: their ids
@@ -429,11 +430,9 @@ inline SmallPlan plan_small(int64_t tensors, Each each) {
     return P;
 }
 
-// Enqueues the step of `tensors` small tensors (A.tensors, or `one` when that is null) as one launch;
-// `ev` as for launch_phases (its time is that of the last place). Returns a cudaError_t value.
-struct TensorDev;
-int launch_small(const StepArgs &A, const TensorDev *one, uint32_t tensors, const SmallPlan &P, void *stream,
-                 void *const *ev);
+// Enqueues the step of `tensors` small tensors as one launch; `ev` as for launch_phases (its time is that
+// of the last place). Returns a cudaError_t value.
+int launch_small(const StepArgs &A, uint32_t tensors, const SmallPlan &P, void *stream, void *const *ev);
 
 
 // Enqueues the phases of `L` as grouped launches (A, F, B, C; with row tiles A + R, F,
