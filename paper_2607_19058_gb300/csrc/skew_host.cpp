@@ -35,7 +35,7 @@ struct TPlan {
     int64_t n = 0, m = 0, numel = 0;
     int64_t moff = -1, voff = -1, roff = -1, coff = -1;  // floats into the state
     uint32_t lcl = 0, strips = 1, rowtiles = 1, tile_rows = 0, ntiles = 0, nfr = 0, nfc = 0, nbc = 0, fvpt = 0;
-    uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0, at_rows = 0, atiles = 0, fci = 0, nu2 = 0;
+    uint32_t rowpath = 0, cr = 0, rt_rows = 0, rtiles = 0, at_rows = 0, atiles = 0, fci = 0, nu2 = 0, keep = 0;
     uint32_t f32 = 0;         // SKEW_F_FP32: fp32 weights and gradient
     // bytes into the workspace
     size_t ws_rowp = 0, ws_colp = 0, ws_bsc = 0, ws_rsum = 0, ws_u2 = 0, ws_pp = 0, ws_rmin = 0, ws_fsum = 0, ws_fmin = 0;
@@ -108,10 +108,10 @@ static bool wg_aligned(const TPlan &p) { return (((uintptr_t)p.w | (uintptr_t)p.
 
 // Tile geometry (plan_geometry): strip tiles of (tile_rows rows) x (8*LC
 // columns) or flat tiles of kFlatTileElems elements, and for the row path whole-row tiles.
-static void geometry(TPlan &p, bool row_aligned, bool small, int64_t rest) {
+static void geometry(TPlan &p, bool row_aligned, bool small, int64_t rest, int64_t rest_c) {
     // the state buffer starts on a 256-byte boundary
     const bool vec = row_vectors(p.f32 != 0, wg_aligned(p), p.moff < 0 || p.moff % 4 == 0, p.m);
-    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, small, p.n, p.m, p.numel, rest);
+    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, small, p.n, p.m, p.numel, rest, rest_c);
     p.lcl = g.lcl;
     p.strips = g.strips;
     p.rowtiles = g.rowtiles;
@@ -196,7 +196,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.tid = (uint32_t)k;
                 q.base = (uint64_t)(e * p.numel);
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
-                geometry(q, row_aligned(q), false, kWholeGroup);  // which path
+                geometry(q, row_aligned(q), false, kWholeGroup, kWholeGroup);  // which path
                 if (q.rowpath == kRowAny) (q.m > kAnyNarrow ? any_wide : any_narrow) += 2 * q.numel;
                 fixed |= q.rowpath == kRowFixed;
                 h->t.push_back(q);
@@ -225,7 +225,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     h->state_bytes = size_t(off) * 4;
 
     // Tiles, now that the paths and the state's alignment are known: the row tiles by the bytes that
-    // follow, from the last matrix back.
+    // follow in each phase.
     const AnyWidths any = any_widths(any_narrow, any_wide, fixed);
     int64_t rest = 0, light = 0, fact = 0;  // elements off the row path, and of factored tensors
     for (TPlan &q : h->t) {
@@ -233,11 +233,29 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         if (!q.rowpath) light += q.numel;
         if (q.kind == kKindFactored) fact += q.numel;
     }
+    std::vector<int64_t> upto;  // bytes of G of the row-path matrices up to each (phase C starts with the last)
+    try {
+        upto.reserve(h->t.size());
+    } catch (...) {
+        delete h;
+        return fail(nullptr, SKEW_ENOMEM, "out of host memory");
+    }
+    int64_t sum = 0;
+    int64_t total = 0, again = 0;  // bytes that phase C reads again: of all, and from a matrix on
+    for (const TPlan &q : h->t) {
+        upto.push_back(sum += q.rowpath ? 2 * q.numel : 0);
+        total += q.rowpath ? (q.momentum ? 4 : 2) * q.numel : 0;
+    }
+    const bool reverse = total > kKeepBytes;  // phase C's row tiles (in fewer bytes all stay in L2 anyway)
     for (size_t k = h->t.size(); k-- > 0;) {
         TPlan &q = h->t[k];
         const bool row = q.rowpath != kRowNone;
-        if (row) rest += 2 * q.numel;
-        geometry(q, row, fact < kSmallStrip, rest);
+        if (row) {
+            rest += 2 * q.numel;
+            again += (q.momentum ? 4 : 2) * q.numel;
+        }
+        geometry(q, row, fact < kSmallStrip, rest, reverse ? upto[k] : rest);
+        q.keep = row && again <= kKeepBytes && total >= kKeepTotal;
         h->n_rowpath += row;
     }
     h->ride = h->n_rowpath && light <= kRideElems;
@@ -261,7 +279,6 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             const bool fact = p.kind == kKindFactored;
             if (p.rowpath) {
                 all(p.rowpath == kRowAny && p.m > kAnyNarrow ? itemsRW : itemsR, q, p.rtiles);
-                all(itemsCR, q, p.atiles);
             } else {
                 if (fact) all(h->itemsA, q, p.ntiles);
                 // flat tiles of phase B need no earlier phase: riding, they go with phase A
@@ -270,6 +287,9 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             }
             if (fact) all(h->itemsF, q, p.nfr + p.nfc);
         }
+        for (int q = 0; q < n_plans; ++q)
+            if (h->t[q].rowpath) all(itemsCR, q, h->t[q].atiles);
+        if (reverse) std::reverse(itemsCR.begin(), itemsCR.end());
         h->nA = (uint32_t)h->itemsA.size();
         h->nC = (uint32_t)h->itemsC.size();
         // the last phase-C row tiles run as two half tiles each (small tiles and tile indices past
@@ -458,6 +478,7 @@ int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace
         T.at_rows = p.at_rows;
         T.atiles = p.atiles;
         T.fci = p.fci;
+        T.keep = p.keep;
         T.srows = 0;
         if (h->small.ctas) {
             if (!fact) {  // stepped as numel x 1

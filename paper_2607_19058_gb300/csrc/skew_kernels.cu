@@ -647,6 +647,16 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 
+// L2 policy of a bulk-copied read: kept for the next phase, or passing through.
+__device__ __forceinline__ uint64_t read_policy(bool keep) {
+    uint64_t p;
+    if (keep)
+        asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    else
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
 // Threads of the row-path kernels (256 or 512).
 #ifndef SKEW_ROW_THREADS
 #define SKEW_ROW_THREADS 256
@@ -764,8 +774,7 @@ __device__ void rowsq_tile(const StepArgs &A, const TensorDev &T, TensorScal &S,
     static_assert(K == 4 || K == 8, "rows per thread per chunk");
     static_assert(CS <= 32, "chunk rows");
     const L lay;
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    const uint64_t pol = read_policy(T.keep);
     const uint32_t nch = (uint32_t)min((int64_t)(T.rt_rows / T.cr), (T.n - int64_t(tile) * T.rt_rows + T.cr - 1) / T.cr);
     if (threadIdx.x == 0) {
         for (int st = 0; st < kRowStages; ++st) mbar_init(&sm.full[st], 1);
@@ -2370,8 +2379,7 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
     auto issue = [&](uint32_t c, uint32_t st) {
         const uint32_t rows = min(cr, rows_t - c * cr), bx = rows * m * 2u;
         const int64_t e0 = (int64_t(tile) * T.rt_rows + c * cr) * T.m;
-        uint64_t pol;
-        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+        const uint64_t pol = read_policy(!MOM && T.keep);
         mbar_expect_tx(&sm.full[st], MOM ? 3u * bx : bx);
         bulk_g2s(ring + st * slot, T.g + e0, bx, &sm.full[st], pol);
         if (MOM) bulk_g2s(ring + st * slot + gbytes, T.M + e0, 2u * bx, &sm.full[st], pol);

@@ -130,6 +130,15 @@ struct TileGeom {
     uint32_t fci = 0;  // columns per finalize item (kFinChunk / fci threads per column)
 };
 
+// Phase C takes the matrices in the reverse of phase A's order, so that it starts with the G (with
+// momentum the M) that phase A read (wrote) last, and phase A asks L2 to keep the last kKeepBytes of it
+// (the L2 holds 126 MB, and R, W and the partials pass through it meanwhile), in steps whose phase C
+// reads kKeepTotal bytes or more again: the 6.78B set 8316 -> 8215 us (k_apply_rows 5862 -> 5765: more
+// than the kept bytes, so the rest of its stream gains too), one MoE layer 2088 -> 2066; without the hint
+// 8295 and 2086. Smaller steps lose by the hint what else the L2 would hold for them (65M parameters in
+// 768 x 488 experts 161 -> 168 us with it).
+constexpr int64_t kKeepBytes = int64_t(64) << 20, kKeepTotal = int64_t(256) << 20;
+
 constexpr int64_t kWholeGroup = int64_t(1) << 60;  // as `rest`: full-sized tiles
 
 // Chunks (of `chunk` bytes) in the row tiles of a matrix of `own` bytes when the step's row-path
@@ -178,11 +187,11 @@ inline AnyWidths any_widths(int64_t narrow, int64_t wide, bool fixed) {
 
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
 // gradient pointers are 16-byte aligned; `vec`: row-vectors may be 16-byte accesses (row_vectors);
-// `small`: the step's factored matrices hold fewer than kSmallStrip elements; `rest`: bytes of G of the step's row-path
-// matrices from this one on. Counts fit 32 bits for n, m <= 2^40
+// `small`: the step's factored matrices hold fewer than kSmallStrip elements; `rest`, `rest_c`: bytes of G of the step's
+// row-path matrices from this one on in phase A's order and in phase C's. Counts fit 32 bits for n, m <= 2^40
 // and n*m <= 2^62 only when the caller has checked the tile count (planner).
 inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, bool vec, bool small, int64_t n,
-                              int64_t m, int64_t numel, int64_t rest) {
+                              int64_t m, int64_t numel, int64_t rest, int64_t rest_c) {
     TileGeom g;
     if (kind == kKindFactored) {
         const int64_t vecs = (m + 7) / 8;  // 8-column groups per row
@@ -210,7 +219,7 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
                 g.cr = (uint32_t)(chunk / (2 * m));
                 const int64_t most = momentum ? kMomChunks : m == 4096 && n >= 2048 ? kRowChunksWide : kRowChunks;
                 g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, 65536 / chunk, most, (12 << 20) / (8 * m));
-                const uint32_t at = row_tile_chunks(own, rest, 3, chunk, 32768 / chunk, (1 << 20) / chunk, 0);
+                const uint32_t at = row_tile_chunks(own, rest_c, 3, chunk, 32768 / chunk, (1 << 20) / chunk, 0);
                 g.at_rows = g.cr * (momentum ? (at + 1) / 2 * 2 : at);  // a half tile is whole phase-C chunks
             } else {
                 const int nv = m > 2048 ? 2 : 1, warps = m > kAnyNarrow ? 16 : 8;
@@ -220,7 +229,7 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
                 g.rt_rows = g.cr * row_tile_chunks(own, rest, momentum ? 2 : 1, chunk, least < 1 ? 1 : least,
                                                    (warps / 8) * kAnyTileBytes / chunk,
                                                    (12 << 20) / (8 * m));
-                int64_t at = 2 * row_tile_chunks(own, rest, 3, 4 * m, (32768 + 4 * m - 1) / (4 * m), kAnyTileBytes / (4 * m), 0);
+                int64_t at = 2 * row_tile_chunks(own, rest_c, 3, 4 * m, (32768 + 4 * m - 1) / (4 * m), kAnyTileBytes / (4 * m), 0);
                 const int64_t fit = (m > kAnyNarrow ? kFlatWideScales : kFlatScales) - m;
                 if (at > fit) at = fit;
                 g.at_rows = (uint32_t)(at / 2 * 2);
@@ -313,6 +322,7 @@ struct TensorDev {
     uint32_t fci;       // columns per finalize item
     uint32_t at_rows;   // row path: rows per phase-C row tile (<= 1024 at the fixed widths)
     uint32_t atiles;    // row path: phase-C row tiles
+    uint32_t keep;      // row path: phase C finds this G in L2 if phase A leaves it there
     uint32_t srows;     // k_small: rows (full: elements, m = 1) of a CTA's slice
 };
 
