@@ -263,6 +263,13 @@ __device__ __forceinline__ float row_scale(float Ri, float rbar_s, int rbar_e) {
 // ---------------------------------------------------------------------------
 // Reductions
 // ---------------------------------------------------------------------------
+// Eight fp32 values in shared memory (16-byte aligned).
+__device__ __forceinline__ void lds8(const float *p, float (&o)[8]) {
+    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
+    o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+}
+
 // Error-free sum (Knuth's TwoSum): s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
@@ -1262,7 +1269,6 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
     float *__restrict__ M_ = T.M;
     const int64_t n = T.n, m = T.m, row0 = F.row0, RG = F.RG, col0 = F.col0;
     const float b1 = A.b1, c1 = grad_scale(A).c1, ce = A.ce;
-    const bool mnew = MOM && T.rowpath;  // phase B of a queued row-path tensor: M is already new
     const float *rows = meta.rows + F.rg;
     const int vpt = (int)(T.tile_rows / F.RG);
     float b[8];
@@ -1294,14 +1300,9 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
                     if (MOM) {
                         const float4 m0 = mraw[MOM ? q : 0][0], m1 = mraw[MOM ? q : 0][1];
                         const float mm[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-                        if (mnew) {  // the row path already stored this step's momentum
 #pragma unroll
-                            for (int c = 0; c < 8; ++c) y[c] = mm[c];
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) y[c] = fmaf(b1, mm[c], c1 * y[c]);
-                            store_f8(M_ + i * m + col0, true, 8, y);
-                        }
+                        for (int c = 0; c < 8; ++c) y[c] = fmaf(b1, mm[c], c1 * y[c]);
+                        store_f8(M_ + i * m + col0, true, 8, y);
                     }
                     rms_row(y, rows[(k0 + q) * RG], b, 8, ce, acc);
                 }
@@ -1524,13 +1525,6 @@ __device__ void phase_B_fact(const StepArgs &A, const TensorDev &T, uint32_t t, 
         phase_B_strip(A, T, t, local, sm, meta, pol);
     else
         phase_B_flat(A, T, t, local, sm, meta, pol);
-}
-
-// The same for k_fallback's own items, out of line: inlined beside the queue's tiles, which are strip
-// tiles, it makes those spill (a queue of 62M elements of 1024 and 496 columns 56 us slower).
-__device__ __noinline__ void phase_B_own(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm,
-                                         Meta &meta) {
-    phase_B_fact(A, T, t, local, sm, meta, Pol());
 }
 
 // ---------------------------------------------------------------------------
@@ -2819,6 +2813,91 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     if (sum && done) publish_sum(A, T, S, item, rows_t, acc, sm.sum);
 }
 
+// Phase B of a queued row-path tensor: sum(U^2) over the rows of a phase-C tile, from a ring of G (or the
+// new M, which phase A stored) alone. Chunks run on from tile to tile (`turn` counts them), so that the
+// barriers keep their phases. Bound by HBM: with all of 65M parameters in 768 x 488 experts queued a step
+// takes 185 us, 205 when the queue ran on strip tiles (118M in 816 x 408 experts: 275 and 297).
+template <bool MOM>
+struct SumRing {
+    static constexpr uint32_t kChunk = MOM ? 512 : 1024, kSlot16 = 1024, kStages = 4;  // vectors; 16 KB slots
+    static constexpr uint32_t kWords = kSlot16 * kStages;
+};
+constexpr int kSumScales = kFlatBytes / 4 - 4 * (int)SumRing<false>::kWords;
+static_assert(kSumScales >= kFlatWideScales && kSumScales >= 4096 + 128, "the planner's rows fit");
+
+template <bool MOM>
+__device__ bool sum_tile(const StepArgs &A, const TensorDev &T, TensorScal &S, uint32_t tile, uint32_t &turn, FlatSmem &sm) {
+    using F = SumRing<MOM>;
+    const int tid = threadIdx.x;
+    const int64_t r0 = int64_t(tile) * T.at_rows;
+    const uint32_t m = (uint32_t)T.m, V = m / 8u, rows_t = (uint32_t)min((int64_t)T.at_rows, T.n - r0), total = rows_t * V;
+    const uint32_t nch = (total + F::kChunk - 1) / F::kChunk;
+    const uint64_t pol = read_policy(false);
+    const char *src = MOM ? reinterpret_cast<const char *>(T.M + r0 * T.m) : reinterpret_cast<const char *>(T.g + r0 * T.m);
+    const uint32_t t0 = turn;
+    auto issue = [&](uint32_t c) {
+        const uint32_t st = (t0 + c) % F::kStages, bytes = min(F::kChunk, total - c * F::kChunk) * (MOM ? 32u : 16u);
+        mbar_expect_tx(&sm.full[st], bytes);
+        bulk_g2s(sm.data + st * F::kSlot16, src + uint64_t(c) * F::kChunk * (MOM ? 32u : 16u), bytes, &sm.full[st], pol);
+    };
+    if (tid == 0) {
+        fence_proxy_async_smem();
+        for (uint32_t c = 0; c < nch && c < F::kStages; ++c) issue(c);
+    }
+    float *ab = reinterpret_cast<float *>(sm.data + F::kWords);
+    const float rbar_s = __ldcg(&S.rbar_s), ce = A.ce;
+    const int rbar_e = __ldcg(&S.rbar_e);
+    for (uint32_t j = tid; j < m / 4; j += kThreads)
+        reinterpret_cast<float4 *>(ab)[j] = __ldcg(reinterpret_cast<const float4 *>(T.bsc) + j);
+    for (uint32_t r = tid; r < rows_t; r += kThreads) ab[m + r] = row_scale(__ldcg(T.R + r0 + r), rbar_s, rbar_e);
+    __syncthreads();
+    const float *sb = ab, *sa = ab + m;
+    uint32_t row = tid / V, col = tid - row * V;
+    const uint32_t dq = kThreads / V, dr = kThreads - dq * V;
+    Acc2 acc;
+    for (uint32_t c = 0; c < nch; ++c) {
+        const uint32_t cnt = min(F::kChunk, total - c * F::kChunk), st = (t0 + c) % F::kStages;
+        const bool ok = mbar_wait(&sm.full[st], ((t0 + c) / F::kStages) & 1u);
+        const uint4 *by = sm.data + st * F::kSlot16;
+#pragma unroll
+        for (uint32_t k = 0; k < F::kChunk / kThreads; ++k) {
+            const uint32_t f = k * kThreads + tid;
+            if (f < cnt) {
+                const float a = sa[row];
+                const float4 b0 = *reinterpret_cast<const float4 *>(sb + 8 * col);
+                const float4 b1 = *reinterpret_cast<const float4 *>(sb + 8 * col + 4);
+                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                float y[8], u[8];
+                if constexpr (MOM)
+                    lds8(reinterpret_cast<const float *>(by) + 8 * f, y);
+                else
+                    unpack_bf8(by[f], y);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) u[q] = y[q] * fminf(a * b[q], ce);
+                acc.add(sumsq8(u));
+            }
+            row += dq;
+            col += dr;
+            if (col >= V) {
+                col -= V;
+                ++row;
+            }
+        }
+        if (__syncthreads_or(!ok)) {  // every thread is done with the slot: refill it
+            if (tid == 0) drain_copies(A.err, sm.full, F::kStages, t0 + c, t0 + min(nch, c + F::kStages));
+            return false;
+        }
+        if (tid == 0 && c + F::kStages < nch) {
+            fence_proxy_async_smem();
+            issue(c + F::kStages);
+        }
+    }
+    turn = t0 + nch;
+    publish_sum(A, T, S, tile, rows_t, acc, sm.sum);
+    __syncthreads();  // the scales and sums are free for the next tile
+    return true;
+}
+
 // ---------------------------------------------------------------------------
 // A step of small tensors only (k_small): a cluster of CTAs takes one tensor through the whole step.
 // Each CTA keeps a slice of it (whole rows of a factored tensor) in shared memory as fp32, so G is read
@@ -2847,13 +2926,7 @@ struct SmallSlice {
     }
 };
 
-// Eight fp32 values in shared memory (16-byte aligned; all eight are there, whatever is valid).
-__device__ __forceinline__ void lds8(const float *p, float (&o)[8]) {
-    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
-    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
-    o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-}
-
+// Eight fp32 values to shared memory (16-byte aligned).
 __device__ __forceinline__ void sts8(float *p, const float (&o)[8]) {
     reinterpret_cast<float4 *>(p)[0] = make_float4(o[0], o[1], o[2], o[3]);
     reinterpret_cast<float4 *>(p)[1] = make_float4(o[4], o[5], o[6], o[7]);
@@ -3261,33 +3334,43 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     }
 }
 
-// Phase B of the row-path tensors whose finalize found that a clamp may bind
-// (queued in A.fb): the CTAs of this grid share the tiles of all queued tensors, laid end to end
-// (starting every tensor at CTA 0 would give the first CTAs a tile of each small one).
-// The first nB CTAs run the phase-B strip tiles of the other tensors.
+// Phase B of the row-path tensors whose finalize found that a clamp may bind and the update be clipped
+// (queued in A.fb): the CTAs of this grid share the phase-C tiles of all queued tensors, laid end to end
+// (starting every tensor at CTA 0 would give the first CTAs a tile of each small one). The first nB CTAs
+// run the phase-B strip and flat tiles of the other tensors.
 __global__ void __launch_bounds__(kThreads, 2)
     k_fallback(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items, uint32_t nB) {
-    __shared__ Smem sm;
-    __shared__ Meta meta;
+    extern __shared__ uint4 dyn_smem[];
+    __shared__ TensorDev td;
     if (blockIdx.x < nB) {
-        __shared__ TensorDev td;
+        struct Own {
+            Smem sm;
+            Meta meta;
+        };
+        Own &o = *reinterpret_cast<Own *>(dyn_smem);
+        static_assert(sizeof(Own) <= sizeof(FlatSmem), "k_fallback's shared memory");
         const uint2 it = begin_item(items, A, td);
-        phase_B_own(A, td, it.x, it.y, sm, meta);
+        phase_B_fact(A, td, it.x, it.y, o.sm, o.meta, Pol());
         return;
     }
     let_next_launch_start();
     wait_previous_launch();
-    const Pol pol;
     const uint32_t cnt = __ldcg(A.fb), ctas = gridDim.x - nB;
-    uint32_t tile = blockIdx.x - nB;  // of queued tensor q
+    if (!cnt) return;
+    FlatSmem &sm = *reinterpret_cast<FlatSmem *>(dyn_smem);
+    if (threadIdx.x == 0) {
+        for (uint32_t st = 0; st < 4; ++st) mbar_init(&sm.full[st], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    uint32_t tile = blockIdx.x - nB, turn = 0;  // of queued tensor q
     for (uint32_t q = 0; q < cnt; ++q) {
         const uint32_t t = __ldcg(A.fb + 1 + q);
         const TensorDev &T = A.tensors ? A.tensors[t] : A.one;
-        const uint32_t nt = T.nbc;
-        for (; tile < nt; tile += ctas) {
-            phase_B_strip(A, T, t, tile, sm, meta, pol);
-            __syncthreads();
-        }
+        const uint32_t nt = T.atiles;
+        for (; tile < nt; tile += ctas)
+            if (!(T.momentum ? sum_tile<true>(A, T, A.scal[t], tile, turn, sm) : sum_tile<false>(A, T, A.scal[t], tile, turn, sm)))
+                return;
         tile -= nt;
     }
 }
@@ -3433,7 +3516,10 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     mark(3);
     if (L.nB > rB) run(launch(k_rms, L.nB, kThreads, 0, s, A, L.itemsB));
     mark(4);
-    if (rows) run(launch(k_fallback, rB + L.nFB, kThreads, 0, s, A, L.itemsB, rB));
+    if (rows) {
+        run(cudaFuncSetAttribute(k_fallback, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FlatSmem)));
+        run(launch(k_fallback, rB + L.nFB, kThreads, sizeof(FlatSmem), s, A, L.itemsB, rB));
+    }
     mark(5);
     if (L.nC > rC) run(launch(k_apply, L.nC, kThreads, 0, s, A, L.itemsC));
     mark(6);
