@@ -148,14 +148,14 @@ def byte_model(opt, n_tensors):
     N = N_mom = N_full = N_fact = N_nomom = N_row = N_rowm = 0
     rc = rc_row = 0
     infos = [opt.info(k) for k in range(n_tensors)]
-    # whole-row tiles: the fixed widths, and any multiple of 8 from 128 to 4096 where such matrices hold
-    # 2 MiB of gradient or more, to 8192 where those above 4096 hold 64 MiB (2 without other row tiles)
+    # whole-row tiles: the fixed widths, and any multiple of 8 from 128 to 4096 where these all hold
+    # 32 MiB of gradient or more, to 8192 where those above 4096 hold 64 MiB (32 without other row tiles)
     def other(lo, hi):
         return 2 * sum(i.numel for i in infos if i.kind == 1 and not i.rowpath and i.vectorized and lo <= i.cols <= hi)
 
-    narrow, wide, fixed = other(128, 4096), other(4097, 8192), any(i.rowpath for i in infos)
-    wide_rows = wide >= 64 << 20 or (not fixed and narrow < 2 << 20 <= wide)
-    narrow_rows = narrow >= 2 << 20 or (wide_rows and narrow > 0)
+    narrow, wide, fixed = other(128, 4096), other(4097, 8192), 2 * sum(i.numel for i in infos if i.rowpath)
+    wide_rows = wide >= 64 << 20 or (not fixed and narrow < 32 << 20 <= wide)
+    narrow_rows = narrow > 0 and (narrow + fixed >= 32 << 20 or wide_rows)
     for i in infos:
         E = max(1, i.stack)  # a stack of E matrices: rows / cols are one matrix's
         N += i.numel

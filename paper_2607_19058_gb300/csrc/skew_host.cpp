@@ -162,8 +162,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     const int64_t kMaxExtent = int64_t(1) << 40;
     // whole-row tiles are for bf16 rows on 16-byte boundaries
     auto row_aligned = [](const TPlan &q) { return !q.f32 && wg_aligned(q); };
-    int64_t any_narrow = 0, any_wide = 0;  // bytes of G of the matrices that only kRowAny's row tiles serve
-    bool fixed = false;                    // matrices of the fixed widths
+    int64_t any_narrow = 0, any_wide = 0, fixed = 0;  // bytes of G: matrices that only kRowAny serves, fixed widths
     for (int32_t k = 0; k < n_params; ++k) {
         const skew_param_desc_t &d = params[k];
         TPlan p;
@@ -198,7 +197,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
                 geometry(q, row_aligned(q), false, kWholeGroup, kWholeGroup);  // which path
                 if (q.rowpath == kRowAny) (q.m > kAnyNarrow ? any_wide : any_narrow) += 2 * q.numel;
-                fixed |= q.rowpath == kRowFixed;
+                if (q.rowpath == kRowFixed) fixed += 2 * q.numel;
                 h->t.push_back(q);
             }
         } catch (...) {

@@ -2,18 +2,20 @@
 //
 // One SkewAdam step (paper Sec. 3, Eq. 1, Algorithm 1) as grouped launches in stream
 // order, each over an item table of (tensor, tile) pairs; a step with row-path tensors
-// takes k_rowsq, k_finalize, k_fallback and k_apply_rows, which also run its strip and flat
-// tiles, any other k_sumsq, k_finalize, k_rms and k_apply:
+// takes k_rowsq (and k_rowsq_wide), k_finalize, k_fallback and k_apply_rows, which also
+// run its strip and flat tiles while these are few; any other takes k_sumsq, k_finalize,
+// k_rms and k_apply, and a step of small tensors k_small alone:
 //   k_sumsq      phase A, strip tiles: per-row and per-column sums of g^2 of a
 //                factored matrix (Eq. 1), column partials per row tile (no atomics);
-//   k_rowsq      phase A, whole-row tiles of factored matrices 512 to 4096 wide:
-//                chunks of whole rows bulk-copied into a shared-memory ring; R_i
-//                formed in the tile (Eq. 1), per-column partials of g^2 and of
-//                g^2 / R_i (or M^2 / R_i after the momentum update, stored here),
-//                from which the finalize forms sum(U^2) by the bilinear identity;
+//   k_rowsq      phase A, whole-row tiles of factored matrices 128 to 4096 wide
+//                (k_rowsq_wide: to 8192): chunks of whole rows bulk-copied into a
+//                shared-memory ring; R_i formed in the tile (Eq. 1), per-column partials
+//                of g^2 and of g^2 / R_i (or M^2 / R_i after the momentum update, stored
+//                here), from which the finalize forms sum(U^2) by the bilinear identity;
 //   k_finalize   R / C moving averages (strip path) or C (row path), 1/sqrt(C_j),
-//                mean(R); on the row path also sum(U^2) and the clip factor, or the
-//                tensor is queued for phase B when the 1/sqrt(eps) clamp may bind;
+//                mean(R); on the row path also sum(U^2) and the clip factor; when the
+//                1/sqrt(eps) clamp may bind, either the clip factor (provably 1; phase C
+//                then sums U^2) or an entry in the queue for phase B;
 //   k_rms        phase B, strip and flat tiles: momentum / exact second-moment
 //                update, U up to its scalar and a compensated sum(U^2) per tile;
 //                the last tile forms RMS(U) and the clip factor (Sec. 3);
@@ -21,7 +23,8 @@
 //   k_apply      phase C, strip and flat tiles: x = w (1 - lr*lambda) - lr*kappa*U
 //                in fp32 and the dithered bf16 write-back (Philox-4x32-10);
 //   k_apply_rows phase C, whole-row tiles: the same on bulk-copied rows of W and
-//                G (or the new M).
+//                G (or the new M);
+//   k_small      all phases of a small tensor, one cluster of CTAs each.
 // The reconstructed second moment of a factored matrix is never formed:
 // 1/sqrt(max(R_i C_j / Rbar, eps)) = min(a_i * b_j, 1/sqrt(eps)) with
 // a_i = 1/sqrt(R_i / Rbar) per row and b_j = 1/sqrt(C_j) per column.

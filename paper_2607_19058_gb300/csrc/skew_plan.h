@@ -164,24 +164,27 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
     return (uint32_t)t;
 }
 
-// Below this many bytes of G in all the matrices that only kRowAny serves, the strip tiles' second
-// read of G costs a step no more than k_fallback and the row tiles' ramps: 2048 x 1408 on its own
-// (5.8 MB) takes 51 us on strip tiles and 44 us on row tiles, the smallest steps the reverse.
-constexpr int64_t kAnyGroupBytes = 2 << 20;
+// Below this many bytes of G in all row-path matrices, those that only kRowAny serves take strip tiles (beside
+// larger row tiles a 4095 x 1000 matrix of 8 MB costs 43 us more on strip tiles): their second read
+// of G (much of it from L2) costs a step no more than k_fallback and the row tiles' ramps: 10M parameters
+// of a 256-wide model, most of them its embedding's, 69 us on strip tiles and 89 on row tiles (21 MB of G),
+// 2048 x 1408 alone 28 and 32; 20M of another 256-wide model 96 and 70 (41 MB), 29M of a 432-wide one 151
+// and 113.
+constexpr int64_t kAnyGroupBytes = 32 << 20;
 // Beside row tiles of other widths, those above kAnyNarrow need a launch of their own, and below this
 // many bytes of G the strip tiles, which ride along, are faster (260M parameters, 23 MB of them 5632
 // wide: 379 us against 407; 1.16B parameters of 4864 and 7128 columns: 2314 against 1653).
 constexpr int64_t kWideGroupBytes = 64 << 20;
 
 // Which widths that only kRowAny serves take row tiles in a step: `narrow` and `wide` bytes of G of its
-// matrices up to and above kAnyNarrow columns, `fixed`: it has matrices of the fixed widths.
+// matrices up to and above kAnyNarrow columns, `fixed`: of those of the fixed widths.
 struct AnyWidths {
     bool narrow, wide;
 };
-inline AnyWidths any_widths(int64_t narrow, int64_t wide, bool fixed) {
+inline AnyWidths any_widths(int64_t narrow, int64_t wide, int64_t fixed) {
     AnyWidths w;
-    w.wide = wide >= kWideGroupBytes || (!fixed && narrow < kAnyGroupBytes && wide >= kAnyGroupBytes);
-    w.narrow = narrow >= kAnyGroupBytes || (w.wide && narrow > 0);
+    w.wide = wide >= kWideGroupBytes || (fixed == 0 && narrow < kAnyGroupBytes && wide >= kAnyGroupBytes);
+    w.narrow = narrow > 0 && (narrow + fixed >= kAnyGroupBytes || w.wide);
     return w;
 }
 

@@ -13,9 +13,9 @@ E, B = WL.TIER_EXPERT, WL.TIER_BACKBONE
 #          rows, width: rows of half a warp; 64-row chunks; 2 warps a row; 5 of 8 warps; a partial last warp; 1 row side by side;
 #          two vectors a thread, the second for few lanes; three quarters of the warps; the widest of 8 warps
 SHAPES = [(2113, 128), (700, 200), (2113, 256), (1, 256), (700, 264), (333, 776), (517, 1032), (131, 1408), (9, 2040), (130, 2056), (257, 2880),
-          (301, 3072), (5, 4088), (267, 4088)]
+          (301, 3072), (5, 4088), (2049, 4088)]
 # 16 warps a row tile (in a step without the others: see the planner's any_widths)
-WIDE = [(1, 4104), (130, 4104), (77, 5632), (131, 7128), (300, 8192)]
+WIDE = [(1, 4104), (130, 4104), (77, 5632), (131, 7128), (1500, 8192)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -27,17 +27,22 @@ def _built():
 
 
 def _workload(shapes):
+    """More than the 32 MiB of gradient from which these widths take row tiles."""
     specs = [WL.Spec(f"{'eb'[t]}{n}x{m}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1)
              for k, (n, m) in enumerate(shapes) for t in (0, 1)]
     m0, m1 = (1536, 768) if shapes is SHAPES else (4800, 5000)
     specs += [WL.Spec("se", (3, 130, m0), E), WL.Spec("sb", (2, 67, m1), B)]
+    assert 2 * sum(torch.Size(s.shape).numel() for s in specs) >= 32 << 20
     return WL.Workload("widths", specs, WL.HP(), "toy", steps=3)
 
 
 @pytest.mark.parametrize("shapes", [SHAPES, WIDE], ids=["to4096", "to8192"])
-@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05)], ids=["eps1e-30", "paper"])
+@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05),
+                                dict(eps=1e-8, lr=3e-4, weight_decay=0.05, clip_d=0.05)],
+                         ids=["eps1e-30", "paper", "clipped"])
 def test_any_width_rows(shapes, hp):
-    """eps = 1e-8 binds the clamp at step 1; experts 5 to 7 have zero gradients on odd steps."""
+    """eps = 1e-8 binds the clamp at step 1 (and d = 0.05 clips, so that every tensor takes phase B); experts
+    5 to 7 have zero gradients on odd steps."""
     import parity
     h = parity.Harness(_workload(shapes), hp_override=hp)
     for t in range(1, 4):
@@ -46,7 +51,9 @@ def test_any_width_rows(shapes, hp):
     h.close()
 
 
-@pytest.mark.parametrize("shape,tier", [((700, 264), E), ((517, 1032), B), ((301, 3072), E), ((2049, 1408), E), ((300, 7128), B), ((700, 8192), E)])
+# (16.8M elements are what takes such a matrix to row tiles when it is alone)
+@pytest.mark.parametrize("shape,tier", [((700, 264), E), ((12001, 1408), E), ((5601, 3072), B), ((2400, 7128), E),
+                                        ((2051, 8192), B)])
 def test_noalloc_matches_the_handle(shape, tier):
     torch.manual_seed(0)
     w0 = (torch.randn(shape, device="cuda") * 0.02).to(torch.bfloat16)
