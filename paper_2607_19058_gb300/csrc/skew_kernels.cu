@@ -3461,7 +3461,8 @@ int launch_small(const StepArgs &A, uint32_t tensors, const SmallPlan &P, void *
     static_assert(kSmallHeadBytes >= (sizeof(SmallSmem) + 15) / 16 * 16, "k_small's shared memory");
     if (ev)
         for (int k = 0; k < kLaunches; ++k) cudaEventRecord((cudaEvent_t)ev[k], s);
-    cudaError_t e = cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
+    // (always the most that a step may take: the attribute is the process's, and other threads launch too)
+    cudaError_t e = cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
     if (e != cudaSuccess) return (int)e;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
