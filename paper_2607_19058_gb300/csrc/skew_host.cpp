@@ -225,7 +225,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
 
     // Tiles, now that the paths and the state's alignment are known: the row tiles by the bytes that
     // follow in each phase.
-    const AnyWidths any = any_widths(any_narrow, any_wide, fixed);
+    const AnyWidths any = any_widths(any_narrow, any_wide, fixed, h->hp.eps);
     int64_t rest = 0, light = 0, fact = 0;  // elements off the row path, and of factored tensors
     for (TPlan &q : h->t) {
         if (q.rowpath == kRowAny && !(q.m > kAnyNarrow ? any.wide : any.narrow)) q.rowpath = kRowNone;

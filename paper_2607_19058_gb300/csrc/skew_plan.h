@@ -171,20 +171,28 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
 // 2048 x 1408 alone 28 and 32; 20M of another 256-wide model 96 and 70 (41 MB), 29M of a 432-wide one 151
 // and 113.
 constexpr int64_t kAnyGroupBytes = 32 << 20;
+// An eps that the clamp may bind at (kBindEps: a row's or column's mean g^2 of 1e-12 is g = 1e-6) can queue
+// matrices for k_fallback, which reads them again, M included; a step of these widths alone then gains from
+// row tiles from twice that on. 256 wide, eps = 1e-8, clipped gradients, half or more of it with momentum:
+// 37 MiB of G 113 us on strip tiles and 121 to 139 on row tiles, 43 MiB 119 and 131, 65 MiB 165 and 155,
+// 110 MiB 241 and 229; eps = 1e-30, 37 MiB: 112 and 90.
+constexpr int64_t kAnyBindBytes = 64 << 20;
+constexpr float kBindEps = 1e-12f;
 // Beside row tiles of other widths, those above kAnyNarrow need a launch of their own, and below this
 // many bytes of G the strip tiles, which ride along, are faster (260M parameters, 23 MB of them 5632
 // wide: 379 us against 407; 1.16B parameters of 4864 and 7128 columns: 2314 against 1653).
 constexpr int64_t kWideGroupBytes = 64 << 20;
 
 // Which widths that only kRowAny serves take row tiles in a step: `narrow` and `wide` bytes of G of its
-// matrices up to and above kAnyNarrow columns, `fixed`: of those of the fixed widths.
+// matrices up to and above kAnyNarrow columns, `fixed`: of those of the fixed widths; `eps`: the clamp's.
 struct AnyWidths {
     bool narrow, wide;
 };
-inline AnyWidths any_widths(int64_t narrow, int64_t wide, int64_t fixed) {
+inline AnyWidths any_widths(int64_t narrow, int64_t wide, int64_t fixed, float eps) {
+    const int64_t least = fixed < kAnyGroupBytes && eps > kBindEps ? kAnyBindBytes : kAnyGroupBytes;
     AnyWidths w;
-    w.wide = wide >= kWideGroupBytes || (fixed == 0 && narrow < kAnyGroupBytes && wide >= kAnyGroupBytes);
-    w.narrow = narrow > 0 && (narrow + fixed >= kAnyGroupBytes || w.wide);
+    w.wide = wide >= kWideGroupBytes || (fixed == 0 && narrow < least && wide >= least);
+    w.narrow = narrow > 0 && (narrow + fixed >= least || w.wide);
     return w;
 }
 

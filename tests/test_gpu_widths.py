@@ -26,13 +26,15 @@ def _built():
     oracle.build()
 
 
-def _workload(shapes):
-    """More than the 32 MiB of gradient from which these widths take row tiles."""
+def _workload(shapes, eps=1e-30):
+    """More than the 32 MiB of gradient from which these widths take row tiles (64 with an eps that may bind)."""
     specs = [WL.Spec(f"{'eb'[t]}{n}x{m}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1)
              for k, (n, m) in enumerate(shapes) for t in (0, 1)]
     m0, m1 = (1536, 768) if shapes is SHAPES else (4800, 5000)
     specs += [WL.Spec("se", (3, 130, m0), E), WL.Spec("sb", (2, 67, m1), B)]
-    assert 2 * sum(torch.Size(s.shape).numel() for s in specs) >= 32 << 20
+    if eps > 1e-12:
+        specs.append(WL.Spec("more", (6000, 1400) if shapes is SHAPES else (1000, 4200), B))
+    assert 2 * sum(torch.Size(s.shape).numel() for s in specs) >= (64 if eps > 1e-12 else 32) << 20
     return WL.Workload("widths", specs, WL.HP(), "toy", steps=3)
 
 
@@ -44,7 +46,7 @@ def test_any_width_rows(shapes, hp):
     """eps = 1e-8 binds the clamp at step 1 (and d = 0.05 clips, so that every tensor takes phase B); experts
     5 to 7 have zero gradients on odd steps."""
     import parity
-    h = parity.Harness(_workload(shapes), hp_override=hp)
+    h = parity.Harness(_workload(shapes, **{k: v for k, v in hp.items() if k == "eps"}), hp_override=hp)
     for t in range(1, 4):
         h.step(t, seed=17 * t, **({"gscale": 0.37} if t == 2 else {}))
     h.opt.sync_status()
