@@ -42,10 +42,11 @@ unsigned char *scratch_base() {
     return static_cast<unsigned char *>(p);
 }
 
-// Where one tensor's scratch lies in the fixed array, its item counts and the bytes it takes.
+// Where one tensor's scratch lies in the fixed array, its item counts and the bytes it takes. (Its
+// descriptor is a kernel parameter and its items are counted off in order, so neither takes room.)
 struct Layout {
     uint32_t nA, nR, nF, nB, nC, nCR;
-    size_t scal, fb, tens, iA, iR, iF, iB, iC, iCR, rowp, colp, bsc, rsum, pp, rmin, fsum, fmin, u2, bytes;
+    size_t scal, fb, rowp, colp, bsc, rsum, pp, rmin, fsum, fmin, u2, bytes;
 };
 
 Layout layout_of(const TileGeom &G, uint32_t kind, int64_t n, int64_t m) {
@@ -64,13 +65,6 @@ Layout layout_of(const TileGeom &G, uint32_t kind, int64_t n, int64_t m) {
     };
     put(o.scal, sizeof(TensorScal));
     put(o.fb, 8);
-    put(o.tens, sizeof(TensorDev));
-    put(o.iA, sizeof(uint2) * o.nA);
-    put(o.iR, sizeof(uint2) * o.nR);
-    put(o.iF, sizeof(uint2) * o.nF);
-    put(o.iB, sizeof(uint2) * o.nB);
-    put(o.iC, sizeof(uint2) * o.nC);
-    put(o.iCR, sizeof(uint2) * o.nCR);
     if (fact && !row) {
         put(o.rowp, 4 * size_t(G.strips) * n);
         put(o.colp, 4 * size_t(G.rowtiles) * m);

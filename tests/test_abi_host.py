@@ -283,6 +283,17 @@ def test_noalloc_scratch_limit_on_the_host():
     assert _noalloc(rows=1 << 20, cols=8192) == S.SKEW_ETOOBIG
 
 
+@pytest.mark.parametrize("rows,cols,flags,off", [(4124839, 1, 0, 0), (357164, 1416, 0, 0), (69422, 7488, 0, 2),
+                                                 (237068, 2144, S.F_FP32, 0), (3861952, 64, 0, 2)])
+def test_noalloc_takes_tensors_whose_partials_fill_the_scratch(rows, cols, flags, off):
+    """Only what the kernels use counts against the scratch: these matrices' row and column partials,
+    column scales and tile sums fit it, if barely. Twice the rows are SKEW_ETOOBIG."""
+    import torch
+    if not torch.cuda.is_available():  # (with a GPU the fake pointers would reach the kernels)
+        assert _noalloc(rows=rows, cols=cols, flags=flags, weight=0x10000000000 + off) == S.SKEW_ECUDA
+    assert _noalloc(rows=2 * rows, cols=cols, flags=flags, weight=0x10000000000 + off) == S.SKEW_ETOOBIG
+
+
 def test_random_plans_tile_the_state():
     """Random parameter lists (vectors, matrices, stacks; every tier; no-decay and fp32
     flags; every policy): the planner's state is the oracle's closed form, each tensor's
