@@ -667,16 +667,10 @@ __device__ __forceinline__ uint64_t read_policy(bool keep) {
     return p;
 }
 
-// Threads of the row-path kernels (256 or 512).
-#ifndef SKEW_ROW_THREADS
-#define SKEW_ROW_THREADS 256
-#endif
-constexpr int kRowThreads = SKEW_ROW_THREADS;
-
 struct RowSmem {
     uint4 buf[kRowStages][kRowChunkBytes / 16];  // the chunk ring (first member: 16-byte aligned)
     uint64_t full[kRowStages];                   // one mbarrier per ring slot
-    float part[kRowThreads / 32][8];             // per-warp row partial sums of the chunk
+    float part[kThreads / 32][8];             // per-warp row partial sums of the chunk
     float inv[32];                               // 1 / R_i of the chunk's rows (0: no contribution)
     int fail;
 };
@@ -1782,7 +1776,7 @@ struct ApplyRowSmem {
     uint4 buf[kRowStages][kRowChunkBytes / 16];  // [W rows | G rows] per slot
     uint64_t full[kRowStages];
     float a[kRowChunks * 32];                    // row scales a_i of the tile (at_rows <= 1024)
-    float red[2 * kRowThreads / 32];
+    float red[2 * kThreads / 32];
     SumSmem sum;
 };
 
@@ -1961,7 +1955,7 @@ constexpr int kMomSlot16 = 3 * kMomGBytes / 16;  // 16-byte words per slot: 16 K
 struct MomRowSmem {
     uint4 buf[kMomStages][kMomSlot16];  // [G rows | M rows] per slot
     uint64_t full[kMomStages];
-    float part[kRowThreads / 32][8];
+    float part[kThreads / 32][8];
     float inv[32];
     int fail;
 };
@@ -2170,7 +2164,7 @@ struct MomApplySmem {
     uint4 buf[kMomStages][kMomSlot16];  // [W rows | M rows] per slot
     uint64_t full[kMomStages];
     float a[kRowChunks * 32];           // row scales a_i of the tile (at_rows <= 1024)
-    float red[2 * kRowThreads / 32];
+    float red[2 * kThreads / 32];
     SumSmem sum;
 };
 
@@ -2632,7 +2626,7 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
 // Above 4096 columns the column scales take 16 to 32 KB, and the ring's chunks are half as long.
 struct FlatSmem {
     uint64_t full[4];
-    float red[2 * kRowThreads / 32];
+    float red[2 * kThreads / 32];
     SumSmem sum;
     uint4 data[kFlatBytes / 16];  // the ring, then b_j [m] and a_i of the tile's rows
 };
@@ -2682,15 +2676,15 @@ __device__ bool apply_flat_body(const StepArgs &A, const TensorDev &T, int64_t r
     const Pol sp;
     const float *__restrict__ sb = F::scales(sm), *__restrict__ sa = sb + 8 * V;
     uint32_t row = tid / V, col = tid - row * V;  // of vector tid of the tile
-    const uint32_t dq = kRowThreads / V, dr = kRowThreads - dq * V;
+    const uint32_t dq = kThreads / V, dr = kThreads - dq * V;
     uint32_t st = 0, par = 0;
     for (uint32_t c = 0; c < nch; ++c) {
         const uint32_t cnt = min(kFlatChunk, total - c * kFlatChunk);
         const bool ok = mbar_wait(&sm.full[st], par);
         const uint4 *bw = sm.data + st * kSlot16, *by = bw + kFlatChunk;
 #pragma unroll
-        for (uint32_t k = 0; k < kFlatChunk / kRowThreads; ++k) {
-            const uint32_t f = k * kRowThreads + tid;
+        for (uint32_t k = 0; k < kFlatChunk / kThreads; ++k) {
+            const uint32_t f = k * kThreads + tid;
             if (f < cnt) {
                 const float a = sa[row];
                 const float4 b0 = *reinterpret_cast<const float4 *>(sb + 8 * col);
@@ -2779,12 +2773,12 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     float ma = 0.f, mb = 0.f;
     const float4 *bsc = reinterpret_cast<const float4 *>(T.bsc);  // (the stores may alias the descriptor)
     const float *R = T.R + r0;
-    for (uint32_t j = threadIdx.x; j < m / 4; j += kRowThreads) {
+    for (uint32_t j = threadIdx.x; j < m / 4; j += kThreads) {
         const float4 b = __ldcg(bsc + j);
         reinterpret_cast<float4 *>(ab)[j] = b;
         mb = fmaxf(fmaxf(mb, fmaxf(nan_to_inf(b.x), nan_to_inf(b.y))), fmaxf(nan_to_inf(b.z), nan_to_inf(b.w)));
     }
-    for (uint32_t r = threadIdx.x; r < rows_t; r += kRowThreads) {
+    for (uint32_t r = threadIdx.x; r < rows_t; r += kThreads) {
         const float a = row_scale(__ldcg(R + r), rbar_s, rbar_e);
         ab[m + r] = a;
         ma = fmaxf(ma, nan_to_inf(a));
@@ -2796,14 +2790,14 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
     }
     if ((threadIdx.x & 31) == 0) {
         sm.red[threadIdx.x >> 5] = ma;
-        sm.red[kRowThreads / 32 + (threadIdx.x >> 5)] = mb;
+        sm.red[kThreads / 32 + (threadIdx.x >> 5)] = mb;
     }
     __syncthreads();
     ma = mb = 0.f;
 #pragma unroll
-    for (int w = 0; w < kRowThreads / 32; ++w) {
+    for (int w = 0; w < kThreads / 32; ++w) {
         ma = fmaxf(ma, sm.red[w]);
-        mb = fmaxf(mb, sm.red[kRowThreads / 32 + w]);
+        mb = fmaxf(mb, sm.red[kThreads / 32 + w]);
     }
     const float coefC = __ldcg(&S.coefC);
     const bool sum = __ldcg(&S.fallback) == kSumInC;
@@ -3225,7 +3219,7 @@ __global__ void __launch_bounds__(kThreads, SKEW_MINB_SUMSQ)
 
 // Row path, phase A: one row tile per CTA (dynamic shared memory: RowSmem), and before them the
 // phase-A strip tiles and phase-B flat tiles.
-__global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
+__global__ void __launch_bounds__(kThreads, 2)
     k_rowsq(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
     RowSmem &sm = *reinterpret_cast<RowSmem *>(dyn_smem);
@@ -3260,18 +3254,18 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     if (T.momentum) {
         MomRowSmem &ms = *reinterpret_cast<MomRowSmem *>(dyn_smem);
         switch (T.m) {
-            case 4096: rowsq_mom_tile<kRowThreads, 512>(A, T, S, it.y, ms); break;
-            case 2048: rowsq_mom_tile<kRowThreads, 256>(A, T, S, it.y, ms); break;
-            case 1024: rowsq_mom_tile<kRowThreads, 128>(A, T, S, it.y, ms); break;
-            default: rowsq_mom_tile<kRowThreads, 64>(A, T, S, it.y, ms); break;  // 512
+            case 4096: rowsq_mom_tile<kThreads, 512>(A, T, S, it.y, ms); break;
+            case 2048: rowsq_mom_tile<kThreads, 256>(A, T, S, it.y, ms); break;
+            case 1024: rowsq_mom_tile<kThreads, 128>(A, T, S, it.y, ms); break;
+            default: rowsq_mom_tile<kThreads, 64>(A, T, S, it.y, ms); break;  // 512
         }
         return;
     }
     switch (T.m) {
-        case 4096: rowsq_tile<kRowThreads, 512>(A, T, S, it.y, sm); break;
-        case 2048: rowsq_tile<kRowThreads, 256>(A, T, S, it.y, sm); break;
-        case 1024: rowsq_tile<kRowThreads, 128>(A, T, S, it.y, sm); break;
-        default: rowsq_tile<kRowThreads, 64>(A, T, S, it.y, sm); break;  // 512
+        case 4096: rowsq_tile<kThreads, 512>(A, T, S, it.y, sm); break;
+        case 2048: rowsq_tile<kThreads, 256>(A, T, S, it.y, sm); break;
+        case 1024: rowsq_tile<kThreads, 128>(A, T, S, it.y, sm); break;
+        default: rowsq_tile<kThreads, 64>(A, T, S, it.y, sm); break;  // 512
     }
 }
 
@@ -3291,7 +3285,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 
 // Row path, phase C: one row tile per CTA (dynamic shared memory: ApplyRowSmem), and before them
 // the phase-C strip and flat tiles.
-__global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
+__global__ void __launch_bounds__(kThreads, 2)
     k_apply_rows(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
     extern __shared__ uint4 dyn_smem[];
     ApplyRowSmem &sm = *reinterpret_cast<ApplyRowSmem *>(dyn_smem);
@@ -3322,18 +3316,18 @@ __global__ void __launch_bounds__(kRowThreads, 512 / kRowThreads)
     if (T.momentum) {
         MomApplySmem &ms = *reinterpret_cast<MomApplySmem *>(dyn_smem);
         switch (T.m) {
-            case 4096: apply_rows_mom_tile<kRowThreads, 512>(A, T, S, it.y, ms); break;
-            case 2048: apply_rows_mom_tile<kRowThreads, 256>(A, T, S, it.y, ms); break;
-            case 1024: apply_rows_mom_tile<kRowThreads, 128>(A, T, S, it.y, ms); break;
-            default: apply_rows_mom_tile<kRowThreads, 64>(A, T, S, it.y, ms); break;  // 512
+            case 4096: apply_rows_mom_tile<kThreads, 512>(A, T, S, it.y, ms); break;
+            case 2048: apply_rows_mom_tile<kThreads, 256>(A, T, S, it.y, ms); break;
+            case 1024: apply_rows_mom_tile<kThreads, 128>(A, T, S, it.y, ms); break;
+            default: apply_rows_mom_tile<kThreads, 64>(A, T, S, it.y, ms); break;  // 512
         }
         return;
     }
     switch (T.m) {
-        case 4096: apply_rows_tile<kRowThreads, 512>(A, T, S, it.y, sm); break;
-        case 2048: apply_rows_tile<kRowThreads, 256>(A, T, S, it.y, sm); break;
-        case 1024: apply_rows_tile<kRowThreads, 128>(A, T, S, it.y, sm); break;
-        default: apply_rows_tile<kRowThreads, 64>(A, T, S, it.y, sm); break;  // 512
+        case 4096: apply_rows_tile<kThreads, 512>(A, T, S, it.y, sm); break;
+        case 2048: apply_rows_tile<kThreads, 256>(A, T, S, it.y, sm); break;
+        case 1024: apply_rows_tile<kThreads, 128>(A, T, S, it.y, sm); break;
+        default: apply_rows_tile<kThreads, 64>(A, T, S, it.y, sm); break;  // 512
     }
 }
 
@@ -3507,7 +3501,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
     if (rows) {
         constexpr size_t kSm = max3(sizeof(RowSmem), sizeof(MomRowSmem), sizeof(GenSmem<8>));
         run(cudaFuncSetAttribute(k_rowsq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm));
-        if (rA + L.nR > L.nRW) run(launch(k_rowsq, rA + L.nR - L.nRW, kRowThreads, kSm, s, A, past(L.itemsA, L.nA - rA)));
+        if (rA + L.nR > L.nRW) run(launch(k_rowsq, rA + L.nR - L.nRW, kThreads, kSm, s, A, past(L.itemsA, L.nA - rA)));
         constexpr size_t kWide = sizeof(GenSmem<16>);
         static_assert(kWide + 1024 <= 227 * 1024, "one CTA per SM");
         if (L.nRW) {
@@ -3532,7 +3526,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
         static_assert(2 * (kSm + 1024 + (sizeof(TensorDev) + 127) / 128 * 128) <= 228 * 1024, "two CTAs per SM");
         static_assert(sizeof(Meta) <= kSm && sizeof(Smem) <= kSm, "light tiles");
         run(cudaFuncSetAttribute(k_apply_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSm));
-        run(launch(k_apply_rows, rC + L.nCR, kRowThreads, kSm, s, A, past(L.itemsC, L.nC - rC)));
+        run(launch(k_apply_rows, rC + L.nCR, kThreads, kSm, s, A, past(L.itemsC, L.nC - rC)));
     }
     mark(7);
     return (int)e;

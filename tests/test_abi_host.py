@@ -68,6 +68,17 @@ def test_struct_layout_matches_header():
     assert got == want
 
 
+def test_cta_size_is_no_build_option():
+    """The row kernels run strip and flat tiles and share reductions that are laid out for 256 threads, so
+    no macro of the build changes their CTA size (the preprocessed source stays the same)."""
+    src = os.path.join(_build.CSRC, "skew_kernels.cu")
+
+    def expand(*macros):
+        return subprocess.check_output([_build.nvcc(), "-E", *_build.NVCC_FLAGS, *macros, src])
+
+    assert expand() == expand("-DSKEW_ROW_THREADS=512")
+
+
 def _descs(wl, base=0x100000):
     out = []
     for k, s in enumerate(wl.specs):
