@@ -3170,7 +3170,10 @@ __device__ void phase_C(const StepArgs &A, const TensorDev &T, const TensorScal 
 // The launches of a step are programmatic dependents of one another: a launch may start when every
 // CTA of the one before has, so that its launch latency (and the load of its item) passes while that
 // one ends, and it waits here, before it touches anything another launch writes, until that one is
-// complete and its writes are visible. Each launch waits, so completion is transitive. `items`: the
+// complete and its writes are visible. Each launch waits, so completion is transitive. A step's last launch
+// releases nothing: the next step begins with an ordinary launch, and a programmatic dependent of the caller's
+// would start while phase C still writes the weights (one that stamps its start and its wait's end: up to
+// 43 us apart behind 160M parameters). `items`: the
 // CTA's (tensor, tile) table, written at bind; null: tensor 0, tiles in order.
 // A step of 296K elements in 39 tensors 37 -> 28 us, 2048 x 1408 alone 43 -> 35, the 6.78B set 8357 -> 8322.
 __device__ __forceinline__ void wait_previous_launch() {
@@ -3184,10 +3187,12 @@ __device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepc
 // read before the wait; the no-alloc step, without tables, passes its descriptor as a parameter.
 // Against reading fields from L2: 24 ragged tensors 150 -> 135 us, a 432-wide model 69 -> 61, a 2048-wide
 // one 378 -> 369, the 6.78B set 8349 -> 8318.
-__device__ __forceinline__ uint2 begin_item(const uint2 *__restrict__ items, const StepArgs &A, TensorDev &td) {
+// `release`: another launch of the step follows.
+__device__ __forceinline__ uint2 begin_item(const uint2 *__restrict__ items, const StepArgs &A, TensorDev &td,
+                                            bool release = true) {
     constexpr uint32_t kWords = sizeof(TensorDev) / 4;
     static_assert(sizeof(TensorDev) % 4 == 0 && kWords <= kThreads, "one word per thread");
-    let_next_launch_start();
+    if (release) let_next_launch_start();
     const uint2 it = items ? items[blockIdx.x] : make_uint2(0u, blockIdx.x);
     if (threadIdx.x < kWords)
         reinterpret_cast<uint32_t *>(&td)[threadIdx.x] =
@@ -3290,7 +3295,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     extern __shared__ uint4 dyn_smem[];
     ApplyRowSmem &sm = *reinterpret_cast<ApplyRowSmem *>(dyn_smem);
     __shared__ TensorDev td;
-    const uint2 it = begin_item(items, A, td);
+    const uint2 it = begin_item(items, A, td, false);
     const TensorDev &T = td;
     TensorScal &S = A.scal[it.x];
     if (T.rowpath == kRowNone) {
@@ -3393,10 +3398,10 @@ __global__ void __launch_bounds__(kThreads, SKEW_MINB_RMS)
 }
 
 __global__ void __launch_bounds__(kThreads, SKEW_MINB_APPLY)
-    k_apply(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items) {
+    k_apply(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items, bool last) {
     __shared__ Meta meta;
     __shared__ TensorDev td;
-    const uint2 it = begin_item(items, A, td);
+    const uint2 it = begin_item(items, A, td, !last);
     phase_C(A, td, A.scal[it.x], it.y, meta, Pol());
 }
 
@@ -3519,7 +3524,7 @@ int launch_phases(const StepArgs &A, const LaunchPlan &L, void *stream, void *co
         run(launch(k_fallback, rB + L.nFB, kThreads, sizeof(FlatSmem), s, A, L.itemsB, rB));
     }
     mark(5);
-    if (L.nC > rC) run(launch(k_apply, L.nC, kThreads, 0, s, A, L.itemsC));
+    if (L.nC > rC) run(launch(k_apply, L.nC, kThreads, 0, s, A, L.itemsC, !rows));
     mark(6);
     if (rows) {
         constexpr size_t kSm = max3(sizeof(ApplyRowSmem), sizeof(MomApplySmem), sizeof(FlatSmem));
