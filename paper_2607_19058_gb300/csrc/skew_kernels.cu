@@ -1342,126 +1342,195 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
 // element and 32 rows per thread one after another (k_apply, 42829 x 58 bf16: 103 -> 17 us; 3467 x
 // 1072 fp32 with momentum: 45 -> 22; 24 ragged tensors of 13M elements in all: a step 215 -> 161).
 // ---------------------------------------------------------------------------
-struct FlatPos {
-    int64_t row, col;    // of element e0
-    int64_t dq, dr;      // one round of the CTA, 8 kThreads elements, in rows and columns
-    __device__ FlatPos(const TensorDev &T, int64_t e0) {
-        if (T.numel < (int64_t(1) << 31)) {  // 64-bit divides are long here
-            row = (uint32_t)e0 / (uint32_t)T.m;
-            dq = 8u * kThreads / (uint32_t)T.m;
-        } else {
-            row = e0 / T.m;
-            dq = (8 * kThreads) / T.m;
-        }
-        col = e0 - row * T.m;
-        dr = 8 * kThreads - dq * T.m;
+// The scales of a tile (a_i of its rows, b_j of its columns) stay in shared memory, and a round is one
+// vector per thread; FlatTile says which, FlatScales what its elements are scaled by. The b_j of columns 8
+// apart lie side by side, so that the lanes of a warp, 8 columns apart, read different banks: column k + s is at
+// [s][k / 8] for every k that is a multiple of 8 and s below 15, so that a vector from any column on
+// reads one word of 8 consecutive of these 15 lists, and 7 columns more than the tile has repeat the first, which
+// a vector may run on into. (With the b_j in column order every load was an 8-way bank conflict: a step of 28160 x
+// 4096 bf16 off a 16-byte boundary, converted beside its loads too, 926 us, 958 with momentum, and on strip tiles of
+// narrow loads 747 and 938; 624 and 690 so.)
+struct FlatVec {
+    int64_t e;  // its first element; at or past numel: none in this round
+    int r, j;   // row and column, from the tile's first
+};
+
+template <bool WIDE>
+struct FlatScales {
+    const float *a, *b;
+    int pitch;  // of the lists
+    int end;    // the column at which the next row begins
+    static constexpr int kLists = 15;
+    // room for `cols` + 7 columns, 4 words past a multiple of 32 (the lanes that fill the lists: different banks)
+    static __host__ __device__ constexpr int pitch_for(int cols) { return ((cols + 14) / 8 + 27) / 32 * 32 + 4; }
+    static __device__ __forceinline__ void put(float *pool, int pitch, int k, float bk) {
+        const int s = k & 7, q = k >> 3;
+        pool[s * pitch + q] = bk;
+        if (s < 7 && q > 0) pool[(s + 8) * pitch + q - 1] = bk;
     }
-    __device__ void next(int64_t m) {
-        row += dq;
-        col += dr;
-        if (col >= m) {
-            col -= m;
-            ++row;
+    // min(a_i b_j, 1/sqrt(eps)) of the vector's `valid` elements, some finite value past them
+    __device__ __forceinline__ void operator()(const FlatVec &v, int valid, float ce, float (&sc)[8]) const {
+        if (!WIDE && end < 8) {  // rows shorter than a vector: b_j in order
+            int r = v.r, j = v.j;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                sc[c] = c < valid ? fminf(a[r] * b[j], ce) : 0.f;
+                const bool wrap = ++j == end;
+                j = wrap ? 0 : j;
+                r += wrap;
+            }
+            return;
+        }
+        const float *p = b + (v.j & 7) * pitch + (v.j >> 3);
+        const int here = end - v.j;  // elements in this row
+        const float ar = a[v.r], an = here < valid ? a[v.r + 1] : 0.f;
+        if (!WIDE && end < 8 * 32) {  // a warp holds the end of a row
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sc[c] = fminf((c < here ? ar : an) * p[c * pitch], ce);
+            return;
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) sc[c] = fminf(ar * p[c * pitch], ce);
+        if (here < valid) {
+#pragma unroll
+            for (int c = 1; c < 8; ++c)
+                if (c >= here) sc[c] = fminf(an * p[c * pitch], ce);
         }
     }
 };
 
-// The scales of a flat tile: a_i of its rows, then b_j of all columns, in shared memory where they
-// fit (`in`; read from L2 by every thread, the few columns of a narrow matrix are one hot line).
-struct FlatMeta {
-    const float *a, *b;
-    int64_t row0;
-    float rbar_s;
-    int rbar_e;
-    bool in;
-    __device__ FlatMeta(const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta) {
-        const int64_t elems = int64_t(8 * kThreads) * T.fvpt, e0 = int64_t(tile) * elems;
-        const int64_t e1 = min(e0 + elems, T.numel) - 1, m = T.m;
-        const bool narrow = T.numel < (int64_t(1) << 31);  // 64-bit divides are long here
-        row0 = narrow ? (uint32_t)e0 / (uint32_t)m : e0 / m;
-        const int64_t rows = (narrow ? (uint32_t)e1 / (uint32_t)m : e1 / m) - row0 + 1;
-        rbar_s = __ldcg(&S.rbar_s);
-        rbar_e = __ldcg(&S.rbar_e);
-        float *pool = reinterpret_cast<float *>(&meta);
-        in = rows + m <= kSmemFloats + kStripCols;
-        a = pool;
-        b = pool + rows;
-        if (in) {
-            // (pointers held apart from the descriptor, which the stores to shared memory may alias)
-            const float *R = T.R + row0, *bsc = T.bsc;
-            for (int r = threadIdx.x; r < (int)rows; r += kThreads) pool[r] = row_scale(__ldcg(R + r), rbar_s, rbar_e);
-            for (int j = threadIdx.x; j < (int)m; j += kThreads) pool[rows + j] = __ldcg(bsc + j);
-            __syncthreads();
+// Matrices of at most kFlatCols columns: 2048 fvpt consecutive elements, and b_j of all columns.
+template <bool WIDE>
+struct FlatTile {
+    FlatScales<WIDE> scales;
+    int64_t e0;
+    int at, r, j;   // of the next round's vector: elements from e0, row, column
+    int dq, dr, m;  // one round of the CTA, 8 kThreads elements, in rows and columns
+    __device__ FlatTile(const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta) {
+        const int64_t elems = int64_t(8 * kThreads) * T.fvpt;
+        e0 = int64_t(tile) * elems;
+        const int count = (int)min(elems, T.numel - e0);
+        m = (int)T.m;
+        // (64-bit divides are long here)
+        const int64_t row0 = T.numel < (int64_t(1) << 31) ? (uint32_t)e0 / (uint32_t)m : e0 / m;
+        const int col0 = (int)(e0 - row0 * m), rows = (int)((uint32_t)(col0 + count - 1) / (uint32_t)m) + 1;
+        const float rbar_s = __ldcg(&S.rbar_s);
+        const int rbar_e = __ldcg(&S.rbar_e);
+        const int pitch = m < 8 ? 1 : FlatScales<WIDE>::pitch_for(m);
+        float *pool = reinterpret_cast<float *>(&meta), *pa = pool + FlatScales<WIDE>::kLists * pitch;
+        __builtin_assume(__isShared(pool));
+        scales = FlatScales<WIDE>{pa, pool, pitch, m};
+        // (pointers held apart from the descriptor, which the stores to shared memory may alias)
+        const float *R = T.R + row0, *bsc = T.bsc;
+        for (int k = threadIdx.x; k < rows; k += kThreads) pa[k] = row_scale(__ldcg(R + k), rbar_s, rbar_e);
+        for (int k = threadIdx.x; k < m; k += kThreads) {
+            const float bj = __ldcg(bsc + k);
+            FlatScales<WIDE>::put(pool, pitch, k, bj);
+            if (k < 7 && m >= 8) FlatScales<WIDE>::put(pool, pitch, m + k, bj);
         }
+        __syncthreads();
+        at = 8 * threadIdx.x;
+        r = (int)((uint32_t)(col0 + at) / (uint32_t)m);
+        j = col0 + at - r * m;
+        dq = 8 * kThreads / m;
+        dr = 8 * kThreads - dq * m;
     }
-    // min(a_i b_j, 1/sqrt(eps)) of the `valid` elements from (row, col) on
-    __device__ __forceinline__ void scales(const TensorDev &T, const FlatPos &P, int valid, float ce, float (&sc)[8]) const {
-        const int64_t m = T.m;
-        if (in) {
-            int r = (int)(P.row - row0), j = (int)P.col;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                sc[c] = c < valid ? fminf(a[r] * b[j], ce) : 0.f;
-                const bool wrap = ++j == (int)m;
-                j = wrap ? 0 : j;
-                r += wrap;
-            }
-        } else {
-            int64_t r = P.row, j = P.col;
-            float ar = row_scale(__ldcg(T.R + r), rbar_s, rbar_e);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                sc[c] = c < valid ? fminf(ar * __ldcg(T.bsc + j), ce) : 0.f;
-                if (++j == m) {
-                    j = 0;
-                    if (++r < T.n) ar = row_scale(__ldcg(T.R + r), rbar_s, rbar_e);
-                }
-            }
+    __device__ __forceinline__ FlatVec next() {
+        const FlatVec v{e0 + at, r, j};
+        at += 8 * kThreads;
+        r += dq;
+        j += dr;
+        if (j >= m) {
+            j -= m;
+            ++r;
         }
+        return v;
+    }
+};
+
+// Wider ones: kFlatStrip columns, 2 rows to a round, so that a tile needs kFlatStrip + 7 column
+// scales whatever the width. A vector starts at a multiple of 8 of the matrix and belongs to the strip that its
+// first element lies in; from the last strip it may run on into the next row. Reading every b_j from L2 instead
+// (tiles of consecutive elements), a step of 2295 x 50257 bf16 took 1400 us, 1433 with momentum, and on strip tiles
+// of narrow loads 925 and 1088; 461 and 557 so.
+template <>
+struct FlatTile<true> {
+    FlatScales<true> scales;
+    static constexpr int kLanes = kFlatStrip / 8, kRows = kThreads / kLanes;  // threads of a row; rows of a round
+    int64_t first, m, numel;  // the first element, in the strip, of the thread's row of the next round
+    int width, r, rows;       // columns of the strip; that row; rows of the tile
+    __device__ FlatTile(const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta) {
+        const uint32_t strips = (uint32_t)((T.m + kFlatStrip - 1) / kFlatStrip), rt = tile / strips;
+        const int64_t c0 = int64_t(tile - rt * strips) * kFlatStrip, i0 = int64_t(rt) * kRows * T.fvpt;
+        m = T.m;
+        numel = T.numel;
+        width = (int)min(m - c0, int64_t(kFlatStrip));
+        rows = (int)min(int64_t(kRows) * T.fvpt, T.n - i0);
+        r = (int)threadIdx.x / kLanes;
+        first = (i0 + r) * m + c0;
+        const float rbar_s = __ldcg(&S.rbar_s);
+        const int rbar_e = __ldcg(&S.rbar_e);
+        constexpr int kPitch = FlatScales<true>::pitch_for(kFlatStrip), kWords = FlatScales<true>::kLists * kPitch;
+        static_assert(kWords + kRows * kVecPerThread + 1 <= kSmemFloats && kRows * kVecPerThread < kThreads, "the scales fit");
+        float *pool = reinterpret_cast<float *>(&meta), *pa = pool + kWords;
+        __builtin_assume(__isShared(pool));
+        scales = FlatScales<true>{pa, pool, kPitch, (int)min(m - c0, int64_t(2 * kFlatStrip))};
+        const float *R = T.R + i0, *bsc = T.bsc;
+        // (and of the row that the tile's last vector may run into)
+        if (threadIdx.x <= rows && i0 + threadIdx.x < T.n) pa[threadIdx.x] = row_scale(__ldcg(R + threadIdx.x), rbar_s, rbar_e);
+        for (int k = threadIdx.x; k < width + 7; k += kThreads)
+            FlatScales<true>::put(pool, kPitch, k, __ldcg(bsc + (c0 + k < m ? c0 + k : c0 + k - m)));
+        __syncthreads();
+    }
+    __device__ __forceinline__ FlatVec next() {
+        const int j = (-(int)first & 7) + 8 * (int)(threadIdx.x % kLanes);  // from the strip's first column
+        const FlatVec v{r < rows && j < width ? first + j : numel, r, j};
+        first += kRows * m;
+        r += kRows;
+        return v;
     }
 };
 constexpr uint32_t kFlatAhead = 2;  // rounds of a flat tile whose loads are issued together
 
+template <bool WIDE>
 __device__ Acc2 rms_flat_tile(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
                               const Pol &pol) {
     const GScale gsc = grad_scale(A);
-    const FlatMeta F(T, S, tile, meta);
+    FlatTile<WIDE> F(T, S, tile, meta);
     Acc2 acc;
     const int64_t numel = T.numel;
-    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
-    FlatPos P(T, e0);
-    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
-        float y[kFlatAhead][8], mm[kFlatAhead][8];
-        FlatPos Q[kFlatAhead] = {P, P};
+    for (uint32_t k = 0; k < T.fvpt; k += kFlatAhead) {
+        Raw8 g[kFlatAhead];
+        float mm[kFlatAhead][8];
+        FlatVec Q[kFlatAhead];
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
-            const int64_t e = e0 + h * 8 * kThreads;
-            Q[h] = P;
+            Q[h] = F.next();
+            const int64_t e = Q[h].e;
             if (e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
+                load8_raw(T.g, T.f32, T.wal, e, valid, g[h], pol);
                 if (T.momentum) load_f8(T.M + e, T.sal, valid, mm[h]);
             }
-            P.next(T.m);
         }
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
-            const int64_t e = e0 + h * 8 * kThreads;
+            const int64_t e = Q[h].e;
             if (e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                float sc[8], u[8];
+                float y[8], sc[8], u[8];
+                values8(g[h], T.f32, y);
                 if (T.momentum) {
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) y[h][c] = fmaf(A.b1, mm[h][c], gsc.c1 * y[h][c]);
-                    store_f8(T.M + e, T.sal, valid, y[h]);
+                    for (int c = 0; c < 8; ++c) y[c] = fmaf(A.b1, mm[h][c], gsc.c1 * y[c]);
+                    store_f8(T.M + e, T.sal, valid, y);
                 }
-                F.scales(T, Q[h], valid, A.ce, sc);
+                F.scales(Q[h], valid, A.ce, sc);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) u[c] = c < valid ? y[h][c] * sc[c] : 0.f;
+                for (int c = 0; c < 8; ++c) u[c] = y[c] * sc[c];  // 0 past the end
                 acc.add(sumsq8(u));
             }
         }
-        e0 += kFlatAhead * 8 * kThreads;
     }
     return acc;
 }
@@ -1539,7 +1608,9 @@ __device__ void phase_B_strip(const StepArgs &A, const TensorDev &T, uint32_t t,
 }
 
 __device__ void phase_B_flat(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
-    finish_B(A, T, t, local, rms_flat_tile(A, T, A.scal[t], local, meta, pol), sm);
+    finish_B(A, T, t, local,
+             T.m > kFlatCols ? rms_flat_tile<true>(A, T, A.scal[t], local, meta, pol)
+                             : rms_flat_tile<false>(A, T, A.scal[t], local, meta, pol), sm);
 }
 
 __device__ void phase_B_fact(const StepArgs &A, const TensorDev &T, uint32_t t, uint32_t local, Smem &sm, Meta &meta, const Pol &pol) {
@@ -1678,45 +1749,50 @@ __device__ void apply_fact_tile(const StepArgs &A, const TensorDev &T, const Ten
     }
 }
 
+template <bool WIDE>
 __device__ void apply_flat_any(const StepArgs &A, const TensorDev &T, const TensorScal &S, uint32_t tile, Meta &meta,
                                const Pol &pol) {
-    const FlatMeta F(T, S, tile, meta);
+    FlatTile<WIDE> F(T, S, tile, meta);
     const float coefC = __ldcg(&S.coefC);
     const float wdf = T.decay ? A.wdf : 1.0f;
     const Dith d = dith_of(A, T);
     const int64_t numel = T.numel;
-    int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
-    FlatPos P(T, e0);
-    for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
-        float y[kFlatAhead][8], w[kFlatAhead][8];
-        FlatPos Q[kFlatAhead] = {P, P};
+    for (uint32_t k = 0; k < T.fvpt; k += kFlatAhead) {
+        Raw8 g[kFlatAhead], w[kFlatAhead];
+        float mm[kFlatAhead][8];
+        FlatVec Q[kFlatAhead];
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
-            const int64_t e = e0 + h * 8 * kThreads;
-            Q[h] = P;
+            Q[h] = F.next();
+            const int64_t e = Q[h].e;
             if (e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
                 if (T.momentum)
-                    load_f8(T.M + e, T.sal, valid, y[h]);
+                    load_f8(T.M + e, T.sal, valid, mm[h]);
                 else
-                    load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
-                load8_elem(T.w, T.f32, T.wal, e, valid, w[h], pol);
+                    load8_raw(T.g, T.f32, T.wal, e, valid, g[h], pol);
+                load8_raw(T.w, T.f32, T.wal, e, valid, w[h], pol);
             }
-            P.next(T.m);
         }
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
-            const int64_t e = e0 + h * 8 * kThreads;
+            const int64_t e = Q[h].e;
             if (e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                float sc[8], x[8];
-                F.scales(T, Q[h], valid, A.ce, sc);
+                float y[8], v[8], sc[8], x[8];
+                if (T.momentum) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[h][c] * sc[c], w[h][c] * wdf);
+                    for (int c = 0; c < 8; ++c) y[c] = mm[h][c];
+                } else {
+                    values8(g[h], T.f32, y);
+                }
+                values8(w[h], T.f32, v);
+                F.scales(Q[h], valid, A.ce, sc);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[c] * sc[c], v[c] * wdf);
                 store8_elem(T, d, e, valid, x, pol);
             }
         }
-        e0 += kFlatAhead * 8 * kThreads;
     }
 }
 
@@ -3175,7 +3251,10 @@ __device__ void phase_C(const StepArgs &A, const TensorDev &T, const TensorScal 
     if (T.kind != kKindFactored) {
         apply_full_tile(A, T, S, tile, pol);
     } else if (!T.vec) {
-        apply_flat_any(A, T, S, tile, meta, pol);
+        if (T.m > kFlatCols)
+            apply_flat_any<true>(A, T, S, tile, meta, pol);
+        else
+            apply_flat_any<false>(A, T, S, tile, meta, pol);
     } else {
         const bool fast = fill_meta(T, S, tile, A.ce, meta);
         if (T.momentum) {

@@ -143,9 +143,7 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     TileGeom most = plan_geometry(kind, momentum, wg_aligned, vec, false, n, m, numel, kWholeGroup, kWholeGroup);
     const bool any = most.rowpath == kRowAny;
     if (any) most = plan_geometry(kind, momentum, false, vec, false, n, m, numel, kWholeGroup, kWholeGroup);
-    TileGeom limit = most;
-    limit.nbc = limit.ntiles;
-    if (layout_of(limit, kind, n, m).bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
+    if (layout_of(most, kind, n, m).bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
     const AnyWidths w = m > kAnyNarrow ? any_widths(0, 2 * numel, 0, H.eps) : any_widths(2 * numel, 0, 0, H.eps);
     const bool on_rows = any ? (m > kAnyNarrow ? w.wide : w.narrow) : most.rowpath != kRowNone;
     TileGeom G = plan_geometry(kind, momentum, on_rows, vec, numel < kSmallStrip, n, m, numel, 2 * numel, 2 * numel);

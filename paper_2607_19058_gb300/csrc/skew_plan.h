@@ -30,6 +30,10 @@ constexpr int64_t kSmallStrip = int64_t(2 * 2 * 152) * 65536;
 constexpr int64_t kRideElems = int64_t(32) << 20;
 constexpr int kFlatVecPerThread = 4;
 constexpr int64_t kFlatTileElems = int64_t(kThreads) * kFlatVecPerThread * 8;
+// Flat tiles of factored tensors with at most kFlatCols columns: consecutive elements, the scales of all columns
+// and of the tile's rows in shared memory; of wider ones: kFlatStrip columns of 2 fvpt rows (as many elements).
+constexpr int64_t kFlatCols = 4096;
+constexpr int kFlatStrip = 1024;
 constexpr int kFinChunk = 256;  // rows / columns per finalize item
 
 // Row-tile path (phase A on whole rows, no phase B unless a clamp may bind):
@@ -263,10 +267,13 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
         }
         g.nbc = g.ntiles;
         if (!g.rowpath && !vec) {
-            // (big tiles of a narrow matrix would hold more rows than their scales have room for)
-            g.fvpt = (uint32_t)(small || (m < 64 && rest < kWholeGroup) ? kFlatVecPerThread : kVecPerThread);
+            // (big tiles of a narrow matrix would hold more rows than their scales have room for, below 8 columns
+            // at any rate)
+            g.fvpt = (uint32_t)(small || (m < 64 && rest < kWholeGroup) ? kFlatVecPerThread
+                                : m < 8                                 ? kFlatVecPerThread * m : kVecPerThread);
             const int64_t tile = int64_t(kThreads) * 8 * g.fvpt;
-            g.nbc = (uint32_t)((numel + tile - 1) / tile);
+            g.nbc = (uint32_t)(m > kFlatCols ? ((m + kFlatStrip - 1) / kFlatStrip) * ((n + 2 * g.fvpt - 1) / (2 * g.fvpt))
+                                             : (numel + tile - 1) / tile);
         }
     } else {
         // one round per thread spreads a small tensor over more CTAs

@@ -40,3 +40,22 @@ def test_flat_and_strip_tiles(many, hp):
     for t in (1, 2):
         h.step(t, seed=23 * t, **({"gscale": 0.37} if t == 2 else {}))
     h.close()
+
+
+@pytest.mark.parametrize("many", [False, True], ids=["few", "many"])
+@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05, clip_d=0.05)], ids=["eps1e-30", "clip"])
+def test_wide_flat_tiles(many, hp):
+    """More columns than a tile's shared memory has room for: tiles of 1024 columns by 8 or (many) 64 rows, whose
+    vectors straddle strips and rows; and the widest that need none. Last strips of 1, 7 and 1024 columns, one-row matrices, rows past a tile."""
+    import parity
+    shapes = [(5, 4095), (9, 4096), (7, 4097), (1, 8193), (5, 10241), (9, 10247), (66, 8450), (33, 50257), (4, 16384), (35, 9001)]
+    specs = [WL.Spec(f"{'eb'[t]}{n}x{m}{'f' if f else ''}", (n, m), (E, B)[t], expert=k % 8 if t == 0 else -1, fp32=f)
+             for k, (n, m) in enumerate(shapes) for t in (0, 1) for f in (False, True)]
+    specs += [WL.Spec("s3x5x8201", (3, 5, 8201), E), WL.Spec("s2x9x10243", (2, 9, 10243), B)]
+    misalign = tuple(range(0, len(specs), 3))
+    if many:  # tiles grow to 64 rows
+        specs.append(WL.Spec("e4100x8200", (4100, 8200), E, expert=0))
+    h = parity.Harness(WL.Workload("wide", specs, WL.HP(), "toy", steps=2), hp_override=hp, misalign=misalign)
+    for t in (1, 2):
+        h.step(t, seed=31 * t, **({"gscale": 0.37} if t == 2 else {}))
+    h.close()

@@ -53,10 +53,10 @@ def test_any_width_rows(shapes, hp):
     h.close()
 
 
-# (16.8M elements are what takes such a matrix to row tiles when it is alone; the last one's row sums
-# fill the no-alloc scratch)
+# (16.8M elements are what takes such a matrix to row tiles when it is alone; the row sums of 4124839 x 1
+# fill the no-alloc scratch; the last takes wide flat tiles)
 @pytest.mark.parametrize("shape,tier", [((700, 264), E), ((12001, 1408), E), ((5601, 3072), B), ((2400, 7128), E),
-                                        ((2051, 8192), B), ((4124839, 1), E)])
+                                        ((2051, 8192), B), ((4124839, 1), E), ((70, 10247), B)])
 def test_noalloc_matches_the_handle(shape, tier):
     torch.manual_seed(0)
     w0 = (torch.randn(shape, device="cuda") * 0.02).to(torch.bfloat16)
