@@ -2920,7 +2920,12 @@ struct SumRing {
     static constexpr uint32_t kChunk = MOM ? 512 : 1024, kSlot16 = 1024, kStages = 4;  // vectors; 16 KB slots
     static constexpr uint32_t kWords = kSlot16 * kStages;
 };
-constexpr int kSumScales = kFlatBytes / 4 - 4 * (int)SumRing<false>::kWords;
+// What k_fallback has read of the queue of such tensors.
+struct alignas(16) QueueSmem {
+    uint32_t id[kThreads], end[kThreads];  // queued tensors, and the tiles up to and with each
+    uint32_t warp[kThreads / 32];
+};
+constexpr int kSumScales = (kFlatBytes - (int)sizeof(QueueSmem)) / 4 - 4 * (int)SumRing<false>::kWords;
 static_assert(kSumScales >= kFlatWideScales && kSumScales >= 4096 + 128, "the planner's rows fit");
 
 template <bool MOM>
@@ -3444,6 +3449,31 @@ __global__ void __launch_bounds__(kThreads, 2)
 // (queued in A.fb): the CTAs of this grid share the phase-C tiles of all queued tensors, laid end to end
 // (starting every tensor at CTA 0 would give the first CTAs a tile of each small one). The first nB CTAs
 // run the phase-B strip and flat tiles of the other tensors.
+// A CTA reads the queue kThreads tensors at a time, one per thread, and finds its tiles among the running
+// sums of their tile counts: walking from tensor to tensor cost two dependent trips to L2 for each, which every
+// CTA paid (82 MiB of G, 121 of its matrices queued, no momentum: k_fallback 78 us so, 45 now, the step 171 and 138).
+// Loads queue entries [q0, q0 + kThreads) (ids and running tile counts); returns the tiles they hold.
+__device__ uint32_t load_queue(const StepArgs &A, uint32_t q0, uint32_t cnt, QueueSmem &qs) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint32_t t = 0, n = 0;
+    if (q0 + tid < cnt) {
+        t = __ldcg(A.fb + 1 + q0 + tid);
+        n = A.tensors ? __ldg(&A.tensors[t].atiles) : A.one.atiles;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t p = __shfl_up_sync(kAll, n, o);
+        if (lane >= o) n += p;
+    }
+    if (lane == 31) qs.warp[warp] = n;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) n += qs.warp[w];
+    qs.id[tid] = t;
+    qs.end[tid] = n;
+    __syncthreads();
+    return qs.end[kThreads - 1];
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
     k_fallback(const __grid_constant__ StepArgs A, const uint2 *__restrict__ items, uint32_t nB) {
     extern __shared__ uint4 dyn_smem[];
@@ -3464,20 +3494,30 @@ __global__ void __launch_bounds__(kThreads, 2)
     const uint32_t cnt = __ldcg(A.fb), ctas = gridDim.x - nB;
     if (!cnt) return;
     FlatSmem &sm = *reinterpret_cast<FlatSmem *>(dyn_smem);
+    QueueSmem &qs = *reinterpret_cast<QueueSmem *>(sm.data + (kFlatBytes - sizeof(QueueSmem)) / 16);  // past the scales
     if (threadIdx.x == 0) {
         for (uint32_t st = 0; st < 4; ++st) mbar_init(&sm.full[st], 1);
         fence_mbar_init();
     }
-    __syncthreads();
-    uint32_t tile = blockIdx.x - nB, turn = 0;  // of queued tensor q
-    for (uint32_t q = 0; q < cnt; ++q) {
-        const uint32_t t = __ldcg(A.fb + 1 + q);
-        const TensorDev &T = A.tensors ? A.tensors[t] : A.one;
-        const uint32_t nt = T.atiles;
-        for (; tile < nt; tile += ctas)
-            if (!(T.momentum ? sum_tile<true>(A, T, A.scal[t], tile, turn, sm) : sum_tile<false>(A, T, A.scal[t], tile, turn, sm)))
+    uint32_t tile = blockIdx.x - nB, turn = 0;  // of the tensors from queue entry q0 on
+    for (uint32_t q0 = 0; q0 < cnt; q0 += kThreads) {
+        const uint32_t total = load_queue(A, q0, cnt, qs);
+        for (; tile < total; tile += ctas) {
+            uint32_t k = 0;  // the first entry whose tiles go past this one
+#pragma unroll
+            for (uint32_t step = kThreads / 2; step; step >>= 1)
+                if (qs.end[k + step - 1] <= tile) k += step;
+            const uint32_t t = qs.id[k], local = tile - (k ? qs.end[k - 1] : 0u);
+            if (threadIdx.x < sizeof(TensorDev) / 4)
+                reinterpret_cast<uint32_t *>(&td)[threadIdx.x] =
+                    A.tensors ? __ldg(reinterpret_cast<const uint32_t *>(A.tensors + t) + threadIdx.x)
+                              : reinterpret_cast<const uint32_t *>(&A.one)[threadIdx.x];
+            __syncthreads();
+            TensorScal &S = A.scal[t];
+            if (!(td.momentum ? sum_tile<true>(A, td, S, local, turn, sm) : sum_tile<false>(A, td, S, local, turn, sm)))
                 return;
-        tile -= nt;
+        }
+        tile -= total;
     }
 }
 

@@ -33,3 +33,18 @@ def test_clamped_tensors(clip_d):
         assert (rep.clipped > 0) == (clip_d < 1.0)
     h.opt.sync_status()
     h.close()
+
+
+def test_more_queued_matrices_than_a_cta_reads_at_once():
+    """300 matrices whose update is clipped (d = 0.05), queued for phase B: k_fallback reads its queue 256 at a
+    time; one to five phase-C tiles each, with and without momentum, fixed and general widths, a stack."""
+    import parity
+    shapes = [(40, 512), (1100, 512), (70, 2048), (300, 776), (5, 4096), (600, 1032)]
+    specs = [WL.Spec(f"{'eb'[k % 2]}{k}", shapes[k % 6], (E, B)[k % 2], expert=k % 5 if k % 2 == 0 else -1) for k in range(240)]
+    specs.append(WL.Spec("s60x33x1024", (60, 33, 1024), E))
+    h = parity.Harness(WL.Workload("queue", specs, WL.HP(), "toy", steps=2),
+                       hp_override=dict(eps=1e-8, lr=3e-4, weight_decay=0.05, clip_d=0.05))
+    for t in (1, 2):
+        assert h.step(t, seed=7 * t).clipped > 256
+    h.opt.sync_status()
+    h.close()
