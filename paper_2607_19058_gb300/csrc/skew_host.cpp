@@ -106,12 +106,14 @@ static void resolve(int ndim, int tier, int policy, uint32_t flags, TPlan &p) {
 
 static bool wg_aligned(const TPlan &p) { return (((uintptr_t)p.w | (uintptr_t)p.g) & 15) == 0; }
 
+// Whether a factored tensor's row-vectors may be 16-byte accesses (the state buffer starts on a 256-byte boundary).
+static bool vectors(const TPlan &p) { return row_vectors(p.f32 != 0, wg_aligned(p), p.moff < 0 || p.moff % 4 == 0, p.m); }
+
 // Tile geometry (plan_geometry): strip tiles of (tile_rows rows) x (8*LC
 // columns) or flat tiles of kFlatTileElems elements, and for the row path whole-row tiles.
-static void geometry(TPlan &p, bool row_aligned, bool small, int64_t rest, int64_t rest_c) {
-    // the state buffer starts on a 256-byte boundary
-    const bool vec = row_vectors(p.f32 != 0, wg_aligned(p), p.moff < 0 || p.moff % 4 == 0, p.m);
-    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, small, p.n, p.m, p.numel, rest, rest_c);
+static void geometry(TPlan &p, bool row_aligned, bool ride, int64_t strip, int64_t rest, int64_t rest_c) {
+    const bool vec = vectors(p);
+    const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, ride, strip, p.n, p.m, p.numel, rest, rest_c);
     p.lcl = g.lcl;
     p.strips = g.strips;
     p.rowtiles = g.rowtiles;
@@ -195,7 +197,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
                 q.tid = (uint32_t)k;
                 q.base = (uint64_t)(e * p.numel);
                 q.f32 = (d.flags & SKEW_F_FP32) ? 1u : 0u;
-                geometry(q, row_aligned(q), false, kWholeGroup, kWholeGroup);  // which path
+                geometry(q, row_aligned(q), false, kWholeGroup, kWholeGroup, kWholeGroup);  // which path
                 if (q.rowpath == kRowAny) (q.m > kAnyNarrow ? any_wide : any_narrow) += 2 * q.numel;
                 if (q.rowpath == kRowFixed) fixed += 2 * q.numel;
                 h->t.push_back(q);
@@ -226,11 +228,13 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     // Tiles, now that the paths and the state's alignment are known: the row tiles by the bytes that
     // follow in each phase.
     const AnyWidths any = any_widths(any_narrow, any_wide, fixed, h->hp.eps);
-    int64_t rest = 0, light = 0, fact = 0;  // elements off the row path, and of factored tensors
+    int64_t rest = 0, light = 0, strip = 0;  // elements off the row path, and of factored tensors there
     for (TPlan &q : h->t) {
         if (q.rowpath == kRowAny && !(q.m > kAnyNarrow ? any.wide : any.narrow)) q.rowpath = kRowNone;
-        if (!q.rowpath) light += q.numel;
-        if (q.kind == kKindFactored) fact += q.numel;
+        if (!q.rowpath) {
+            light += q.numel;
+            if (q.kind == kKindFactored) strip += q.numel;
+        }
     }
     std::vector<int64_t> upto;  // bytes of G of the row-path matrices up to each (phase C starts with the last)
     try {
@@ -245,6 +249,7 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
         upto.push_back(sum += q.rowpath ? 2 * q.numel : 0);
         total += q.rowpath ? (q.momentum ? 4 : 2) * q.numel : 0;
     }
+    h->ride = sum > 0 && light <= kRideElems;
     const bool reverse = total > kKeepBytes;  // phase C's row tiles (in fewer bytes all stay in L2 anyway)
     for (size_t k = h->t.size(); k-- > 0;) {
         TPlan &q = h->t[k];
@@ -253,11 +258,10 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
             rest += 2 * q.numel;
             again += (q.momentum ? 4 : 2) * q.numel;
         }
-        geometry(q, row, fact < kSmallStrip, rest, reverse ? upto[k] : rest);
+        geometry(q, row, h->ride, strip, rest, reverse ? upto[k] : rest);
         q.keep = row && again <= kKeepBytes && total >= kKeepTotal;
         h->n_rowpath += row;
     }
-    h->ride = h->n_rowpath && light <= kRideElems;
 
     // a step of small tensors only: one launch
     h->small = plan_small(n_plans, [&](auto &&f) {

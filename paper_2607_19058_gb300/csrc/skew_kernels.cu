@@ -414,7 +414,7 @@ struct Meta {
     float red[2 * kThreads / 32];  // per-warp maxima of the row / column scales
 };
 
-// Geometry of a factored tile: LC lanes along a row, RG row groups, 16 rows per thread.
+// Geometry of a factored tile: LC lanes along a row, RG row groups, tile_rows / RG rows per thread.
 struct FactTile {
     uint32_t LC, RG, lane, rg, s, rt;
     int64_t col0, row0;
@@ -507,7 +507,7 @@ __device__ void sumsq_tile(const TensorDev &T, uint32_t tile, Smem &sm, const Po
     const int64_t n = T.n, m = T.m, row0 = F.row0, RG = F.RG, col0 = F.col0;
     const uint32_t LC = F.LC;
     const bool act = F.act, lane0 = F.lane == 0;
-    const int vpt = (int)(T.tile_rows / F.RG);  // rows per thread: 8 or kVecPerThread
+    const int vpt = (int)(T.tile_rows / F.RG);  // rows per thread (strip_rows)
     float col[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if constexpr (VEC) {
         constexpr int KCH = 8;  // row-vectors requested before the first is used

@@ -140,13 +140,13 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
     // full-sized strip tiles at the others; a matrix whose own tiles (as skew_step cuts it) need more
     // scratch than there is runs on those.
     const bool vec = row_vectors(f32, (((uintptr_t)weight | (uintptr_t)grad) & 15) == 0, ((uintptr_t)M & 15) == 0, m);
-    TileGeom most = plan_geometry(kind, momentum, wg_aligned, vec, false, n, m, numel, kWholeGroup, kWholeGroup);
+    TileGeom most = plan_geometry(kind, momentum, wg_aligned, vec, false, kWholeGroup, n, m, numel, kWholeGroup, kWholeGroup);
     const bool any = most.rowpath == kRowAny;
-    if (any) most = plan_geometry(kind, momentum, false, vec, false, n, m, numel, kWholeGroup, kWholeGroup);
+    if (any) most = plan_geometry(kind, momentum, false, vec, false, kWholeGroup, n, m, numel, kWholeGroup, kWholeGroup);
     if (layout_of(most, kind, n, m).bytes > SKEW_NOALLOC_SCRATCH_BYTES) return SKEW_ETOOBIG;  // too large for the fixed array
     const AnyWidths w = m > kAnyNarrow ? any_widths(0, 2 * numel, 0, H.eps) : any_widths(2 * numel, 0, 0, H.eps);
     const bool on_rows = any ? (m > kAnyNarrow ? w.wide : w.narrow) : most.rowpath != kRowNone;
-    TileGeom G = plan_geometry(kind, momentum, on_rows, vec, numel < kSmallStrip, n, m, numel, 2 * numel, 2 * numel);
+    TileGeom G = plan_geometry(kind, momentum, on_rows, vec, false, numel, n, m, numel, 2 * numel, 2 * numel);
     Layout o = layout_of(G, kind, n, m);
     if (o.bytes > SKEW_NOALLOC_SCRATCH_BYTES) {
         G = most;

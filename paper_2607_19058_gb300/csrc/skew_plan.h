@@ -11,19 +11,29 @@
 
 namespace skew {
 
-// Every kernel runs 256-thread CTAs; a thread owns 8 consecutive bf16 elements
-// (one 16-byte vector) of up to kVecPerThread rows (strip tiles: 64 Ki elements)
-// or of kFlatVecPerThread flat vectors (full-second-moment tiles: 8 Ki elements,
-// so that the router and the vectors, small, spread over many CTAs). Where a step's
-// strip-path matrices hold fewer than kSmallStrip elements, strip tiles have
-// kVecSmall rows per thread and flat tiles of factored tensors kFlatVecPerThread
-// vectors, else kVecPerThread of both: 608 full tiles fill two waves of two CTAs
-// per SM, and below that a tile's rounds, one after another, set the time (296K
-// elements in 39 tensors: a step 46 -> 37 us).
+// Every kernel runs 256-thread CTAs; a thread owns 8 consecutive elements (one 16-byte vector of bf16) of
+// strip_rows rows (strip tiles), of flat_rounds flat vectors (flat tiles of factored tensors), or of up to
+// kFlatVecPerThread (full-second-moment tiles: 8 Ki elements, so that the router and the vectors, small, spread
+// over many CTAs).
 constexpr int kThreads = 256;
 constexpr int kVecPerThread = 32;
-constexpr int kVecSmall = 8;
-constexpr int64_t kSmallStrip = int64_t(2 * 2 * 152) * 65536;
+constexpr int64_t kFullTile = int64_t(kThreads) * 8 * kVecPerThread;  // elements
+
+// Heights of the tiles of factored tensors off the row path, which hold `strip` elements in a step: where these
+// give an SM few tiles, a tile's rounds, one after another, set the time; where they give it many, the tiles' own
+// start and the partials they leave do. Measured at 8, 16 and 32 rows (4, 8, 16 and 32 rounds), one matrix without
+// momentum: 768 columns 4M elements 29 31 40 us, 8M 44 38 44, 13M 63 59 56, 26M 110 95 94; 4095 columns 2M 33 38 53 72,
+// 6M 63 60 63 85, 13M 113 94 98 96, 20M 164 139 135 149, 36M 271 218 189 178; 24 ragged tensors of 13M 114 102 113 125.
+// (`vec`: row-vectors of 16 bytes; the others' phase A, too, gains from more tiles. `ride`: in the launches of row
+// tiles, which fill what full tiles leave idle: 12M elements beside 60M, 16 and 8: 188 us, full 181; fp32 217 and 205.)
+inline int strip_rows(bool vec, bool ride, int64_t strip) {
+    return strip < (vec ? 76 : 38) * kFullTile ? 8 : strip < (ride ? 152 : 228) * kFullTile ? 16 : kVecPerThread;
+}
+inline int flat_rounds(bool ride, int64_t strip) {
+    return strip < 38 * kFullTile                     ? 4
+           : strip < (ride ? 152 : 228) * kFullTile   ? 8
+           : strip < (ride ? 152 : 456) * kFullTile   ? 16 : kVecPerThread;
+}
 // A step with row tiles runs its strip and flat tiles in their launches while these hold at most
 // kRideElems elements: more of them are faster in launches of their own, where four CTAs share an SM
 // (1.15B elements of 4864 and 7128 columns beside one 4095 x 1000 matrix: 2316 against 2586 us).
@@ -202,10 +212,10 @@ inline AnyWidths any_widths(int64_t narrow, int64_t wide, int64_t fixed, float e
 
 // `kind`, `momentum` as resolved by the tier policy; `wg_aligned`: weight and
 // gradient pointers are 16-byte aligned; `vec`: row-vectors may be 16-byte accesses (row_vectors);
-// `small`: the step's factored matrices hold fewer than kSmallStrip elements; `rest`, `rest_c`: bytes of G of the step's
+// `strip`: elements of the step's factored tensors off the row path, `ride`: whether in the row tiles' launches; `rest`, `rest_c`: bytes of G of the step's
 // row-path matrices from this one on in phase A's order and in phase C's. Counts fit 32 bits for n, m <= 2^40
 // and n*m <= 2^62 only when the caller has checked the tile count (planner).
-inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, bool vec, bool small, int64_t n,
+inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned, bool vec, bool ride, int64_t strip, int64_t n,
                               int64_t m, int64_t numel, int64_t rest, int64_t rest_c) {
     TileGeom g;
     if (kind == kKindFactored) {
@@ -216,7 +226,7 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
             ++g.lcl;
         }
         g.strips = (uint32_t)((m + 8 * lc - 1) / (8 * lc));
-        g.tile_rows = (uint32_t)((small ? kVecSmall : kVecPerThread) * (kThreads / lc));
+        g.tile_rows = (uint32_t)(strip_rows(vec, ride, strip) * (kThreads / lc));
         g.rowtiles = (uint32_t)((n + g.tile_rows - 1) / g.tile_rows);
         g.ntiles = g.strips * g.rowtiles;
         g.nfc = (uint32_t)((m + kFinChunk - 1) / kFinChunk);
@@ -267,10 +277,9 @@ inline TileGeom plan_geometry(uint32_t kind, uint32_t momentum, bool wg_aligned,
         }
         g.nbc = g.ntiles;
         if (!g.rowpath && !vec) {
-            // (big tiles of a narrow matrix would hold more rows than their scales have room for, below 8 columns
-            // at any rate)
-            g.fvpt = (uint32_t)(small || (m < 64 && rest < kWholeGroup) ? kFlatVecPerThread
-                                : m < 8                                 ? kFlatVecPerThread * m : kVecPerThread);
+            // (with more rounds a tile of a matrix of fewer than 8 columns has more rows than room for their scales)
+            g.fvpt = (uint32_t)flat_rounds(ride, strip);
+            if (m < 8 && g.fvpt > kFlatVecPerThread * m) g.fvpt = (uint32_t)(kFlatVecPerThread * m);
             const int64_t tile = int64_t(kThreads) * 8 * g.fvpt;
             g.nbc = (uint32_t)(m > kFlatCols ? ((m + kFlatStrip - 1) / kFlatStrip) * ((n + 2 * g.fvpt - 1) / (2 * g.fvpt))
                                              : (numel + tile - 1) / tile);
@@ -329,7 +338,7 @@ struct TensorDev {
     uint32_t lcl;       // factored: log2 of lanes along a row (LC)
     uint32_t strips;    // factored: column strips of 8*LC columns
     uint32_t rowtiles;  // factored: row tiles of tile_rows rows; full: flat tiles
-    uint32_t tile_rows; // factored: rows per tile = 32 * (256 / LC)
+    uint32_t tile_rows; // factored: rows per strip tile (strip_rows times its row groups)
     uint32_t ntiles;    // strip tiles (full: flat tiles) of this tensor
     uint32_t nbc, fvpt; // tiles of phases B and C; vectors per thread of a flat tile
     uint32_t nfr, nfc;  // factored: finalize items over rows / columns
@@ -447,13 +456,13 @@ inline SmallPlan plan_small(int64_t tensors, Each each) {
     while (c < 8 && tensors * c * 2 <= kSmallCtas &&
            !each([c](int64_t n, int64_t m) { return small_rows(n, 2 * c) * m < 4 * kSmallThreads; }))
         c *= 2;
-    P.ctas = c;
     int64_t most = 0;
     each([&](int64_t n, int64_t m) {
         const int64_t b = small_bytes(n, m, c);
         most = b > most ? b : most;
         return true;
     });
+    P.ctas = c;
     P.smem = size_t(most);
     return P;
 }

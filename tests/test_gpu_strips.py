@@ -59,3 +59,20 @@ def test_wide_flat_tiles(many, hp):
     for t in (1, 2):
         h.step(t, seed=31 * t, **({"gscale": 0.37} if t == 2 else {}))
     h.close()
+
+
+@pytest.mark.parametrize("rows", [10007, 50007, 166669, 300007])
+@pytest.mark.parametrize("hp", [{}, dict(eps=1e-8, lr=3e-4, weight_decay=0.05, clip_d=0.05)], ids=["eps1e-30", "clip"])
+def test_tile_heights(rows, hp):
+    """One matrix of 120 columns sets the step's strip elements (1.2M, 6M, 20M, 36M) and so the rows per strip tile (8,
+    16, 32, 32 of each thread) and the rounds of a flat tile (4, 8, 16, 32), for 16-byte row-vectors of 3 to 31
+    lanes a row and more, odd widths, fp32 and unaligned tensors beside it."""
+    import parity
+    shapes = [(1100, 24), (2100, 64), (257, 248), (300, 776), (33, 8200), (700, 7), (4100, 3), (129, 1001), (9, 4095), (70, 9001)]
+    specs = [WL.Spec(f"{'eb'[t]}{n}x{m}{'f' if f else ''}", (n, m), (E, B)[t], fp32=f)
+             for k, (n, m) in enumerate(shapes) for t, f in ((k % 2, False), (1 - k % 2, k % 3 == 0))]
+    specs.append(WL.Spec(f"e{rows}x120", (rows, 120), (E, B)[rows % 2]))
+    h = parity.Harness(WL.Workload("heights", specs, WL.HP(), "toy", steps=2), hp_override=hp, misalign=tuple(range(0, len(specs) - 1, 4)))
+    for t in (1, 2):
+        h.step(t, seed=37 * t, **({"gscale": 0.37} if t == 2 else {}))
+    h.close()
