@@ -264,7 +264,12 @@ int skew_create(const skew_param_desc_t *params, int32_t n_params, const skew_hp
     }
 
     // a step of small tensors only: one launch
-    h->small = plan_small(n_plans, [&](auto &&f) {
+    int64_t all_elems = 0, vec_elems = 0;
+    for (const TPlan &q : h->t) {
+        all_elems += q.numel;
+        if (q.kind == kKindFactored && vectors(q)) vec_elems += q.numel;
+    }
+    h->small = plan_small(n_plans, 2 * vec_elems > all_elems, [&](auto &&f) {
         for (const TPlan &q : h->t)
             if (!f(q.kind == kKindFactored ? q.n : q.numel, q.kind == kKindFactored ? q.m : 1)) return false;
         return true;

@@ -419,6 +419,7 @@ constexpr int kLaunches = 7;  // kernels a step may launch in turn
 constexpr int kSmallThreads = 512;
 constexpr size_t kSmallHeadBytes = 4096;                     // fixed part of its shared memory
 constexpr size_t kSmallSmem = 224 * 1024;                    // most that it takes
+constexpr size_t kSmallHalf = 112 * 1024;                    // up to which an SM holds two CTAs
 constexpr int64_t kSmallCtas = 256;                          // CTAs of a launch
 struct SmallPlan {
     uint32_t ctas = 0;  // 0: not a step for k_small
@@ -443,9 +444,13 @@ inline bool small_fits(int64_t n, int64_t m, uint32_t ctas) {
 
 // The rule: every tensor of the step fits, with at most kSmallCtas CTAs in all (two waves at one CTA per
 // SM, one at two): beyond, the strip tiles' four launches are as fast. Slices are then halved while that
-// holds: the toy MoE's 39 tensors take 21 us in clusters of two, 17 in clusters of four.
+// holds: the toy MoE's 39 tensors take 21 us in clusters of two, 17 in clusters of four. `vec`: matrices with 16-byte
+// row-vectors hold more than half of the elements. Their strip tiles are fast, so that slices too large for two CTAs
+// on an SM lose to them, unless one wave of small clusters holds all (48 matrices of 256 x 776 bf16 81 us so, 51 in
+// four launches; 16 of 640 x 640 79 and 35; 76 of 256 x 256, clusters of two, 30 and 30, with momentum 35 and 38).
+// Tensors without row-vectors gain up to the full room (64 of 256 x 776 fp32 86 and 94, 128 of 200 x 333 bf16 64 and 74).
 template <typename Each>
-inline SmallPlan plan_small(int64_t tensors, Each each) {
+inline SmallPlan plan_small(int64_t tensors, bool vec, Each each) {
     SmallPlan P;
     if (tensors < 1 || tensors > kSmallCtas) return P;
     auto fits = [&](uint32_t c) { return each([c](int64_t n, int64_t m) { return small_fits(n, m, c); }); };
@@ -462,6 +467,7 @@ inline SmallPlan plan_small(int64_t tensors, Each each) {
         most = b > most ? b : most;
         return true;
     });
+    if (vec && most > (int64_t)kSmallHalf && (c > 2 || tensors * c > 152)) return P;
     P.ctas = c;
     P.smem = size_t(most);
     return P;

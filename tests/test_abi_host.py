@@ -360,3 +360,28 @@ def test_random_plans_tile_the_state():
             S.skew_destroy(h)
 
     check()
+
+
+def _launches(specs):
+    """Launches of one step over [(shape, fp32, tier)], planned on fake pointers."""
+    descs = [_one(shape, tier=tier, weight=0x100000000 * (k + 1), grad=0x100000000 * (k + 1) + 0x80000000,
+                  flags=S.F_FP32 if f32 else 0) for k, (shape, f32, tier) in enumerate(specs)]
+    h = S.skew_create(descs, S.hparams())
+    n = S.skew_launches_per_step(h)
+    S.skew_destroy(h)
+    return n
+
+
+@pytest.mark.parametrize("specs,small", [
+    ([((256, 776), False, S.TIER_EXPERT)] * 32, True),     # clusters of eight, slices of 104 KB: two to an SM
+    ([((256, 776), False, S.TIER_EXPERT)] * 38, False),    # of four, 200 KB
+    ([((256, 256), False, S.TIER_EXPERT)] * 76, True),     # of two, 137 KB, one wave
+    ([((256, 256), False, S.TIER_EXPERT)] * 77, False),    # more than one
+    ([((640, 640), False, S.TIER_BACKBONE)] * 8, False),
+    ([((256, 776), True, S.TIER_EXPERT)] * 48, True),      # without row-vectors: as long as it fits
+    ([((200, 333), False, S.TIER_EXPERT)] * 128, True),
+    ([((256, 776), False, S.TIER_EXPERT)] * 48 + [((776,), True, S.TIER_BACKBONE)] * 4, False),
+    ([((256, 776), False, S.TIER_EXPERT)] * 4 + [((256, 776), True, S.TIER_EXPERT)] * 6, True),
+])
+def test_small_step_is_one_launch_where_its_slices_share_an_sm(specs, small):
+    assert (_launches(specs) == 1) == small
