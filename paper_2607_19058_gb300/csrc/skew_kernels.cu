@@ -1026,6 +1026,14 @@ __device__ void set_rbar(TensorScal &S, double rbar) {
     }
 }
 
+// The exponent of gamma (floor of its log2; 0 where that has no value), within an fp32 factor's range.
+__device__ __forceinline__ int gamma_exponent(float gam) {
+    if (!(gam > 0.f && gam < __int_as_float(0x7F800000))) return 0;
+    int e;
+    frexpf(gam, &e);
+    return min(max(e - 1, -126), 126);
+}
+
 // U = coef * y / D: a momentum-free tensor's y is g, so its coef carries gamma (M already does).
 __device__ __forceinline__ double update_coef(const StepArgs &A, const TensorDev &T) {
     return T.momentum ? A.coef_mom : A.coef_plain * (double)grad_scale(A).gam;
@@ -1092,6 +1100,11 @@ __device__ void phase_F_row(const StepArgs &A, const TensorDev &T, uint32_t t, u
                 }
         }
     }
+    // without momentum P_j grows with 1 / gamma^2, and P_j / C_j with more than that: P_j is taken times 2^2e for
+    // gamma's exponent e, which is exact, and the sum in fp64 divided by it (a gamma of 2^-45 overflowed, to a clip
+    // factor of 0)
+    const int ge = T.momentum ? 0 : gamma_exponent(grad_scale(A).gam);
+    const float pscale = __int_as_float((ge + 127) << 23);
     // the column's tpc parts in slice order
     float *red = sm.colred;  // [3][kFinChunk]: sum g^2, hi, lo
     red[threadIdx.x] = cs;
@@ -1115,7 +1128,7 @@ __device__ void phase_F_row(const StepArgs &A, const TensorDev &T, uint32_t t, u
         T.bsc[j] = __frsqrt_rn(Cn);
         if (P > 0.f) {
             if (Cn > 0.f && Cn < inf) {
-                contrib.add(__fdiv_rn(P, Cn));
+                contrib.add(__fdiv_rn(P * pscale * pscale, Cn));
                 cmin = Cn;
             } else {
                 atomicOr(&S.zflag, 1u);  // gradient in a column whose C_j is 0 or not finite
@@ -1191,12 +1204,14 @@ __device__ void phase_F_row(const StepArgs &A, const TensorDev &T, uint32_t t, u
         }
         const double rbar = rs * T.inv_n;
         set_rbar(S, rbar);
+        const double sum = fs * rbar * __hiloint2double((1023 - 2 * ge) << 20, 0);
         // max_i a_i^2 = Rbar / min R_i over rows with R_i > 0; max_j b_j^2 = 1 / min C_j over columns
         // holding gradient (0 without any). Multiplied out: fp64 divides are slow here.
         const bool some = rmn < inf && cmn < inf;
         const double ce2 = (double)A.ce * (double)A.ce;
-        if (__ldcg(&S.zflag) == 0u && (!some || rbar <= ce2 * (1.0 - 1e-6) * ((double)rmn * (double)cmn))) {
-            set_clip(A, T, S, fs * rbar);
+        // (a sum that overflowed fp32, from gradients of 1e-16 with a lower eps still: phase B or phase C adds it up)
+        if (__ldcg(&S.zflag) == 0u && isfinite(sum) && (!some || rbar <= ce2 * (1.0 - 1e-6) * ((double)rmn * (double)cmn))) {
+            set_clip(A, T, S, sum);
         } else {
             // A clamp may bind, and it only lowers |U|: no element is above its unclamped value or
             // coef |y| / sqrt(eps), so sum(U^2) is at most the bilinear sum, and (without momentum,
@@ -1205,7 +1220,7 @@ __device__ void phase_F_row(const StepArgs &A, const TensorDev &T, uint32_t t, u
             // whatever sum(U^2) is, and phase C, which forms every U anyway, adds it up: at the
             // paper's hyper-parameters (eps 1e-8 above most g^2) that saves every tensor's phase B,
             // 850M parameters 1724 -> 1205 us (phase B 572 us, the sums 32 us of phase C).
-            const double ub = T.momentum ? fs * rbar : fmin(fs * rbar, gs * ce2);
+            const double ub = T.momentum ? sum : fmin(sum, gs * ce2);
             const double coef = update_coef(A, T);
             if (__ldcg(&S.zflag) == 0u && ub * coef * coef * T.inv_numel <= (double)A.clip_d * (double)A.clip_d * (1.0 - 1e-4)) {
                 S.kappa = 1.0;

@@ -139,3 +139,56 @@ def test_grad_scale_adafactor_comparator():
         for t, g in ((1, 0.6), (2, 0.37), (3, 1.0)):
             h.step(t, seed=17 * t, gscale=g)
         h.close()
+
+
+def _steps_at(shapes, k, gamma, eps=1e-30, steps=2):
+    """Weights, state and scalars after steps on gradients scaled by 2^k, with the device scalar gamma."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    ps = []
+    for shape, tier in shapes:
+        w = torch.empty(shape, device="cuda").normal_(0, 0.02, generator=gen).to(torch.bfloat16)
+        ps.append((w, torch.empty_like(w), tier))
+    opt = S.SkewAdam(ps, S.hparams(eps=eps))
+    gs = torch.tensor([gamma], dtype=torch.float32, device="cuda")
+    for t in range(1, steps + 1):
+        for w, g, _ in ps:
+            g.copy_((torch.empty(g.shape, device="cuda").normal_(0, 1e-3, generator=gen).to(torch.bfloat16).double() * 2.0 ** k))
+        opt.step(t, 1e-3, 5, grad_scale=gs)
+    opt.sync_status()
+    sc = [opt.scalars(i) for i in range(len(ps))]
+    out = [w.view(torch.int16).clone() for w, _, _ in ps], opt.state.clone(), sc
+    opt.close()
+    return out
+
+
+E_, B_ = WL.TIER_EXPERT, WL.TIER_BACKBONE
+ROWS = {"to4096": [((300, 4096), E_), ((257, 2048), B_), ((1500, 4088), E_), ((1800, 3072), B_), ((1900, 1000), E_), ((1500, 2056), E_)],
+        "to8192": [((1100, 8192), E_), ((1200, 7128), B_)],
+        "strips": [((300, 1001), E_), ((40, 13), B_), ((3, 50001), E_)]}
+
+
+@pytest.mark.parametrize("name,k", [("to4096", 20), ("to4096", 45), ("to8192", 45), ("strips", 45)])
+def test_tiny_grad_scale_is_exact(name, k):
+    """Gradients 2^k times as large with gamma = 2^-k are the same gradients: every product with a power of
+    two is exact, so weights, state and scalars are the same bits (a gradient norm of 2^45 clipped to 1)."""
+    (w0, s0, c0), (w1, s1, c1) = _steps_at(ROWS[name], 0, 1.0), _steps_at(ROWS[name], k, 2.0 ** -k)
+    assert torch.equal(s0, s1)
+    assert c0 == c1
+    assert all(torch.equal(a, b) for a, b in zip(w0, w1))
+
+
+@pytest.mark.parametrize("name", ["to4096", "to8192", "strips"])
+def test_tiny_gradients_are_clipped_alike(name):
+    """Gradients of 1e-3 and 2^-40 times that, neither near eps = 1e-38 (V is 1e-9 and 1e-33): the update does not
+    depend on the gradient's scale. The sum of U^2 may be formed in another order: RMS and clip factor to 1e-6, so
+    at a rounding threshold a weight moves by one ulp (2^-7 of it), or where the update cancels the weight by 1e-6 of
+    the terms of x, |w| below 0.15 and lr |U| with |U| below 20; fewer than 1e-4 of them."""
+    (w0, _, c0), (w1, _, c1) = _steps_at(ROWS[name], 0, 1.0, 1e-38), _steps_at(ROWS[name], -40, 1.0, 1e-38)
+    for a, b in zip(c0, c1):
+        assert a["rms"] == pytest.approx(b["rms"], rel=1e-6) and a["kappa"] == pytest.approx(b["kappa"], rel=1e-6)
+    for a, b in zip(w0, w1):
+        a, b = a.view(torch.bfloat16).float(), b.view(torch.bfloat16).float()
+        d = (a - b).abs()
+        assert (d <= 2.0 ** -7 * a.abs() + 1e-6 * (0.15 + 1e-3 * 20)).all()
+        assert int((d > 0).sum()) <= 1e-4 * d.numel() + 1
