@@ -183,8 +183,9 @@ def test_tiny_gradients_are_clipped_alike(name):
     """Gradients of 1e-3 and 2^-40 times that, neither near eps = 1e-38 (V is 1e-9 and 1e-33): the update does not
     depend on the gradient's scale. The sum of U^2 may be formed in another order: RMS and clip factor to 1e-6, so
     at a rounding threshold a weight moves by one ulp (2^-7 of it), or where the update cancels the weight by 1e-6 of
-    the terms of x, |w| below 0.15 and lr |U| with |U| below 20; fewer than 1e-4 of them."""
-    (w0, _, c0), (w1, _, c1) = _steps_at(ROWS[name], 0, 1.0, 1e-38), _steps_at(ROWS[name], -40, 1.0, 1e-38)
+    the terms of x, |w| below 0.15 and lr |U| with |U| below 20; fewer than 1e-4 of them. (One step: a second would
+    start from the moved weights.)"""
+    (w0, _, c0), (w1, _, c1) = (_steps_at(ROWS[name], k, 1.0, 1e-38, steps=1) for k in (0, -40))
     for a, b in zip(c0, c1):
         assert a["rms"] == pytest.approx(b["rms"], rel=1e-6) and a["kappa"] == pytest.approx(b["kappa"], rel=1e-6)
     for a, b in zip(w0, w1):
