@@ -2518,7 +2518,10 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
     }
     const uint32_t kr = tid / rpp, w0 = (tid - kr * rpp) * wpr;  // threads < cr: chunk row tid is k = kr of row-in-pass tid % rpp
     const GScale gsc = grad_scale(A);
-    const float b2 = A.b2, c2m = __fdiv_rn(gsc.c2, (float)m);
+    // c2 / m, without a step into the subnormals that c2 itself does not take (a tiny gamma): c2 over m times kLead, at
+    // most 2, and the row's sum times kLead
+    constexpr float kLead = W == 16 ? 1.f / 4096.f : NV == 2 ? 1.f / 2048.f : 1.f / 1024.f;
+    const float b2 = A.b2, c2m = __fdiv_rn(gsc.c2, (float)m * kLead);
     const float2 b12 = make_float2(A.b1, A.b1), c12 = make_float2(gsc.c1, gsc.c1);
     // per column pair: sums of g^2, the compensated (hi, lo) sum of y^2 / R_i (y = g, or the new
     // M with momentum) and its open fp32 part
@@ -2597,7 +2600,7 @@ __device__ void rowsq_gen_tile(const StepArgs &A, const TensorDev &T, TensorScal
                 for (int w = 0; w < W / 2; ++w)
                     if (w < h) p[w] += p[w + h];
             sum = p[0];
-            Rn = fmaf(b2, rold, c2m * sum);  // c2m = c2 / m, rounded once
+            Rn = fmaf(b2, rold, c2m * (sum * kLead));  // c2 / m, rounded once
             sm.inv[tid] = Rn > 0.f && Rn < inf ? __frcp_rn(Rn) : 0.f;
         }
         __syncthreads();
