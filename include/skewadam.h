@@ -349,8 +349,9 @@ int skew_noalloc_sync_status(void *stream);
 int skew_noalloc_selftest_wait_timeout(void *stream);
 
 /*
- * Kernel launches one skew_step performs (its grouped launches over item
- * tables; 0 for NULL or an empty handle).
+ * Kernel launches one skew_step performs: the one that clears the per-step
+ * scalars and the grouped launches over item tables, or the single launch of a
+ * step of small tensors; 0 for NULL or an empty handle.
  */
 int64_t skew_launches_per_step(const skew_handle_t *h);
 

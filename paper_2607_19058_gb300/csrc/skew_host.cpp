@@ -382,9 +382,10 @@ int32_t skew_num_tensors(const skew_handle_t *h) { return h ? (int32_t)h->desc.s
 int64_t skew_launches_per_step(const skew_handle_t *h) {
     if (!h) return 0;
     if (h->small.ctas) return 1;
-    // with row tiles k_rowsq, k_fallback and k_apply_rows; the others where they have items of their own
+    if (h->t.empty()) return 0;
+    // k_reset; with row tiles k_rowsq, k_fallback and k_apply_rows; the others where they have items of their own
     const uint32_t rows = h->n_rowpath > 0, rA = h->ride ? h->nA : 0;
-    return 2 * rows + int64_t(rA + (h->itemsA.size() - h->nA) > h->nRW) + int64_t(h->nRW > 0) + int64_t(!h->itemsF.empty()) +
+    return 1 + 2 * rows + int64_t(rA + (h->itemsA.size() - h->nA) > h->nRW) + int64_t(h->nRW > 0) + int64_t(!h->itemsF.empty()) +
            (h->ride ? 0 : int64_t(h->nA > 0) + int64_t(!h->itemsB.empty()) + int64_t(h->nC > 0));
 }
 

@@ -385,3 +385,18 @@ def _launches(specs):
 ])
 def test_small_step_is_one_launch_where_its_slices_share_an_sm(specs, small):
     assert (_launches(specs) == 1) == small
+
+
+@pytest.mark.parametrize("specs,launches", [
+    ([], 0),
+    ([((64, 128), False, S.TIER_EXPERT)], 1),                              # k_small
+    ([((9000, 64), False, S.TIER_EXPERT)] * 8, 5),                         # k_reset, k_sumsq, k_finalize, k_rms, k_apply
+    ([((1 << 20,), False, S.TIER_BACKBONE)], 3),                           # a vector: k_reset, k_rms, k_apply
+    ([((4096, 4096), False, S.TIER_EXPERT)], 5),                           # k_reset, k_rowsq, k_finalize, k_fallback, k_apply_rows
+    ([((4096, 4096), False, S.TIER_EXPERT), ((999, 333), False, S.TIER_BACKBONE)], 5),    # the strips ride along
+    ([((4096, 4096), False, S.TIER_EXPERT), ((40000, 1001), False, S.TIER_BACKBONE)], 8),  # too many of them to
+    ([((8000, 5632), False, S.TIER_EXPERT)], 5),                           # k_rowsq_wide in k_rowsq's place
+    ([((4096, 4096), False, S.TIER_EXPERT), ((8000, 5632), False, S.TIER_EXPERT)], 6),
+])
+def test_launches_per_step_counts_every_kernel(specs, launches):
+    assert _launches(specs) == launches
