@@ -147,16 +147,10 @@ def byte_model(opt, n_tensors):
     """Algorithmic minimum bytes of one step and of each kernel's own traffic."""
     N = N_mom = N_full = N_fact = N_nomom = N_row = N_rowm = 0
     rc = rc_row = 0
+    from paper_2607_19058_gb300 import skewadam as S
     infos = [opt.info(k) for k in range(n_tensors)]
-    # whole-row tiles: the fixed widths, and any multiple of 8 from 128 to 4096 where these all hold
-    # 32 MiB of gradient or more, to 8192 where those above 4096 hold 64 MiB (32 without other row tiles)
-    def other(lo, hi):
-        return 2 * sum(i.numel for i in infos if i.kind == 1 and not i.rowpath and i.vectorized and lo <= i.cols <= hi)
-
-    narrow, wide, fixed = other(128, 4096), other(4097, 8192), 2 * sum(i.numel for i in infos if i.rowpath)
-    wide_rows = wide >= 64 << 20 or (not fixed and narrow < 32 << 20 <= wide)
-    narrow_rows = narrow > 0 and (narrow + fixed >= 32 << 20 or wide_rows)
-    for i in infos:
+    routes = [opt.route(k) for k in range(n_tensors)]
+    for i, route in zip(infos, routes):
         E = max(1, i.stack)  # a stack of E matrices: rows / cols are one matrix's
         N += i.numel
         if i.momentum:
@@ -165,7 +159,7 @@ def byte_model(opt, n_tensors):
             N_nomom += i.numel
         if i.kind == 0:
             N_full += i.numel
-        elif i.rowpath or (i.vectorized and ((narrow_rows and 128 <= i.cols <= 4096) or (wide_rows and 4096 < i.cols <= 8192))):
+        elif route == S.ROUTE_ROWS:
             N_row += i.numel
             N_rowm += i.numel if i.momentum else 0
             rc_row += E * (i.rows + i.cols)
@@ -180,17 +174,19 @@ def byte_model(opt, n_tensors):
     rms_full = 2 * N_full + 8 * mom_full + 8 * N_full             # read G; M, v read + write
     rms_fact = 2 * N_fact + 8 * (mom_rest - mom_full)
     apply = 4 * N_rest + 2 * (N_nomom - (N_row - N_rowm)) + 4 * mom_rest + 4 * N_full
-    rows = N_row > 0  # the row path's launches then run the strip and flat tiles too
+    ride = S.ROUTE_RIDING in routes  # the strip and flat tiles run in the row path's launches
     kernels = {
-        "k_sumsq": 0 if rows else sumsq,
+        "k_sumsq": 0 if ride else sumsq,
         # read G (and M r/w) of row-path matrices; R r/w
-        "k_rowsq": 2 * N_row + 8 * N_rowm + 8 * rc_row + (sumsq + rms_full if rows else 0),
+        "k_rowsq": 2 * N_row + 8 * N_rowm + 8 * rc_row + (sumsq + rms_full if ride else 0),
         "k_finalize": 8 * (rc + rc_row),                         # R, C read + write
-        "k_rms": 0 if rows else rms_full + rms_fact,
-        "k_fallback": rms_fact if rows else 0,                    # and phase B of queued row-path tensors
-        "k_apply": 0 if rows else apply,
-        "k_apply_rows": 6 * N_row - 2 * N_rowm + 4 * N_rowm + (apply if rows else 0),  # W r/w and G (or the new M) read
+        "k_rms": 0 if ride else rms_full + rms_fact,
+        "k_fallback": rms_fact if ride else 0,                    # and phase B of queued row-path tensors
+        "k_apply": 0 if ride else apply,
+        "k_apply_rows": 6 * N_row - 2 * N_rowm + 4 * N_rowm + (apply if ride else 0),  # W r/w and G (or the new M) read
     }
+    if S.ROUTE_SMALL in routes:  # one launch, timed in the last place: G, M, v and R, C once, W r/w
+        kernels = {name: 0 for name in kernels} | {"k_apply_rows": step_min}
     return dict(N=N, N_mom=N_mom, N_full=N_full, rc=rc, step_min=step_min, kernels=kernels)
 
 

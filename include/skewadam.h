@@ -150,7 +150,7 @@ typedef struct {
     int64_t rows, cols, numel;
     int64_t m_offset, v_offset, r_offset, c_offset;
     int32_t rowpath;    /* 1 at the widths 512, 1024, 2048 and 4096 (bf16, 16-byte */
-                        /* aligned), whose phase A always runs on whole rows       */
+                        /* aligned); what a step runs on: skew_tensor_route        */
     int32_t stack;      /* matrices of a stacked tensor (ndim 3), else 0; then   */
                         /* rows / cols are one matrix's, numel the whole stack's, */
                         /* and each state array holds the E matrices' in order   */
@@ -264,6 +264,17 @@ int skew_matrix_scalars(skew_handle_t *h, int32_t tid, int32_t e, double out[4],
 
 /* Resolved policy and state offsets of tensor `tid`. Errors: SKEW_EINVAL. */
 int skew_tensor_info(const skew_handle_t *h, int32_t tid, skew_tensor_info_t *out);
+
+/*
+ * Which launches step tensor `tid` (every matrix of a stack alike), as skew_create
+ * planned them: a SKEW_ROUTE_* value, or SKEW_EINVAL. Inspection, tests and byte
+ * accounting; results do not depend on it beyond the summation order.
+ */
+#define SKEW_ROUTE_OWN 0    /* strip or flat tiles: k_sumsq, k_finalize, k_rms, k_apply              */
+#define SKEW_ROUTE_RIDING 1 /* the same tiles in the row tiles' launches                            */
+#define SKEW_ROUTE_ROWS 2   /* whole-row tiles: k_rowsq, k_finalize, k_fallback, k_apply_rows        */
+#define SKEW_ROUTE_SMALL 3  /* the whole step is one launch, k_small                                 */
+int skew_tensor_route(const skew_handle_t *h, int32_t tid);
 
 /*
  * Benchmark support: launch timing. After skew_profile_begin(h, n), each of the

@@ -411,6 +411,12 @@ int skew_tensor_info(const skew_handle_t *h, int32_t tid, skew_tensor_info_t *ou
     return SKEW_OK;
 }
 
+int skew_tensor_route(const skew_handle_t *h, int32_t tid) {
+    if (!h || tid < 0 || tid >= (int32_t)h->desc.size()) return SKEW_EINVAL;
+    if (h->small.ctas) return SKEW_ROUTE_SMALL;
+    return h->t[h->first[tid]].rowpath ? SKEW_ROUTE_ROWS : h->ride ? SKEW_ROUTE_RIDING : SKEW_ROUTE_OWN;
+}
+
 int skew_bind(skew_handle_t *h, void *state, size_t state_bytes, void *workspace, size_t workspace_bytes, void *stream) {
     if (!h) return SKEW_EINVAL;
     if (state_bytes != h->state_bytes) return fail(h, SKEW_EINVAL, "state buffer is %zu bytes, need exactly %zu", state_bytes, h->state_bytes);

@@ -25,12 +25,13 @@ POLICY_TIERED, POLICY_EXPERT_MOMENTUM, POLICY_FACTORED_ROUTER, POLICY_UNIFORM, P
 F_NO_DECAY = 1
 F_FP32 = 2
 KIND_FULL, KIND_FACTORED = 0, 1
+ROUTE_OWN, ROUTE_RIDING, ROUTE_ROWS, ROUTE_SMALL = 0, 1, 2, 3
 
 EXPORTS = ["skew_create", "skew_destroy", "skew_state_bytes", "skew_workspace_bytes", "skew_bind", "skew_step",
            "skew_sync_status", "skew_tensor_scalars", "skew_matrix_scalars", "skew_tensor_info", "skew_num_tensors", "skew_last_error",
            "skew_profile_begin", "skew_profile_end", "skew_kernel_name", "skew_step_tensor_noalloc",
            "skew_launches_per_step", "skew_selftest_wait_timeout", "skew_noalloc_sync_status", "skew_step_scaled",
-           "skew_noalloc_selftest_wait_timeout"]
+           "skew_noalloc_selftest_wait_timeout", "skew_tensor_route"]
 
 
 class SkewError(RuntimeError):
@@ -96,6 +97,8 @@ def load(path: Optional[str] = None) -> C.CDLL:
         L.skew_matrix_scalars.restype = C.c_int
         L.skew_tensor_info.argtypes = [vp, i32, C.POINTER(TensorInfo)]
         L.skew_tensor_info.restype = C.c_int
+        L.skew_tensor_route.argtypes = [vp, i32]
+        L.skew_tensor_route.restype = C.c_int
         L.skew_launches_per_step.argtypes = [vp]
         L.skew_launches_per_step.restype = i64
         L.skew_num_tensors.argtypes = [vp]
@@ -185,6 +188,14 @@ def skew_tensor_info(h, tid: int) -> TensorInfo:
     info = TensorInfo()
     _check(load().skew_tensor_info(h, tid, C.byref(info)), h)
     return info
+
+
+def skew_tensor_route(h, tid: int) -> int:
+    """ROUTE_*: which launches step the tensor."""
+    r = load().skew_tensor_route(h, tid)
+    if r < 0:
+        raise SkewError(r, f"tensor {tid} out of range")
+    return r
 
 
 def skew_launches_per_step(h) -> int:
@@ -328,6 +339,9 @@ class SkewAdam:
 
     def info(self, tid: int) -> TensorInfo:
         return skew_tensor_info(self.h, tid)
+
+    def route(self, tid: int) -> int:
+        return skew_tensor_route(self.h, tid)
 
     def state_views(self, tid: int):
         """fp32 views (M, v, R, C; None when absent) into the state buffer."""

@@ -400,3 +400,59 @@ def test_small_step_is_one_launch_where_its_slices_share_an_sm(specs, small):
 ])
 def test_launches_per_step_counts_every_kernel(specs, launches):
     assert _launches(specs) == launches
+
+
+R_OWN, R_RIDE, R_ROWS, R_SMALL = S.ROUTE_OWN, S.ROUTE_RIDING, S.ROUTE_ROWS, S.ROUTE_SMALL
+
+
+@pytest.mark.parametrize("specs,eps,routes", [
+    ([((64, 128), False, S.TIER_EXPERT)] * 2, 1e-30, [R_SMALL] * 2),
+    ([((4096, 4096), False, S.TIER_EXPERT), ((4096, 4096), True, S.TIER_EXPERT), ((999, 333), False, S.TIER_EXPERT),
+      ((4096,), True, S.TIER_BACKBONE)], 1e-30, [R_ROWS, R_RIDE, R_RIDE, R_RIDE]),
+    ([((4096, 4096), False, S.TIER_EXPERT), ((40000, 1001), False, S.TIER_EXPERT)], 1e-30, [R_ROWS, R_OWN]),
+    # other widths take row tiles from 32 MiB of gradient on, 64 where eps may bind, beside fixed widths' 32 always
+    ([((12000, 1408), False, S.TIER_EXPERT)], 1e-30, [R_ROWS]),
+    ([((11000, 1408), False, S.TIER_EXPERT)], 1e-30, [R_OWN]),
+    ([((12000, 1408), False, S.TIER_EXPERT)], 1e-8, [R_OWN]),
+    ([((24000, 1408), False, S.TIER_EXPERT)], 1e-8, [R_ROWS]),
+    ([((1000, 1408), False, S.TIER_EXPERT), ((4096, 4096), False, S.TIER_EXPERT)], 1e-8, [R_ROWS, R_ROWS]),
+    ([((3, 4200, 1408), False, S.TIER_EXPERT), ((3000, 104), False, S.TIER_EXPERT)], 1e-30, [R_ROWS, R_RIDE]),
+    # above 4096 columns, 64 MiB beside other row tiles
+    ([((3000, 5632), False, S.TIER_EXPERT)], 1e-30, [R_ROWS]),
+    ([((3000, 5632), False, S.TIER_EXPERT), ((4096, 4096), False, S.TIER_EXPERT)], 1e-30, [R_RIDE, R_ROWS]),
+    ([((6000, 5632), False, S.TIER_EXPERT), ((4096, 4096), False, S.TIER_EXPERT)], 1e-30, [R_ROWS, R_ROWS]),
+    ([((3000, 8200), False, S.TIER_EXPERT)], 1e-30, [R_OWN]),
+])
+def test_tensor_route(specs, eps, routes):
+    descs = [_one(shape, tier=tier, weight=0x100000000 * (k + 1), grad=0x100000000 * (k + 1) + 0x80000000,
+                  flags=S.F_FP32 if f32 else 0) for k, (shape, f32, tier) in enumerate(specs)]
+    h = S.skew_create(descs, S.hparams(eps=eps))
+    assert [S.skew_tensor_route(h, k) for k in range(len(specs))] == routes
+    with pytest.raises(S.SkewError):
+        S.skew_tensor_route(h, len(specs))
+    S.skew_destroy(h)
+
+
+@pytest.mark.parametrize("eps", [1e-30, 1e-8])
+def test_bench_byte_model_follows_the_routes(eps):
+    """A kernel's bytes are 0 where it does not run: 16M elements of 1408 columns are row tiles unless eps may bind;
+    small tensors are one launch, whose bytes are the step's."""
+    import bench
+
+    class Opt:
+        def __init__(self, specs):
+            descs = [_one(shape, tier=tier, weight=0x100000000 * (k + 1), grad=0x100000000 * (k + 1) + 0x80000000)
+                     for k, (shape, tier) in enumerate(specs)]
+            self.h = S.skew_create(descs, S.hparams(eps=eps))
+            self.info, self.route = (lambda k: S.skew_tensor_info(self.h, k)), (lambda k: S.skew_tensor_route(self.h, k))
+
+    bm = bench.byte_model(Opt([((12000, 1408), S.TIER_EXPERT), ((700, 64), S.TIER_BACKBONE)]), 2)["kernels"]
+    rows = eps < 1e-12
+    assert [k for k, v in bm.items() if v] == (["k_rowsq", "k_finalize", "k_fallback", "k_apply_rows"] if rows else
+                                                ["k_sumsq", "k_finalize", "k_rms", "k_apply"])
+    n, e, r = 12000 * 1408, 700 * 64, 8 * (12000 + 1408)
+    assert bm["k_rowsq" if rows else "k_sumsq"] == 2 * n + 2 * e + (r if rows else 0)
+    assert bm["k_apply_rows" if rows else "k_apply"] == 6 * n + 8 * e
+    bm = bench.byte_model(Opt([((64, 128), S.TIER_EXPERT), ((64,), S.TIER_BACKBONE)]), 2)
+    assert [k for k, v in bm["kernels"].items() if v] == ["k_apply_rows"]
+    assert bm["kernels"]["k_apply_rows"] == bm["step_min"] == 6 * (8192 + 64) + 8 * 64 + 8 * 64 + 8 * (64 + 128)
