@@ -28,10 +28,13 @@ def _set(seed, shapes):
     return ps, S.SkewAdam(ps, S.hparams(eps=1e-30))
 
 
-@pytest.mark.parametrize("shapes", [SHAPES, SHAPES[2:]], ids=["rows", "light"])
-def test_captured_step_equals_direct(shapes):
+# row tiles with strip and flat tiles beside them; strip and flat tiles alone; the single launch of small tensors
+@pytest.mark.parametrize("shapes,launches", [(SHAPES, 5), (SHAPES[2:] + [((9000, 64), 0), ((8000, 72), 1), ((20000, 41), 0)], 5), (SHAPES[2:], 1)],
+                         ids=["rows", "light", "small"])
+def test_captured_step_equals_direct(shapes, launches):
     pa, a = _set(1, shapes)
     pb, b = _set(1, shapes)
+    assert S.skew_launches_per_step(b.h) == launches
     stream = torch.cuda.Stream()
     stream.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(stream):

@@ -3,6 +3,7 @@ phase C where a bound proves that the update is not clipped (d = 1), and by phas
 (d = 0.05). Weights, state and the scalars (sum(U^2), RMS, clip factor) against the oracle; whole and
 half phase-C tiles, last tiles without a second half, one-row matrices, stacks, zero-gradient experts."""
 import pytest
+import torch
 
 from paper_2607_19058_gb300 import workloads as WL
 
@@ -19,6 +20,16 @@ def _built():
     oracle.build()
 
 
+BILINEAR, PHASE_B, PHASE_C = 0, 1, 2
+
+
+def _sum_from(opt):
+    """Where the last step took each matrix's sum(U^2) from: the word at byte 52 of its 64-byte scalars, with which
+    the workspace starts."""
+    count = sum(max(1, opt.info(k).stack) for k in range(len(opt.params)))
+    return opt.workspace[: 64 * count].cpu().view(torch.int32).view(count, 16)[:, 13].tolist()
+
+
 @pytest.mark.parametrize("clip_d", [1.0, 0.05])
 def test_clamped_tensors(clip_d):
     import parity
@@ -31,6 +42,13 @@ def test_clamped_tensors(clip_d):
     for t in range(1, 4):
         rep = h.step(t, seed=5 * t, **({"gscale": 0.37} if t == 2 else {}))
         assert (rep.clipped > 0) == (clip_d < 1.0)
+        for src, where in zip(_sum_from(h.opt), [sp for sp in specs for _ in range(sp.shape[0] if len(sp.shape) == 3 else 1)]):
+            if t % 2 and where.expert >= 5:
+                assert src == BILINEAR, where      # no gradient
+            elif clip_d < 1.0:
+                assert src == PHASE_B, where
+            elif t > 1 or where.tier == E:
+                assert src == PHASE_C, where       # (momentum's first step is near d: either)
     h.opt.sync_status()
     h.close()
 

@@ -42,7 +42,7 @@ def _mixed_workload():
 
 
 def test_grad_scale_toy():
-    """The toy set (strip and flat tiles, zero-gradient experts) with gamma = 0.37."""
+    """The toy set (one launch; zero-gradient experts) with gamma = 0.37."""
     h = _harness(WL.toy())
     for t in range(1, 5):
         h.step(t, seed=5, gscale=0.37)
@@ -60,7 +60,7 @@ def test_grad_scale_every_path(gammas):
 
 
 def test_grad_scale_with_clamp_fallback():
-    """eps = 1e-8 (App. A): the clamp binds, so the row-path tensors take phase B."""
+    """eps = 1e-8 (App. A): the clamp binds, so the row-path tensors take phase B or C for sum(U^2)."""
     h = _harness(_mixed_workload(), hp_override=dict(eps=1e-8, lr=3e-4, weight_decay=0.05))
     for t in range(1, 4):
         h.step(t, seed=77, gscale=0.6)
@@ -133,7 +133,7 @@ def test_grad_scale_fp32_tensors():
 
 def test_grad_scale_adafactor_comparator():
     """The Adafactor comparator's annealed beta2_t with gamma: every increment (1 - beta2_t)
-    gamma^2 g^2, on the strip path (toy) and the whole-row path."""
+    gamma^2 g^2, in the single launch of small tensors (toy) and on the whole-row path."""
     for wl in (WL.toy(), _mixed_workload()):
         h = _harness(wl, hp_override=dict(policy=WL.POLICY_ADAFACTOR))
         for t, g in ((1, 0.6), (2, 0.37), (3, 1.0)):

@@ -219,8 +219,8 @@ def test_row_path_bilinear_sum():
 
 
 def test_row_path_tiny_matrices():
-    """Momentum-free row-path matrices with fewer rows than one chunk (1 to 5 rows; a stack
-    of one-row matrices): every tile is one ragged chunk."""
+    """Momentum-free matrices of the fixed widths with 1 to 5 rows, and a stack of one-row matrices (alone one
+    launch of small tensors; on row tiles, where every tile is one ragged chunk, in test_gpu_routes)."""
     E = WL.TIER_EXPERT
     specs = [WL.Spec("e1x4096", (1, 4096), E, expert=0), WL.Spec("e2x1024", (2, 1024), E, expert=1),
              WL.Spec("e3x512", (3, 512), E, expert=2), WL.Spec("e5x2048", (5, 2048), E, expert=3),
@@ -234,7 +234,8 @@ def test_row_path_tiny_matrices():
 
 def test_row_path_clamp_falls_back_to_phase_b():
     """eps = 1e-8 (App. A): the clamp binds at step 1, so the finalize queues the
-    tensors for phase B and sum(U^2) is taken element by element."""
+    tensors for phase B, or phase C where the clip factor is provably 1, and sum(U^2) is taken element by
+    element (which of the two: test_gpu_clamp_routes)."""
     h = _harness(_row_path_workload(), hp_override=dict(eps=1e-8, lr=3e-4, weight_decay=0.05))
     for t in range(1, 4):
         h.step(t, seed=77)
@@ -285,7 +286,8 @@ def test_stacked_appb_experts_full_size_subset():
 
 def test_adafactor_comparator():
     """The Adafactor comparator (every matrix factored, no momentum, beta2_t = 1 - t^-0.8, no
-    bias correction) on the toy set (strip path, exact vectors, zero-gradient experts at t = 1)
+    bias correction) on the toy set (one launch, exact vectors, zero-gradient experts at t = 1; the strip
+    path: test_gpu_routes)
     and on the whole-row path, over steps whose decay changes every step."""
     h = _harness(WL.toy(), hp_override=dict(policy=WL.POLICY_ADAFACTOR))
     assert all(h.opt.info(k).momentum == 0 for k in range(len(h.wl.specs)))

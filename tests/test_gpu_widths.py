@@ -47,6 +47,7 @@ def test_any_width_rows(shapes, hp):
     5 to 7 have zero gradients on odd steps."""
     import parity
     h = parity.Harness(_workload(shapes, **{k: v for k, v in hp.items() if k == "eps"}), hp_override=hp)
+    assert all(h.opt.route(k) == S.ROUTE_ROWS for k in range(len(h.wl.specs)))
     for t in range(1, 4):
         h.step(t, seed=17 * t, **({"gscale": 0.37} if t == 2 else {}))
     h.opt.sync_status()

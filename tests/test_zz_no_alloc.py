@@ -24,8 +24,7 @@ pytestmark = pytest.mark.gpu
 
 # (8192, 4096) expert: a momentum-free matrix on the whole-row path; (50304, 4096)
 # backbone: the paper's embedding, the largest tensor the fixed scratch is sized for;
-# (4096, 4096) and (3001, 2048) experts: matrices that skew_step runs in its pipelined
-# launch, which the no-alloc entry point must match with the separate launches.
+# (4096, 4096) and (3001, 2048) experts: row tiles cut by the work left, as skew_step cuts them.
 SHAPES = [((300, 1000), S.TIER_EXPERT), ((517, 136), S.TIER_BACKBONE), ((4096, 127), S.TIER_ROUTER),
           ((100003,), S.TIER_BACKBONE), ((8192, 4096), S.TIER_EXPERT), ((50304, 4096), S.TIER_BACKBONE),
           ((4096, 4096), S.TIER_EXPERT), ((3001, 2048), S.TIER_EXPERT)]
