@@ -1556,13 +1556,14 @@ __device__ Acc2 rms_full_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
     Acc2 acc;
     int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
     for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
-        float g[kFlatAhead][8], v[kFlatAhead][8], mm[kFlatAhead][8];
+        Raw8 raw[kFlatAhead];
+        float v[kFlatAhead][8], mm[kFlatAhead][8];
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
             const int64_t e = e0 + h * 8 * kThreads;
             if (k + h < T.fvpt && e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                load8_elem(T.g, T.f32, T.wal, e, valid, g[h], pol);
+                load8_raw(T.g, T.f32, T.wal, e, valid, raw[h], pol);
                 load_f8(T.v + e, T.sal, valid, v[h]);
                 if (T.momentum) load_f8(T.M + e, T.sal, valid, mm[h]);
             }
@@ -1572,17 +1573,18 @@ __device__ Acc2 rms_full_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
             const int64_t e = e0 + h * 8 * kThreads;
             if (k + h < T.fvpt && e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                float u[8];
+                float g[8], u[8];
+                values8(raw[h], T.f32, g);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) v[h][c] = fmaf(A.b2, v[h][c], gsc.c2 * (g[h][c] * g[h][c]));
+                for (int c = 0; c < 8; ++c) v[h][c] = fmaf(A.b2, v[h][c], gsc.c2 * (g[c] * g[c]));
                 store_f8(T.v + e, T.sal, valid, v[h]);
                 if (T.momentum) {
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) g[h][c] = fmaf(A.b1, mm[h][c], gsc.c1 * g[h][c]);
-                    store_f8(T.M + e, T.sal, valid, g[h]);
+                    for (int c = 0; c < 8; ++c) g[c] = fmaf(A.b1, mm[h][c], gsc.c1 * g[c]);
+                    store_f8(T.M + e, T.sal, valid, g);
                 }
 #pragma unroll
-                for (int c = 0; c < 8; ++c) u[c] = c < valid ? g[h][c] * fminf(__frsqrt_rn(v[h][c]), A.ce) : 0.f;
+                for (int c = 0; c < 8; ++c) u[c] = c < valid ? g[c] * fminf(__frsqrt_rn(v[h][c]), A.ce) : 0.f;
                 acc.add(sumsq8(u));
             }
         }
@@ -1819,18 +1821,19 @@ __device__ void apply_full_tile(const StepArgs &A, const TensorDev &T, const Ten
     const int64_t numel = T.numel;
     int64_t e0 = 8 * (int64_t(tile) * kThreads * T.fvpt + threadIdx.x);
     for (uint32_t k = 0; k < T.fvpt && e0 < numel; k += kFlatAhead) {
-        float y[kFlatAhead][8], v[kFlatAhead][8], w[kFlatAhead][8];
+        Raw8 g[kFlatAhead], w[kFlatAhead];
+        float mm[kFlatAhead][8], v[kFlatAhead][8];
 #pragma unroll
         for (uint32_t h = 0; h < kFlatAhead; ++h) {
             const int64_t e = e0 + h * 8 * kThreads;
             if (k + h < T.fvpt && e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
                 if (T.momentum)
-                    load_f8(T.M + e, T.sal, valid, y[h]);
+                    load_f8(T.M + e, T.sal, valid, mm[h]);
                 else
-                    load8_elem(T.g, T.f32, T.wal, e, valid, y[h], pol);
+                    load8_raw(T.g, T.f32, T.wal, e, valid, g[h], pol);
                 load_f8(T.v + e, T.sal, valid, v[h]);
-                load8_elem(T.w, T.f32, T.wal, e, valid, w[h], pol);
+                load8_raw(T.w, T.f32, T.wal, e, valid, w[h], pol);
             }
         }
 #pragma unroll
@@ -1838,10 +1841,16 @@ __device__ void apply_full_tile(const StepArgs &A, const TensorDev &T, const Ten
             const int64_t e = e0 + h * 8 * kThreads;
             if (k + h < T.fvpt && e < numel) {
                 const int valid = (int)min(int64_t(8), numel - e);
-                float x[8];
+                float y[8], wv[8], x[8];
+                if (T.momentum) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    x[c] = fmaf(-coefC, y[h][c] * fminf(__frsqrt_rn(v[h][c]), A.ce), w[h][c] * wdf);
+                    for (int c = 0; c < 8; ++c) y[c] = mm[h][c];
+                } else {
+                    values8(g[h], T.f32, y);
+                }
+                values8(w[h], T.f32, wv);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) x[c] = fmaf(-coefC, y[c] * fminf(__frsqrt_rn(v[h][c]), A.ce), wv[c] * wdf);
                 store8_elem(T, d, e, valid, x, pol);
             }
         }
