@@ -150,11 +150,26 @@ __device__ __forceinline__ void values8(const Raw8 &r, bool f32, float (&o)[8]) 
     }
 }
 
+// The same for one vector at a time, as values.
 __device__ __forceinline__ void load8_elem(const uint16_t *base, bool f32, bool wide, int64_t e0, int valid,
                                            float (&o)[8], const Pol &pol) {
-    Raw8 r;
-    load8_raw(base, f32, wide, e0, valid, r, pol);
-    values8(r, f32, o);
+    if (f32) {
+        const float *p = reinterpret_cast<const float *>(base) + e0;
+        if (wide && valid == 8) {
+            const uint4 a = ld16_hint(p, pol.drop), b = ld16_hint(p + 4, pol.drop);
+            const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] = __uint_as_float(w[c]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) o[c] = c < valid ? p[c] : 0.f;
+        }
+    } else if (wide && valid == 8) {
+        unpack_bf8(ld16_hint(base + e0, pol.drop), o);
+    } else {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) o[c] = c < valid ? bf16_to_f32(base[e0 + c]) : 0.f;
+    }
 }
 
 // Eight fp32 state values (`wide`: on a 16-byte boundary), read through L2 (an earlier launch of
