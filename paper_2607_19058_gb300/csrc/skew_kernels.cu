@@ -712,7 +712,6 @@ struct RowSmem {
     uint64_t full[kRowStages];                   // one mbarrier per ring slot
     float part[kThreads / 32][8];             // per-warp row partial sums of the chunk
     float inv[32];                               // 1 / R_i of the chunk's rows (0: no contribution)
-    int fail;
 };
 
 // Rows `i` of chunk `c` of row tile `tile`: [i0, i0 + rows).
@@ -823,7 +822,6 @@ __device__ void rowsq_tile(const StepArgs &A, const TensorDev &T, TensorScal &S,
     if (threadIdx.x == 0) {
         for (int st = 0; st < kRowStages; ++st) mbar_init(&sm.full[st], 1);
         fence_mbar_init();
-        sm.fail = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0)
@@ -2097,7 +2095,6 @@ struct MomRowSmem {
     uint64_t full[kMomStages];
     float part[kThreads / 32][8];
     float inv[32];
-    int fail;
 };
 
 // Issues the bulk copies of chunk c of the tile whose first row is r0 (rows of x = G in phase A,
@@ -2128,7 +2125,6 @@ __device__ void rowsq_mom_tile(const StepArgs &A, const TensorDev &T, TensorScal
     if (threadIdx.x == 0) {
         for (int st = 0; st < kMomStages; ++st) mbar_init(&sm.full[st], 1);
         fence_mbar_init();
-        sm.fail = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0)

@@ -235,7 +235,6 @@ extern "C" int skew_step_tensor_noalloc(void *weight, const void *grad, int32_t 
         nFB = (uint32_t)(2 * (sms > 0 ? sms : 1));
     }
 
-    cudaStream_t s = (cudaStream_t)stream;
     const SmallPlan sp = plan_small(1, fact && vec, [&](auto &&f) { return f(fact ? n : numel, fact ? m : 1); });
     if (sp.ctas) {  // one launch, which needs of the scratch only the scalars
         if (!fact) {
