@@ -4,7 +4,8 @@
 // order, each over an item table of (tensor, tile) pairs; a step with row-path tensors
 // takes k_rowsq (and k_rowsq_wide), k_finalize, k_fallback and k_apply_rows, which also
 // run its strip and flat tiles while these are few; any other takes k_sumsq, k_finalize,
-// k_rms and k_apply, and a step of small tensors k_small alone:
+// k_rms and k_apply, each after k_reset (an ordinary launch, which clears the per-step scalars), and a step
+// of small tensors k_small alone:
 //   k_sumsq      phase A, strip tiles: per-row and per-column sums of g^2 of a
 //                factored matrix (Eq. 1), column partials per row tile (no atomics);
 //   k_rowsq      phase A, whole-row tiles of factored matrices 128 to 4096 wide
@@ -1367,8 +1368,8 @@ __device__ Acc2 rms_fact_tile(const StepArgs &A, const TensorDev &T, uint32_t ti
 // multiple of 8, unaligned pointers): flat tiles of 8 consecutive elements per thread and round, which
 // are loaded wide wherever the arrays start on a 16-byte boundary and draw one Philox block, whatever
 // the width. Bound by latency; the row-vectors' layout had 8 narrow loads per row, a Philox block per
-// element and 32 rows per thread one after another (k_apply, 42829 x 58 bf16: 103 -> 17 us; 3467 x
-// 1072 fp32 with momentum: 45 -> 22; 24 ragged tensors of 13M elements in all: a step 215 -> 161).
+// element and 32 rows per thread one after another (k_apply, 42829 x 58 bf16: 103 -> 18 us; 3467 x
+// 1072 fp32 with momentum: 45 -> 20; 24 ragged tensors of 13M elements in all: a step 215 -> 102).
 // ---------------------------------------------------------------------------
 // The scales of a tile (a_i of its rows, b_j of its columns) stay in shared memory, and a round is one
 // vector per thread; FlatTile says which, FlatScales what its elements are scaled by. The b_j of columns 8
@@ -2951,8 +2952,8 @@ __device__ void apply_flat_tile(const StepArgs &A, const TensorDev &T, TensorSca
 
 // Phase B of a queued row-path tensor: sum(U^2) over the rows of a phase-C tile, from a ring of G (or the
 // new M, which phase A stored) alone. Chunks run on from tile to tile (`turn` counts them), so that the
-// barriers keep their phases. Bound by HBM: with all of 65M parameters in 768 x 488 experts queued a step
-// takes 185 us, 205 when the queue ran on strip tiles (118M in 816 x 408 experts: 275 and 297).
+// barriers keep their phases. With all of 65M parameters in 173 matrices of 768 x 488 queued a step takes 188 us,
+// 119 with none (118M in 354 of 816 x 408: 304 and 191).
 template <bool MOM>
 struct SumRing {
     static constexpr uint32_t kChunk = MOM ? 512 : 1024, kSlot16 = 1024, kStages = 4;  // vectors; 16 KB slots
@@ -3366,7 +3367,7 @@ __global__ void __launch_bounds__(kThreads, SKEW_MINB_SUMSQ)
 
 // A step with row-path tensors runs its strip and flat tiles in the row path's launches, ahead of
 // the row tiles, unless there are many of them (kRideElems): phase B of the flat tiles needs nothing from phase A or the finalize, so it comes
-// with phase A. Such a step has four launches instead of seven, and the light tiles' latency (a
+// with phase A. Such a step has four launches (after k_reset) instead of seven, and the light tiles' latency (a
 // launch of its own took 12 to 25 us each for phases A, B and C) hides behind the row tiles.
 
 // Row path, phase A: one row tile per CTA (dynamic shared memory: RowSmem), and before them the

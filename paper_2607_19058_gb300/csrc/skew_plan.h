@@ -178,23 +178,27 @@ inline uint32_t row_tile_chunks(int64_t own, int64_t rest, int64_t waves, int64_
     return (uint32_t)t;
 }
 
-// Below this many bytes of G in all row-path matrices, those that only kRowAny serves take strip tiles (beside
-// larger row tiles a 4095 x 1000 matrix of 8 MB costs 43 us more on strip tiles): their second read
-// of G (much of it from L2) costs a step no more than k_fallback and the row tiles' ramps: 10M parameters
-// of a 256-wide model, most of them its embedding's, 69 us on strip tiles and 89 on row tiles (21 MB of G),
-// 2048 x 1408 alone 28 and 32; 20M of another 256-wide model 96 and 70 (41 MB), 29M of a 432-wide one 151
-// and 113.
+// Below this many bytes of G in all row-path matrices, those that only kRowAny serves take strip tiles: beside
+// larger row tiles a 4095 x 1000 matrix of 8 MB costs 43 us more there, but alone the second read of G (much of it
+// from L2) costs a step little. One matrix, strip and row tiles: 2048 x 1408 27 and 32 us, 768 columns of 16 MiB of G
+// 37 and 40, 32 MiB 59 and 51, 52 MiB 91 and 73; with momentum 16 MiB 52 and 46, 32 MiB 79 and 69. Models of 256
+// columns, most of it the embedding's: 20 MiB 67 and 57, 42 MiB 104 and 78; all matrices queued for phase B (below):
+// 68 and 83, 107 and 116.
 constexpr int64_t kAnyGroupBytes = 32 << 20;
 // An eps that the clamp may bind at (kBindEps: a row's or column's mean g^2 of 1e-12 is g = 1e-6) can queue
-// matrices for k_fallback, which reads them again, M included; a step of these widths alone then gains from
-// row tiles from twice that on. 256 wide, eps = 1e-8, clipped gradients, half or more of it with momentum:
-// 37 MiB of G 113 us on strip tiles and 121 to 139 on row tiles, 43 MiB 119 and 131, 65 MiB 165 and 155,
-// 110 MiB 241 and 229; eps = 1e-30, 37 MiB: 112 and 90.
+// matrices for k_fallback, which reads them again, M included; a step of these widths alone then takes row tiles
+// from twice that on. What binds is eps against g^2, which no plan knows: 768 columns, strip and row tiles, in MiB of G,
+// where all is queued 32: 60 and 69 us, 52: 95 and 99, 68: 104 and 112, 100: 150 and 149, 180: 231 and 216 (momentum 82
+// and 88, 132 and 158, 142 and 176, 208 and 239, 333 and 372); where the clamp does not bind 59 and 51, 91 and 73, 100
+// and 80, 146 and 102, 225 and 158 (79 and 69, 129 and 118, 141 and 133, 206 and 177, 329 and 291). Where it binds in
+// the first steps only, or the clip factor is provably 1, the latter holds for most of a run.
 constexpr int64_t kAnyBindBytes = 64 << 20;
 constexpr float kBindEps = 1e-12f;
 // Beside row tiles of other widths, those above kAnyNarrow need a launch of their own, and below this
 // many bytes of G the strip tiles, which ride along, are faster (260M parameters, 23 MB of them 5632
-// wide: 379 us against 407; 1.16B parameters of 4864 and 7128 columns: 2314 against 1653).
+// wide: 379 us against 407; 1.16B parameters of 4864 and 7128 columns: 2314 against 1653). 5632 columns alone, as
+// above: not bound 32 MiB 58 and 57, 68 MiB 104 and 93 (momentum 79 and 78, 143 and 140), queued 60 and 76, 108 and 139
+// (82 and 100, 145 and 196); with momentum 7168 columns and more gain nothing to 100 MiB (8192: 80 and 91 at 32 MiB).
 constexpr int64_t kWideGroupBytes = 64 << 20;
 
 // Which widths that only kRowAny serves take row tiles in a step: `narrow` and `wide` bytes of G of its
