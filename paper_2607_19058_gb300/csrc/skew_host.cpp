@@ -110,7 +110,7 @@ static bool wg_aligned(const TPlan &p) { return (((uintptr_t)p.w | (uintptr_t)p.
 static bool vectors(const TPlan &p) { return row_vectors(p.f32 != 0, wg_aligned(p), p.moff < 0 || p.moff % 4 == 0, p.m); }
 
 // Tile geometry (plan_geometry): strip tiles of (tile_rows rows) x (8*LC
-// columns) or flat tiles of kFlatTileElems elements, and for the row path whole-row tiles.
+// columns) or flat tiles, and for the row path whole-row tiles.
 static void geometry(TPlan &p, bool row_aligned, bool ride, int64_t strip, int64_t rest, int64_t rest_c) {
     const bool vec = vectors(p);
     const TileGeom g = plan_geometry(p.kind, p.momentum, row_aligned, vec, ride, strip, p.n, p.m, p.numel, rest, rest_c);

@@ -73,8 +73,8 @@ constexpr int kMomChunks = 64;
 // (rowsq_gen_tile, apply_flat_tile): rows per thread and phase-A chunk at NV vectors per
 // thread and row, and the floats of shared memory that hold phase C's scales.
 // Below 128 columns a row fills less than half a warp (20M parameters of a 256-wide model with experts
-// of 248 columns: strip tiles below 256 91 us, below 128 72 us), and above 4096 the column sums of a row do
-// not fit the registers of two 256-thread CTAs per SM: both stay on the strip tiles. Against
+// of 248 columns: strip tiles below 256 91 us, below 128 72 us), and above 8192 the column sums of a row do
+// not fit the registers of one CTA: both stay on the strip tiles. (Above 4096, 16-warp CTAs, one per SM.) Against
 // the strip tiles (three reads of G): 930M parameters in 3072 x 1536 experts 1872 -> 1259 us.
 enum RowPath : uint32_t { kRowNone = 0, kRowFixed = 1, kRowAny = 2 };
 constexpr int64_t kAnyMin = 128, kAnyNarrow = 4096, kAnyMax = 8192;
